@@ -1,0 +1,255 @@
+"""The work a user of this library has it do, as cases that can be timed.
+
+A case of kind "gnn" is one inference pass of a whole model over a whole graph through the public calls: for every
+layer taurus_layer_begin, every chunk pushed in order (GAT: its three passes), taurus_layer_end.  The context (graph,
+weights, pool), the input rows and the output matrices are what the program holds before the call.  Kind "reorder" is
+the one-time preprocessing of a graph: Algorithm 1, relabelling of the topology, permutation of the feature rows.
+
+Graphs are made on the GPU from the seed: power-law out-degrees (at least one edge each), destinations half local (a band
+around the source, as in a graph whose labelling has been ordered) and half power-law hubs, or uniform; optionally with
+every edge's reverse.  Input rows are N(0, 1), weights Xavier-uniform, as in this repository's workload table.
+"""
+import math
+
+import torch
+
+import paper_2607_17374_b200 as tb
+
+MODES = {"sage": tb.SAGE_MEAN, "gcn": tb.GCN_SYM, "gin": tb.GIN_SUM, "gat": tb.GAT}
+
+
+def _gnn(name, V, E, dims, mode="sage", chunk=65536, graph="banded", symmetric=False, pool=1.0, hubs=0.0, fanout="", bf16=False,
+         heads=1, output="dense", host=False, push=0):
+    """pool, hubs: share of V.  fanout: per layer, "" = exact.  output: "dense" (finished rows go to a matrix), "drain" (drained
+    into it after every chunk), "runs" (sorted runs that the next layer reads back).  host: input and result in pinned host
+    memory.  push: sources per push where it is not the chunk size the context was made for."""
+    c = dict(kind="gnn", V=V, E=E, dims=dims, mode=mode, chunk=chunk, graph=graph, symmetric=symmetric, pool=pool, hubs=hubs,
+             fanout=fanout, bf16=bf16, heads=heads, output=output, host=host, push=push)
+    if name:
+        c["name"] = name
+    return c
+
+
+def listed():
+    return [
+        # one small query graph, one chunk: the latency of a call sequence
+        _gnn("single_chunk", 700, 5_600, "47-33", chunk=1024, graph="uniform"),
+        # the "tiny" workload of the table: 10 small chunks a layer, launch-bound
+        _gnn("tiny", 10_000, 100_000, "64-64-16", chunk=1024, graph="uniform"),
+        # a pass whose rows the program takes after every chunk, pushes that are not cells of the chunk grid, odd widths
+        _gnn("gin_drain_ragged", 120_001, 1_700_003, "37-130-47", mode="gin", chunk=16384, output="drain", push=10_007),
+        # the "mid" workload at full size: exact inference, the accumulator pool holds all of V
+        _gnn("mid", 2_450_000, 124_000_000, "100-256-256-47", symmetric=True),
+        # the same kind of graph at the size of one machine's share, several attention heads
+        _gnn("gat_heads", 400_000, 20_000_000, "100-128-128", mode="gat", symmetric=True, heads=4),
+        # the "large" shape: bounded pool, hubs in their own store, evicted rows in pinned host memory
+        _gnn("large_evict", 600_000, 8_640_000, "128-256-256", chunk=4096, pool=0.27, hubs=0.001),
+        # the "sampled" shape: fanout-sampled layers over the same kind of graph, the pool holds the active set
+        _gnn("sampled", 1_500_000, 21_600_000, "128-256-256-256", fanout="15-10-5", hubs=0.001),
+        # the "stress" shape: wide input rows, GCN, bf16 projection, a pool that just covers the active set
+        _gnn("stress_bf16", 900_000, 13_400_000, "512-256-256", mode="gcn", chunk=16384, pool=0.8, hubs=0.001, bf16=True),
+        # layers chained through sorted runs, no dense V x H matrix between them
+        _gnn("runs_chain", 500_000, 12_500_000, "128-128-64", output="runs"),
+        # rows streamed from pinned host memory and the result written back there
+        _gnn("host_stream", 500_000, 12_500_000, "128-64-32", mode="gcn", host=True),
+        # preprocessing of a graph: five iterations, relabel, permute the rows
+        dict(name="reorder", kind="reorder", V=400_000, E=5_800_000, width=128, iterations=5),
+    ]
+
+
+def _log(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def draw(rng):
+    if rng.random() < 0.1:
+        V = _log(rng, 20_000, 500_000)
+        return dict(kind="reorder", V=V, E=int(V * rng.uniform(8, 20)), width=rng.choice([64, 100, 128]), iterations=rng.randint(3, 5))
+    mode = rng.choice(["sage", "sage", "sage", "gcn", "gcn", "gin", "gat"])
+    layers = rng.choice([1, 2, 2, 3])
+    widths = [rng.choice([16, 33, 47, 64, 100, 128, 128, 256, 256, 512])]
+    heads = rng.choice([1, 2, 4]) if mode == "gat" else 1
+    for l in range(layers):
+        widths.append(rng.choice([16, 47, 64, 100, 128, 130, 256, 256]) if mode != "gat" else rng.choice([32, 64, 128, 256]))
+    bounded = rng.random() < 0.25
+    V = _log(rng, 3_000, 250_000) if bounded else _log(rng, 500, 1_000_000)
+    degree = rng.uniform(8, 16) if bounded else rng.uniform(8, 50)
+    E = int(min(V * degree, 30_000_000)) // 2 * 2
+    chunk = max(64, int(V * rng.uniform(0.004, 0.01))) if bounded else min(65536, max(256, _log(rng, V / 40, V)))
+    output = "dense" if bounded else rng.choice(["dense", "dense", "dense", "drain", "runs"])
+    return _gnn("", V, E, "-".join(map(str, widths)), mode=mode, chunk=chunk, graph=rng.choice(["banded", "banded", "uniform"]),
+                symmetric=rng.random() < 0.4, pool=rng.uniform(0.5, 0.8) if bounded else 1.0, hubs=rng.choice([0.0, 0.001]),
+                fanout="-".join(rng.choice(["0", "5", "10", "15"]) for _ in range(layers)) if rng.random() < 0.3 else "",
+                bf16=mode != "gat" and rng.random() < 0.2, heads=heads, output=output, host=rng.random() < 0.2,
+                push=int(chunk * rng.uniform(0.3, 0.95)) if not bounded and output == "drain" and rng.random() < 0.5 else 0)
+
+
+# ---------------------------------------------------------------------------------------------------------------- inputs
+
+def _graph(V, E, shape, symmetric, band, gen, dev):
+    """(row_ptr int64 [V+1], col int32 [E], in_degree int32 [V]), exactly E edges."""
+    n = E // 2 if symmetric else E
+    # out-degrees: one edge each, the rest by power-law weights
+    base = 1 if n >= V else 0
+    w = (1.0 - torch.rand(V, generator=gen, device=dev, dtype=torch.float64)).pow(-1.0 / 1.1).clamp_(max=20_000.0 * max(1e-3, (V / 2.45e6)) ** 0.5)
+    cut = (torch.cumsum(w, 0) * ((n - base * V) / float(w.sum()))).round_().to(torch.int64)
+    cut[-1] = n - base * V
+    degree = torch.diff(cut, prepend=cut.new_zeros(1)) + base
+    src = torch.repeat_interleave(torch.arange(V, device=dev, dtype=torch.int32), degree, output_size=n)
+    del w, cut
+    if shape == "uniform":
+        dst = torch.randint(0, V, (n,), generator=gen, device=dev, dtype=torch.int32)
+    else:
+        x = torch.rand(n, generator=gen, device=dev, dtype=torch.float32)
+        coin = torch.randint(0, 4, (n,), generator=gen, device=dev, dtype=torch.int8)
+        step = (torch.log1p(-x) * -float(band)).to(torch.int64)
+        local = torch.remainder(src + torch.where(coin == 0, step, -step), V).to(torch.int32)
+        s, r0 = 1.0 - 1.0 / 1.1, max(1.0, 1e-4 * V)   # P(rank) ~ (rank + r0)^-(1/1.1)
+        rank = ((r0 ** s + x.double() * ((V + r0) ** s - r0 ** s)).pow(1.0 / s) - r0).to(torch.int64).clamp_(0, V - 1)
+        a = int(V * 0.6180339887) | 1
+        while math.gcd(a, V) != 1:
+            a += 2
+        dst = torch.where(coin < 2, local, torch.remainder(rank * a + 13, V).to(torch.int32))
+        del x, coin, step, local, rank
+    if symmetric:
+        src, dst = torch.cat([src, dst]), torch.cat([dst, src])
+        src, order = torch.sort(src, stable=True)
+        dst = dst[order]
+        del order
+        degree = torch.bincount(src, minlength=V)
+    row_ptr = torch.zeros(V + 1, dtype=torch.int64, device=dev)
+    row_ptr[1:] = torch.cumsum(degree, 0)
+    return row_ptr, dst.contiguous(), torch.bincount(dst, minlength=V).to(torch.int32)
+
+
+def _xavier(rows, cols, gen):
+    bound = math.sqrt(6.0 / (rows + cols))
+    return (torch.rand(rows, cols, generator=gen) * 2 - 1).mul_(bound)
+
+
+def prepare(case, seed):
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(seed)
+    cpu = torch.Generator()
+    cpu.manual_seed(seed)
+    V, E = case["V"], case["E"]
+    if case["kind"] == "reorder":
+        row_ptr, col, _ = _graph(V, E, "banded", False, V / 40, gen, dev)
+        shuffle = torch.randperm(V, generator=gen, device=dev)   # a labelling that has not been ordered yet
+        degree = torch.diff(row_ptr)
+        degree_new = torch.empty_like(degree)
+        degree_new[shuffle] = degree
+        src = shuffle[torch.repeat_interleave(torch.arange(V, device=dev), degree, output_size=E)]
+        col = shuffle[col.long()].to(torch.int32)[torch.sort(src, stable=True)[1]]
+        row_ptr[1:] = torch.cumsum(degree_new, 0)
+        rows = torch.randn(V, case["width"], generator=gen, device=dev)
+        return dict(case=case, row_ptr=row_ptr.cpu().numpy(), col=col.cpu().numpy(), rows=rows, out=torch.empty_like(rows),
+                    rank=torch.empty(V, dtype=torch.int32, device=dev))
+    row_ptr, col, din = _graph(V, E, case["graph"], case["symmetric"], min(4 * case["chunk"], max(V // 8, 1)), gen, dev)
+    dims = [int(d) for d in case["dims"].split("-")]
+    L, mode = len(dims) - 1, MODES[case["mode"]]
+    W = [_xavier(dims[l], dims[l + 1], cpu) for l in range(L)]
+    Ws = [_xavier(dims[l], dims[l + 1], cpu) if mode == tb.SAGE_MEAN else W[l] for l in range(L)]
+    bias = [_xavier(1, dims[l + 1], cpu)[0].contiguous() for l in range(L)]
+    att = [[_xavier(dims[l + 1], 1, cpu)[:, 0].contiguous() for l in range(L)] for _ in range(2)] if mode == tb.GAT else [None, None]
+    fanout = [int(f) for f in case["fanout"].split("-")] if case["fanout"] else None
+    hubs = int(V * case["hubs"])
+    pool = V if case["pool"] >= 1.0 else max(1, int(V * case["pool"]))
+    bounded = pool < V - hubs
+    half_rows = case["output"] == "runs" or (case["host"] and case["output"] == "dense")
+    ctx = tb.Context(V, E, row_ptr, col, din, mode, dims, W, Ws, bias, [1] * (L - 1) + [0], case["chunk"], pool, hubs, fanout, 1 + seed,
+                     V - hubs if bounded else 0, 2 * V if half_rows else V, tb.GEMM_BF16 if case["bf16"] else tb.GEMM_FP32, 0, 0, 0.1,
+                     att[0], att[1], 0.2, case["heads"])
+    x = torch.randn(V, dims[0], generator=gen, device=dev)
+    push = case["push"] or case["chunk"]
+    s = dict(case=case, ctx=ctx, dims=dims, x=x.cpu().pin_memory() if case["host"] else x, chunks=[(b, min(b + push, V)) for b in range(0, V, push)],
+             between=[torch.empty(V * max(dims[1:]), device=dev) for _ in range(2 if L > 2 else L - 1)] if case["output"] != "runs" else None,
+             out=torch.empty(V, dims[-1]).pin_memory() if case["host"] and case["output"] != "runs" else torch.empty(V, dims[-1], device=dev))
+    if mode == tb.GAT:
+        s["hprime"] = torch.empty(V * max(dims[1:]), device=dev)
+    if case["output"] == "runs":
+        s["runs"] = [tb.Runs(V, dims[l + 1], 16, max(64, V // 64), store_rows=V, max_append_rows=V, max_chunk_rows=case["chunk"],
+                             store_kind=tb.RUNS_DEVICE) for l in range(L)]
+    return s
+
+
+# ---------------------------------------------------------------------------------------------------------------- one pass
+
+def _reorder(s):
+    c = s["case"]
+    rank, positions, J, span = tb.reorder(c["V"], c["E"], s["row_ptr"], s["col"], None, c["iterations"])
+    row_ptr, col, din = tb.relabel_csr(c["V"], c["E"], s["row_ptr"], s["col"], rank)
+    s["rank"].copy_(torch.from_numpy(rank))
+    tb.permute_rows(c["V"], c["width"], s["rows"], c["width"], s["rank"], s["out"], c["width"], torch.cuda.current_stream())
+    return dict(rank=rank, positions=positions, dispersion=J, span=span.astype("float64"), row_ptr=row_ptr, col=col, in_degree=din, rows=s["out"])
+
+
+def run(s):
+    if s["case"]["kind"] == "reorder":
+        return _reorder(s)
+    ctx, dims, chunks, output = s["ctx"], s["dims"], s["chunks"], s["case"]["output"]
+    V, L, gat, stream = s["case"]["V"], len(s["dims"]) - 1, s["case"]["mode"] == "gat", torch.cuda.current_stream()
+    feat, counts = s["x"], []
+    for l in range(L):
+        d = dims[l + 1]
+        out = s["out"] if l == L - 1 else s["between"][l % len(s["between"])][:V * d].view(V, d) if output != "runs" else None
+        from_runs = output == "runs" and l > 0
+        ctx.layer_begin(l, stream)
+        src = feat
+        if gat:
+            src = s["hprime"][:V * d].view(V, d)
+            for b, e in chunks:
+                if from_runs:
+                    ctx.gat_project_chunk_from_runs(b, e, s["runs"][l - 1], src[b:e], d, stream)
+                else:
+                    ctx.gat_project_chunk(b, e, feat[b:e], src[b:e], d, stream)
+            ctx.gat_attention(stream)
+        if output == "runs":
+            s["runs"][l].reset()
+            ctx.layer_set_run_output(s["runs"][l])
+        elif output == "dense":
+            ctx.layer_set_dense_output(out, d)
+        for b, e in chunks:
+            if from_runs and not gat:
+                ctx.push_chunk_from_runs(b, e, s["runs"][l - 1], stream)
+            else:
+                ctx.push_chunk(b, e, src[b:e], stream)
+            if output == "drain":
+                ctx.drain_dense(out, d, V)
+        st = ctx.layer_end()
+        counts.append([st[k] for k in ("total_messages", "completed", "evictions", "reloads", "hub_messages", "peak_occupancy", "chunks")])
+        feat = out
+    if output == "runs":   # the result in vertex order
+        for b, e in chunks:
+            s["runs"][L - 1].read_chunk(b, e, s["out"][b:e], dims[-1], stream)
+    return dict(rows=s["out"], counts=torch.tensor(counts))
+
+
+# ---------------------------------------------------------------------------------------------------------------- bounds
+
+def work(case):
+    V, E = case["V"], case["E"]
+    graph = 8 * (V + 1) + 4 * E
+    if case["kind"] == "reorder":
+        # two sweeps over the edges an iteration (means over in-lists, then over out-lists), the relabelled graph, the rows
+        return dict(bytes=case["iterations"] * 2 * (graph + 16 * V) + 2 * graph + 8 * V + 8 * V * case["width"], flops=case["iterations"] * 4 * E)
+    dims = [int(d) for d in case["dims"].split("-")]
+    fanout = [int(f) for f in case["fanout"].split("-")] if case["fanout"] else [0] * (len(dims) - 1)
+    total, flops = 0, 0
+    for l in range(len(dims) - 1):
+        K, N = dims[l], dims[l + 1]
+        messages = min(E, fanout[l] * V) if fanout[l] else E
+        total += graph + 4 * V * (K + N) + 4 * K * N * (2 if case["mode"] == "sage" else 1)
+        flops += 2 * V * K * N * (2 if case["mode"] == "sage" else 1) + (2 if case["mode"] == "gat" else 1) * messages * min(K, N)
+    return dict(bytes=total, flops=flops)
+
+
+def tolerance(case):
+    """About four times what the present path differs by from the same pass in 64 bits (measured on six of the listed cases: relative
+    0.4e-6 .. 3.2e-6 and largest 1.2e-5 in 32 bits, 1.7e-3 and 4.4e-2 with bf16 operands)."""
+    if case["kind"] == "reorder":
+        return {"rel": 1e-9, "max": 1e-7, "differ": 1e-4}   # fp64 sums; a near-tie in the positions can swap two ranks
+    if case["bf16"]:
+        return {"rel": 7e-3, "max": 2e-1}
+    return {"rel": 1.2e-5, "max": 1e-4}
