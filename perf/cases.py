@@ -127,14 +127,31 @@ def _xavier(rows, cols, gen):
     return (torch.rand(rows, cols, generator=gen) * 2 - 1).mul_(bound)
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
+    """Graph, input rows and weights of a "gnn" case."""
     dev = torch.device("cuda:0")
     gen = torch.Generator(device=dev)
     gen.manual_seed(seed)
     cpu = torch.Generator()
     cpu.manual_seed(seed)
     V, E = case["V"], case["E"]
+    row_ptr, col, din = _graph(V, E, case["graph"], case["symmetric"], min(4 * case["chunk"], max(V // 8, 1)), gen, dev)
+    dims = [int(d) for d in case["dims"].split("-")]
+    L, mode = len(dims) - 1, MODES[case["mode"]]
+    W = [_xavier(dims[l], dims[l + 1], cpu) for l in range(L)]
+    Ws = [_xavier(dims[l], dims[l + 1], cpu) if mode == tb.SAGE_MEAN else W[l] for l in range(L)]
+    bias = [_xavier(1, dims[l + 1], cpu)[0].contiguous() for l in range(L)]
+    att = [[_xavier(dims[l + 1], 1, cpu)[:, 0].contiguous() for l in range(L)] for _ in range(2)] if mode == tb.GAT else [None, None]
+    x = torch.randn(V, dims[0], generator=gen, device=dev)
+    return dict(row_ptr=row_ptr, col=col, din=din, dims=dims, W=W, Ws=Ws, bias=bias, att=att, x=x)
+
+
+def prepare(case, seed):
+    V, E = case["V"], case["E"]
     if case["kind"] == "reorder":
+        dev = torch.device("cuda:0")
+        gen = torch.Generator(device=dev)
+        gen.manual_seed(seed)
         row_ptr, col, _ = _graph(V, E, "banded", False, V / 40, gen, dev)
         shuffle = torch.randperm(V, generator=gen, device=dev)   # a labelling that has not been ordered yet
         degree = torch.diff(row_ptr)
@@ -146,22 +163,17 @@ def prepare(case, seed):
         rows = torch.randn(V, case["width"], generator=gen, device=dev)
         return dict(case=case, row_ptr=row_ptr.cpu().numpy(), col=col.cpu().numpy(), rows=rows, out=torch.empty_like(rows),
                     rank=torch.empty(V, dtype=torch.int32, device=dev))
-    row_ptr, col, din = _graph(V, E, case["graph"], case["symmetric"], min(4 * case["chunk"], max(V // 8, 1)), gen, dev)
-    dims = [int(d) for d in case["dims"].split("-")]
+    g = _inputs(case, seed)
+    dims, x, att, dev = g["dims"], g["x"], g["att"], g["x"].device
     L, mode = len(dims) - 1, MODES[case["mode"]]
-    W = [_xavier(dims[l], dims[l + 1], cpu) for l in range(L)]
-    Ws = [_xavier(dims[l], dims[l + 1], cpu) if mode == tb.SAGE_MEAN else W[l] for l in range(L)]
-    bias = [_xavier(1, dims[l + 1], cpu)[0].contiguous() for l in range(L)]
-    att = [[_xavier(dims[l + 1], 1, cpu)[:, 0].contiguous() for l in range(L)] for _ in range(2)] if mode == tb.GAT else [None, None]
     fanout = [int(f) for f in case["fanout"].split("-")] if case["fanout"] else None
     hubs = int(V * case["hubs"])
     pool = V if case["pool"] >= 1.0 else max(1, int(V * case["pool"]))
     bounded = pool < V - hubs
     half_rows = case["output"] == "runs" or (case["host"] and case["output"] == "dense")
-    ctx = tb.Context(V, E, row_ptr, col, din, mode, dims, W, Ws, bias, [1] * (L - 1) + [0], case["chunk"], pool, hubs, fanout, 1 + seed,
+    ctx = tb.Context(V, E, g["row_ptr"], g["col"], g["din"], mode, dims, g["W"], g["Ws"], g["bias"], [1] * (L - 1) + [0], case["chunk"], pool, hubs, fanout, 1 + seed,
                      V - hubs if bounded else 0, 2 * V if half_rows else V, tb.GEMM_BF16 if case["bf16"] else tb.GEMM_FP32, 0, 0, 0.1,
                      att[0], att[1], 0.2, case["heads"])
-    x = torch.randn(V, dims[0], generator=gen, device=dev)
     push = case["push"] or case["chunk"]
     s = dict(case=case, ctx=ctx, dims=dims, x=x.cpu().pin_memory() if case["host"] else x, chunks=[(b, min(b + push, V)) for b in range(0, V, push)],
              between=[torch.empty(V * max(dims[1:]), device=dev) for _ in range(2 if L > 2 else L - 1)] if case["output"] != "runs" else None,
@@ -224,6 +236,62 @@ def run(s):
         for b, e in chunks:
             s["runs"][L - 1].read_chunk(b, e, s["out"][b:e], dims[-1], stream)
     return dict(rows=s["out"], counts=torch.tensor(counts))
+
+
+# ---------------------------------------------------------------------------------------------------------------- 64 bits
+
+def exact(case, seed):
+    """The rows of a "gnn" case in 64 bits with plain torch.  A sampled layer has no such value (which in-edges it keeps is the
+    library's own choice), nor have the counters, nor the ordering (an iteration whose ties may fall either way)."""
+    if case["kind"] == "reorder" or case["fanout"]:
+        return None
+    g = _inputs(case, seed)
+    V, dims, mode, dev = case["V"], g["dims"], case["mode"], g["x"].device
+    row_ptr, col = g["row_ptr"], g["col"]
+    dout, din = torch.diff(row_ptr).double(), g["din"].double()
+    step = max(1, int(3e8 / max(dims)))
+    spans = [(b, min(b + step, case["E"])) for b in range(0, case["E"], step)]
+    source = torch.repeat_interleave(torch.arange(V, device=dev, dtype=torch.int32), torch.diff(row_ptr), output_size=case["E"])
+
+    def gather(rows, weight=None):   # sum over the in-edges (u -> v) of weight * rows[u]
+        out = torch.zeros(V, rows.shape[1], dtype=torch.float64, device=dev)
+        for b, e in spans:
+            m = rows[source[b:e].long()]
+            out.index_add_(0, col[b:e].long(), m if weight is None else m * weight(b, e))
+        return out
+
+    x = g["x"].double()
+    for l in range(len(dims) - 1):
+        W, Ws, bias = (t[l].to(dev).double() for t in (g["W"], g["Ws"], g["bias"]))
+        if mode == "sage":
+            x = (gather(x) / din.clamp(min=1)[:, None]) @ W + x @ Ws
+        elif mode == "gcn":
+            c = (1.0 / torch.sqrt(dout + 1))[:, None]
+            x = (gather(x * c) + x * c) @ W / torch.sqrt(din + 1)[:, None]
+        elif mode == "gin":
+            x = (gather(x) + 1.1 * x) @ W
+        else:
+            heads, h = case["heads"], x @ W
+            s, t = ((h * g["att"][k][l].to(dev).double()).view(V, heads, -1).sum(2) for k in range(2))
+
+            def score(b, e):
+                return torch.nn.functional.leaky_relu(s[source[b:e].long()] + t[col[b:e].long()], 0.2)
+            own = torch.nn.functional.leaky_relu(s + t, 0.2)
+            top = own.clone()
+            for b, e in spans:
+                top.scatter_reduce_(0, col[b:e].long()[:, None].expand(e - b, heads), score(b, e), "amax")
+            own = torch.exp(own - top)
+            norm, x = own.clone(), torch.zeros(V, heads, dims[l + 1] // heads, dtype=torch.float64, device=dev)
+            hh = h.view(V, heads, -1)
+            for b, e in spans:
+                w = torch.exp(score(b, e) - top[col[b:e].long()])
+                norm.index_add_(0, col[b:e].long(), w)
+                x.index_add_(0, col[b:e].long(), hh[source[b:e].long()] * w[:, :, None])
+            x = ((x + own[:, :, None] * hh) / norm[:, :, None]).reshape(V, -1)
+        x = x + bias
+        if l < len(dims) - 2:
+            x = torch.relu(x)
+    return dict(rows=x.cpu() if case["host"] and case["output"] != "runs" else x, counts=None)
 
 
 # ---------------------------------------------------------------------------------------------------------------- bounds
