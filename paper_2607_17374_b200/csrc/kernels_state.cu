@@ -165,7 +165,6 @@ static __device__ void plan_chunk(const ChunkArgs& a, DevCtl* ctl, ChunkCtl* pc)
   pc->victim_count = 0;
   for (int l = 0; l <= TAURUS_SEL_LEVELS; ++l) { pc->sel_k[l] = 0; pc->sel_min[l] = ~0ull; pc->sel_max[l] = 0ull; pc->sel_count[l] = 0; }
   pc->sel_k[0] = deficit;
-  pc->sel_final_level = deficit > 0 ? TAURUS_SEL_LEVELS + 1 : -1;
   // Slots are handed out by list index, not by per-item atomics: need-list entry i < deficit takes over the slot
   // of victim deficit - 1 - i, entry i >= deficit pops free_stack[F + deficit - 1 - i].  The counter is brought to
   // its end-of-chunk value here.
@@ -212,8 +211,8 @@ static __device__ __forceinline__ int sel_shift_of(unsigned long long lo, unsign
   return top >= TAURUS_SEL_BITS ? top - (TAURUS_SEL_BITS - 1) : 0;
 }
 
-// Block-wide minimum / maximum / count of the eligible keys a thread saw, folded into level `lvl` of the control block.
-static __device__ __forceinline__ void sel_fold(ChunkCtl* pc, int lvl, unsigned long long kmin, unsigned long long kmax, int cnt) {
+// Minimum / maximum / count of the eligible keys a thread saw, folded into level `lvl` of the control block.
+static __device__ __forceinline__ void sel_fold(ChunkCtl* pc, int lvl, unsigned long long kmin, unsigned long long kmax, int cnt, bool with_count) {
   for (int o = 16; o; o >>= 1) {
     const unsigned long long m = __shfl_xor_sync(FULL, kmin, o), M = __shfl_xor_sync(FULL, kmax, o);
     if (m < kmin) kmin = m;
@@ -223,84 +222,57 @@ static __device__ __forceinline__ void sel_fold(ChunkCtl* pc, int lvl, unsigned 
   if (lane_id() == 0 && cnt) {
     atomicMin(&pc->sel_min[lvl], kmin);
     atomicMax(&pc->sel_max[lvl], kmax);
-    atomicAdd(&pc->sel_count[lvl], cnt);
+    if (with_count) atomicAdd(&pc->sel_count[lvl], cnt);
   }
 }
 
-// The passes over the pool work on tiles of SEL_TILE slots.  A block takes the tiles of its own number, or, where row
-// transfers may run beside the kernel (dynamic_spans), the next tile of a counter: blocks on SMs that also host transfer
-// warps are several times slower, and with a fixed deal the pass would wait for them.
-#define SEL_ITEMS 8
-#define SEL_TILE (256 * SEL_ITEMS)
-static __device__ __forceinline__ long long next_tile(bool dyn, unsigned int* counter, long long it, long long* s_tile) {
-  if (!dyn) return (long long)blockIdx.x + it * gridDim.x;
-  __syncthreads();   // every thread has read the previous value
-  if (threadIdx.x == 0) *s_tile = (long long)atomicAdd(counter, 1u);
-  __syncthreads();
-  return *s_tile;
-}
+#define MR_THREADS 1024
+#define MR_ITEMS 2
+#define MR_TILE (MR_THREADS * MR_ITEMS)   // slots or candidates a block takes per step
 
-__global__ void __launch_bounds__(256) select_keys_kernel(ChunkArgs a) {   // key of every slot; range of the eligible keys
-  DevCtl* ctl = a.ctl;
-  ChunkCtl* pc = a.pc;
-  if (ctl->error || pc->sel_final_level < 0) return;
+// Key of every slot; range and number of the eligible ones.
+static __device__ __forceinline__ void select_keys(const ChunkArgs& a, ChunkCtl* pc) {
   unsigned long long kmin = ~0ull, kmax = 0ull;
   int cnt = 0;
-  __shared__ long long s_tile;
-  for (long long it = 0;; ++it) {
-    const long long base = next_tile(a.dynamic_spans != 0, &pc->tile_next[0], it, &s_tile) * SEL_TILE;
-    if (base >= a.pool_slots) break;
+  for (long long base = (long long)blockIdx.x * MR_TILE; base < a.pool_slots; base += (long long)gridDim.x * MR_TILE) {
 #pragma unroll
-  for (int j = 0; j < SEL_ITEMS; ++j) {
-    const long long s = base + j * 256 + threadIdx.x;
-    if (s >= a.pool_slots) break;
-    const int v = a.owner[s];
-    unsigned long long key = ~0ull;
-    if (v >= 0) {
-      const int t = a.slot_touch[s];   // = touch[v]
-      if (t != a.epoch) {
-        unsigned score;
-        if (a.evict_policy == TAURUS_EVICT_FIFO) score = (unsigned)a.slot_epoch[s];
-        else if (a.evict_policy == TAURUS_EVICT_LRU) score = (unsigned)t;
-        else if (a.evict_policy == TAURUS_EVICT_RANDOM) score = evict_hash(a.seed, (unsigned long long)v, (unsigned long long)(a.epoch - 1));
-        else score = (unsigned)a.slot_pend[s];   // = pend[v]: v was not touched since the copy was taken
-        key = ((unsigned long long)score << 31) | (unsigned long long)v;
-        if (key < kmin) kmin = key;
-        if (key > kmax) kmax = key;
-        cnt++;
+    for (int j = 0; j < MR_ITEMS; ++j) {
+      const long long s = base + j * MR_THREADS + threadIdx.x;
+      if (s >= a.pool_slots) break;
+      const int v = a.owner[s];
+      unsigned long long key = ~0ull;
+      if (v >= 0) {
+        const int t = a.slot_touch[s];   // = touch[v]
+        if (t != a.epoch) {
+          unsigned score;
+          if (a.evict_policy == TAURUS_EVICT_FIFO) score = (unsigned)a.slot_epoch[s];
+          else if (a.evict_policy == TAURUS_EVICT_LRU) score = (unsigned)t;
+          else if (a.evict_policy == TAURUS_EVICT_RANDOM) score = evict_hash(a.seed, (unsigned long long)v, (unsigned long long)(a.epoch - 1));
+          else score = (unsigned)a.slot_pend[s];   // = pend[v]: v was not touched since the copy was taken
+          key = ((unsigned long long)score << 31) | (unsigned long long)v;
+          if (key < kmin) kmin = key;
+          if (key > kmax) kmax = key;
+          cnt++;
+        }
       }
+      a.keys[s] = key;
     }
-    a.keys[s] = key;
   }
-  }
-  sel_fold(pc, 0, kmin, kmax, cnt);
+  sel_fold(pc, 0, kmin, kmax, cnt, true);
 }
 
 // Histogram of the level's digit over the keys entering the level.  Threads of a warp that hit the same bin add
 // once (most keys of a level often share a bin).
-__global__ void __launch_bounds__(256) select_hist_kernel(ChunkArgs a, int level) {
-  DevCtl* ctl = a.ctl;
-  ChunkCtl* pc = a.pc;
-  if (ctl->error || pc->sel_final_level < level) return;
-  const long long k = pc->sel_k[level];
+static __device__ __forceinline__ void select_hist(const ChunkArgs& a, ChunkCtl* pc, int level, int shift, unsigned int* sh) {
   const long long n = level == 0 ? a.pool_slots : (long long)pc->sel_count[level];
-  if (pc->sel_count[level] < k) {   // fewer eligible victims than needed
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicCAS(&ctl->error, 0, level == 0 ? TAURUS_ERR_POOL_TOO_SMALL : TAURUS_ERR_INTERNAL);
-    return;
-  }
-  __shared__ unsigned int sh[TAURUS_SEL_BINS];
-  for (int i = threadIdx.x; i < TAURUS_SEL_BINS; i += blockDim.x) sh[i] = 0;
+  if ((long long)blockIdx.x * MR_TILE >= n) return;
+  for (int i = threadIdx.x; i < TAURUS_SEL_BINS; i += MR_THREADS) sh[i] = 0;
   __syncthreads();
-  const int shift = sel_shift_of(pc->sel_min[level], pc->sel_max[level]);
-  const int32_t* __restrict__ cand = level == 0 ? nullptr : a.cand[level & 1];
-  __shared__ long long s_tile;
-  const bool dyn = level == 0 && a.dynamic_spans != 0;   // deeper levels see short candidate lists
-  for (long long it = 0;; ++it) {
-    const long long base = next_tile(dyn, &pc->tile_next[1], it, &s_tile) * SEL_TILE;
-    if (base >= n) break;
+  const int32_t* cand = level == 0 ? nullptr : a.cand[level & 1];   // written by other blocks of this launch: no read-only loads
+  for (long long base = (long long)blockIdx.x * MR_TILE; base < n; base += (long long)gridDim.x * MR_TILE) {
 #pragma unroll
-    for (int j = 0; j < SEL_ITEMS; ++j) {
-      const long long i = base + j * 256 + threadIdx.x;
+    for (int j = 0; j < MR_ITEMS; ++j) {
+      const long long i = base + j * MR_THREADS + threadIdx.x;
       unsigned long long key = ~0ull;
       if (i < n) key = a.keys[level == 0 ? i : (long long)cand[i]];
       const bool on = key != ~0ull;
@@ -311,113 +283,96 @@ __global__ void __launch_bounds__(256) select_hist_kernel(ChunkArgs a, int level
   }
   __syncthreads();
   unsigned int* hist = pc->hist[level & 1];
-  for (int b = threadIdx.x; b < TAURUS_SEL_BINS; b += blockDim.x)
+  for (int b = threadIdx.x; b < TAURUS_SEL_BINS; b += MR_THREADS)
     if (sh[b]) atomicAdd(&hist[b], sh[b]);
 }
 
 // Every block finds the digit that holds rank k from the level's histogram; keys below it are victims, keys inside
-// it go to the next level (or are victims too when the digit holds exactly the ranks still missing).
-__global__ void __launch_bounds__(256) select_split_kernel(ChunkArgs a, int level) {
-  DevCtl* ctl = a.ctl;
-  ChunkCtl* pc = a.pc;
-  if (ctl->error || pc->sel_final_level < level) return;
-  __shared__ unsigned int sh[TAURUS_SEL_BINS];
-  __shared__ unsigned int part[256];
-  __shared__ int s_digit;
-  __shared__ long long s_rest;
+// it go to the next level (or are victims too when the digit holds exactly the ranks still missing).  Returns 1 when
+// the level listed the last victims, 0 when another level follows, -1 when the selection cannot be completed; the
+// answer is the same in every block.
+static __device__ __forceinline__ int select_split(const ChunkArgs& a, ChunkCtl* pc, int level, int shift, unsigned int* sh, unsigned int* part,
+                                                   int* s_digit, long long* s_rest) {
   const unsigned int* hist = pc->hist[level & 1];
   const long long k = pc->sel_k[level];
-  // bins per thread: TAURUS_SEL_BINS / 256 consecutive ones
-  constexpr int PER = TAURUS_SEL_BINS / 256;
-  unsigned int mine[PER], sum = 0;
-#pragma unroll
-  for (int j = 0; j < PER; ++j) { mine[j] = hist[threadIdx.x * PER + j]; sh[threadIdx.x * PER + j] = mine[j]; sum += mine[j]; }
-  part[threadIdx.x] = sum;
-  if (threadIdx.x == 0) s_digit = -1;
+  constexpr int PER = TAURUS_SEL_BINS / MR_THREADS;   // consecutive bins per thread
+  unsigned int sum = 0;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    long long cum = 0;
-    int t = 0;
-    for (; t < 256; ++t) { if (cum + part[t] >= k) break; cum += part[t]; }
-    if (t < 256) {
-      int b = t * PER;
-      for (; b < t * PER + PER; ++b) { if (cum + sh[b] >= k) break; cum += sh[b]; }
-      s_digit = b;
-      s_rest = k - cum;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) { const unsigned m = __ldcg(&hist[threadIdx.x * PER + j]); sh[threadIdx.x * PER + j] = m; sum += m; }
+  unsigned incl = sum;   // inclusive prefix over the block: warp scan, then scan of the warp totals
+  for (int o = 1; o < 32; o <<= 1) { const unsigned y = __shfl_up_sync(FULL, incl, o); if (lane_id() >= o) incl += y; }
+  if (lane_id() == 31) part[threadIdx.x >> 5] = incl;
+  if (threadIdx.x == 0) *s_digit = -1;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    unsigned w = part[threadIdx.x];
+    for (int o = 1; o < 32; o <<= 1) { const unsigned y = __shfl_up_sync(FULL, w, o); if (lane_id() >= o) w += y; }
+    part[threadIdx.x] = w;
+  }
+  __syncthreads();
+  incl += threadIdx.x >= 32 ? part[(threadIdx.x >> 5) - 1] : 0;
+  long long cum = (long long)incl - sum;
+  if (cum < k && (long long)incl >= k) {   // exactly one thread's bins cross rank k
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      const unsigned m = sh[threadIdx.x * PER + j];
+      if (cum < k && cum + m >= k) { *s_digit = threadIdx.x * PER + j; *s_rest = k - cum; }
+      cum += m;
     }
   }
   __syncthreads();
-  const int digit_k = s_digit;
-  if (digit_k < 0) {   // the histogram holds fewer keys than k: cannot happen after the count check
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
-    return;
-  }
-  const long long rest = s_rest;
+  const int digit_k = *s_digit;
+  if (digit_k < 0) return -1;   // the histogram holds fewer keys than k: cannot happen after the count check
+  const long long rest = *s_rest;
   const bool final = rest == (long long)sh[digit_k];   // the whole digit is victims: nothing left to resolve
-  const int shift = sel_shift_of(pc->sel_min[level], pc->sel_max[level]);
+  if (!final && (level == TAURUS_SEL_LEVELS - 1 || shift == 0)) return -1;   // unique keys always end in a final level
   const long long n = level == 0 ? a.pool_slots : (long long)pc->sel_count[level];
-  const int32_t* __restrict__ cand = level == 0 ? nullptr : a.cand[level & 1];
-  int32_t* __restrict__ next = a.cand[(level + 1) & 1];
+  const int32_t* cand = level == 0 ? nullptr : a.cand[level & 1];   // written by other blocks of this launch: no read-only loads
+  int32_t* next = a.cand[(level + 1) & 1];
   if (blockIdx.x == 0) {
     unsigned int* other = pc->hist[(level + 1) & 1];   // the next level's histogram (read last by the level above this one)
-    for (int b = threadIdx.x; b < TAURUS_SEL_BINS; b += blockDim.x) other[b] = 0;
-    if (threadIdx.x == 0) {
-      if (final) pc->sel_final_level = level;
-      else if (level == TAURUS_SEL_LEVELS - 1 || shift == 0) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);   // unique keys always end in a final level
-      else pc->sel_k[level + 1] = rest;
-    }
+    for (int b = threadIdx.x; b < TAURUS_SEL_BINS; b += MR_THREADS) other[b] = 0;
+    if (threadIdx.x == 0 && !final) pc->sel_k[level + 1] = rest;
   }
   unsigned long long kmin = ~0ull, kmax = 0ull;
   int cnt = 0;
   const unsigned lt = (1u << lane_id()) - 1;
-  __shared__ long long s_tile;
-  const bool dyn = level == 0 && a.dynamic_spans != 0;
-  for (long long it = 0;; ++it) {
-    const long long base = next_tile(dyn, &pc->tile_next[2], it, &s_tile) * SEL_TILE;
-    if (base >= n) break;
-#pragma unroll 2
-  for (int j = 0; j < SEL_ITEMS; ++j) {
-    const long long i = base + j * 256 + threadIdx.x;
-    unsigned long long key = ~0ull;
-    int slot = -1;
-    if (i < n) { slot = level == 0 ? (int)i : cand[i]; key = a.keys[slot]; }
-    const bool on = key != ~0ull;
-    const int digit = on ? (int)((unsigned)(key >> shift) & (TAURUS_SEL_BINS - 1)) : TAURUS_SEL_BINS;
-    const bool victim = digit < digit_k || (final && digit == digit_k);
-    const bool keep = !final && digit == digit_k;
-    const unsigned mv = __ballot_sync(FULL, victim), mk = __ballot_sync(FULL, keep);
-    if (mv) {
-      int idx = 0;
-      const int leader = __ffs(mv) - 1;
-      if (lane_id() == leader) idx = atomicAdd(&pc->victim_count, __popc(mv));
-      idx = __shfl_sync(FULL, idx, leader) + __popc(mv & lt);
-      if (victim && idx < a.victim_capacity) a.victims[idx].x = slot;
-    }
-    if (mk) {
-      int idx = 0;
-      const int leader = __ffs(mk) - 1;
-      if (lane_id() == leader) idx = atomicAdd(&pc->sel_count[level + 1], __popc(mk));
-      idx = __shfl_sync(FULL, idx, leader) + __popc(mk & lt);
-      if (keep) {
-        next[idx] = slot;   // at most pool_slots keys enter any level
-        if (key < kmin) kmin = key;
-        if (key > kmax) kmax = key;
-        cnt++;
+  for (long long base = (long long)blockIdx.x * MR_TILE; base < n; base += (long long)gridDim.x * MR_TILE) {
+#pragma unroll
+    for (int j = 0; j < MR_ITEMS; ++j) {
+      const long long i = base + j * MR_THREADS + threadIdx.x;
+      unsigned long long key = ~0ull;
+      int slot = -1;
+      if (i < n) { slot = level == 0 ? (int)i : cand[i]; key = a.keys[slot]; }
+      const bool on = key != ~0ull;
+      const int digit = on ? (int)((unsigned)(key >> shift) & (TAURUS_SEL_BINS - 1)) : TAURUS_SEL_BINS;
+      const bool victim = digit < digit_k || (final && digit == digit_k);
+      const bool keep = !final && digit == digit_k;
+      const unsigned mv = __ballot_sync(FULL, victim), mk = __ballot_sync(FULL, keep);
+      if (mv) {
+        int idx = 0;
+        const int leader = __ffs(mv) - 1;
+        if (lane_id() == leader) idx = atomicAdd(&pc->victim_count, __popc(mv));
+        idx = __shfl_sync(FULL, idx, leader) + __popc(mv & lt);
+        if (victim && idx < a.victim_capacity) a.victims[idx].x = slot;
+      }
+      if (mk) {
+        int idx = 0;
+        const int leader = __ffs(mk) - 1;
+        if (lane_id() == leader) idx = atomicAdd(&pc->sel_count[level + 1], __popc(mk));
+        idx = __shfl_sync(FULL, idx, leader) + __popc(mk & lt);
+        if (keep) {
+          next[idx] = slot;   // at most pool_slots keys enter any level
+          if (key < kmin) kmin = key;
+          if (key > kmax) kmax = key;
+          cnt++;
+        }
       }
     }
   }
-  }
-  // sel_count of the next level is already counted by the appends: fold only the key range
-  for (int o = 16; o; o >>= 1) {
-    const unsigned long long m = __shfl_xor_sync(FULL, kmin, o), M = __shfl_xor_sync(FULL, kmax, o);
-    if (m < kmin) kmin = m;
-    if (M > kmax) kmax = M;
-    cnt += __shfl_xor_sync(FULL, cnt, o);
-  }
-  if (lane_id() == 0 && cnt) {
-    atomicMin(&pc->sel_min[level + 1], kmin);
-    atomicMax(&pc->sel_max[level + 1], kmax);
-  }
+  sel_fold(pc, level + 1, kmin, kmax, cnt, false);   // the appends have counted the next level already
+  return final ? 1 : 0;
 }
 
 // ---- host store: where a victim's row goes
@@ -444,15 +399,8 @@ static __device__ __forceinline__ long long next_sender(const ChunkArgs& a, int 
   return ns;
 }
 
-__global__ void __launch_bounds__(256) victim_bucket_kernel(ChunkArgs a) {
-  DevCtl* ctl = a.ctl;
-  ChunkCtl* pc = a.pc;
-  if (ctl->error || pc->deficit == 0) return;
-  const int n = pc->deficit;
-  if (pc->victim_count != n) {   // the select must have produced exactly `deficit` victims
-    if (threadIdx.x == 0 && blockIdx.x == 0) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
-    return;
-  }
+// Bucket and rank of every victim.
+static __device__ __forceinline__ void victim_bucket(const ChunkArgs& a, DevCtl* ctl, int n) {
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const int slot = a.victims[i].x;
@@ -467,10 +415,7 @@ __global__ void __launch_bounds__(256) victim_bucket_kernel(ChunkArgs a) {
 // One block.  First the tails of the buckets whose grid cell ends inside this push are closed (no victim can be
 // filed there any more: its next sender would lie behind the push); then every bucket that received victims gets
 // the extents it lacks from the free stack.
-__global__ void __launch_bounds__(1024) extent_plan_kernel(ChunkArgs a) {
-  DevCtl* ctl = a.ctl;
-  ChunkCtl* pc = a.pc;
-  if (ctl->error) return;
+static __device__ void extent_plan(const ChunkArgs& a, DevCtl* ctl, int deficit) {
   const int E = 1 << a.ext_shift;
   __shared__ int warp_sum[32];
   __shared__ long long s_running;
@@ -508,7 +453,7 @@ __global__ void __launch_bounds__(1024) extent_plan_kernel(ChunkArgs a) {
     }
   }
   __syncthreads();
-  if (pc->deficit == 0) return;
+  if (deficit == 0) return;
   // phase 2: extents needed per bucket, exclusive prefix over the buckets
   for (long long base = 0; base < a.n_buckets; base += blockDim.x) {
     const long long b = base + threadIdx.x;
@@ -541,7 +486,7 @@ __global__ void __launch_bounds__(1024) extent_plan_kernel(ChunkArgs a) {
   }
   const long long total = s_running;
   if (total > ctl->ext_free_top) {
-    if (threadIdx.x == 0) atomicCAS(&ctl->error, 0, TAURUS_ERR_HOST_STORE_FULL);
+    if (threadIdx.x == 0) { atomicCAS(&ctl->error, 0, TAURUS_ERR_HOST_STORE_FULL); a.pc->room_fail = 1; }
     return;
   }
   const long long stack_base = ctl->ext_free_top - total;
@@ -566,11 +511,8 @@ __global__ void __launch_bounds__(1024) extent_plan_kernel(ChunkArgs a) {
   }
 }
 
-__global__ void __launch_bounds__(256) victim_place_kernel(ChunkArgs a) {
-  DevCtl* ctl = a.ctl;
-  ChunkCtl* pc = a.pc;
-  if (ctl->error || pc->deficit == 0) return;
-  const int n = pc->deficit;
+// Host row of every victim.
+static __device__ __forceinline__ void victim_place(const ChunkArgs& a, int n) {
   const int E = 1 << a.ext_shift;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -583,6 +525,85 @@ __global__ void __launch_bounds__(256) victim_place_kernel(ChunkArgs a) {
     a.victims[i].y = (ext << a.ext_shift) + idx;
     a.bk_new[pl.x] = 0;   // same value from every victim of the bucket; nothing reads the count after the plan
   }
+}
+
+// Barrier of a cooperative grid.  Arrivals are counted in pc->grid_arrivals, which the chunk's commit clears.  The wait
+// is bounded: a block that runs out sets the sticky error and goes on; the others then run out too, or have passed.
+static __device__ __forceinline__ bool grid_barrier(DevCtl* ctl, ChunkCtl* pc, unsigned int& round, int* s_ok) {
+  __syncthreads();
+  round += 1;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(&pc->grid_arrivals, 1u);
+    const unsigned int want = round * gridDim.x;
+    bool ok = false;
+    for (unsigned i = 0; i < (1u << 22) && !ok; ++i) {
+      unsigned int got;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(&pc->grid_arrivals) : "memory");
+      ok = got >= want;
+    }
+    if (!ok) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
+    *s_ok = ok ? 1 : 0;
+  }
+  __syncthreads();
+  return *s_ok != 0;
+}
+
+// Plan, victim select and placement of a bounded pool in ONE cooperative launch.  As seventeen launches this step took
+// longer than the row transfers it has to hide behind: most of the launches resolve nothing (the select usually ends at its
+// second or third level) and a launch costs 2.5 us on an idle GPU and 4 to 10 us while rows cross the host link, a barrier
+// of this grid about 1.5 us.  Every branch around a barrier depends only on values that were written before an earlier
+// barrier and are not written again until a later one, so all blocks take the same number of barriers.
+__global__ void __launch_bounds__(MR_THREADS, 1) make_room_kernel(ChunkArgs a) {
+  DevCtl* ctl = a.ctl;
+  ChunkCtl* pc = a.pc;
+  __shared__ unsigned int sh[TAURUS_SEL_BINS];
+  __shared__ unsigned int part[32];
+  __shared__ int s_digit, s_ok;
+  __shared__ long long s_rest;
+  unsigned int round = 0;
+  if (blockIdx.x == 0) {
+    for (int i = threadIdx.x; i < 2 * TAURUS_SEL_BINS; i += MR_THREADS) (&pc->hist[0][0])[i] = 0;
+    if (threadIdx.x == 0) {
+      pc->room_go = 0;
+      if (!ctl->error) { plan_chunk(a, ctl, pc); pc->room_go = ctl->error ? 0 : 1; }
+    }
+  }
+  if (!grid_barrier(ctl, pc, round, &s_ok)) return;
+  if (!pc->room_go) return;
+  const int deficit = pc->deficit;
+  if (deficit == 0) {
+    if (blockIdx.x == 0) extent_plan(a, ctl, 0);
+    return;
+  }
+  select_keys(a, pc);
+  if (!grid_barrier(ctl, pc, round, &s_ok)) return;
+  for (int level = 0;; ++level) {
+    if ((long long)pc->sel_count[level] < pc->sel_k[level]) {   // fewer eligible victims than needed
+      if (blockIdx.x == 0 && threadIdx.x == 0) atomicCAS(&ctl->error, 0, level == 0 ? TAURUS_ERR_POOL_TOO_SMALL : TAURUS_ERR_INTERNAL);
+      return;
+    }
+    const int shift = sel_shift_of(pc->sel_min[level], pc->sel_max[level]);
+    select_hist(a, pc, level, shift, sh);
+    if (!grid_barrier(ctl, pc, round, &s_ok)) return;
+    const int done = select_split(a, pc, level, shift, sh, part, &s_digit, &s_rest);
+    if (done < 0) {
+      if (blockIdx.x == 0 && threadIdx.x == 0) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
+      return;
+    }
+    if (!grid_barrier(ctl, pc, round, &s_ok)) return;
+    if (done) break;
+  }
+  if (pc->victim_count != deficit) {   // the select must have produced exactly `deficit` victims
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
+    return;
+  }
+  victim_bucket(a, ctl, deficit);
+  if (!grid_barrier(ctl, pc, round, &s_ok)) return;
+  if (blockIdx.x == 0) extent_plan(a, ctl, deficit);
+  if (!grid_barrier(ctl, pc, round, &s_ok)) return;
+  if (pc->room_fail) return;
+  victim_place(a, deficit);
 }
 
 // One warp per vertex that needs a slot.  Need-list entry i < deficit takes over the slot of victim
@@ -684,77 +705,99 @@ __global__ void alloc_kernel(ChunkArgs a) {
   if (lane_id() == 0 && reloaded) atomicAdd(&pc->reloaded, reloaded);
 }
 
+// ---- rows across the host link
+static __device__ __forceinline__ unsigned xf_smem(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+static __device__ __forceinline__ bool xf_wait(unsigned long long* bar, unsigned parity) {   // bounded; false when it ran out
+  for (unsigned i = 0; i < (1u << 22); ++i) {
+    unsigned ok;
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(xf_smem(bar)), "r"(parity) : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+static __device__ __forceinline__ void xf_load(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(xf_smem(dst)), "l"(src), "r"(bytes), "r"(xf_smem(bar)) : "memory");
+}
+
 // The rows of one chunk across the host link: the staged row of the victim whose slot a need-list entry took over
 // goes to its pinned host row (device -> host), and the host row of a vertex that was EVICTED is added into its new
-// slot (host -> device), so both directions of the link are busy at once.  A warp takes R entries per round, R chosen so
-// that it has four float4 per lane and direction in flight whatever the row width (R = 4 for rows of up to 32 float4,
-// 2 up to 64, else 1): the link is fed by bytes in flight, and narrow rows otherwise leave it short.  An extent whose
-// last row has come back is listed for the free stack (taken back two chunks later by extent_plan_kernel).
-template <int R>
-__global__ void __launch_bounds__(256) transfer_kernel(ChunkArgs a) {
+// slot (host -> device), so both directions of the link are busy at once.
+// Every thread carries one entry at a time through its own pair of row buffers in shared memory with untiled bulk
+// copies: host row and staged row in (one barrier for both), then an fp32 add-reduction into the slot and a store to
+// the host row.
+// Bound by the host link, and by what it does to the kernels beside it: rows waiting for the link fill the queues between
+// the SMs and L2, and everything else on the GPU waits in them.  So the rows in flight are kept to what the link needs,
+// on four SMs of their own (a block takes all the shared memory of its SM, so no block of another kernel shares it).
+// 600 k vertices, 4 096-source chunks, pool 0.27 V, 147 pushes of each of two layers (rows of 128 and 256 floats): one
+// block of eight warps per SM with 4 float4 per lane and direction in flight took 250 us a push and stretched the scatter
+// beside it from 30 to 260 us, 135 ms a pass; blocks of this kernel: 2 115 ms, 3 101, 4 98.7, 6 98.9, 8 99.1 with the one-
+// launch make-room step, 4 115.6, 16 124, 64 135 without it.  Fewer entries per block cost more than they relieve (32
+// instead of 112 rows of 1 KB in each of four blocks: 283 ms).
+// An extent whose last row has come back is listed for the free stack (taken back two chunks later by
+// extent_plan_kernel).
+#define XF_SMEM (224 * 1024)
+#define XF_THREADS 256
+__global__ void __launch_bounds__(XF_THREADS) transfer_kernel(ChunkArgs a, int lanes) {   // lanes: entries in flight per block
+  extern __shared__ __align__(128) unsigned char xf_rows[];
+  __shared__ unsigned long long bars[XF_THREADS];
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
   if (ctl->error) return;
-  constexpr int QPR = 4 / R;   // float4 steps of one row per round
+  if ((int)threadIdx.x >= lanes) return;
   const int n = pc->need_count;
-  const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
-  const int vec = a.Hp >> 2;
+  const unsigned bytes = (unsigned)a.Hp * 4u;
+  unsigned char* in = xf_rows + (size_t)threadIdx.x * 2 * bytes;
+  unsigned char* out = in + bytes;
+  unsigned long long* bar = &bars[threadIdx.x];
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(xf_smem(bar)) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   const int par = a.epoch & 1;
-  for (long long i0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * R; i0 < n; i0 += warps * R) {
-    int4 x[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) x[r] = i0 + r < n ? a.xfer_list[i0 + r] : make_int4(0, -1, -1, 0);   // same address for the whole warp
-    for (int k0 = 0; k0 < vec; k0 += 32 * QPR) {
-      float4 keep[4], in[4];
-#pragma unroll
-      for (int s4 = 0; s4 < 4; ++s4) {
-        const int r = s4 / QPR, k = k0 + (s4 % QPR) * 32 + lane_id();
-        if (k < vec) {
-          if (x[r].z >= 0) keep[s4] = reinterpret_cast<const float4*>(a.stage_out + (size_t)(i0 + r) * a.Hp)[k];
-          if (x[r].y >= 0) in[s4] = reinterpret_cast<const float4*>(a.host_store + (size_t)x[r].y * a.Hp)[k];
-        }
-      }
-#pragma unroll
-      for (int s4 = 0; s4 < 4; ++s4) {
-        const int r = s4 / QPR, k = k0 + (s4 % QPR) * 32 + lane_id();
-        if (k < vec) {
-          if (x[r].z >= 0) reinterpret_cast<float4*>(a.host_store + (size_t)x[r].z * a.Hp)[k] = keep[s4];
-          if (x[r].y >= 0) {
-            float* row = a.acc + (size_t)x[r].x * a.Hp + 4 * k;
-            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(row), "f"(in[s4].x), "f"(in[s4].y), "f"(in[s4].z), "f"(in[s4].w) : "memory");
-          }
-        }
-      }
+  unsigned phase = 0;
+  for (long long i = (long long)threadIdx.x * gridDim.x + blockIdx.x; i < n; i += (long long)lanes * gridDim.x) {
+    const int4 x = a.xfer_list[i];   // (slot, host row coming back or -1, host row to fill or -1)
+    if (x.y < 0 && x.z < 0) continue;
+    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the stores of the last entry have read the buffers
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                 ::"r"(xf_smem(bar)), "r"((x.y >= 0 ? bytes : 0u) + (x.z >= 0 ? bytes : 0u)) : "memory");
+    if (x.y >= 0) xf_load(in, a.host_store + (size_t)x.y * a.Hp, bytes, bar);
+    if (x.z >= 0) xf_load(out, a.stage_out + (size_t)i * a.Hp, bytes, bar);
+    if (!xf_wait(bar, phase)) { atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL); xf_wait(bar, phase); break; }
+    phase ^= 1;
+    if (x.y >= 0)
+      asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;"
+                   ::"l"(a.acc + (size_t)x.x * a.Hp), "r"(xf_smem(in)), "r"(bytes) : "memory");
+    if (x.z >= 0)
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                   ::"l"(a.host_store + (size_t)x.z * a.Hp), "r"(xf_smem(out)), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    if (x.y >= 0) {
+      const int e = x.y >> a.ext_shift;
+      if (atomicSub(&a.ext_live[e], 1) == 1) a.ext_ret[par][atomicAdd(&ctl->ext_ret_count[par], 1)] = e;   // last row of the extent
     }
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-      if (lane_id() == r && x[r].y >= 0) {
-        const int e = x[r].y >> a.ext_shift;
-        if (atomicSub(&a.ext_live[e], 1) == 1) a.ext_ret[par][atomicAdd(&ctl->ext_ret_count[par], 1)] = e;   // last row of the extent
-      }
   }
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-void launch_make_room(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, cudaEvent_t before_moves) {
-  const int blocks = c->sm_count * 8;
-  if (!a.direct) {   // direct-mapped pools plan inside alloc_kernel
+int launch_make_room(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, cudaEvent_t before_moves) {
+  if (c->pool_slots < c->V - c->hub_count) {
+    // one block per SM that the row transfers leave free; blocks that a small pool has no tile for only cost barrier time
+    long long blocks = (a.pool_slots + MR_TILE - 1) / MR_TILE;
+    if (blocks > c->sm_count - TAURUS_XFER_BLOCKS) blocks = c->sm_count - TAURUS_XFER_BLOCKS;
+    if (blocks < 1) blocks = 1;
+    ChunkArgs args = a;
+    void* params[1] = {&args};
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)make_room_kernel, dim3((unsigned)blocks), dim3(MR_THREADS), params, 0, st);
+    if (e != cudaSuccess) { taurus_note_cuda_error(e, "make_room_kernel"); return TAURUS_ERR_CUDA; }
+    c->launches += 1;
+  } else if (!a.direct) {   // eviction is impossible when every non-hub vertex has a slot; direct-mapped pools plan inside alloc_kernel
     plan_kernel<<<1, 256, 0, st>>>(a);
     c->launches += 1;
   }
-  if (c->pool_slots < c->V - c->hub_count) {   // eviction is impossible when every non-hub vertex has a slot
-    select_keys_kernel<<<blocks, 256, 0, st>>>(a);
-    for (int l = 0; l < TAURUS_SEL_LEVELS; ++l) {
-      // deeper levels work on what is left of one digit of the level above: a handful of blocks is enough
-      const int b = l == 0 ? blocks : l == 1 ? c->sm_count * 2 : c->sm_count;
-      select_hist_kernel<<<b, 256, 0, st>>>(a, l);
-      select_split_kernel<<<b, 256, 0, st>>>(a, l);
-    }
-    victim_bucket_kernel<<<c->sm_count * 8, 256, 0, st>>>(a);
-    extent_plan_kernel<<<1, 1024, 0, st>>>(a);
-    victim_place_kernel<<<c->sm_count * 2, 256, 0, st>>>(a);
-    c->launches += 2 * TAURUS_SEL_LEVELS + 4;
-  }
   if (before_moves) cudaEventRecord(before_moves, st);
+  return TAURUS_OK;
 }
 
 // Slots handed out, victims' rows staged, new rows cleared (S4, device side).
@@ -763,15 +806,17 @@ void launch_alloc(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
   c->launches += 1;
 }
 // Rows across the host link (bounded pools only).
-void launch_transfer(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
-  // One block per SM.  The warps spend their time waiting for the host link; measured on the "large" workload, fewer
-  // blocks leave the link short of requests (64 blocks: 36 + 33 GB/s, 148: 38 + 34, 1 184: 39 + 35), more blocks only
-  // take thread slots from the scatter and select kernels that run beside the transfers on the compute stream.
-  const int vec = a.Hp >> 2;
-  if (vec <= 32) transfer_kernel<4><<<c->sm_count, 256, 0, st>>>(a);
-  else if (vec <= 64) transfer_kernel<2><<<c->sm_count, 256, 0, st>>>(a);
-  else transfer_kernel<1><<<c->sm_count, 256, 0, st>>>(a);
+int launch_transfer(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
+  int lanes = XF_SMEM / (2 * a.Hp * 4);
+  if (lanes > XF_THREADS) lanes = XF_THREADS;
+  if (!c->xfer_smem_set) {   // once per context (the attribute belongs to the context's device)
+    const cudaError_t e = cudaFuncSetAttribute(transfer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, XF_SMEM);
+    if (e != cudaSuccess) { taurus_note_cuda_error(e, "transfer_kernel"); return TAURUS_ERR_CUDA; }
+    c->xfer_smem_set = true;
+  }
+  transfer_kernel<<<TAURUS_XFER_BLOCKS, XF_THREADS, XF_SMEM, st>>>(a, lanes);
   c->launches += 1;
+  return TAURUS_OK;
 }
 
 // ------------------------------------------------------------------------------------------------ finalise (S6 tail, S7)
@@ -781,7 +826,9 @@ void launch_transfer(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
 // Each lane takes CD_ITEMS entries per round so that their scattered reads (pending count, slot) are in flight
 // together and one pair of counter round trips serves CD_ITEMS * 32 entries.
 #define CD_ITEMS 4
-__global__ void compact_done_kernel(ChunkArgs a) {
+static __device__ void commit_counts(const ChunkArgs& a, DevCtl* ctl, ChunkCtl* pc);
+// write_record: the last block to finish folds the chunk's counters into the layer totals.
+__global__ void compact_done_kernel(ChunkArgs a, int write_record) {
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
   if (ctl->error) return;
@@ -849,6 +896,13 @@ __global__ void compact_done_kernel(ChunkArgs a) {
     }
   }
   if (__any_sync(FULL, bad) && lane_id() == 0) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
+  if (write_record) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      if (atomicAdd(&pc->done_blocks, 1u) == gridDim.x - 1) { __threadfence(); commit_counts(a, ctl, pc); }
+    }
+  }
 }
 
 // Completed vertices (listed by compact_done_kernel) in batches of 32 per warp: each lane first fetches the
@@ -931,22 +985,22 @@ __global__ void finalise_kernel(ChunkArgs a) {
 
 // After the chunk's completions are listed: fold the chunk's counters into the layer totals, write the chunk record.
 static __device__ void commit_counts(const ChunkArgs& a, DevCtl* ctl, ChunkCtl* pc) {   // one thread
-  long long c = ctl->chunks;
+  // every word is read before the first is written, so that the reads overlap (L2: other blocks of the launch wrote some)
+  const int hs = __ldcg(&pc->hs), ns = __ldcg(&pc->ns), ev = __ldcg(&pc->ev), gs = __ldcg(&pc->gs), need = __ldcg(&pc->need_count);
+  const int deficit = __ldcg(&pc->deficit), reloaded = __ldcg(&pc->reloaded), done = __ldcg(&pc->done_count);
+  const long long c = ctl->chunks, f = __ldcg(&ctl->free_top), s0 = ctl->sum_hs, s1 = ctl->sum_ns, s2 = ctl->sum_ev, s3 = ctl->sum_gs;
+  const long long e0 = ctl->evictions, r0 = ctl->reloads, d0 = ctl->completed;
   if (c < a.log_capacity) {
     long long* r = a.chunk_log + c * TAURUS_CK_COLUMNS;
-    r[TAURUS_CK_HS] = pc->hs; r[TAURUS_CK_NS] = pc->ns; r[TAURUS_CK_EV] = pc->ev; r[TAURUS_CK_GS] = pc->gs;
-    r[TAURUS_CK_NEED] = pc->need_count; r[TAURUS_CK_EVICTED] = pc->deficit; r[TAURUS_CK_RELOADED] = pc->reloaded;
-    r[TAURUS_CK_COMPLETED] = pc->done_count; r[TAURUS_CK_OCCUPANCY] = a.pool_slots - ctl->free_top;
+    r[TAURUS_CK_HS] = hs; r[TAURUS_CK_NS] = ns; r[TAURUS_CK_EV] = ev; r[TAURUS_CK_GS] = gs;
+    r[TAURUS_CK_NEED] = need; r[TAURUS_CK_EVICTED] = deficit; r[TAURUS_CK_RELOADED] = reloaded;
+    r[TAURUS_CK_COMPLETED] = done; r[TAURUS_CK_OCCUPANCY] = a.pool_slots - f;
   }
-  ctl->sum_hs += pc->hs; ctl->sum_ns += pc->ns; ctl->sum_ev += pc->ev; ctl->sum_gs += pc->gs;
-  ctl->evictions += pc->deficit;
-  ctl->reloads += pc->reloaded;
-  ctl->completed += pc->done_count;
+  ctl->sum_hs = s0 + hs; ctl->sum_ns = s1 + ns; ctl->sum_ev = s2 + ev; ctl->sum_gs = s3 + gs;
+  ctl->evictions = e0 + deficit;
+  ctl->reloads = r0 + reloaded;
+  ctl->completed = d0 + done;
   ctl->chunks = c + 1;
-}
-__global__ void commit_counts_kernel(ChunkArgs a) {
-  if (threadIdx.x != 0 || a.ctl->error) return;
-  commit_counts(a, a.ctl, a.pc);
 }
 // One thread, after the chunk's rows are finalised: the graduation buffer's row count, and the chunk's counters are
 // cleared for the chunk after next.  with_counts: the chunk record has not been written yet (no transfers in flight:
@@ -962,14 +1016,16 @@ __global__ void commit_kernel(ChunkArgs a, int with_counts) {
   pc->hs = pc->ns = pc->ev = pc->gs = 0;
   pc->need_count = 0; pc->done_count = 0; pc->touched_count = 0; pc->deficit = 0; pc->victim_count = 0; pc->reloaded = 0;
   pc->span_next = 0; pc->self_next = 0;
-  pc->tile_next[0] = pc->tile_next[1] = pc->tile_next[2] = pc->tile_next[3] = 0;
+  pc->grid_arrivals = 0; pc->done_blocks = 0; pc->room_go = 0; pc->room_fail = 0;
 }
 
 // S6: completions listed, slots released, chunk record written.
 void launch_compact_done(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, bool write_record) {
-  compact_done_kernel<<<c->sm_count * 8, 256, 0, st>>>(a);
-  if (write_record) commit_counts_kernel<<<1, 32, 0, st>>>(a);
-  c->launches += write_record ? 2 : 1;
+  // a warp takes 32 * CD_ITEMS entries per round: no more blocks than the longest list of any chunk can feed
+  const long long need = (a.touched_capacity + 8 * 32 * CD_ITEMS - 1) / (8 * 32 * CD_ITEMS);
+  const int blocks = (int)(need < 1 ? 1 : need < c->sm_count * 8 ? need : c->sm_count * 8);
+  compact_done_kernel<<<blocks, 256, 0, st>>>(a, write_record ? 1 : 0);
+  c->launches += 1;
 }
 void launch_commit(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
   commit_kernel<<<1, 32, 0, st>>>(a, c->pipelined ? 0 : 1);

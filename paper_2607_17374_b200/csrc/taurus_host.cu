@@ -279,7 +279,9 @@ static int init_impl(taurus_ctx* c, const taurus_graph* g, const taurus_model* m
     ALLOC(c->d_ext_ret[0], c->n_ext); ALLOC(c->d_ext_ret[1], c->n_ext);
     ALLOC(c->d_xfer_list, std::min<long long>(c->pool_slots, c->touched_capacity));   // one entry per need-list entry: a chunk needs at most what it touches
     ALLOC(c->d_stage_out, (size_t)c->victim_capacity * c->Hmax);
-    CU(cudaStreamCreateWithFlags(&c->xfer_stream, cudaStreamNonBlocking));
+    int prio_low = 0, prio_high = 0;
+    CU(cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
+    CU(cudaStreamCreateWithPriority(&c->xfer_stream, cudaStreamNonBlocking, prio_high));
     CU(cudaEventCreateWithFlags(&c->moves_ready, cudaEventDisableTiming));
     CU(cudaEventCreateWithFlags(&c->xfer_done, cudaEventDisableTiming));
     c->pipelined = true;
@@ -677,7 +679,7 @@ static int push_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const fl
   const bool grouped = c->d_gdst != nullptr && src_begin % c->chunk_sources == 0 &&
                        src_end == std::min<long long>(c->V, src_begin + c->chunk_sources);
   if (grouped) launch_classify_grouped(c, a, st); else launch_classify(c, a, st);
-  launch_make_room(c, a, st, timing ? pev[3] : nullptr);   // pev[3]: victims chosen and placed, rows not yet moved
+  { int rc = launch_make_room(c, a, st, timing ? pev[3] : nullptr); if (rc) { c->h_ctl->error = rc; return rc; } }   // pev[3]: victims chosen and placed, rows not yet moved
   // The chunk before this one: its rows have been crossing the host link since its slots were handed out.  Its
   // finalise runs now, before this chunk takes over the slots it released.
   int run_rc = finish_chunk(c, st);
@@ -688,7 +690,7 @@ static int push_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const fl
     CU(cudaEventRecord(c->moves_ready, st));
     CU(cudaStreamWaitEvent(c->xfer_stream, c->moves_ready, 0));
     if (timing) cudaEventRecord(pev[10], c->xfer_stream);
-    launch_transfer(c, a, c->xfer_stream);
+    { int rc = launch_transfer(c, a, c->xfer_stream); if (rc) { c->h_ctl->error = rc; return rc; } }
     if (timing) cudaEventRecord(pev[11], c->xfer_stream);
     CU(cudaEventRecord(c->xfer_done, c->xfer_stream));
   }

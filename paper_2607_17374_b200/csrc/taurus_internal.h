@@ -15,6 +15,7 @@
 #define TAURUS_MAX_TIMED_PUSHES 16384
 #define TAURUS_PUSH_EVENTS 12                   // CUDA events per timed push
 #define TAURUS_PHASES 9                         // durations reported per timed push
+#define TAURUS_XFER_BLOCKS 4                     // SMs that carry rows across the host link (one block each, all of its shared memory)
 #define TAURUS_SEL_BITS 11                      // radix-select digit width
 #define TAURUS_SEL_BINS (1 << TAURUS_SEL_BITS)
 #define TAURUS_SEL_LEVELS 6                     // 6 x 11 = 66 bits >= the 62-bit (score, id) key
@@ -32,14 +33,15 @@ struct ChunkCtl {
   int32_t reloaded;       // reloads
   unsigned int span_next; // scatter: next span of the chunk's edge list to hand to a warp
   unsigned int self_next; // scatter: next tile of 32 self messages to hand to a warp
-  unsigned int tile_next[4];  // pool passes of the victim select: next tile of slots to hand to a block
+  unsigned int grid_arrivals; // make-room step: blocks that reached its barriers so far
+  unsigned int done_blocks;   // completion list: blocks that have finished
+  int32_t room_go, room_fail; // make-room step: the plan went through / the host store could not take the victims
   long long alloc_base;   // need-list entry i takes free_stack[alloc_base - 1 - i]
   // Victim select, level by level (level 0 scans the pool, deeper levels the candidates the level above left):
   long long sel_k[TAURUS_SEL_LEVELS + 1];               // rank still to resolve among the keys entering the level
   unsigned long long sel_min[TAURUS_SEL_LEVELS + 1];    // smallest / largest key entering the level: the digit of a level
   unsigned long long sel_max[TAURUS_SEL_LEVELS + 1];    //   starts at the highest bit in which they differ
   int32_t sel_count[TAURUS_SEL_LEVELS + 1];             // keys entering the level
-  int32_t sel_final_level;                              // level that listed the last victims; kernels of deeper levels return
   unsigned int hist[2][TAURUS_SEL_BINS];                // digit histogram, alternating between levels
 };
 
@@ -184,6 +186,7 @@ struct taurus_ctx {
   // weights per layer: Wcat is [Kp x Ncat] row-major fp32 (P columns then T columns), bias [Hp]
   float* d_Wcat[TAURUS_MAX_LAYERS] = {nullptr};
   float* d_bias[TAURUS_MAX_LAYERS] = {nullptr};
+  bool xfer_smem_set = false;                      // the same for the row transfer kernel
   bool tc_smem_set = false;                        // dynamic shared memory limit of the projection kernel raised
   void* tc_image[TAURUS_MAX_LAYERS] = {nullptr};   // tensor-core operand images of Wcat (owned by kernels_gemm_tc.cu)
   void* tc_image_af[TAURUS_MAX_LAYERS] = {nullptr};   // SAGE aggregate-first layers: image of [W_neigh ; W_self] stacked along K
@@ -309,9 +312,9 @@ static inline int taurus_proj_width(int mode, int Hp, int heads = 1) {
 // ---- kernels_state.cu
 void launch_layer_reset(taurus_ctx* c, int layer, cudaStream_t st);
 void launch_classify(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);
-void launch_make_room(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, cudaEvent_t before_moves = nullptr);   // plan, select, placement, [event]
+int launch_make_room(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, cudaEvent_t before_moves = nullptr);   // plan, select, placement, [event]
 void launch_alloc(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);       // slots handed out, victims' rows staged, new rows cleared
-void launch_transfer(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);    // staged rows to the host store, reloaded rows added into their slots
+int launch_transfer(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);    // staged rows to the host store, reloaded rows added into their slots
 void launch_finalise(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);    // finalise + commit (after launch_compact_done)
 void launch_compact_done(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, bool write_record);   // completions listed (and the chunk record written)
 void launch_commit(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);
