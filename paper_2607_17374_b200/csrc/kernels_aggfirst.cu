@@ -101,7 +101,7 @@ __global__ void af_finish_kernel(ChunkArgs a, const float* __restrict__ O, long 
     if (threadIdx.x == 0 && blockIdx.x == 0) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
     return;
   }
-  const long long base = a.dense_half >= 0 ? a.grad_off : ctl->grad_count;
+  const long long base = a.resident ? pc->grad_base : a.dense_half >= 0 ? a.grad_off : ctl->grad_count;
   const long long limit = a.dense_half >= 0 ? a.grad_off + a.grad_cap : a.drain_rows;
   const int vec = a.Hout >> 2;
   const bool vec_ok = a.dense_direct && (a.dense_ld & 3) == 0 && (reinterpret_cast<uintptr_t>(a.dense_direct) & 15) == 0;
@@ -158,8 +158,10 @@ int launch_af_finalise(taurus_ctx* c, const ChunkArgs& a, int layer, long long r
     }
     const bool sage = c->mode == TAURUS_SAGE_MEAN;
     const int Ka = sage ? 2 * a.Hp : a.Hp;               // columns of the gathered matrix
-    af_gather_kernel<<<grid, 256, 0, st>>>(a, c->d_af_A, rows, sage ? c->d_af_X : nullptr);
-    c->launches += 1;
+    if (!a.resident) {   // (a resident pool's gather has left the sums in d_af_A)
+      af_gather_kernel<<<grid, 256, 0, st>>>(a, c->d_af_A, rows, sage ? c->d_af_X : nullptr);
+      c->launches += 1;
+    }
     void* image = sage ? c->tc_image_af[layer] : c->tc_image[layer];
     const bool tc = gemm_plain_tc_usable(c, image, c->d_af_A, Ka, O, a.Hout);
     // rows that go straight into the caller's matrix leave the tensor-core kernel finished (bias, activation, state)
@@ -169,7 +171,7 @@ int launch_af_finalise(taurus_ctx* c, const ChunkArgs& a, int layer, long long r
       fin.bias = a.bias; fin.act = a.act;
       int rc = launch_gemm_plain_tc(c, image, 0, a.Hout, c->d_af_A, Ka, Ka, (int)rows, O, a.Hout, st, &fin, &a.pc->done_count);
       if (rc) return rc;
-      launch_commit(c, a, st);
+      if (!a.resident) launch_commit(c, a, st);
       return TAURUS_OK;
     }
     if (tc) {
@@ -184,6 +186,6 @@ int launch_af_finalise(taurus_ctx* c, const ChunkArgs& a, int layer, long long r
     af_finish_kernel<<<grid, 256, 0, st>>>(a, O, rows);
     c->launches += 1;
   }
-  launch_commit(c, a, st);
+  if (!a.resident) launch_commit(c, a, st);
   return TAURUS_OK;
 }

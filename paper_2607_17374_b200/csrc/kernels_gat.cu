@@ -140,6 +140,7 @@ void launch_gat_scores(taurus_ctx* c, int layer, const float* X, int ldx, int n,
 }
 
 void launch_gat_attention(taurus_ctx* c, cudaStream_t st) {
+  if (c->resident) { launch_resident_attention(c, st); return; }
   const int grid = c->sm_count * 8;
   if (c->heads == 1) gat_edge_max_kernel<true><<<grid, 256, 0, st>>>(c->V, 1, c->d_row_ptr, c->d_col, c->d_mask_cur, c->d_att_s, c->d_att_max);
   else gat_edge_max_kernel<false><<<grid, 256, 0, st>>>(c->V, c->heads, c->d_row_ptr, c->d_col, c->d_mask_cur, c->d_att_s, c->d_att_max);

@@ -1,0 +1,997 @@
+// Pools that hold every vertex (pool_slots >= V): the pull form of a layer.
+//
+// Nothing is ever evicted from such a pool, so no partial sum has to be kept between chunks: the memory of the
+// accumulator rows keeps the rows that the sources send instead (projected rows, or input rows in aggregate-first layers),
+// filed under their source, and a vertex's sum is formed once, when its last message has arrived, from its in-list
+// (Sect. 3.1's messages, 3.4's counts and 3.6's graduation in another order of the same additions).  One message then
+// costs one row read, where the push form reads the row and read-modify-writes the destination's row once per (chunk,
+// destination) group.
+//
+// A push is
+//   rows     : the chunk's rows into the store (by the projection, or a copy)
+//   account  : pending counts, states, completion list and the chunk record, one item per (chunk, destination) group
+//   gather   : one warp per completed vertex sums the rows of its in-list and finishes the row; long in-lists are cut
+//              into segments that different warps sum
+// Integer accounting (counts, states, chunk records) is that of the push form.
+#include <cub/cub.cuh>
+
+#include <algorithm>
+#include <type_traits>
+#include <vector>
+
+#include "taurus_internal.h"
+
+#define FULL 0xffffffffu
+#define HEAVY_DEGREE 256     // in-lists longer than this are summed in segments
+#define HEAVY_SEGMENT 128
+
+namespace {
+
+__device__ __forceinline__ int rl() { return threadIdx.x & 31; }
+__device__ __forceinline__ float r_lrelu(float x, float slope) { return x > 0.f ? x : slope * x; }
+__device__ __forceinline__ void red_v4(float* addr, const float4& v) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ void add4(float4& s, const float4& r) { s.x += r.x; s.y += r.y; s.z += r.z; s.w += r.w; }
+__device__ __forceinline__ void fma4(float4& s, float w, const float4& r) {
+  s.x = fmaf(w, r.x, s.x); s.y = fmaf(w, r.y, s.y); s.z = fmaf(w, r.z, s.z); s.w = fmaf(w, r.w, s.w);
+}
+
+// ------------------------------------------------------------------------------------------------ layer reset
+__global__ void resident_reset_kernel(long long V, const int32_t* din, int fanout, int32_t* pend, uint8_t* state, int32_t* touch,
+                                      int32_t* reload, long long pool_slots, DevCtl* ctl) {
+  const long long stride = (long long)gridDim.x * blockDim.x, tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  for (long long v = tid; v < V; v += stride) {
+    const int d = din[v];
+    pend[v] = ((fanout > 0 && d > fanout) ? fanout : d) + 1;
+    state[v] = TAURUS_NOT_STARTED;
+    touch[v] = 0;
+    reload[v] = 0;
+  }
+  long long* words = reinterpret_cast<long long*>(ctl);
+  for (long long i = tid; i < (long long)(sizeof(DevCtl) / 8); i += stride) words[i] = words + i == &ctl->free_top ? pool_slots : 0;
+}
+
+// ------------------------------------------------------------------------------------------------ account
+// Items of a grid chunk: every vertex the chunk can touch, in ascending order, each once: destinations of the chunk's edges
+// (begin, count: their entries in the destination's in-list) and the chunk's own vertices (self message; the count may
+// be zero).  No two items share a vertex, so nothing here needs an atomic or an epoch stamp.
+struct Items { const int32_t* v; const uint32_t* begin; const int32_t* count; };
+
+__device__ __forceinline__ int mask_bits(const uint32_t* mask, unsigned long long b, int n) {   // set bits of [b, b + n)
+  if (n <= 0) return 0;
+  const unsigned long long e = b + (unsigned)n - 1;
+  const long long w0 = (long long)(b >> 5), w1 = (long long)(e >> 5);
+  const uint32_t first = 0xffffffffu << (b & 31), last = 0xffffffffu >> (31 - (e & 31));
+  if (w0 == w1) return __popc(mask[w0] & first & last);
+  int c = __popc(mask[w0] & first) + __popc(mask[w1] & last);
+  for (long long w = w0 + 1; w < w1; ++w) c += __popc(mask[w]);
+  return c;
+}
+
+// Edges and own vertices of a push that is not a grid cell: pending counts by atomics, first touches listed.
+__global__ void __launch_bounds__(256) account_edges_kernel(ChunkArgs a) {
+  DevCtl* ctl = a.ctl;
+  ChunkCtl* pc = a.pc;
+  if (ctl->error) return;
+  const long long e0 = a.row_ptr[a.src_begin], ne = a.row_ptr[a.src_end] - e0, total = ne + (a.src_end - a.src_begin);
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  __shared__ unsigned int s_msgs, s_hub;
+  if (threadIdx.x == 0) s_msgs = s_hub = 0;
+  __syncthreads();
+  unsigned msgs = 0, hub = 0;
+  int bad = 0;
+  for (long long base = (long long)blockIdx.x * blockDim.x; base < total; base += stride) {
+    const long long i = base + threadIdx.x;
+    int v = -1;
+    if (i < ne) {
+      const long long e = e0 + i;
+      if (a.mask == nullptr || ((a.mask[e >> 5] >> (e & 31)) & 1u)) v = a.col[e];
+      if (v >= 0) { msgs++; if (a.hub && a.hub[v]) hub++; }
+    } else if (i < total) {
+      v = (int)(a.src_begin + (i - ne));
+    }
+    bool first = false;
+    if (v >= 0) {
+      atomicAdd(&a.pend[v], -1);
+      if (a.touch[v] != a.epoch) first = atomicMax(&a.touch[v], a.epoch) != a.epoch;
+    }
+    const unsigned m = __ballot_sync(FULL, first);
+    if (m) {
+      int at = 0;
+      const int leader = __ffs(m) - 1;
+      if (rl() == leader) at = atomicAdd(&pc->touched_count, __popc(m));
+      at = __shfl_sync(FULL, at, leader) + __popc(m & ((1u << rl()) - 1));
+      if (first) { if (at < a.touched_capacity) a.touched_list[at] = v; else bad = 1; }
+    }
+  }
+  if (msgs) atomicAdd(&s_msgs, msgs);
+  if (hub) atomicAdd(&s_hub, hub);
+  if (bad) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_msgs) {
+    atomicAdd((unsigned long long*)&ctl->total_messages, (unsigned long long)s_msgs);
+    atomicAdd((unsigned long long*)&ctl->scatter_groups, (unsigned long long)s_msgs);   // no groups here: one per message
+    if (s_hub) atomicAdd((unsigned long long*)&ctl->hub_messages, (unsigned long long)s_hub);
+  }
+}
+
+// Pending counts, states, completion list; the last block to finish writes the chunk record and brings the layer totals,
+// the free-slot count and the place of the chunk's rows in the graduation buffer up to date, so that a push needs no
+// launch of its own for them.  LISTED: the items are the touched vertices listed by account_edges_kernel, whose pending
+// counts are already down.  Bound by the scattered words of a vertex (4 B count, 1 B state), which ascending items make
+// nearly sequential; ITEMS per thread keep their reads in flight together.
+enum { C_HS, C_NS, C_GS, C_MSGS, C_HUB, C_GROUPS, C_FREED, C_COUNT };
+#define ITEMS 4
+
+template <bool LISTED>
+__global__ void __launch_bounds__(256) account_kernel(ChunkArgs a, Items it, long long i0, long long n_items, const uint32_t* __restrict__ cmask,
+                                                      int4* __restrict__ heavy, int32_t* __restrict__ heavy_left) {
+  DevCtl* ctl = a.ctl;
+  ChunkCtl* pc = a.pc;
+  if (ctl->error) return;
+  __shared__ int s_cnt[2][8], s_base[2];
+  __shared__ unsigned int s_sum[C_COUNT];
+  __shared__ int s_last;
+  if (threadIdx.x < C_COUNT) s_sum[threadIdx.x] = 0;
+  const long long n = LISTED ? (long long)pc->touched_count : n_items;
+  const long long stride = (long long)gridDim.x * blockDim.x * ITEMS;
+  const int warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << rl()) - 1;
+  unsigned sum[C_COUNT] = {0};
+  int bad = 0, par = 0;
+  for (long long base = (long long)blockIdx.x * blockDim.x * ITEMS; base < n; base += stride, par ^= 1) {
+    int v[ITEMS], msgs[ITEMS], dec[ITEMS], p[ITEMS], st[ITEMS];
+#pragma unroll
+    for (int q = 0; q < ITEMS; ++q) {
+      const long long i = base + q * 256 + threadIdx.x;
+      v[q] = -1; msgs[q] = dec[q] = 0;
+      if (i < n) {
+        if (LISTED) v[q] = a.touched_list[i];
+        else {
+          v[q] = it.v[i0 + i];
+          msgs[q] = it.count[i0 + i];
+          if (cmask) msgs[q] = mask_bits(cmask, it.begin[i0 + i], msgs[q]);
+          dec[q] = msgs[q] + (v[q] >= a.src_begin && v[q] < a.src_end ? 1 : 0);
+          if (dec[q] == 0) v[q] = -1;   // a sampled layer kept none of the group's messages
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < ITEMS; ++q)
+      if (v[q] >= 0) { p[q] = a.pend[v[q]] - dec[q]; st[q] = a.state[v[q]]; }
+    bool done[ITEMS];
+    unsigned md[ITEMS];
+    int wd = 0;
+#pragma unroll
+    for (int q = 0; q < ITEMS; ++q) {
+      done[q] = false;
+      if (v[q] >= 0) {
+        const bool hub = a.hub && a.hub[v[q]];
+        done[q] = p[q] == 0;
+        if (p[q] < 0 || st[q] == TAURUS_COMPLETED) bad = 1;   // a completed vertex cannot receive a message
+        if (!LISTED) a.pend[v[q]] = p[q];
+        const int to = done[q] ? TAURUS_COMPLETED : hub ? TAURUS_ON_GPU : TAURUS_IN_BUFFER;
+        if (to != st[q]) a.state[v[q]] = (uint8_t)to;
+        if (hub) sum[C_GS]++;
+        else if (st[q] == TAURUS_NOT_STARTED) sum[C_NS]++;
+        else sum[C_HS]++;
+        if (done[q] && !hub) sum[C_FREED]++;
+        sum[C_MSGS] += (unsigned)msgs[q];
+        if (msgs[q] > 0) sum[C_GROUPS]++;
+        if (hub) sum[C_HUB] += (unsigned)msgs[q];
+      }
+      md[q] = __ballot_sync(FULL, done[q]);
+      wd += __popc(md[q]);
+    }
+    // appended per block: single-address atomics would bound this kernel
+    if (rl() == 0) s_cnt[par][warp] = wd;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int t = 0;
+      for (int w = 0; w < 8; ++w) { const int c = s_cnt[par][w]; s_cnt[par][w] = t; t += c; }
+      s_base[par] = t ? atomicAdd(&pc->done_count, t) : 0;
+    }
+    __syncthreads();
+    int at = s_base[par] + s_cnt[par][warp];
+#pragma unroll
+    for (int q = 0; q < ITEMS; ++q) {
+      if (done[q]) {
+        const int i = at + __popc(md[q] & lt);
+        if (i < a.grad_cap) a.done_list[i] = v[q]; else bad = 1;
+        if (heavy && i < a.grad_cap) {
+          const int d = a.din[v[q]];
+          if (d > HEAVY_DEGREE) {
+            const int segs = (d + HEAVY_SEGMENT - 1) / HEAVY_SEGMENT;
+            const int row = atomicAdd(&ctl->heavy_rows, 1), e = atomicAdd(&pc->heavy_count, segs);
+            heavy_left[row] = segs;
+            for (int s = 0; s < segs; ++s) heavy[e + s] = make_int4(i, s, row, segs);
+          }
+        }
+      }
+      at += __popc(md[q]);
+    }
+  }
+  if (bad) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
+#pragma unroll
+  for (int c = 0; c < C_COUNT; ++c) {
+    unsigned x = sum[c];
+    for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
+    if (rl() == 0 && x) atomicAdd(&s_sum[c], x);
+  }
+  __syncthreads();
+  if (threadIdx.x < C_COUNT && s_sum[threadIdx.x]) atomicAdd(&pc->acc[threadIdx.x], (unsigned long long)s_sum[threadIdx.x]);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&pc->done_blocks, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  // the counters of the next chunk (the other set; its last reader, the chunk before this one, is through)
+  ChunkCtl* next = pc == &ctl->pc[0] ? &ctl->pc[1] : &ctl->pc[0];
+  for (int i = threadIdx.x; i < (int)(offsetof(ChunkCtl, sel_k) / 4); i += blockDim.x) reinterpret_cast<int32_t*>(next)[i] = 0;
+  if (threadIdx.x != 0) return;
+  __threadfence();
+  long long c[C_COUNT];
+  for (int k = 0; k < C_COUNT; ++k) c[k] = (long long)__ldcg(&pc->acc[k]);
+  const long long done = __ldcg(&pc->done_count);
+  const long long F = ctl->free_top - c[C_NS], at = ctl->chunks, grad = ctl->grad_count, peak = ctl->peak_occupancy;
+  if (a.pool_slots - F > peak) ctl->peak_occupancy = a.pool_slots - F;
+  ctl->free_top = F + c[C_FREED];
+  if (at < a.log_capacity) {
+    long long* r = a.chunk_log + at * TAURUS_CK_COLUMNS;
+    r[TAURUS_CK_HS] = c[C_HS]; r[TAURUS_CK_NS] = c[C_NS]; r[TAURUS_CK_EV] = 0; r[TAURUS_CK_GS] = c[C_GS];
+    r[TAURUS_CK_NEED] = c[C_NS]; r[TAURUS_CK_EVICTED] = 0; r[TAURUS_CK_RELOADED] = 0;
+    r[TAURUS_CK_COMPLETED] = done; r[TAURUS_CK_OCCUPANCY] = a.pool_slots - (F + c[C_FREED]);
+  }
+  ctl->chunks = at + 1;
+  ctl->sum_hs += c[C_HS]; ctl->sum_ns += c[C_NS]; ctl->sum_gs += c[C_GS];
+  ctl->completed += done;
+  if (!LISTED) { ctl->total_messages += c[C_MSGS]; ctl->scatter_groups += c[C_GROUPS]; ctl->hub_messages += c[C_HUB]; }
+  pc->grad_base = a.dense_half >= 0 ? a.grad_off : grad;
+  if (a.dense_direct) { /* rows go straight into the caller's matrix */ }
+  else if (a.dense_half >= 0) ctl->out_count[a.dense_half] = done;
+  else {
+    if (grad + done > a.drain_rows) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
+    ctl->grad_count = grad + done;
+  }
+}
+
+// ------------------------------------------------------------------------------------------------ gather
+struct GatherArgs {
+  const float4* rows;        // the store: row of source u at u * pitch (float4 units)
+  int pitch, vec;            // pitch and width of a gathered row in float4
+  const int32_t* src;        // sources of the in-lists: entries [csc_ptr[v], csc_ptr[v + 1]), or, where a layer is
+  int keep;                  //   sampled (keep > 0), the kept ones at v * keep
+  const long long* csc_ptr;
+  const int32_t* done_list;
+  const int4* heavy;         // (index in done_list, segment, partial row, segments) of the long in-lists
+  float4* heavy_rows;        // partial sums, zero between vertices
+  int32_t* heavy_left;
+  DevCtl* ctl;
+  ChunkCtl* pc;
+  const float4* bias;
+  const float* att_s;
+  const float2* att_tm;
+  const double* att_z;
+  float4* A;                 // aggregate-first: finished sums (SAGE: followed by the vertex's own row), pitch a_pitch float4; else NULL
+  int a_pitch;
+  float* dense;              // the caller's matrix, or NULL: graduation buffer
+  long long dense_ld;
+  float* grad_rows;
+  long long* grad_ids;
+  int d_out, act, mode, heads, head_vec;
+  float gin_self, leaky;
+};
+
+#define G_WARPS 4            // warps per block
+#define BATCH 8              // items a warp takes at a time
+struct Item {                // fetched by one lane each: one chain of dependent reads for the whole batch
+  int v, i, len, row;        // vertex, place in done_list, entries to sum (-1: nothing), partial row (-1: the whole in-list)
+  uint32_t begin;            // first entry
+  float scale, self, bw;     // factor of the finished row, weight of the own row, weight of the bias
+};
+struct HeadTerm { float t, top, scale, self, bw; };   // GAT: destination term and maximum of the scores; the same three per head
+
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+// One warp per item (a completed vertex, or a segment of a long in-list), LPE lanes x VPL float4 per row and 32 / LPE rows
+// side by side.  What bounds it is how many random row reads an SM has in flight, so the rows of a batch's in-lists run
+// as one stream through a ring in shared memory: a step is U rows per lane group, D steps are always on their way, and
+// the vertex's own row is the last step of its item.  Every lane copies and reads back its own 16 bytes: no barrier.
+// With the same loads held in registers (4 rows per warp, 32 warps per SM) DRAM ran at 38 %, L2 at 27 %, the schedulers
+// issued in 20 % of the cycles.  The U rows of a step are added up before they join the running sum and long in-lists
+// are cut: fewer additions in sequence than the push form has.
+// GAT: most heads the ring is sized for (0: no attention).  The scores of a block of 32 sources travel with the block's
+// first step; the lanes turn them into coefficients, one source each, when the block is reached.
+template <int VPL, int U, int D, int GAT>
+struct Ring {
+  float4 row[D + 1][U][VPL][32];
+  float att[GAT ? D + 3 : 1][GAT ? 32 * GAT : 4];   // blocks between the producer and the consumer: at most one per step
+  Item item[BATCH];
+  HeadTerm head[GAT ? BATCH : 1][GAT ? GAT : 1];
+};
+
+template <int LPE, int VPL, int U, int D, int GAT>
+__global__ void __launch_bounds__(32 * G_WARPS) gather_kernel(const __grid_constant__ GatherArgs g) {
+  extern __shared__ __align__(16) unsigned char g_smem[];
+  ChunkCtl* const pc = g.pc;
+  if (g.ctl->error) return;
+  constexpr int EPS = 32 / LPE, STEP = U * EPS;
+  static_assert(STEP <= 32 && 32 % STEP == 0, "a block of 32 sources is a whole number of steps");
+  typedef Ring<VPL, U, D, GAT> R;
+  const int lane = rl(), sub = lane / LPE, c4 = lane % LPE, wid = threadIdx.x >> 5;
+  R& ring = reinterpret_cast<R*>(g_smem)[wid];
+  const int warps = (int)((gridDim.x * blockDim.x) >> 5);
+  const int n = pc->done_count, nh = g.heavy ? pc->heavy_count : 0;
+  const int total = n + nh;
+  bool on[VPL];
+  int hk[VPL];
+#pragma unroll
+  for (int k = 0; k < VPL; ++k) {
+    on[k] = c4 + k * LPE < g.vec;
+    hk[k] = 0;
+    if (GAT && g.heads > 1) { hk[k] = (c4 + k * LPE) / g.head_vec; if (hk[k] >= g.heads) hk[k] = g.heads - 1; }
+  }
+  // lanes behind the end of a row carry its last float4 along (same sectors, never stored): no predicates in the stream
+  int col[VPL];
+#pragma unroll
+  for (int k = 0; k < VPL; ++k) col[k] = (on[k] ? c4 + k * LPE : g.vec - 1) * 16;
+  const char* const rows = reinterpret_cast<const char*>(g.rows);
+  const unsigned pitch = (unsigned)g.pitch * 16u;
+  const bool sage = g.mode == TAURUS_SAGE_MEAN;
+  const int own_off = sage && !g.A ? g.vec * 16 : 0;   // SAGE, projected rows: the self message T_v sits behind P_v
+
+  int per = total / (warps * 2);
+  per = per < 1 ? 1 : per > BATCH ? BATCH : per;
+  for (int i0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per; i0 < total; i0 += warps * per) {
+    const int cnt = total - i0 < per ? total - i0 : per;
+    __syncwarp();
+    if (lane < cnt) {
+      Item x;
+      int i = i0 + lane - nh, seg = 0;   // segments first
+      x.row = -1;
+      if (i < 0) { const int4 h = g.heavy[i0 + lane]; i = h.x; seg = h.y; x.row = h.z; }
+      x.i = i;
+      x.v = g.done_list[i];
+      const long long b = g.csc_ptr[x.v];
+      int d = (int)(g.csc_ptr[x.v + 1] - b);
+      x.scale = x.self = x.bw = 1.f;
+      if (g.mode == TAURUS_GCN_SYM) {
+        x.bw = (float)sqrt((double)d + 1.0);
+        x.scale = (float)(1.0 / sqrt((double)d + 1.0));
+      } else if (g.mode == TAURUS_GIN_SUM) {
+        x.self = g.gin_self;
+      }
+      x.begin = (uint32_t)b;
+      if (g.keep) { x.begin = (uint32_t)x.v * (unsigned)g.keep; if (d > g.keep) d = g.keep; }
+      if (sage) x.scale = 1.0f / (float)(d > 1 ? d : 1);
+      x.len = d;
+      if (x.row >= 0) { x.begin += (unsigned)(seg * HEAVY_SEGMENT); x.len = d - seg * HEAVY_SEGMENT < HEAVY_SEGMENT ? d - seg * HEAVY_SEGMENT : HEAVY_SEGMENT; }
+      else if (g.heavy && d > HEAVY_DEGREE) x.len = -1;
+      ring.item[lane] = x;
+    }
+    __syncwarp();
+    if (GAT) {
+      for (int x = lane; x < cnt * g.heads; x += 32) {
+        const int j = x / g.heads, h = x - j * g.heads;
+        const size_t at = (size_t)ring.item[j].v * g.heads + h;
+        const float2 tm = g.att_tm[at];
+        const double z = g.att_z[at];
+        HeadTerm e;
+        e.t = tm.x; e.top = tm.y;
+        e.self = __expf(r_lrelu(g.att_s[at] + tm.x, g.leaky) - tm.y);
+        e.bw = (float)z;
+        e.scale = (float)(1.0 / z);
+        ring.head[j][h] = e;
+      }
+      __syncwarp();
+    }
+
+    // sources, 32 at a time: `u` the block the producer is in, `un` the one after it (item fj, entries from fb on)
+    int u = 0, un = 0, fj = 0, fb = -32;
+    auto fetch = [&]() {
+      fb += 32;
+      while (fj < cnt && fb >= ring.item[fj].len) { ++fj; fb = 0; }
+      if (fj < cnt) un = fb + lane < ring.item[fj].len ? g.src[ring.item[fj].begin + fb + lane] : 0;
+    };
+    // producer: next step to request (item pj, entries from pp on; pp at the end: the own row)
+    int pj = -1, pp = 0, plen = 0, slot = 0;
+    int pblk = 0, cblk = 0;     // GAT: block slots of the producer and the consumer
+    auto next_block = [&]() {
+      u = un;
+      if (GAT) {
+        pblk = pblk == D + 2 ? 0 : pblk + 1;
+        if (pp + lane < plen) {
+          const float* s = g.att_s + (size_t)(unsigned)u * g.heads;
+          float* to = &ring.att[GAT ? pblk : 0][lane * g.heads];
+          if ((g.heads & 3) == 0) for (int h = 0; h < g.heads; h += 4) copy16(to + h, s + h);
+          else for (int h = 0; h < g.heads; ++h) copy4(to + h, s + h);
+        }
+      }
+      fetch();
+    };
+    auto enter = [&]() {
+      do ++pj; while (pj < cnt && ring.item[pj].len < 0);
+      if (pj < cnt) {
+        pp = 0;
+        plen = ring.item[pj].len;
+        if (plen > 0) next_block();
+      }
+    };
+    auto produce = [&](int to) {
+      if (pj < cnt) {
+        if (pp < plen) {
+          const int at = (pp & 31) + sub;
+          if (pp + STEP <= plen) {
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+              const char* src = rows + (unsigned long long)(unsigned)__shfl_sync(FULL, u, at + q * EPS) * pitch;
+#pragma unroll
+              for (int k = 0; k < VPL; ++k) copy16(&ring.row[to][q][k][lane], src + col[k]);
+            }
+          } else {
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+              const char* src = rows + (unsigned long long)(unsigned)__shfl_sync(FULL, u, at + q * EPS) * pitch;
+              if (pp + q * EPS + sub < plen)
+#pragma unroll
+                for (int k = 0; k < VPL; ++k) copy16(&ring.row[to][q][k][lane], src + col[k]);
+            }
+          }
+          pp += STEP;
+          if (pp < plen && (pp & 31) == 0) next_block();
+        } else {
+          if (sub == 0 && ring.item[pj].row < 0) {
+            const char* src = rows + (size_t)ring.item[pj].v * pitch + own_off;
+#pragma unroll
+            for (int k = 0; k < VPL; ++k) copy16(&ring.row[to][0][k][lane], src + col[k]);
+          }
+          enter();
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fetch();
+    enter();
+#pragma unroll 1
+    for (int d = 0; d < D; ++d) produce(d);
+
+#pragma unroll 1
+    for (int j = 0; j < cnt; ++j) {
+      const int len = ring.item[j].len;
+      if (len < 0) continue;
+      float4 sum[VPL];
+#pragma unroll
+      for (int k = 0; k < VPL; ++k) sum[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+      for (int p = 0; p < len; p += STEP) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(D - 1) : "memory");
+        if (GAT && (p & 31) == 0) {   // scores of the block -> coefficients
+          cblk = cblk == D + 2 ? 0 : cblk + 1;
+          if (p + lane < len) {
+            float* const w = &ring.att[GAT ? cblk : 0][lane * g.heads];
+            for (int h = 0; h < g.heads; ++h) w[h] = __expf(r_lrelu(w[h] + ring.head[j][GAT ? h : 0].t, g.leaky) - ring.head[j][GAT ? h : 0].top);
+          }
+          __syncwarp();
+        }
+        auto add_step = [&](auto full) {
+#pragma unroll
+          for (int k = 0; k < VPL; ++k) {
+            float4 r[U];
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+              if (full || p + q * EPS + sub < len) {
+                r[q] = ring.row[slot][q][k][lane];
+                if (GAT) {
+                  const float w = ring.att[GAT ? cblk : 0][((p & 31) + q * EPS + sub) * g.heads + hk[k]];
+                  r[q].x *= w; r[q].y *= w; r[q].z *= w; r[q].w *= w;
+                }
+              } else {
+                r[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+              }
+            }
+#pragma unroll
+            for (int o = 1; o < U; o <<= 1)
+#pragma unroll
+              for (int q = 0; q + o < U; q += 2 * o) add4(r[q], r[q + o]);
+            add4(sum[k], r[0]);
+          }
+        };
+        if (p + STEP <= len) add_step(std::true_type()); else add_step(std::false_type());
+        produce(slot == 0 ? D : slot - 1);   // the slot of the step before this one: its rows have been added
+        slot = slot == D ? 0 : slot + 1;
+      }
+      // the sub-groups' sums
+#pragma unroll
+      for (int o = LPE; o < 32; o <<= 1)
+#pragma unroll
+        for (int k = 0; k < VPL; ++k) {
+          sum[k].x += __shfl_xor_sync(FULL, sum[k].x, o); sum[k].y += __shfl_xor_sync(FULL, sum[k].y, o);
+          sum[k].z += __shfl_xor_sync(FULL, sum[k].z, o); sum[k].w += __shfl_xor_sync(FULL, sum[k].w, o);
+        }
+      // the own row
+      asm volatile("cp.async.wait_group %0;" ::"n"(D - 1) : "memory");
+      float4 x[VPL];
+#pragma unroll
+      for (int k = 0; k < VPL; ++k) {
+        x[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (sub == 0 && on[k]) x[k] = ring.row[slot][0][k][lane];
+      }
+      produce(slot == 0 ? D : slot - 1);
+      slot = slot == D ? 0 : slot + 1;
+
+      const int v = ring.item[j].v, i = ring.item[j].i, row = ring.item[j].row;
+      if (row >= 0) {
+        // partial sums meet in a row of their own; the segment that arrives last finishes the vertex
+        float4* const part = g.heavy_rows + (size_t)row * g.vec;
+        if (sub == 0)
+#pragma unroll
+          for (int k = 0; k < VPL; ++k)
+            if (on[k]) red_v4(reinterpret_cast<float*>(part + c4 + k * LPE), sum[k]);
+        __threadfence();
+        __syncwarp();
+        int left = 0;
+        if (lane == 0) left = atomicSub(&g.heavy_left[row], 1);
+        left = __shfl_sync(FULL, left, 0);
+        if (left != 1) continue;
+        __threadfence();
+        if (sub == 0)
+#pragma unroll
+          for (int k = 0; k < VPL; ++k)
+            if (on[k]) {
+              sum[k] = __ldcg(part + c4 + k * LPE);
+              part[c4 + k * LPE] = make_float4(0.f, 0.f, 0.f, 0.f);
+              x[k] = *reinterpret_cast<const float4*>(rows + (size_t)v * pitch + own_off + col[k]);
+            }
+      }
+      // finished row
+      if (sub == 0) {
+        float scale = ring.item[j].scale, self = ring.item[j].self, bw = ring.item[j].bw;
+        const long long base = g.A || g.dense ? 0 : pc->grad_base;
+        const bool vec_ok = g.A || !g.dense || ((g.dense_ld & 3) == 0 && (reinterpret_cast<uintptr_t>(g.dense) & 15) == 0);
+        float* const out = g.A ? reinterpret_cast<float*>(g.A + (size_t)i * g.a_pitch)
+                               : g.dense ? g.dense + (size_t)v * g.dense_ld : g.grad_rows + (size_t)(base + i) * g.vec * 4;
+        const int width = g.dense && !g.A ? g.d_out : g.vec * 4;
+#pragma unroll
+        for (int k = 0; k < VPL; ++k) {
+          const int c = c4 + k * LPE;
+          if (!on[k]) continue;
+          if (GAT) { const HeadTerm& h = ring.head[j][hk[k]]; scale = h.scale; self = h.self; bw = h.bw; }
+          float4 y = sum[k];
+          if (g.A) {   // the weights, the bias and the activation are applied by the transform
+            if (sage) reinterpret_cast<float4*>(out)[g.vec + c] = x[k];
+            else fma4(y, self, x[k]);
+            y.x *= scale; y.y *= scale; y.z *= scale; y.w *= scale;
+          } else {
+            if (sage) add4(y, x[k]);   // T_v: own row times W_self, plus bias, times the message count
+            else {
+              const float4 b = g.bias[c];
+              add4(y, make_float4(x[k].x * self + b.x * bw, x[k].y * self + b.y * bw, x[k].z * self + b.z * bw, x[k].w * self + b.w * bw));
+            }
+            y.x *= scale; y.y *= scale; y.z *= scale; y.w *= scale;
+            if (g.act) { y.x = fmaxf(y.x, 0.f); y.y = fmaxf(y.y, 0.f); y.z = fmaxf(y.z, 0.f); y.w = fmaxf(y.w, 0.f); }
+          }
+          const int c0 = c << 2;
+          if (vec_ok && c0 + 3 < width) {
+            reinterpret_cast<float4*>(out)[c] = y;
+          } else {   // ragged last columns, or a matrix whose rows are not 16-byte aligned
+            if (c0 < width) out[c0] = y.x;
+            if (c0 + 1 < width) out[c0 + 1] = y.y;
+            if (c0 + 2 < width) out[c0 + 2] = y.z;
+            if (c0 + 3 < width) out[c0 + 3] = y.w;
+          }
+        }
+        if (c4 == 0 && !g.dense && !g.A) g.grad_ids[base + i] = v;
+      }
+    }
+  }
+}
+
+template <int LPE, int VPL, int U, int D, int GAT>
+int launch_g(taurus_ctx* c, const GatherArgs& g, long long bound, cudaStream_t st) {
+  const size_t smem = sizeof(Ring<VPL, U, D, GAT>) * G_WARPS;
+  static int per_sm = 0;
+  if (per_sm == 0) {
+    int b = 0;
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(gather_kernel<LPE, VPL, U, D, GAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TAURUS_ERR_CUDA;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, gather_kernel<LPE, VPL, U, D, GAT>, 32 * G_WARPS, smem) != cudaSuccess || b < 1) b = 1;
+    per_sm = b;
+  }
+  // no more warps than items: a completed vertex each, and the segments of long in-lists
+  const long long items = bound + c->n_heavy_segments;
+  const int grid = (int)std::max<long long>(1, std::min<long long>((items + G_WARPS - 1) / G_WARPS, (long long)c->sm_count * per_sm));
+  gather_kernel<LPE, VPL, U, D, GAT><<<grid, 32 * G_WARPS, smem, st>>>(g);
+  return TAURUS_OK;
+}
+template <int LPE, int VPL, int U, int D>
+int launch_g2(taurus_ctx* c, const GatherArgs& g, long long bound, cudaStream_t st) {
+  if (g.mode != TAURUS_GAT) return launch_g<LPE, VPL, U, D, 0>(c, g, bound, st);
+  constexpr int DG = D > 3 ? 3 : 2;   // the scores take room in the ring
+  return g.heads <= 4 ? launch_g<LPE, VPL, U, DG, 4>(c, g, bound, st) : launch_g<LPE, VPL, U, DG, 16>(c, g, bound, st);
+}
+
+// ------------------------------------------------------------------------------------------------ rows into the store
+// out[r] = scale * X[r], zero-padded from K to Kp columns; scale = 1, or 1 / sqrt(out-degree + 1) with GCN.
+__global__ void store_rows_kernel(const float* __restrict__ X, long long ldx, int n, int K, int Kp, long long src_begin, int gcn,
+                                  const long long* __restrict__ row_ptr, float* __restrict__ out) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  const int vec = Kp >> 2;
+  const bool wide = (ldx & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < (long long)n * vec; i += stride) {
+    const long long r = i / vec;
+    const int c = (int)(i - r * vec) * 4;
+    const float* src = X + r * ldx + c;
+    float4 x;
+    if (wide && c + 3 < K) x = *reinterpret_cast<const float4*>(src);
+    else x = make_float4(c < K ? src[0] : 0.f, c + 1 < K ? src[1] : 0.f, c + 2 < K ? src[2] : 0.f, c + 3 < K ? src[3] : 0.f);
+    if (gcn) {
+      const long long u = src_begin + r;
+      const float s = (float)(1.0 / sqrt((double)(row_ptr[u + 1] - row_ptr[u]) + 1.0));
+      x.x *= s; x.y *= s; x.z *= s; x.w *= s;
+    }
+    reinterpret_cast<float4*>(out)[i] = x;
+  }
+}
+
+// ------------------------------------------------------------------------------------------------ attention
+// tm[v] = (t_v, LeakyReLU(max_u s_u + t_v)) and z[v] = sum over v itself and its in-list of exp(e_uv - max): two sweeps
+// over the in-list, (entry, head) pairs across the lanes, the second one in double.  Bound by the latency of the scalars'
+// reads (heads x 4 B per entry, from L2), so a lane holds the first HELD of its scores for the second sweep.  The push form
+// of the same sweeps pays one atomic per edge, head and sweep: 4.7 ms for two layers of 400 k vertices, 20 M edges, four
+// heads.  WARPS = 1: a warp per vertex, long in-lists left out; else a block of so many warps per listed vertex with an
+// in-list of more than `above` and at most `upto` entries.
+#define HELD 8
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS == 1 ? 256 : 32 * WARPS)
+attention_kernel(long long V, int heads, const long long* __restrict__ csc_ptr, const int32_t* __restrict__ csc_src, const uint32_t* __restrict__ cmask,
+                 const float* __restrict__ att_s, const float* __restrict__ att_t, float slope, float2* __restrict__ tm, double* __restrict__ z,
+                 const int32_t* __restrict__ list, int above, int upto) {
+  constexpr bool LONG = WARPS > 1;
+  __shared__ float s_max[LONG ? WARPS * 16 : 1];
+  __shared__ double s_sum[LONG ? WARPS * 16 : 1];
+  const int lane = rl(), wid = threadIdx.x >> 5;
+  const int eps = 32 / heads, sub = lane / heads, h = lane - sub * heads;   // eps entries side by side; lanes behind them idle
+  const bool live = sub < eps;
+  int top = 1;                       // power of two >= eps
+  while (top < eps) top <<= 1;
+  const long long stride = LONG ? gridDim.x : ((long long)gridDim.x * blockDim.x) >> 5;
+  const int step = WARPS * eps, first = LONG ? wid * eps + sub : sub;
+  for (long long i = LONG ? blockIdx.x : ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < V; i += stride) {
+    const long long v = LONG ? list[i] : i;
+    const long long b = csc_ptr[v];
+    const int d = (int)(csc_ptr[v + 1] - b);
+    if (d <= above || d > upto) continue;
+    const float own = live ? att_s[v * heads + h] : 0.f, t = live ? att_t[v * heads + h] : 0.f;
+    float x[HELD];
+    unsigned has = 0;                // which of the held scores are kept entries
+    auto load = [&](int p0) {
+      has = 0;
+#pragma unroll
+      for (int q = 0; q < HELD; ++q) {
+        const int p = p0 + q * step + first;
+        x[q] = own;
+        if (live && p < d && (!cmask || ((cmask[(b + p) >> 5] >> ((b + p) & 31)) & 1u))) {
+          x[q] = att_s[(long long)csc_src[b + p] * heads + h];
+          has |= 1u << q;
+        }
+      }
+    };
+    float mx = own;   // the self message takes part in the maximum
+    for (int p0 = 0; p0 < d; p0 += HELD * step) {
+      load(p0);
+#pragma unroll
+      for (int q = 0; q < HELD; ++q) mx = fmaxf(mx, x[q]);
+    }
+    for (int o = top >> 1; o; o >>= 1) {
+      const float y = __shfl_down_sync(FULL, mx, o * heads);
+      if (sub + o < eps) mx = fmaxf(mx, y);
+    }
+    if (LONG) {
+      if (lane < heads) s_max[wid * 16 + lane] = mx;
+      __syncthreads();
+      if (lane < heads) for (int w = 0; w < WARPS; ++w) mx = fmaxf(mx, s_max[w * 16 + lane]);
+    }
+    mx = __shfl_sync(FULL, mx, h);
+    const float m = r_lrelu(mx + t, slope);
+    double sum = 0.0;
+    for (int p0 = 0; p0 < d; p0 += HELD * step) {
+      if (d > HELD * step) load(p0);   // else the scores are still held
+#pragma unroll
+      for (int q = 0; q < HELD; ++q)
+        if ((has >> q) & 1u) sum += (double)__expf(r_lrelu(x[q] + t, slope) - m);
+    }
+    for (int o = top >> 1; o; o >>= 1) {
+      const double y = __shfl_down_sync(FULL, sum, o * heads);
+      if (sub + o < eps) sum += y;
+    }
+    if (LONG) {
+      if (lane < heads) s_sum[wid * 16 + lane] = sum;
+      __syncthreads();
+      if (wid == 0 && lane < heads) { sum = 0.0; for (int w = 0; w < WARPS; ++w) sum += s_sum[w * 16 + lane]; }
+    }
+    if (lane < heads && (!LONG || wid == 0)) {
+      tm[v * heads + lane] = make_float2(t, m);
+      z[v * heads + lane] = sum + (double)__expf(r_lrelu(own + t, slope) - m);
+    }
+    if (LONG) __syncthreads();   // the partial results are rewritten for the block's next vertex
+  }
+}
+
+// ------------------------------------------------------------------------------------------------ build (init)
+__global__ void edge_sources_kernel(long long V, const long long* __restrict__ row_ptr, int32_t* __restrict__ src) {
+  const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
+  for (long long u = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < V; u += warps)
+    for (long long k = row_ptr[u] + rl(); k < row_ptr[u + 1]; k += 32) src[k] = (int32_t)u;
+}
+__global__ void degrees_kernel(long long V, const int32_t* __restrict__ din, long long* __restrict__ out) {   // out[V] = 0: room for the total
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v <= V; v += stride) out[v] = v < V ? din[v] : 0;
+}
+
+// Items of vertex v, ascending by chunk: one per chunk that holds a source of its in-list, and one for v's own chunk.
+// Pass 0 counts them, pass 1 writes (chunk, vertex, first entry) from the vertex's offset on.
+template <int PASS>
+__global__ void items_kernel(long long V, unsigned cs, const long long* __restrict__ csc_ptr, const int32_t* __restrict__ csc_src,
+                             long long* __restrict__ at, int32_t* __restrict__ chunk, int32_t* __restrict__ item_v, uint32_t* __restrict__ item_b,
+                             unsigned long long* __restrict__ heavy) {   // heavy[0..1]: vertices with long in-lists, their segments
+  const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
+  const int lane = rl();
+  for (long long v = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < V; v += warps) {
+    const long long b = csc_ptr[v], e = csc_ptr[v + 1];
+    const unsigned own = (unsigned)v / cs;
+    uint32_t put = PASS ? (uint32_t)at[v] : 0u, n = 0;
+    unsigned prev = 0xffffffffu;    // chunk of the entry before the batch
+    bool own_done = false;
+    for (long long p0 = b; p0 < e; p0 += 32) {
+      const long long p = p0 + lane;
+      const unsigned k = p < e ? (unsigned)csc_src[p] / cs : 0xffffffffu;
+      unsigned before = __shfl_up_sync(FULL, k, 1);
+      if (lane == 0) before = prev;
+      const bool head = p < e && k != before;
+      const unsigned heads = __ballot_sync(FULL, head);
+      const unsigned past = __ballot_sync(FULL, p < e && k >= own);   // the first such entry is where the own chunk's item starts
+      int extra_lane = 32;
+      if (!own_done && past) {
+        own_done = true;
+        const int f = __ffs(past) - 1;
+        const unsigned kf = __shfl_sync(FULL, k, f);
+        if (kf != own) {   // no source of the own chunk: an item without messages in front of this entry (a head, as its chunk is a later one)
+          extra_lane = f;
+          if (PASS && lane == f) {
+            const uint32_t i = put + __popc(heads & ((1u << f) - 1));
+            chunk[i] = (int32_t)own; item_v[i] = (int32_t)v; item_b[i] = (uint32_t)p;
+          }
+        }
+      }
+      if (PASS && head) {
+        const uint32_t i = put + __popc(heads & ((1u << lane) - 1)) + (lane >= extra_lane ? 1u : 0u);
+        chunk[i] = (int32_t)k; item_v[i] = (int32_t)v; item_b[i] = (uint32_t)p;
+      }
+      const uint32_t got = (uint32_t)__popc(heads) + (extra_lane < 32 ? 1u : 0u);
+      put += got; n += got;
+      prev = __shfl_sync(FULL, k, 31);
+    }
+    if (!own_done) {   // every source lies in an earlier chunk
+      if (PASS && lane == 0) { chunk[put] = (int32_t)own; item_v[put] = (int32_t)v; item_b[put] = (uint32_t)e; }
+      n += 1;
+    }
+    if (!PASS && lane == 0) {
+      at[v] = n;
+      if (e - b > HEAVY_DEGREE) {
+        atomicAdd(&heavy[0], 1ull);
+        atomicAdd(&heavy[1], (unsigned long long)((e - b + HEAVY_SEGMENT - 1) / HEAVY_SEGMENT));
+      }
+    }
+  }
+}
+__global__ void items_order_kernel(long long M, const int32_t* __restrict__ order, const int32_t* __restrict__ v_in, const uint32_t* __restrict__ b_in,
+                                   const long long* __restrict__ csc_ptr, int32_t* __restrict__ v_out, uint32_t* __restrict__ b_out,
+                                   int32_t* __restrict__ n_out) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += stride) {
+    const int32_t j = order[i];
+    const int32_t v = v_in[j];
+    const uint32_t b = b_in[j];
+    const uint32_t e = (long long)j + 1 < M && v_in[(long long)j + 1] == v ? b_in[j + 1] : (uint32_t)csc_ptr[v + 1];
+    v_out[i] = v; b_out[i] = b; n_out[i] = (int32_t)(e - b);
+  }
+}
+__global__ void items_bounds_kernel(long long M, long long n_chunks, const int32_t* __restrict__ key, long long* __restrict__ ptr) {
+  const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k > n_chunks) return;
+  long long lo = 0, hi = M;   // first item of a chunk >= k
+  while (lo < hi) { const long long mid = (lo + hi) >> 1; if ((long long)key[mid] < k) lo = mid + 1; else hi = mid; }
+  ptr[k] = lo;
+}
+__global__ void iota32_kernel(long long n, int32_t* out) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) out[i] = (int32_t)i;
+}
+// The vertices with long in-lists.
+__global__ void heavy_kernel(long long V, const int32_t* __restrict__ din, int32_t* __restrict__ list, long long capacity, unsigned long long* __restrict__ count) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += stride)
+    if (din[v] > HEAVY_DEGREE) {
+      const long long i = (long long)atomicAdd(count, 1ull);
+      if (i < capacity) list[i] = (int32_t)v;
+    }
+}
+
+// One allocation handed out in pieces: the build is mostly allocations otherwise.
+struct Arena {
+  char* base = nullptr;
+  size_t size = 0, used = 0;
+  template <class T> void plan(size_t n) { size += (n * sizeof(T) + 255) / 256 * 256; }
+  bool get() { return cudaMalloc((void**)&base, size > 0 ? size : 256) == cudaSuccess; }
+  template <class T> T* take(size_t n) { T* p = reinterpret_cast<T*>(base + used); used += (n * sizeof(T) + 255) / 256 * 256; return p; }
+  ~Arena() { cudaFree(base); }
+};
+
+template <class T>
+bool take_mem(T** p, size_t n) { return cudaMalloc((void**)p, (n > 0 ? n : 1) * sizeof(T)) == cudaSuccess; }
+
+}  // namespace
+
+// Columns of a row of the store for layer l.
+int resident_row(const taurus_ctx* c, int l) {
+  const int Kp = taurus_round_up(c->dims[l], 4), Hp = taurus_round_up(c->dims[l + 1], 4);
+  if (c->agg_first[l]) return Kp;
+  return c->mode == TAURUS_SAGE_MEAN ? 2 * Hp : Hp;
+}
+
+// In-lists (csc_ptr, csc_src; with csc_eid where a layer is sampled: built already), items of the chunk grid, heavy vertices.
+int build_resident(taurus_ctx* c) {
+  const long long V = c->V, E = c->E, cs = c->chunk_sources, n_chunks = (V + cs - 1) / cs;
+  const int grid = c->sm_count * 8;
+  int v_bit = 1, k_bit = 1;
+  while (v_bit < 31 && (1ll << v_bit) < V) ++v_bit;
+  while (k_bit < 31 && (1ll << k_bit) < n_chunks) ++k_bit;
+  const bool have = c->d_csc_eid != nullptr;
+  int32_t* const none = nullptr;
+  long long* const none64 = nullptr;
+  size_t scan_b = 0, sort_b = 0;
+  cub::DeviceScan::ExclusiveSum(nullptr, scan_b, none64, none64, V + 1);
+  if (!have && E > 0) cub::DeviceRadixSort::SortPairs(nullptr, sort_b, none, none, none, none, E, 0, v_bit);
+  Arena a;
+  a.plan<long long>(V + 1); a.plan<unsigned long long>(3); a.plan<char>(scan_b);
+  if (!have) { a.plan<int32_t>(E); a.plan<int32_t>(E); a.plan<char>(sort_b); }
+  if (!take_mem(&c->d_csc_src, (size_t)E) || !a.get()) return TAURUS_ERR_NOMEM;
+  long long* at = a.take<long long>(V + 1);
+  unsigned long long* heavy = a.take<unsigned long long>(3);
+  void* scan = a.take<char>(scan_b);
+  if (have) {
+    const int rc = build_csc_src_from_eid(c);
+    if (rc) return rc;
+  } else {
+    if (!take_mem(&c->d_csc_ptr, (size_t)V + 1)) return TAURUS_ERR_NOMEM;
+    degrees_kernel<<<grid, 256>>>(V, c->d_din, c->d_csc_ptr);
+    if (cub::DeviceScan::ExclusiveSum(scan, scan_b, c->d_csc_ptr, c->d_csc_ptr, V + 1) != cudaSuccess) return TAURUS_ERR_CUDA;
+    if (E > 0) {
+      int32_t *src = a.take<int32_t>(E), *keys = a.take<int32_t>(E);
+      edge_sources_kernel<<<grid, 256>>>(V, c->d_row_ptr, src);
+      if (cub::DeviceRadixSort::SortPairs(a.take<char>(sort_b), sort_b, c->d_col, keys, src, c->d_csc_src, E, 0, v_bit) != cudaSuccess) return TAURUS_ERR_CUDA;
+    }
+  }
+  cudaMemsetAsync(heavy, 0, 3 * sizeof(*heavy));
+  cudaMemsetAsync(at + V, 0, sizeof(*at));
+  items_kernel<0><<<grid, 256>>>(V, (unsigned)cs, c->d_csc_ptr, c->d_csc_src, at, nullptr, nullptr, nullptr, heavy);
+  if (cub::DeviceScan::ExclusiveSum(scan, scan_b, at, at, V + 1) != cudaSuccess) return TAURUS_ERR_CUDA;
+  long long M = 0;
+  unsigned long long count[2] = {0, 0};
+  if (cudaMemcpy(&M, at + V, sizeof(M), cudaMemcpyDeviceToHost) != cudaSuccess || cudaMemcpy(count, heavy, sizeof(count), cudaMemcpyDeviceToHost) != cudaSuccess)
+    return TAURUS_ERR_CUDA;
+  c->n_heavy = (long long)count[0];
+  c->n_heavy_segments = (long long)count[1];
+  cub::DeviceRadixSort::SortPairs(nullptr, sort_b, none, none, none, none, M, 0, k_bit);
+  Arena t;
+  for (int k = 0; k < 6; ++k) t.plan<int32_t>(M);
+  t.plan<char>(sort_b);
+  if (!t.get()) return TAURUS_ERR_NOMEM;
+  int32_t *key_in = t.take<int32_t>(M), *key_out = t.take<int32_t>(M), *idx_in = t.take<int32_t>(M), *idx_out = t.take<int32_t>(M), *v_in = t.take<int32_t>(M);
+  uint32_t* b_in = t.take<uint32_t>(M);
+  // one block of memory for the items, one for the long in-lists (freed through their first members)
+  int width = 4;
+  for (int l = 0; l < c->L; ++l) width = std::max(width, taurus_round_up(c->agg_first[l] ? c->dims[l] : c->dims[l + 1], 4));
+  if (!take_mem(&c->d_item_v, (size_t)M * 3) || !take_mem(&c->d_item_ptr, (size_t)n_chunks + 1)) return TAURUS_ERR_NOMEM;
+  c->d_item_begin = reinterpret_cast<uint32_t*>(c->d_item_v + M);
+  c->d_item_count = c->d_item_v + 2 * M;
+  items_kernel<1><<<grid, 256>>>(V, (unsigned)cs, c->d_csc_ptr, c->d_csc_src, at, key_in, v_in, b_in, nullptr);
+  iota32_kernel<<<grid, 256>>>(M, idx_in);
+  if (cub::DeviceRadixSort::SortPairs(t.take<char>(sort_b), sort_b, key_in, key_out, idx_in, idx_out, M, 0, k_bit) != cudaSuccess) return TAURUS_ERR_CUDA;
+  items_order_kernel<<<grid, 256>>>(M, idx_out, v_in, b_in, c->d_csc_ptr, c->d_item_v, c->d_item_begin, c->d_item_count);
+  items_bounds_kernel<<<(int)((n_chunks + 1 + 255) / 256), 256>>>(M, n_chunks, key_out, c->d_item_ptr);
+  if (c->n_heavy > 0) {
+    if (!take_mem(&c->d_heavy_list, (size_t)c->n_heavy * 2) || !take_mem(&c->d_heavy, (size_t)c->n_heavy_segments) ||
+        !take_mem(&c->d_heavy_rows, (size_t)c->n_heavy * width)) return TAURUS_ERR_NOMEM;
+    c->d_heavy_left = c->d_heavy_list + c->n_heavy;
+    cudaMemsetAsync(c->d_heavy_rows, 0, (size_t)c->n_heavy * width * sizeof(float));
+    heavy_kernel<<<grid, 256>>>(V, c->d_din, c->d_heavy_list, c->n_heavy, heavy + 2);
+  }
+  c->item_ptr.resize((size_t)n_chunks + 1);
+  c->launches += 8;
+  return cudaMemcpy(c->item_ptr.data(), c->d_item_ptr, (size_t)(n_chunks + 1) * sizeof(long long), cudaMemcpyDeviceToHost) == cudaSuccess ? TAURUS_OK : TAURUS_ERR_CUDA;
+}
+
+void launch_resident_reset(taurus_ctx* c, int layer, cudaStream_t st) {
+  const long long work = std::max<long long>(c->V, (long long)(sizeof(DevCtl) / 8));
+  const int grid = (int)std::min<long long>((work + 255) / 256, (long long)c->sm_count * 8);
+  resident_reset_kernel<<<grid, 256, 0, st>>>(c->V, c->d_din, c->fanout[layer], c->d_pend, c->d_state, c->d_touch, c->d_reload, c->pool_slots, c->d_ctl);
+  c->launches += 1;
+}
+
+void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int K, int Kp, long long src_begin, bool gcn, float* out, cudaStream_t st) {
+  const int grid = (int)std::min<long long>(((long long)n * (Kp >> 2) + 255) / 256, (long long)c->sm_count * 8);
+  store_rows_kernel<<<grid, 256, 0, st>>>(X, ldx, n, K, Kp, src_begin, gcn ? 1 : 0, c->d_row_ptr, out);
+  c->launches += 1;
+}
+
+// Accounting of a push.  `cell`: the chunk's number when it is one cell of the chunk grid, else -1.
+void launch_account(taurus_ctx* c, const ChunkArgs& a, long long cell, cudaStream_t st) {
+  const uint32_t* cmask = c->d_mask_cur ? c->d_cmask : nullptr;
+  int4* heavy = c->n_heavy > 0 && !cmask ? c->d_heavy : nullptr;
+  Items it = {c->d_item_v, c->d_item_begin, c->d_item_count};
+  if (cell >= 0) {
+    const long long i0 = c->item_ptr[(size_t)cell], n = c->item_ptr[(size_t)cell + 1] - i0;
+    const int grid = (int)std::max<long long>(1, std::min<long long>((n + 256 * ITEMS - 1) / (256 * ITEMS), (long long)c->sm_count * 6));
+    account_kernel<false><<<grid, 256, 0, st>>>(a, it, i0, n, cmask, heavy, c->d_heavy_left);
+    c->launches += 1;
+    return;
+  }
+  account_edges_kernel<<<c->sm_count * 8, 256, 0, st>>>(a);
+  const int grid = (int)std::max<long long>(1, std::min<long long>((a.touched_capacity + 256 * ITEMS - 1) / (256 * ITEMS), (long long)c->sm_count * 6));
+  account_kernel<true><<<grid, 256, 0, st>>>(a, it, 0, 0, cmask, heavy, c->d_heavy_left);
+  c->launches += 2;
+}
+
+// Sums and finished rows of the vertices the push completed, at most `bound` (aggregate-first layers: sums into A).
+int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitch, float* A, long long bound, cudaStream_t st) {
+  GatherArgs g;
+  const bool sampled = c->d_mask_cur != nullptr;
+  g.rows = reinterpret_cast<const float4*>(rows); g.pitch = pitch >> 2; g.vec = a.Hp >> 2;
+  g.csc_ptr = c->d_csc_ptr; g.src = sampled ? c->d_kept : c->d_csc_src; g.keep = sampled ? a.fanout : 0;
+  g.done_list = a.done_list;
+  g.heavy = c->n_heavy > 0 && !sampled ? c->d_heavy : nullptr;
+  g.heavy_rows = reinterpret_cast<float4*>(c->d_heavy_rows); g.heavy_left = c->d_heavy_left;
+  g.ctl = a.ctl; g.pc = a.pc;
+  g.bias = reinterpret_cast<const float4*>(a.bias);
+  g.att_s = a.att_s; g.att_tm = a.att_tm; g.att_z = a.att_z;
+  g.A = reinterpret_cast<float4*>(A); g.a_pitch = (c->mode == TAURUS_SAGE_MEAN ? 2 * a.Hp : a.Hp) >> 2;
+  g.dense = a.dense_direct; g.dense_ld = a.dense_ld; g.grad_rows = a.grad_rows; g.grad_ids = a.grad_ids;
+  g.d_out = a.d_out; g.act = a.act; g.mode = a.mode; g.heads = a.heads; g.head_vec = a.head_vec;
+  g.gin_self = a.gin_self; g.leaky = a.leaky;
+  c->launches += 1;
+  // Rows split over as many lanes as they have float4, steps of about 2 KB per warp.  Measured on the passes of 2.45 M
+  // vertices / 124 M edges (48, 100, 256 floats) and 500 k / 12.5 M (64): 48 floats 16 x 1 lanes, 4 rows, 3 steps 4.1 ms,
+  // 4 x 3 lanes 4.3 to 5.1; 64: 2 rows, 4 steps 0.53, others 0.55 to 0.78; 100: 4 rows, 2 steps 8.5, others 8.4 to 8.8
+  // (64 k completed rows of 128 floats 0.68 against 0.75 to 0.94); 256: 2 rows, 3 steps 16.4, others 16.4 to 16.9.
+  const int Hp = a.Hp;
+  if (Hp <= 16) return launch_g2<4, 1, 2, 4>(c, g, bound, st);
+  if (Hp <= 32) return launch_g2<8, 1, 2, 4>(c, g, bound, st);
+  if (Hp <= 48) return launch_g2<16, 1, 4, 3>(c, g, bound, st);
+  if (Hp <= 64) return launch_g2<16, 1, 2, 4>(c, g, bound, st);
+  if (Hp <= 128) return launch_g2<32, 1, 4, 3>(c, g, bound, st);
+  if (Hp <= 256) return launch_g2<32, 2, 2, 4>(c, g, bound, st);
+  if (Hp <= 512) return launch_g2<32, 4, 1, 4>(c, g, bound, st);
+  return launch_g2<32, 8, 1, 3>(c, g, bound, st);
+}
+
+void launch_resident_attention(taurus_ctx* c, cudaStream_t st) {
+  const uint32_t* cmask = c->d_mask_cur ? c->d_cmask : nullptr;
+  const int grid = (int)std::min<long long>((c->V + 7) / 8, (long long)c->sm_count * 8);
+  attention_kernel<1><<<grid, 256, 0, st>>>(c->V, c->heads, c->d_csc_ptr, c->d_csc_src, cmask, c->d_att_s, c->d_att_t, c->leaky, c->d_att_tm, c->d_att_z,
+                                            nullptr, -1, HEAVY_DEGREE);
+  c->launches += 1;
+  if (c->n_heavy > 0) {
+    attention_kernel<8><<<(int)std::min<long long>(c->n_heavy, (long long)c->sm_count * 8), 256, 0, st>>>(
+        c->n_heavy, c->heads, c->d_csc_ptr, c->d_csc_src, cmask, c->d_att_s, c->d_att_t, c->leaky, c->d_att_tm, c->d_att_z, c->d_heavy_list, HEAVY_DEGREE, 4096);
+    attention_kernel<32><<<(int)std::min<long long>(c->n_heavy, (long long)c->sm_count), 1024, 0, st>>>(
+        c->n_heavy, c->heads, c->d_csc_ptr, c->d_csc_src, cmask, c->d_att_s, c->d_att_t, c->leaky, c->d_att_tm, c->d_att_z, c->d_heavy_list, 4096, 0x7fffffff);
+    c->launches += 2;
+  }
+}

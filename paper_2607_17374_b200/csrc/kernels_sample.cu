@@ -50,7 +50,8 @@ static __device__ void sample_positions(unsigned long long seed, int layer, long
 }
 
 __global__ void sample_mask_kernel(long long V, const int32_t* din, const long long* csc_ptr, const uint32_t* csc_eid,
-                                   unsigned long long seed, int layer, int fanout, uint32_t* mask) {
+                                   unsigned long long seed, int layer, int fanout, uint32_t* mask, uint32_t* cmask,   // cmask: the same bits by in-list entry, or NULL
+                                   const int32_t* csc_src, int32_t* kept) {   // kept [V x fanout]: the kept entries' sources, or NULL
   long long stride = (long long)gridDim.x * blockDim.x;
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += stride) {
     int d = din[v];
@@ -60,12 +61,20 @@ __global__ void sample_mask_kernel(long long V, const int32_t* din, const long l
         uint32_t e = csc_eid[base + p];
         atomicOr(&mask[e >> 5], 1u << (e & 31));
       }
+      if (kept) for (int p = 0; p < d; ++p) kept[v * fanout + p] = csc_src[base + p];
+      if (cmask && d > 0) {   // d <= 64 consecutive bits
+        const unsigned long long b = (unsigned long long)base, t = b + (unsigned)d - 1;
+        for (unsigned long long w = b >> 5; w <= t >> 5; ++w)
+          atomicOr(&cmask[w], (w == b >> 5 ? 0xffffffffu << (b & 31) : 0xffffffffu) & (w == t >> 5 ? 0xffffffffu >> (31 - (t & 31)) : 0xffffffffu));
+      }
     } else {
       int pos[TAURUS_MAX_FANOUT];
       sample_positions(seed, layer, v, d, fanout, pos);
       for (int k = 0; k < fanout; ++k) {
         uint32_t e = csc_eid[base + pos[k]];
         atomicOr(&mask[e >> 5], 1u << (e & 31));
+        if (cmask) atomicOr(&cmask[(base + pos[k]) >> 5], 1u << ((base + pos[k]) & 31));
+        if (kept) kept[v * fanout + k] = csc_src[base + pos[k]];
       }
     }
   }
@@ -74,8 +83,9 @@ __global__ void sample_mask_kernel(long long V, const int32_t* din, const long l
 void launch_sample_mask(taurus_ctx* c, int layer, cudaStream_t st) {
   size_t words = (size_t)((c->E + 31) / 32);
   cudaMemsetAsync(c->d_mask, 0, words * sizeof(uint32_t), st);
+  if (c->d_cmask) cudaMemsetAsync(c->d_cmask, 0, words * sizeof(uint32_t), st);
   sample_mask_kernel<<<c->sm_count * 8, 128, 0, st>>>(c->V, c->d_din, c->d_csc_ptr, c->d_csc_eid, c->seed, layer,
-                                                      c->fanout[layer], c->d_mask);
+                                                      c->fanout[layer], c->d_mask, c->d_cmask, c->d_csc_src, c->d_kept);
   c->launches += 1;
 }
 

@@ -52,6 +52,7 @@ __global__ void reset_pool_kernel(long long pool_slots, long long n_ext, long lo
 }
 
 void launch_layer_reset(taurus_ctx* c, int layer, cudaStream_t st) {
+  if (c->resident) { launch_resident_reset(c, layer, st); return; }
   int blocks = c->sm_count * 8;
   cudaMemsetAsync(c->d_ctl, 0, sizeof(DevCtl), st);
   reset_vertices_kernel<<<blocks, 256, 0, st>>>(c->V, c->d_din, c->fanout[layer], c->d_pend, c->d_state, c->d_loc,

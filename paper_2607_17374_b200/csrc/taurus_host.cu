@@ -84,6 +84,8 @@ extern "C" void taurus_destroy(taurus_ctx* c) {
   cudaFree(c->d_af_A); cudaFree(c->d_af_O); cudaFree(c->d_af_X);
   for (int l = 0; l < TAURUS_MAX_LAYERS; ++l) { cudaFree(c->d_Waf[l]); cudaFree(c->d_att_w[l]); }
   cudaFree(c->d_att_s); cudaFree(c->d_att_t); cudaFree(c->d_att_max); cudaFree(c->d_att_tm); cudaFree(c->d_att_z);
+  cudaFree(c->d_store); cudaFree(c->d_cmask); cudaFree(c->d_kept); cudaFree(c->d_item_v); cudaFree(c->d_item_ptr);
+  cudaFree(c->d_heavy_list); cudaFree(c->d_heavy); cudaFree(c->d_heavy_rows);
   cudaFree(c->d_csc_ptr); cudaFree(c->d_csc_eid); cudaFree(c->d_mask); cudaFree(c->d_vtmp); cudaFree(c->d_rank_hist);
   cudaFree(c->d_gdst); cudaFree(c->d_gedge); cudaFree(c->d_geid); cudaFree(c->d_gmask);
   cudaFree(c->d_ctl); cudaFree(c->d_chunk_log); cudaFree(c->d_reload_hist);
@@ -241,8 +243,22 @@ static int init_impl(taurus_ctx* c, const taurus_graph* g, const taurus_model* m
   // per-vertex state
   ALLOC(c->d_pend, V); ALLOC(c->d_state, V); ALLOC(c->d_loc, V); ALLOC(c->d_touch, V); ALLOC(c->d_reload, V);
   ALLOC(c->d_rank_hist, (V + 63) / 64);
+  // A pool that holds every vertex keeps the rows the sources send instead of accumulators (kernels_resident.cu), where the
+  // in-lists and their build fit beside them; else the push form.
+  const bool grouping = !(c->flags & TAURUS_FLAG_NO_GROUPING);
+  int store_floats = 0;
+  for (int l = 0; l < c->L; ++l) store_floats = std::max(store_floats, resident_row(c, l));
+  int max_fanout = 0;
+  for (int l = 0; l < c->L; ++l) max_fanout = std::max(max_fanout, c->fanout[l]);
+  if (grouping && c->pool_slots >= V && E + V < (1ll << 31) && V * std::max(max_fanout, 1) < (1ll << 31)) {
+    const double rows_b = (double)V * store_floats * 4.0 + (double)c->drain_rows * (c->Hmax + (af_kmax > 0 ? 2 * af_kmax : 0)) * 4.0;
+    const double graph_b = (double)(E + V) * (12.0 + 36.0) + (double)E * 8.0 + (double)V * max_fanout * 4.0;   // in-lists and items, and their build
+    CU(cudaMemGetInfo(&free_b, &total_b));
+    c->resident = rows_b + graph_b + 2e9 < 0.95 * (double)free_b || rows_b + graph_b < 0.5 * (double)free_b;
+  }
   // pool, hub store
-  ALLOC(c->d_acc, (size_t)(c->pool_slots + c->hub_count) * c->Hmax);
+  if (c->resident) ALLOC(c->d_store, (size_t)V * store_floats);
+  else ALLOC(c->d_acc, (size_t)(c->pool_slots + c->hub_count) * c->Hmax);
   {
     // a push of at most chunk_sources sources touches at most its edges plus its own vertices
     long long max_edges = max_window_edges(c);
@@ -250,8 +266,10 @@ static int init_impl(taurus_ctx* c, const taurus_graph* g, const taurus_model* m
     c->touched_capacity = std::min<long long>(V, max_edges + c->chunk_sources);
     ALLOC(c->d_touched_list, c->touched_capacity);
   }
-  ALLOC(c->d_owner, c->pool_slots); ALLOC(c->d_free_stack, c->pool_slots); ALLOC(c->d_need_list, c->pool_slots);
-  ALLOC(c->d_slot_epoch, c->pool_slots);   // written at every slot hand-out, also when no eviction can happen
+  if (!c->resident) {
+    ALLOC(c->d_owner, c->pool_slots); ALLOC(c->d_free_stack, c->pool_slots); ALLOC(c->d_need_list, c->pool_slots);
+    ALLOC(c->d_slot_epoch, c->pool_slots);   // written at every slot hand-out, also when no eviction can happen
+  }
   const bool can_evict = c->pool_slots < V - c->hub_count;
   if (can_evict) {   // a chunk evicts at most what it needs, and it needs at most what it touches
     c->victim_capacity = std::min<long long>(c->pool_slots, c->touched_capacity);
@@ -311,11 +329,10 @@ static int init_impl(taurus_ctx* c, const taurus_graph* g, const taurus_model* m
     ALLOC(c->d_af_A, (size_t)c->drain_rows * af_kmax * (sage ? 2 : 1));
     // rows behind a chunk's finished ones are read (and their products dropped) by the last row tile: keep them finite
     CU(cudaMemset(c->d_af_A, 0, (size_t)c->drain_rows * af_kmax * (sage ? 2 : 1) * sizeof(float)));
-    if (sage) ALLOC(c->d_af_X, (size_t)V * af_kmax);
+    if (sage && !c->resident) ALLOC(c->d_af_X, (size_t)V * af_kmax);
   }
   // In-lists (ascending source id).  Sampled layers pick in-list positions; the host store files an evicted row by the
   // next sender of its vertex, read from the vertex's in-list.
-  const bool grouping = !(c->flags & TAURUS_FLAG_NO_GROUPING);
   const bool need_src = c->n_ext > 0;
   if (any_sampled || (need_src && !grouping)) {
     int rc = build_in_edge_order(c);
@@ -335,8 +352,13 @@ static int init_impl(taurus_ctx* c, const taurus_graph* g, const taurus_model* m
       src_from_groups = true;
     }
   }
+  if (c->resident) {
+    int rc = build_resident(c);
+    if (rc) { cuda_ok(cudaGetLastError(), "build_resident"); return rc; }
+    if (any_sampled) { ALLOC(c->d_cmask, (E + 31) / 32); ALLOC(c->d_kept, (size_t)V * max_fanout); }
+  }
   // destination-grouped edge order of the chunk grid
-  if (grouping) {
+  if (grouping && !c->resident) {
     int rc = build_grouped_order(c, any_sampled, src_from_groups);
     if (rc) { cuda_ok(cudaGetLastError(), "build_grouped_order"); return rc; }
     if (any_sampled) ALLOC(c->d_gmask, (E + 31) / 32);
@@ -466,7 +488,7 @@ static ChunkArgs make_args(taurus_ctx* c, long long s, long long e) {
   ChunkArgs a;
   const int l = c->layer;
   a.row_ptr = c->d_row_ptr; a.col = c->d_col; a.din = c->d_din; a.mask = c->d_mask_cur;
-  a.pend = c->d_pend; a.state = c->d_state; a.loc = c->d_loc; a.touch = c->d_touch; a.reload_count = c->d_reload;
+  a.pend = c->d_pend; a.hub = c->hub_count > 0 ? c->d_hub : nullptr; a.resident = c->resident ? 1 : 0; a.state = c->d_state; a.loc = c->d_loc; a.touch = c->d_touch; a.reload_count = c->d_reload;
   a.acc = c->d_acc; a.owner = c->d_owner; a.free_stack = c->d_free_stack; a.need_list = c->d_need_list; a.slot_epoch = c->d_slot_epoch;
   a.slot_touch = c->d_slot_touch; a.slot_pend = c->d_slot_pend;
   a.touched_list = c->d_touched_list; a.touched_capacity = c->touched_capacity;
@@ -515,24 +537,9 @@ static int finish_run_append(taurus_ctx* c) {
   return TAURUS_OK;
 }
 
-static int finish_chunk(taurus_ctx* c, cudaStream_t st) {
-  if (!c->pending) return TAURUS_OK;
-  c->pending = false;
-  const PendingChunk& p = *c->pend_chunk;
-  const ChunkArgs& a = p.a;
-  const int l = p.layer;
-  cudaEvent_t* pev = p.timed_index >= 0 && c->timing != 2 ? &c->phase_ev[(size_t)p.timed_index * TAURUS_PUSH_EVENTS] : nullptr;
-  if (c->pipelined) {
-    CU(cudaStreamWaitEvent(st, c->xfer_done, 0));   // reloaded partial sums have been added to the chunk's rows
-    if (pev) cudaEventRecord(pev[8], st);           // (without transfers the finalise follows event 7 directly)
-  }
-  if (a.dense_half >= 0 && c->half_used[a.dense_half]) CU(cudaStreamWaitEvent(st, c->out_done[a.dense_half], 0));
-  if (p.af) {
-    int rc = launch_af_finalise(c, a, l, std::min<long long>(p.bound, a.grad_cap), st);
-    if (rc) { c->h_ctl->error = rc; return rc; }   // the chunk is half applied: the layer has to be begun again
-  } else {
-    launch_finalise(c, a, st);
-  }
+// A chunk's finished rows on their way out of the graduation buffer (nothing to do where they sit in the caller's matrix or
+// wait for a drain).
+static int hand_off(taurus_ctx* c, const ChunkArgs& a, int l, long long bound, cudaStream_t st) {
   int run_rc = TAURUS_OK;
   if (a.dense_half >= 0 && c->dense_out) {   // hand this chunk's rows to the output stream (matrix in pinned host memory)
     const int h = a.dense_half, d_out = c->dims[l + 1];
@@ -552,11 +559,33 @@ static int finish_chunk(taurus_ctx* c, cudaStream_t st) {
     if (!run_rc) {
       CU(cudaStreamWaitEvent(c->out_stream, c->fin_done[h], 0));
       const long long off = a.grad_off;
-      run_rc = runs_phase1(c->run_out, c->d_grad_ids + off, c->d_grad_rows + (size_t)off * a.Hout, a.Hout, std::min(p.bound, a.grad_cap),
+      run_rc = runs_phase1(c->run_out, c->d_grad_ids + off, c->d_grad_rows + (size_t)off * a.Hout, a.Hout, std::min(bound, a.grad_cap),
                            &c->d_ctl->out_count[h], 0, c->out_stream);
       if (!run_rc) c->run_pending_half = h;
     }
   }
+  return run_rc;
+}
+
+static int finish_chunk(taurus_ctx* c, cudaStream_t st) {
+  if (!c->pending) return TAURUS_OK;
+  c->pending = false;
+  const PendingChunk& p = *c->pend_chunk;
+  const ChunkArgs& a = p.a;
+  const int l = p.layer;
+  cudaEvent_t* pev = p.timed_index >= 0 && c->timing != 2 ? &c->phase_ev[(size_t)p.timed_index * TAURUS_PUSH_EVENTS] : nullptr;
+  if (c->pipelined) {
+    CU(cudaStreamWaitEvent(st, c->xfer_done, 0));   // reloaded partial sums have been added to the chunk's rows
+    if (pev) cudaEventRecord(pev[8], st);           // (without transfers the finalise follows event 7 directly)
+  }
+  if (a.dense_half >= 0 && c->half_used[a.dense_half]) CU(cudaStreamWaitEvent(st, c->out_done[a.dense_half], 0));
+  if (p.af) {
+    int rc = launch_af_finalise(c, a, l, std::min<long long>(p.bound, a.grad_cap), st);
+    if (rc) { c->h_ctl->error = rc; return rc; }   // the chunk is half applied: the layer has to be begun again
+  } else {
+    launch_finalise(c, a, st);
+  }
+  const int run_rc = hand_off(c, a, l, p.bound, st);
   if (pev) cudaEventRecord(pev[9], st);
   CU(cudaGetLastError());
   return run_rc;
@@ -637,6 +666,44 @@ static int push_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const fl
   { int rc = stage_chunk(c, features, src_runs, src_begin, src_end, K, st, &X, &xbuf); if (rc) return rc; }
   if (timing) cudaEventRecord(pev[1], st);
   ChunkArgs a = make_args(c, src_begin, src_end);
+  if (c->resident) {
+    // rows into the store, accounting, sums and finished rows of the vertices this chunk completes
+    const bool af = c->agg_first[l];
+    const int w = resident_row(c, l);
+    float* rows = c->d_store + (size_t)src_begin * w;
+    if (af) {
+      a.Hout = a.Hp; a.Hp = w; a.self_bias = 0;
+      launch_store_rows(c, X, ldx, n, c->dims[l], w, src_begin, c->mode == TAURUS_GCN_SYM, rows, st);   // (GAT: pass 1 handed the input rows back, pitch dims[l + 1])
+    } else if (gat) {
+      launch_store_rows(c, X, ldx, n, K, w, src_begin, false, rows, st);
+    } else if (project_tc_usable(c, l, X, ldx)) {
+      int rc = launch_project_tc(c, l, X, ldx, src_begin, n, rows, st);
+      if (rc) return rc;
+    } else {
+      launch_project_simt(c, l, X, ldx, src_begin, n, rows, st);
+    }
+    if (xbuf >= 0) { CU(cudaEventRecord(c->x_free[xbuf], st)); c->x_used[xbuf] = true; }
+    if (timing) cudaEventRecord(pev[2], st);
+    if (a.dense_half >= 0 && c->half_used[a.dense_half]) CU(cudaStreamWaitEvent(st, c->out_done[a.dense_half], 0));
+    const bool cell = src_begin % c->chunk_sources == 0 && src_end == std::min<long long>(c->V, src_begin + c->chunk_sources);
+    launch_account(c, a, cell ? src_begin / c->chunk_sources : -1, st);
+    if (timing) cudaEventRecord(pev[3], st);
+    if (scatter_timing) cudaEventRecord(pev[5], st);
+    { int rc = launch_gather(c, a, c->d_store, w, af ? c->d_af_A : nullptr, std::min<long long>(bound, a.grad_cap), st); if (rc) { c->h_ctl->error = rc; return rc; } }
+    if (scatter_timing) cudaEventRecord(pev[6], st);
+    if (timing) cudaEventRecord(pev[7], st);
+    if (af) {
+      int rc = launch_af_finalise(c, a, l, std::min<long long>(bound, a.grad_cap), st);
+      if (rc) { c->h_ctl->error = rc; return rc; }   // the chunk is half applied: the layer has to be begun again
+    }
+    const int rc = hand_off(c, a, l, bound, st);
+    if (timing) cudaEventRecord(pev[9], st);
+    CU(cudaGetLastError());
+    c->next_src = src_end;
+    c->chunk_seq += 1;
+    if (!halves && !direct_dense) c->ub_since_drain += bound;
+    return rc;
+  }
   // S2: projection (GAT: already done in pass 1; rows narrower than their padded width are repacked).
   // Aggregate-first layers push the (scaled, padded) input rows instead and transform the finished rows in S7.
   bool x_in_use = false;
@@ -668,10 +735,10 @@ static int push_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const fl
     if (K == a.Hp && (reinterpret_cast<uintptr_t>(X) & 15) == 0) { a.PT = X; x_in_use = true; }
     else launch_gat_repack(c, X, n, K, a.Hp, st);
   } else if (project_tc_usable(c, l, X, ldx)) {
-    int rc = launch_project_tc(c, l, X, ldx, src_begin, n, st);
+    int rc = launch_project_tc(c, l, X, ldx, src_begin, n, c->d_PT, st);
     if (rc) return rc;
   } else {
-    launch_project_simt(c, l, X, ldx, src_begin, n, st);
+    launch_project_simt(c, l, X, ldx, src_begin, n, c->d_PT, st);
   }
   if (xbuf >= 0 && !x_in_use) { CU(cudaEventRecord(c->x_free[xbuf], st)); c->x_used[xbuf] = true; }
   if (timing) cudaEventRecord(pev[2], st);
@@ -741,10 +808,10 @@ static int gat_project_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, c
     return TAURUS_OK;
   }
   if (project_tc_usable(c, l, X, K)) {
-    int rc = launch_project_tc(c, l, X, K, src_begin, n, st);
+    int rc = launch_project_tc(c, l, X, K, src_begin, n, c->d_PT, st);
     if (rc) return rc;
   } else {
-    launch_project_simt(c, l, X, K, src_begin, n, st);
+    launch_project_simt(c, l, X, K, src_begin, n, c->d_PT, st);
   }
   if (xbuf >= 0) { CU(cudaEventRecord(c->x_free[xbuf], st)); c->x_used[xbuf] = true; }
   launch_gat_split(c, n, Hp, d_out, src_begin, hprime_out, ld, st);

@@ -36,6 +36,9 @@ struct ChunkCtl {
   unsigned int grid_arrivals; // make-room step: blocks that reached its barriers so far
   unsigned int done_blocks;   // completion list: blocks that have finished
   int32_t room_go, room_fail; // make-room step: the plan went through / the host store could not take the victims
+  int32_t heavy_count;    // resident pools: segments of long in-lists to sum
+  long long grad_base;    // resident pools: first row of the chunk's finished rows in the graduation buffer
+  unsigned long long acc[8];  // resident pools: sums over the blocks of the account kernel
   long long alloc_base;   // need-list entry i takes free_stack[alloc_base - 1 - i]
   // Victim select, level by level (level 0 scans the pool, deeper levels the candidates the level above left):
   long long sel_k[TAURUS_SEL_LEVELS + 1];               // rank still to resolve among the keys entering the level
@@ -49,6 +52,7 @@ struct ChunkCtl {
 // the host.  One per context.
 struct DevCtl {
   int32_t error;            // sticky TAURUS_ERR_* found on the device
+  int32_t heavy_rows;       // resident pools: partial rows of long in-lists handed out in this layer
   int32_t ext_ret_count[2]; // extents emptied by the row transfers of the chunks of each parity, waiting to go back on the free stack
   long long free_top;       // entries on the free-slot stack
   long long ext_free_top;   // entries on the free-extent stack of the host store
@@ -72,6 +76,7 @@ struct ChunkArgs {
   // per-vertex state
   int32_t* pend;
   uint8_t* state;
+  const uint8_t* hub;       // [V] 1 = hub-store vertex; NULL without hubs
   int32_t* loc;             // pool slot / hub row (>= pool_slots) / host row while EVICTED; -1 = none
   int32_t* touch;           // chunk epoch of the last touch
   int32_t* reload_count;
@@ -155,6 +160,7 @@ struct ChunkArgs {
   // the padded INPUT width, and the transform runs on the finished rows
   int32_t Hout;             // padded output width (= Hp for project-first layers)
   int32_t self_rows;        // 1: the scatter adds a self row; 0: it only counts the self message (the self term is added after the transform)
+  int32_t resident;         // 1: resident pool, the account kernel has done the graduation bookkeeping
   int32_t self_bias;        // 1: the self row carries the bias (project-first); 0: the bias is added after the transform
 };
 
@@ -223,6 +229,21 @@ struct taurus_ctx {
   float* d_af_O = nullptr;      // [drain_rows x Hmax] transform output when its place in the graduation buffer is known only on the device
   float* d_af_X = nullptr;      // [V x Kp] SAGE: the (padded) input row of every vertex, kept from its chunk until it completes;
                                 //   the scatter reads the chunk's rows from here and the transform multiplies them by W_self
+  // resident pools (every vertex has a slot, nothing is ever evicted): see kernels_resident.cu
+  bool resident = false;
+  float* d_store = nullptr;        // [V x widest row] the rows the sources send, filed under their source
+  uint32_t* d_cmask = nullptr;     // sampled layers: kept entries of the in-lists, as bits,
+  int32_t* d_kept = nullptr;       //   and as [V x fanout] sources
+  int32_t* d_item_v = nullptr;     // items of the chunk grid: vertex, first in-list entry, entries
+  uint32_t* d_item_begin = nullptr;
+  int32_t* d_item_count = nullptr;
+  long long* d_item_ptr = nullptr; // [grid chunks + 1]
+  std::vector<long long> item_ptr;
+  int32_t* d_heavy_list = nullptr; // vertices with long in-lists
+  long long n_heavy = 0, n_heavy_segments = 0;
+  int4* d_heavy = nullptr;         // segments of one push
+  int32_t* d_heavy_left = nullptr; // [n_heavy] segments still to come
+  float* d_heavy_rows = nullptr;   // [n_heavy x widest summed row] partial sums, zero between vertices
   int32_t* d_free_stack = nullptr;
   int32_t* d_need_list = nullptr;
   int32_t* d_touched_list = nullptr;
@@ -350,7 +371,7 @@ void launch_gat_repack(taurus_ctx* c, const float* X, int n, int d_out, int Hp, 
 // ---- kernels_scatter.cu
 void launch_scatter(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);
 // ---- kernels_gemm_simt.cu
-void launch_project_simt(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, cudaStream_t st);
+void launch_project_simt(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, cudaStream_t st);
 void launch_gemm_plain_simt(taurus_ctx* c, const float* W, int ldw, int N, const float* X, int ldx, int K, int n, float* out, long long ld_out,
                             cudaStream_t st);   // out = X . W[:, 0..N), W row-major with pitch ldw
 // ---- kernels_gemm_tc.cu
@@ -373,7 +394,15 @@ int launch_gemm_plain_tc(taurus_ctx* c, void* image, int col0, int N, const floa
 int prepare_tc_weights(taurus_ctx* c, void** slot, const std::vector<float>& cat, int K, int N);   // image of cat [K x N] into *slot
 void free_tc_weights(taurus_ctx* c);
 bool project_tc_usable(const taurus_ctx* c, int layer, const float* X, int ldx);
-int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, cudaStream_t st);
+int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, cudaStream_t st);   // out [n x projection width], 16-byte aligned
+// ---- kernels_resident.cu
+int resident_row(const taurus_ctx* c, int layer);                            // floats per row of the store
+int build_resident(taurus_ctx* c);
+void launch_resident_reset(taurus_ctx* c, int layer, cudaStream_t st);
+void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int K, int Kp, long long src_begin, bool gcn, float* out, cudaStream_t st);
+void launch_account(taurus_ctx* c, const ChunkArgs& a, long long cell, cudaStream_t st);
+int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitch, float* A, long long bound, cudaStream_t st);
+void launch_resident_attention(taurus_ctx* c, cudaStream_t st);
 // ---- kernels_group.cu
 int build_grouped_order(taurus_ctx* c, bool keep_edge_ids, bool fill_csc_src);   // fill_csc_src: also writes csc_src (needs csc_ptr)
 void launch_group_mask(taurus_ctx* c, cudaStream_t st);
