@@ -94,14 +94,12 @@ __global__ void rs_collect_kernel(const MoveSeg* __restrict__ segs, const int32_
   }
 }
 
-// Writes sorted runs: ids and rows in id order, sequentially, into the store (the id ranges are contiguous, so
-// buffers sorted together come out range after range).
-__global__ void rs_gather_kernel(long long n, const int32_t* __restrict__ sid, const int32_t* __restrict__ sidx,
-                                 const float* __restrict__ prows, int width, int32_t* __restrict__ run_ids,
-                                 float* __restrict__ run_rows) {
+// Writes the rows of sorted runs in id order, sequentially, into the store (the id ranges are contiguous, so buffers
+// sorted together come out range after range).  Their ids, sorted already, follow as one copy: written from here, 4 bytes
+// a row into pinned memory, they were what bounded this kernel.
+__global__ void rs_gather_kernel(long long n, const int32_t* __restrict__ sidx, const float* __restrict__ prows, int width, float* __restrict__ run_rows) {
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
-    if (rs_lane() == 0) run_ids[i] = sid[i];
     copy_row(run_rows + (size_t)i * width, prows + (size_t)sidx[i] * width, width);
   }
 }
@@ -114,14 +112,14 @@ __global__ void rs_place_kernel(long long n, const int32_t* __restrict__ sid, co
     copy_row(out + (size_t)(sid[i] - s) * ld, srows + (size_t)i * width, width);
 }
 
-// The same for a store in device memory: slice q of the chunk (rows src .. src + n of the store, their ids staged
-// at dst ..) is read in place, without a staging copy of the rows.
-__global__ void rs_place_slices_kernel(const MoveSeg* __restrict__ segs, const int32_t* __restrict__ sid, const float* __restrict__ store,
+// The same for a store in device memory: slice q of the chunk (rows src .. src + n of the store, ids beside them) is read
+// in place, without staging copies (one small copy of ids per slice took 2.6 us of the stream, thirty a chunk).
+__global__ void rs_place_slices_kernel(const MoveSeg* __restrict__ segs, const int32_t* __restrict__ ids, const float* __restrict__ store,
                                        int width, long long s, float* __restrict__ out, long long ld) {
   const MoveSeg sg = segs[blockIdx.y];
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < sg.n; i += warps)
-    copy_row(out + (size_t)(sid[sg.dst + i] - s) * ld, store + (size_t)(sg.src + i) * width, width);
+    copy_row(out + (size_t)(ids[sg.src + i] - s) * ld, store + (size_t)(sg.src + i) * width, width);
 }
 
 int bits_for(long long values) {   // bits needed to tell `values` different keys apart
@@ -142,8 +140,8 @@ struct taurus_runs {
   // run store
   float* store_dev = nullptr;    // what kernels write: device memory, or the device alias of store_host
   float* store_host = nullptr;   // pinned + mapped (host kind only)
-  int32_t* h_ids = nullptr;      // ids of all runs, pinned + mapped
-  int32_t* d_ids = nullptr;      // device alias of h_ids
+  int32_t* h_ids = nullptr;      // ids of all runs, pinned
+  int32_t* d_ids = nullptr;      // device kind: the same in device memory
   long long store_top = 0;
   std::vector<RunRec> dir;
   std::vector<std::vector<int>> by_part;
@@ -205,7 +203,7 @@ extern "C" void taurus_runs_destroy(taurus_runs* r) {
   cudaFreeHost(r->h_ids); cudaFreeHost(r->h_cnt); cudaFreeHost(r->h_segs);
   cudaFree(r->d_key); cudaFree(r->d_key_s); cudaFree(r->d_idx); cudaFree(r->d_idx_s); cudaFree(r->d_cnt); cudaFree(r->d_segs);
   cudaFree(r->d_fkeys); cudaFree(r->d_fvals); cudaFree(r->d_sid); cudaFree(r->d_sidx); cudaFree(r->d_tmp);
-  cudaFree(r->d_stage_rows); cudaFree(r->d_stage_ids);
+  cudaFree(r->d_stage_rows); cudaFree(r->d_stage_ids); cudaFree(r->d_ids);
   for (int i = 0; i < SEG_RING; ++i) if (r->seg_done[i]) cudaEventDestroy(r->seg_done[i]);
   if (r->cnt_ready) cudaEventDestroy(r->cnt_ready);
   if (r->write_done) cudaEventDestroy(r->write_done);
@@ -244,7 +242,7 @@ extern "C" int taurus_runs_create(taurus_runs** out, const taurus_runs_config* c
     RALLOC(r->store_dev, (size_t)r->store_rows * w);
   }
   RPINNED(r->h_ids, (size_t)r->store_rows);
-  if (cudaHostGetDevicePointer((void**)&r->d_ids, r->h_ids, 0) != cudaSuccess) { cudaGetLastError(); taurus_runs_destroy(r); return TAURUS_ERR_CUDA; }
+  if (r->kind == TAURUS_RUNS_DEVICE) RALLOC(r->d_ids, r->store_rows);
   RALLOC(r->d_key, r->max_append); RALLOC(r->d_key_s, r->max_append); RALLOC(r->d_idx, r->max_append); RALLOC(r->d_idx_s, r->max_append);
   RALLOC(r->d_cnt, r->P + 2);
   RPINNED(r->h_cnt, (size_t)r->P + 2);
@@ -352,7 +350,9 @@ static int flush_many(taurus_runs* r, const std::vector<long long>& parts, cudaS
     RCU(cub::DeviceRadixSort::SortPairs(r->d_tmp, tb, r->d_fkeys, r->d_sid, r->d_fvals, r->d_sidx, (int)m, 0, r->id_bits, st));
     const long long off = r->store_top;
     const int grid = (int)std::min<long long>((m * 32 + 255) / 256, (long long)r->sm_count * 8);
-    rs_gather_kernel<<<grid, 256, 0, st>>>(m, r->d_sid, r->d_sidx, r->d_prows, r->width, r->d_ids + off, r->store_dev + (size_t)off * r->width);
+    rs_gather_kernel<<<grid, 256, 0, st>>>(m, r->d_sidx, r->d_prows, r->width, r->store_dev + (size_t)off * r->width);
+    RCU(cudaMemcpyAsync(r->h_ids + off, r->d_sid, (size_t)m * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    if (r->d_ids) RCU(cudaMemcpyAsync(r->d_ids + off, r->d_sid, (size_t)m * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
     r->launches += 4;
     for (size_t q = first; q < at; ++q) {
       const long long p = parts[q], n = r->fill[(size_t)p];
@@ -461,13 +461,12 @@ int runs_read_into(taurus_runs* r, long long s, long long e, float* out, long lo
     int nseg = 0;
     long long most = 0;
     for (const Slice& sl : slices) {
-      RCU(cudaMemcpyAsync(r->d_stage_ids + at, r->h_ids + sl.off, (size_t)sl.n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
       hs[nseg++] = MoveSeg{sl.off, sl.n, at};
       at += sl.n; most = std::max(most, sl.n);
     }
     { int rc2 = push_segs(r, slot, nseg, st); if (rc2) return rc2; }
     const int gx = (int)std::max<long long>(1, std::min<long long>((most * 32 + 255) / 256, std::max<long long>(1, (long long)r->sm_count * 8 / nseg)));
-    rs_place_slices_kernel<<<dim3(gx, nseg), 256, 0, st>>>(ds, r->d_stage_ids, r->store_dev, r->width, s, out, ld);
+    rs_place_slices_kernel<<<dim3(gx, nseg), 256, 0, st>>>(ds, r->d_ids, r->store_dev, r->width, s, out, ld);
     { int rc2 = release_seg_slot(r, slot, st); if (rc2) return rc2; }
   } else {
     for (const Slice& sl : slices) {
