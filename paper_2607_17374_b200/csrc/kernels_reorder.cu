@@ -80,32 +80,39 @@ __global__ void ro_rank_kernel(long long V, const int32_t* order, int32_t* rank,
     pos[order[i]] = (double)i;
   }
 }
-// J = sum_v 1/d(v) * sum over v's in-neighbours and v itself of (pos(u) - mu(v))^2; span = sum_v (max - min) of ranks.
-__global__ void ro_measure_kernel(long long V, const long long* in_ptr, const int32_t* in_src, const double* pos, const double* mu,
-                                  const int32_t* rank, double* J, unsigned long long* span) {
+// J = sum_v 1/d(v) * sum over v's in-neighbours and v itself of (pos(u) - mu(v))^2 with mu(v) their mean (the optimum for
+// these positions); span = sum_v (max - min) of ranks.  Two sweeps over the in-list in one kernel: the second finds its
+// scattered positions in L1 / L2 (as two kernels the mean went through memory and the positions were fetched twice:
+// 170 us for 400 k vertices, 5.8 M edges).
+__global__ void ro_measure_kernel(long long V, const long long* __restrict__ in_ptr, const int32_t* __restrict__ in_src, const double* __restrict__ pos,
+                                  double* J, unsigned long long* span) {
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
   double jsum = 0.0;
   unsigned long long ssum = 0;
   for (long long v = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < V; v += warps) {
     const long long b = in_ptr[v], e = in_ptr[v + 1];
-    const double m = mu[v];
-    double s = 0.0;
-    int lo = rank[v], hi = rank[v];
+    const double own = pos[v], d = (double)(e - b) + 1.0;
+    double x0 = own, s = 0.0, lo = own, hi = own;   // x0: the lane's first entry, still held in the second sweep
     for (long long p = b + lane(); p < e; p += 32) {
-      const int u = in_src[p];
-      const double dlt = pos[u] - m;
-      s += dlt * dlt;
-      const int ru = rank[u];
-      lo = ru < lo ? ru : lo; hi = ru > hi ? ru : hi;
+      const double x = pos[in_src[p]];
+      if (p < b + 32) x0 = x;
+      s += x;
+      lo = x < lo ? x : lo; hi = x > hi ? x : hi;   // positions are the ranks themselves
     }
     s = warp_sum(s);
+    const double m = (own + s) / d;
+    double q = 0.0;
+    for (long long p = b + lane(); p < e; p += 32) {
+      const double dlt = (p < b + 32 ? x0 : pos[in_src[p]]) - m;
+      q += dlt * dlt;
+    }
+    q = warp_sum(q);
     for (int o = 16; o; o >>= 1) {
-      int l2 = __shfl_xor_sync(FULL, lo, o), h2 = __shfl_xor_sync(FULL, hi, o);
+      const double l2 = __shfl_xor_sync(FULL, lo, o), h2 = __shfl_xor_sync(FULL, hi, o);
       lo = l2 < lo ? l2 : lo; hi = h2 > hi ? h2 : hi;
     }
     if (lane() == 0) {
-      const double dv = pos[v] - m;
-      jsum += (s + dv * dv) / ((double)(e - b) + 1.0);
+      jsum += (q + (own - m) * (own - m)) / d;
       ssum += (unsigned long long)(hi - lo);
     }
   }
@@ -115,15 +122,19 @@ __global__ void ro_measure_kernel(long long V, const long long* in_ptr, const in
   }
 }
 
-struct Buffers {
-  std::vector<void*> ptrs;
-  ~Buffers() { for (void* p : ptrs) cudaFree(p); }
-  template <class T> T* get(size_t n) {
-    void* p = nullptr;
-    if (cudaMalloc(&p, (n > 0 ? n : 1) * sizeof(T)) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    ptrs.push_back(p);
-    return static_cast<T*>(p);
+// One allocation, handed out in pieces once every piece is planned: thirty allocations and as many frees, which wait for
+// the device each, took longer than the kernels between them.
+struct Arena {
+  char* base = nullptr;
+  size_t size = 0;
+  template <class T> size_t plan(size_t n) { const size_t at = size; size += (n * sizeof(T) + 255) / 256 * 256 + 256; return at; }
+  bool get() {
+    if (cudaMalloc((void**)&base, size > 0 ? size : 256) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
   }
+  template <class T> T* at(size_t off) const { return reinterpret_cast<T*>(base + off); }
+  ~Arena() { cudaFree(base); }
 };
 
 }  // namespace
@@ -139,30 +150,37 @@ extern "C" int taurus_reorder(int64_t V, int64_t E, const int64_t* row_ptr, cons
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int grid = sms * 8;
-  Buffers B;
-  long long* d_row = B.get<long long>((size_t)V + 1);
-  int32_t* d_col = B.get<int32_t>((size_t)E);
-  int32_t* d_din = B.get<int32_t>((size_t)V);
-  int32_t* d_init = initial_rank ? B.get<int32_t>((size_t)V) : nullptr;
-  long long* d_inptr = B.get<long long>((size_t)V + 1);
-  int32_t* d_insrc = B.get<int32_t>((size_t)E);
-  int32_t* d_srcedge = B.get<int32_t>((size_t)E);
-  int32_t* d_keys = B.get<int32_t>((size_t)E);
-  double* d_r = B.get<double>((size_t)V);
-  double* d_rsorted = B.get<double>((size_t)V);
-  double* d_mu = B.get<double>((size_t)V);
-  double* d_w1 = B.get<double>((size_t)V);
-  double* d_w2 = B.get<double>((size_t)V);
-  double* d_pos = B.get<double>((size_t)V);
-  int32_t* d_ids = B.get<int32_t>((size_t)V);
-  int32_t* d_order = B.get<int32_t>((size_t)V);
-  int32_t* d_rank = B.get<int32_t>((size_t)V);
-  double* d_J = B.get<double>(1);
-  unsigned long long* d_span = B.get<unsigned long long>(1);
-  int* d_bad = B.get<int>(1);
-  if (!d_row || !d_col || !d_din || (initial_rank && !d_init) || !d_inptr || !d_insrc || !d_srcedge || !d_keys || !d_r ||
-      !d_rsorted || !d_mu || !d_w1 || !d_w2 || !d_pos || !d_ids || !d_order || !d_rank || !d_J || !d_span || !d_bad)
-    return TAURUS_ERR_NOMEM;
+  int end_bit = 1;
+  while (end_bit < 31 && (1ll << end_bit) < V) ++end_bit;
+  size_t t1 = 0, t2 = 0, t3 = 0;
+  {
+    long long* const n64 = nullptr;
+    int32_t* const n32 = nullptr;
+    double* const nd = nullptr;
+    cub::DeviceScan::ExclusiveSum(nullptr, t1, n64, n64, V + 1, st);
+    if (E > 0) cub::DeviceRadixSort::SortPairs(nullptr, t2, n32, n32, n32, n32, E, 0, end_bit, st);
+    cub::DeviceRadixSort::SortPairs(nullptr, t3, nd, nd, n32, n32, V, 0, 64, st);
+  }
+  size_t tmp_bytes = t1 > t2 ? t1 : t2;
+  if (t3 > tmp_bytes) tmp_bytes = t3;
+  const size_t n_meas = (size_t)iterations + 1;
+  Arena B;
+  const size_t o_row = B.plan<long long>((size_t)V + 1), o_col = B.plan<int32_t>((size_t)E), o_din = B.plan<int32_t>((size_t)V),
+               o_init = B.plan<int32_t>(initial_rank ? (size_t)V : 0), o_inptr = B.plan<long long>((size_t)V + 1), o_insrc = B.plan<int32_t>((size_t)E),
+               o_src = B.plan<int32_t>((size_t)E), o_keys = B.plan<int32_t>((size_t)E), o_r = B.plan<double>((size_t)V), o_rs = B.plan<double>((size_t)V),
+               o_mu = B.plan<double>((size_t)V), o_w1 = B.plan<double>((size_t)V), o_w2 = B.plan<double>((size_t)V), o_pos = B.plan<double>((size_t)V),
+               o_ids = B.plan<int32_t>((size_t)V), o_order = B.plan<int32_t>((size_t)V), o_rank = B.plan<int32_t>((size_t)V),
+               o_meas = B.plan<double>(2 * n_meas), o_bad = B.plan<int>(1), o_tmp = B.plan<char>(tmp_bytes);
+  if (!B.get()) return TAURUS_ERR_NOMEM;
+  long long *d_row = B.at<long long>(o_row), *d_inptr = B.at<long long>(o_inptr);
+  int32_t *d_col = B.at<int32_t>(o_col), *d_din = B.at<int32_t>(o_din), *d_init = initial_rank ? B.at<int32_t>(o_init) : nullptr,
+          *d_insrc = B.at<int32_t>(o_insrc), *d_srcedge = B.at<int32_t>(o_src), *d_keys = B.at<int32_t>(o_keys), *d_ids = B.at<int32_t>(o_ids),
+          *d_order = B.at<int32_t>(o_order), *d_rank = B.at<int32_t>(o_rank);
+  double *d_r = B.at<double>(o_r), *d_rsorted = B.at<double>(o_rs), *d_mu = B.at<double>(o_mu), *d_w1 = B.at<double>(o_w1), *d_w2 = B.at<double>(o_w2),
+         *d_pos = B.at<double>(o_pos), *d_J = B.at<double>(o_meas);
+  unsigned long long* d_span = reinterpret_cast<unsigned long long*>(d_J + n_meas);
+  int* d_bad = B.at<int>(o_bad);
+  void* d_tmp = B.at<char>(o_tmp);
 #define RO(call) do { if ((call) != cudaSuccess) { cudaGetLastError(); return TAURUS_ERR_CUDA; } } while (0)
   RO(cudaMemcpyAsync(d_row, row_ptr, (size_t)(V + 1) * sizeof(long long), cudaMemcpyDefault, st));
   if (E > 0) RO(cudaMemcpyAsync(d_col, col_idx, (size_t)E * sizeof(int32_t), cudaMemcpyDefault, st));
@@ -173,16 +191,6 @@ extern "C" int taurus_reorder(int64_t V, int64_t E, const int64_t* row_ptr, cons
   ro_degree_kernel<<<grid, 256, 0, st>>>(E, d_col, V, d_din, d_bad);
   ro_widen_kernel<<<grid, 256, 0, st>>>(V, d_din, d_inptr);
   ro_src_kernel<<<grid, 256, 0, st>>>(V, d_row, d_srcedge);
-  int end_bit = 1;
-  while (end_bit < 31 && (1ll << end_bit) < V) ++end_bit;
-  size_t t1 = 0, t2 = 0, t3 = 0;
-  cub::DeviceScan::ExclusiveSum(nullptr, t1, d_inptr, d_inptr, V + 1, st);
-  if (E > 0) cub::DeviceRadixSort::SortPairs(nullptr, t2, d_col, d_keys, d_srcedge, d_insrc, E, 0, end_bit, st);
-  cub::DeviceRadixSort::SortPairs(nullptr, t3, d_r, d_rsorted, d_ids, d_order, V, 0, 64, st);
-  size_t tmp_bytes = t1 > t2 ? t1 : t2;
-  if (t3 > tmp_bytes) tmp_bytes = t3;
-  void* d_tmp = B.get<char>(tmp_bytes);
-  if (!d_tmp) return TAURUS_ERR_NOMEM;
   size_t tb = tmp_bytes;
   RO(cub::DeviceScan::ExclusiveSum(d_tmp, tb, d_inptr, d_inptr, V + 1, st));
   if (E > 0) { tb = tmp_bytes; RO(cub::DeviceRadixSort::SortPairs(d_tmp, tb, d_col, d_keys, d_srcedge, d_insrc, E, 0, end_bit, st)); }
@@ -193,8 +201,7 @@ extern "C" int taurus_reorder(int64_t V, int64_t E, const int64_t* row_ptr, cons
 
   ro_init_kernel<<<grid, 256, 0, st>>>(V, d_init, d_r);
   ro_iota_kernel<<<grid, 256, 0, st>>>(V, d_ids);
-  std::vector<double> J((size_t)iterations + 1, 0.0);
-  std::vector<unsigned long long> span((size_t)iterations + 1, 0);
+  RO(cudaMemsetAsync(d_J, 0, 2 * n_meas * sizeof(double), st));
   for (int it = 0; it <= iterations; ++it) {
     if (it > 0) {   // one iteration of the update rules on the real-valued positions
       ro_mu_kernel<<<grid, 256, 0, st>>>(V, d_inptr, d_insrc, d_r, d_mu, d_w1, d_w2);
@@ -205,14 +212,13 @@ extern "C" int taurus_reorder(int64_t V, int64_t E, const int64_t* row_ptr, cons
     RO(cub::DeviceRadixSort::SortPairs(d_tmp, tb, d_r, d_rsorted, d_ids, d_order, V, 0, 64, st));
     ro_rank_kernel<<<grid, 256, 0, st>>>(V, d_order, d_rank, d_pos);
     if (out_J || out_span) {   // J and C(pi) of this ordering (positions = ranks, centres = their optimum)
-      RO(cudaMemsetAsync(d_J, 0, sizeof(double), st));
-      RO(cudaMemsetAsync(d_span, 0, sizeof(unsigned long long), st));
-      ro_mu_kernel<<<grid, 256, 0, st>>>(V, d_inptr, d_insrc, d_pos, d_mu, nullptr, nullptr);
-      ro_measure_kernel<<<grid, 256, 0, st>>>(V, d_inptr, d_insrc, d_pos, d_mu, d_rank, d_J, d_span);
-      RO(cudaMemcpyAsync(&J[(size_t)it], d_J, sizeof(double), cudaMemcpyDeviceToHost, st));
-      RO(cudaMemcpyAsync(&span[(size_t)it], d_span, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+      ro_measure_kernel<<<grid, 256, 0, st>>>(V, d_inptr, d_insrc, d_pos, d_J + it, d_span + it);
     }
   }
+  std::vector<double> J(n_meas, 0.0);
+  std::vector<unsigned long long> span(n_meas, 0);
+  RO(cudaMemcpyAsync(J.data(), d_J, n_meas * sizeof(double), cudaMemcpyDeviceToHost, st));
+  RO(cudaMemcpyAsync(span.data(), d_span, n_meas * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
   RO(cudaMemcpyAsync(out_rank, d_rank, (size_t)V * sizeof(int32_t), cudaMemcpyDefault, st));
   if (out_positions) RO(cudaMemcpyAsync(out_positions, d_r, (size_t)V * sizeof(double), cudaMemcpyDefault, st));
   RO(cudaStreamSynchronize(st));
@@ -263,10 +269,12 @@ __global__ void rl_edges_kernel(long long V, const long long* __restrict__ row_p
 __global__ void rl_rows_kernel(long long V, int width, const float* __restrict__ in, long long ld_in, const int32_t* __restrict__ rank,
                                float* __restrict__ out, long long ld_out) {
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
+  const bool wide = ((width | ld_in | ld_out) & 3) == 0 && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
   for (long long v = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < V; v += warps) {
     const float* src = in + (size_t)v * ld_in;
     float* dst = out + (size_t)rank[v] * ld_out;
-    for (int k = lane(); k < width; k += 32) dst[k] = src[k];
+    if (wide) for (int k = lane(); k < (width >> 2); k += 32) reinterpret_cast<float4*>(dst)[k] = reinterpret_cast<const float4*>(src)[k];
+    else for (int k = lane(); k < width; k += 32) dst[k] = src[k];
   }
 }
 
@@ -281,19 +289,21 @@ extern "C" int taurus_relabel_csr(int64_t V, int64_t E, const int64_t* row_ptr, 
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int grid = sms * 8;
-  Buffers B;
-  long long* d_row = B.get<long long>((size_t)V + 1);
-  int32_t* d_col = B.get<int32_t>((size_t)E);
-  int32_t* d_rank = B.get<int32_t>((size_t)V);
-  int32_t* d_seen = B.get<int32_t>((size_t)V);
-  long long* d_nptr = B.get<long long>((size_t)V + 1);
-  int32_t* d_ncol = B.get<int32_t>((size_t)E);
-  int32_t* d_ndin = out_in_degree ? B.get<int32_t>((size_t)V) : nullptr;
-  int* d_bad = B.get<int>(1);
   size_t tb = 0;
-  cub::DeviceScan::ExclusiveSum(nullptr, tb, d_nptr, d_nptr, V + 1, st);
-  void* d_tmp = B.get<char>(tb);
-  if (!d_row || !d_col || !d_rank || !d_seen || !d_nptr || !d_ncol || (out_in_degree && !d_ndin) || !d_bad || !d_tmp) return TAURUS_ERR_NOMEM;
+  {
+    long long* const n64 = nullptr;
+    cub::DeviceScan::ExclusiveSum(nullptr, tb, n64, n64, V + 1, st);
+  }
+  Arena B;
+  const size_t o_row = B.plan<long long>((size_t)V + 1), o_col = B.plan<int32_t>((size_t)E), o_rank = B.plan<int32_t>((size_t)V),
+               o_seen = B.plan<int32_t>((size_t)V), o_nptr = B.plan<long long>((size_t)V + 1), o_ncol = B.plan<int32_t>((size_t)E),
+               o_ndin = B.plan<int32_t>((size_t)V), o_bad = B.plan<int>(1), o_tmp = B.plan<char>(tb);
+  if (!B.get()) return TAURUS_ERR_NOMEM;
+  long long *d_row = B.at<long long>(o_row), *d_nptr = B.at<long long>(o_nptr);
+  int32_t *d_col = B.at<int32_t>(o_col), *d_rank = B.at<int32_t>(o_rank), *d_seen = B.at<int32_t>(o_seen), *d_ncol = B.at<int32_t>(o_ncol),
+          *d_ndin = out_in_degree ? B.at<int32_t>(o_ndin) : nullptr;
+  int* d_bad = B.at<int>(o_bad);
+  void* d_tmp = B.at<char>(o_tmp);
 #define RL(call) do { if ((call) != cudaSuccess) { cudaGetLastError(); return TAURUS_ERR_CUDA; } } while (0)
   RL(cudaMemcpyAsync(d_row, row_ptr, (size_t)(V + 1) * sizeof(long long), cudaMemcpyDefault, st));
   if (E > 0) RL(cudaMemcpyAsync(d_col, col_idx, (size_t)E * sizeof(int32_t), cudaMemcpyDefault, st));

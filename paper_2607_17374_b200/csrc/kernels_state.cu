@@ -1117,9 +1117,11 @@ void launch_place_half(taurus_ctx* c, int half, int d_out, int Hp, cudaStream_t 
   c->launches += 1;
 }
 
-void launch_reload_histogram(taurus_ctx* c, long long* d_hist18, cudaStream_t st) {
-  cudaMemsetAsync(d_hist18, 0, 18 * sizeof(long long), st);
-  reload_histogram_kernel<<<c->sm_count * 4, 256, 0, st>>>(c->V, c->d_reload, d_hist18);
+void launch_reload_histogram(taurus_ctx* c, cudaStream_t st) {
+  if (c->resident) return;   // nothing is ever reloaded; the words are zero from the layer reset on
+  long long* hist = c->d_ctl->reload_hist;
+  cudaMemsetAsync(hist, 0, 18 * sizeof(long long), st);
+  reload_histogram_kernel<<<c->sm_count * 4, 256, 0, st>>>(c->V, c->d_reload, hist);
   c->launches += 1;
 }
 

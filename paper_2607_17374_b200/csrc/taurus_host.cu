@@ -88,7 +88,7 @@ extern "C" void taurus_destroy(taurus_ctx* c) {
   cudaFree(c->d_heavy_list); cudaFree(c->d_heavy); cudaFree(c->d_heavy_rows);
   cudaFree(c->d_csc_ptr); cudaFree(c->d_csc_eid); cudaFree(c->d_mask); cudaFree(c->d_vtmp); cudaFree(c->d_rank_hist);
   cudaFree(c->d_gdst); cudaFree(c->d_gedge); cudaFree(c->d_geid); cudaFree(c->d_gmask);
-  cudaFree(c->d_ctl); cudaFree(c->d_chunk_log); cudaFree(c->d_reload_hist);
+  cudaFree(c->d_ctl); cudaFree(c->d_chunk_log);
   if (c->h_ctl) cudaFreeHost(c->h_ctl);
   if (c->order_event) cudaEventDestroy(c->order_event);
   for (int i = 0; i < 2; ++i) {
@@ -365,7 +365,6 @@ static int init_impl(taurus_ctx* c, const taurus_graph* g, const taurus_model* m
   }
   // control
   ALLOC(c->d_ctl, 1);
-  ALLOC(c->d_reload_hist, 18);
   CU(cudaMemset(c->d_ctl, 0, sizeof(DevCtl)));
   CU(cudaHostAlloc((void**)&c->h_ctl, sizeof(DevCtl), cudaHostAllocDefault));
   memset(c->h_ctl, 0, sizeof(DevCtl));
@@ -418,13 +417,16 @@ extern "C" int taurus_graph_init(taurus_ctx** out, const taurus_graph* g, const 
   return TAURUS_OK;
 }
 
-// Reads the device control block (after synchronising `st`) and returns its sticky error.
+// Reads the device control block up to the chunks' own counters, once everything on `st` and the output stream is through,
+// and returns its sticky error.  One copy into pinned memory and one wait: the calls that block (drains, layer_end, stats)
+// are paid per chunk or per layer.  with_stats: the reload histogram comes along.
 static int finish_chunk(taurus_ctx* c, cudaStream_t st);
-static int read_ctl(taurus_ctx* c, cudaStream_t st) {
+static int read_ctl(taurus_ctx* c, cudaStream_t st, bool with_stats = false) {
   { int rc = finish_chunk(c, st); if (rc) return rc; }   // the last chunk's finalise may still be waiting for a successor
+  if (with_stats) launch_reload_histogram(c, st);
+  CU(cudaMemcpyAsync(c->h_ctl, c->d_ctl, offsetof(DevCtl, pc), cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));
   CU(cudaStreamSynchronize(c->out_stream));
-  CU(cudaMemcpy(c->h_ctl, c->d_ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost));
   return c->h_ctl->error;
 }
 
@@ -944,13 +946,10 @@ extern "C" int taurus_layer_set_dense_output(taurus_ctx* c, float* dense_rows, i
   return TAURUS_OK;
 }
 
-static int fill_stats(taurus_ctx* c, taurus_stats* s) {
+static int fill_stats(const taurus_ctx* c, taurus_stats* s) {   // from the control block read with its statistics
   const DevCtl* h = c->h_ctl;
   memset(s, 0, sizeof(*s));
-  launch_reload_histogram(c, c->d_reload_hist, c->last_stream);
-  long long hist[18];
-  CU(cudaMemcpyAsync(hist, c->d_reload_hist, sizeof(hist), cudaMemcpyDeviceToHost, c->last_stream));
-  CU(cudaStreamSynchronize(c->last_stream));
+  const long long* hist = h->reload_hist;
   long long nonzero = 0;
   for (int i = 1; i < 17; ++i) { s->reload_histogram[i] = hist[i]; nonzero += hist[i]; }
   s->reload_histogram[0] = c->V - nonzero;
@@ -966,7 +965,7 @@ extern "C" int taurus_get_stats(taurus_ctx* c, taurus_stats* stats) {
   if (!c || !stats) return TAURUS_ERR_INVALID_ARG;
   if (c->layer < 0) return TAURUS_ERR_ORDER;
   CU(cudaSetDevice(c->device));
-  int err = read_ctl(c, c->last_stream);
+  int err = read_ctl(c, c->last_stream, true);
   if (err) return err;
   return fill_stats(c, stats);
 }
@@ -981,7 +980,7 @@ extern "C" int taurus_layer_end(taurus_ctx* c, taurus_stats* stats) {
     if (!rc) rc = runs_flush_all(c->run_out, c->out_stream);
     if (rc) return rc;
   }
-  int err = read_ctl(c, c->last_stream);
+  int err = read_ctl(c, c->last_stream, stats != nullptr);
   if (err) return err;
   if (stats) { int rc = fill_stats(c, stats); if (rc) return rc; }
   if (c->next_src != c->V || c->h_ctl->completed != c->V || c->h_ctl->free_top != c->pool_slots) return TAURUS_ERR_ORDER;

@@ -63,6 +63,7 @@ struct DevCtl {
   long long evictions, reloads, peak_occupancy, hub_messages, total_messages, completed;
   long long sum_hs, sum_ns, sum_ev, sum_gs, chunks;
   long long scatter_groups; // accumulator-row reductions issued by the scatter (self messages not counted)
+  long long reload_hist[18]; // filled for the statistics: vertices by reload count 0..16+, most reloads of one vertex
   ChunkCtl pc[2];
 };
 
@@ -303,7 +304,6 @@ struct taurus_ctx {
   int32_t* d_vtmp = nullptr;     // [V] scratch for layer_begin
   int32_t* d_rank_hist = nullptr;
   DevCtl* d_ctl = nullptr;
-  long long* d_reload_hist = nullptr;   // 18 words for the reload histogram of taurus_get_stats
   DevCtl* h_ctl = nullptr;       // pinned
   long long* d_chunk_log = nullptr;
   long long log_capacity = 0;
@@ -341,7 +341,7 @@ void launch_compact_done(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, boo
 void launch_commit(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);
 void launch_place_rows(taurus_ctx* c, float* dense, long long ld, int d_out, int Hp, long long count, cudaStream_t st);
 void launch_place_half(taurus_ctx* c, int half, int d_out, int Hp, cudaStream_t st);   // dense-output mode
-void launch_reload_histogram(taurus_ctx* c, long long* d_hist18, cudaStream_t st);
+void launch_reload_histogram(taurus_ctx* c, cudaStream_t st);               // fills ctl->reload_hist
 void launch_completion_ranks(taurus_ctx* c, cudaStream_t st);                // fills d_rank_hist
 long long max_window_edges(taurus_ctx* c);                                  // most edges of any chunk_sources consecutive sources
 int check_in_degrees(taurus_ctx* c, cudaStream_t st);                        // 0 ok, 1 mismatch
