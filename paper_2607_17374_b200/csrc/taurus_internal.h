@@ -240,6 +240,8 @@ struct taurus_ctx {
   int32_t* d_item_count = nullptr;
   long long* d_item_ptr = nullptr; // [grid chunks + 1]
   std::vector<long long> item_ptr;
+  cudaStream_t account_stream = nullptr;   // the accounting of a push runs here, beside its copy and projection
+  cudaEvent_t account_go = nullptr, account_done = nullptr;
   int32_t* d_heavy_list = nullptr; // vertices with long in-lists
   long long n_heavy = 0, n_heavy_segments = 0;
   int4* d_heavy = nullptr;         // segments of one push
