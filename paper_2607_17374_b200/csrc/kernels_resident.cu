@@ -592,28 +592,33 @@ __global__ void __launch_bounds__(32 * G_WARPS) gather_kernel(const __grid_const
   }
 }
 
+// per_sm: the context's record of the instantiation (blocks per SM, 0 = not launched yet).  The shared-memory limit belongs to
+// the context's device, so nothing is kept process-wide.
 template <int LPE, int VPL, int U, int D, int GAT>
-int launch_g(taurus_ctx* c, const GatherArgs& g, long long bound, cudaStream_t st) {
+int launch_g(taurus_ctx* c, const GatherArgs& g, long long bound, int* per_sm, cudaStream_t st) {
   const size_t smem = sizeof(Ring<VPL, U, D, GAT>) * G_WARPS;
-  static int per_sm = 0;
-  if (per_sm == 0) {
+  if (*per_sm == 0) {
     int b = 0;
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(gather_kernel<LPE, VPL, U, D, GAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TAURUS_ERR_CUDA;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, gather_kernel<LPE, VPL, U, D, GAT>, 32 * G_WARPS, smem) != cudaSuccess || b < 1) b = 1;
-    per_sm = b;
+    cudaError_t e = cudaSuccess;
+    if (smem > 48 * 1024) e = cudaFuncSetAttribute(gather_kernel<LPE, VPL, U, D, GAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, gather_kernel<LPE, VPL, U, D, GAT>, 32 * G_WARPS, smem);
+    if (e != cudaSuccess) { taurus_note_cuda_error(e, "gather_kernel"); return TAURUS_ERR_CUDA; }
+    *per_sm = b < 1 ? 1 : b;
   }
   // no more warps than items: a completed vertex each, and the segments of long in-lists
   const long long items = bound + c->n_heavy_segments;
-  const int grid = (int)std::max<long long>(1, std::min<long long>((items + G_WARPS - 1) / G_WARPS, (long long)c->sm_count * per_sm));
+  const int grid = (int)std::max<long long>(1, std::min<long long>((items + G_WARPS - 1) / G_WARPS, (long long)c->sm_count * *per_sm));
   gather_kernel<LPE, VPL, U, D, GAT><<<grid, 32 * G_WARPS, smem, st>>>(g);
+  const cudaError_t e = cudaGetLastError();   // the accounting has been enqueued: the push must not look as if nothing had happened
+  if (e != cudaSuccess) { taurus_note_cuda_error(e, "gather_kernel"); return TAURUS_ERR_CUDA; }
   return TAURUS_OK;
 }
 template <int LPE, int VPL, int U, int D>
-int launch_g2(taurus_ctx* c, const GatherArgs& g, long long bound, cudaStream_t st) {
-  if (g.mode != TAURUS_GAT) return launch_g<LPE, VPL, U, D, 0>(c, g, bound, st);
+int launch_g2(taurus_ctx* c, const GatherArgs& g, long long bound, int width_class, cudaStream_t st) {
+  int* const per_sm = c->gather_per_sm[width_class];
+  if (g.mode != TAURUS_GAT) return launch_g<LPE, VPL, U, D, 0>(c, g, bound, per_sm, st);
   constexpr int DG = D > 3 ? 3 : 2;   // the scores take room in the ring
-  return g.heads <= 4 ? launch_g<LPE, VPL, U, DG, 4>(c, g, bound, st) : launch_g<LPE, VPL, U, DG, 16>(c, g, bound, st);
+  return g.heads <= 4 ? launch_g<LPE, VPL, U, DG, 4>(c, g, bound, per_sm + 1, st) : launch_g<LPE, VPL, U, DG, 16>(c, g, bound, per_sm + 2, st);
 }
 
 // ------------------------------------------------------------------------------------------------ rows into the store
@@ -971,14 +976,14 @@ int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitc
   // 4 x 3 lanes 4.3 to 5.1; 64: 2 rows, 4 steps 0.53, others 0.55 to 0.78; 100: 4 rows, 2 steps 8.5, others 8.4 to 8.8
   // (64 k completed rows of 128 floats 0.68 against 0.75 to 0.94); 256: 2 rows, 3 steps 16.4, others 16.4 to 16.9.
   const int Hp = a.Hp;
-  if (Hp <= 16) return launch_g2<4, 1, 2, 4>(c, g, bound, st);
-  if (Hp <= 32) return launch_g2<8, 1, 2, 4>(c, g, bound, st);
-  if (Hp <= 48) return launch_g2<16, 1, 4, 3>(c, g, bound, st);
-  if (Hp <= 64) return launch_g2<16, 1, 2, 4>(c, g, bound, st);
-  if (Hp <= 128) return launch_g2<32, 1, 4, 3>(c, g, bound, st);
-  if (Hp <= 256) return launch_g2<32, 2, 2, 4>(c, g, bound, st);
-  if (Hp <= 512) return launch_g2<32, 4, 1, 4>(c, g, bound, st);
-  return launch_g2<32, 8, 1, 3>(c, g, bound, st);
+  if (Hp <= 16) return launch_g2<4, 1, 2, 4>(c, g, bound, 0, st);
+  if (Hp <= 32) return launch_g2<8, 1, 2, 4>(c, g, bound, 1, st);
+  if (Hp <= 48) return launch_g2<16, 1, 4, 3>(c, g, bound, 2, st);
+  if (Hp <= 64) return launch_g2<16, 1, 2, 4>(c, g, bound, 3, st);
+  if (Hp <= 128) return launch_g2<32, 1, 4, 3>(c, g, bound, 4, st);
+  if (Hp <= 256) return launch_g2<32, 2, 2, 4>(c, g, bound, 5, st);
+  if (Hp <= 512) return launch_g2<32, 4, 1, 4>(c, g, bound, 6, st);
+  return launch_g2<32, 8, 1, 3>(c, g, bound, 7, st);
 }
 
 void launch_resident_attention(taurus_ctx* c, cudaStream_t st) {

@@ -242,6 +242,7 @@ struct taurus_ctx {
   std::vector<long long> item_ptr;
   cudaStream_t account_stream = nullptr;   // the accounting of a push runs here, beside its copy and projection
   cudaEvent_t account_go = nullptr, account_done = nullptr;
+  int gather_per_sm[8][3] = {{0}};         // gather: blocks per SM by row width class and attention variant, 0 = not launched yet
   int32_t* d_heavy_list = nullptr; // vertices with long in-lists
   long long n_heavy = 0, n_heavy_segments = 0;
   int4* d_heavy = nullptr;         // segments of one push
