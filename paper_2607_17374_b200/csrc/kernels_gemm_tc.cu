@@ -14,12 +14,6 @@
 // The output columns of a tile are processed in blocks of up to 256; (tile, block) units alternate between two
 // TMEM accumulator buffers, so the epilogue of one unit overlaps the main loop of the next, also across tiles.
 //
-// Two CTAs to a tile (PAIR, cta_group::2): the pair works on 256 rows, each CTA with its own 128 rows of X and its own half of
-// the block's weight columns in shared memory; the leader issues the MMAs, which read both halves, and each CTA finishes its own
-// rows.  A weight tile then crosses L2 once per 256 rows instead of once per 128: the loads of the one-CTA form, 80 KB per SM
-// and K step, 64 KB of them weights, ran L2 at 7 TB/s.  The converters and the epilogue of the second CTA arrive at the
-// leader's barriers; commits reach both CTAs.
-//
 // Every wait on an mbarrier is bounded: after WAIT_LIMIT polls the kernel raises a CTA-wide abort flag,
 // records TAURUS_ERR_INTERNAL in the control block, waits (bounded) for its TMA copies in flight, frees its
 // TMEM and returns.  Every TMA load is a plain load of the issuing CTA alone.
@@ -46,7 +40,7 @@ constexpr int TILE_B_BYTES = BN_MAX * 128;       // 256 rows x 128 B
 constexpr int KS32 = 32;
 constexpr int ROW32 = KS32 * 4;                  // operand row bytes in fp32 mode
 constexpr int A32_BYTES = BM * ROW32;            // one fp32-mode feature tile (raw / hi, or lo)
-constexpr unsigned WAIT_LIMIT = 1u << 20;
+constexpr unsigned WAIT_LIMIT = 1u << 24;
 constexpr int NUM_THREADS = 320;
 constexpr int OUT_TILE_BYTES = 32 * 128;        // epilogue staging tile: 32 rows x 32 fp32, 128B-swizzled
 constexpr int OUT_STAGING_BYTES = 4 * 2 * OUT_TILE_BYTES;   // 4 epilogue warps x 2 tiles
@@ -63,8 +57,6 @@ struct __align__(8) Barriers {
 // narrower runs as many stages as fit (GemmArgs::stages, stage_bytes).
 constexpr int STAGE_BYTES_FP32 = 2 * TILE_A_BYTES + 2 * TILE_B_BYTES;
 constexpr int STAGE_BYTES_BF16 = 3 * TILE_A_BYTES + TILE_B_BYTES;
-constexpr int STAGE_BUDGET = STAGES * STAGE_BYTES_FP32;   // shared memory for the stages
-static_assert(STAGES * STAGE_BYTES_BF16 <= STAGE_BUDGET, "both modes fit their stages");
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -73,11 +65,6 @@ __device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned coun
 }
 __device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// Arrival at the same barrier of the cluster's first CTA, with everything this thread wrote before it.
-__device__ __forceinline__ void mbar_arrive_leader(unsigned long long* bar) {
-  asm volatile("{\n.reg .b32 ra;\nmapa.shared::cluster.u32 ra, %0, 0;\nmbarrier.arrive.release.cluster.shared::cluster.b64 _, [ra];\n}"
-               ::"r"(smem_u32(bar)) : "memory");
 }
 __device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
@@ -88,17 +75,10 @@ __device__ __forceinline__ bool mbar_try(unsigned long long* bar, unsigned parit
                : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ bool mbar_try_cluster(unsigned long long* bar, unsigned parity) {   // sees what the other CTA released
-  unsigned ok;
-  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-               : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-  return ok != 0;
-}
 // Bounded wait.  Returns false when the CTA is aborting (this wait or another one ran out).
-template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, volatile int* abort_flag) {
   for (unsigned i = 0; i < WAIT_LIMIT; ++i) {
-    if (CLUSTER ? mbar_try_cluster(bar, parity) : mbar_try(bar, parity)) return true;
+    if (mbar_try(bar, parity)) return true;
     if ((i & 63u) == 63u && *abort_flag) return false;
   }
   *abort_flag = 1;
@@ -123,37 +103,20 @@ __device__ __forceinline__ unsigned long long umma_desc(unsigned smem_addr) {
   return d;
 }
 
-template <bool PAIR>
 __device__ __forceinline__ void umma(unsigned tmem_d, unsigned long long a, unsigned long long b, unsigned idesc,
                                      unsigned accumulate, bool tf32) {
-  if (PAIR && tf32)
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
-  else if (PAIR)
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
-  else if (tf32)
+  if (tf32)
     asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}"
                  ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
   else
     asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
                  ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
 }
-template <bool PAIR>
 __device__ __forceinline__ void umma_commit(unsigned long long* bar) {
-  if (PAIR) {   // arrives at this barrier in both CTAs
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(smem_u32(bar)), "h"((unsigned short)3) : "memory");
-    return;
-  }
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 
 struct GemmArgs {
   float* PT;            // [n x N]
@@ -173,46 +136,37 @@ struct GemmArgs {
   GemmFinish fin;
 };
 
-template <bool BF16, bool PAIR>
+template <bool BF16>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_b0,
                   const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ CUtensorMap map_out, GemmArgs g) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  constexpr int TILE = PAIR ? 2 * BM : BM;   // rows of a unit
-  unsigned rank = 0;                         // CTA of the pair
-  if (PAIR) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  const int unit0 = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, units_step = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
+  constexpr int STAGE_BYTES_MAX = BF16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32;
   const int STAGE_BYTES = g.stage_bytes;
   const int n_stages = g.stages;
-  unsigned char* out_staging = smem + STAGE_BUDGET;
+  unsigned char* out_staging = smem + STAGES * STAGE_BYTES_MAX;
   Barriers* bars = reinterpret_cast<Barriers*>(out_staging + OUT_STAGING_BYTES);
   volatile int* abort_flag = &bars->abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int n_rows = g.n;
   if (g.done_count) { const int nd = *g.done_count; n_rows = nd < g.n ? nd : g.n; }   // same value in every thread
-  const int n_tiles = (n_rows + TILE - 1) / TILE;
+  const int n_tiles = (n_rows + BM - 1) / BM;
   const int n_blocks = (g.Np + BN_MAX - 1) / BN_MAX;
   const int tmem_cols = 512;   // two accumulator buffers of 256 columns; one CTA per SM
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->conv[s], PAIR ? 256 : 128); mbar_init(&bars->empty[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&bars->acc_full[b], 1); mbar_init(&bars->acc_empty[b], PAIR ? 256 : 128); }
+    for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->conv[s], 128); mbar_init(&bars->empty[s], 1); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&bars->acc_full[b], 1); mbar_init(&bars->acc_empty[b], 128); }
     bars->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {   // TMEM allocation by one full warp
-    if (PAIR) {
-      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem_base)), "r"(tmem_cols) : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    } else {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem_base)), "r"(tmem_cols) : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem_base)), "r"(tmem_cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
-  if (PAIR) cluster_sync();   // the other CTA's barriers are initialised
   tc_fence_after();
   const unsigned tmem_base = bars->tmem_base;
 
@@ -222,14 +176,10 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     // ---------------------------------------------------------------- TMA producer
     if (lane == 0) {
       int it = 0;
-      for (int w = unit0; w < n_tiles * n_blocks && !*abort_flag; w += units_step) {
+      for (int w = blockIdx.x; w < n_tiles * n_blocks && !*abort_flag; w += gridDim.x) {
         const int tile = w / n_blocks, nb = w % n_blocks;
-        const int row0 = tile * TILE + (int)rank * BM;
-        int col0 = nb * BN_MAX;
-        if (PAIR) {   // this CTA's half of the block's columns
-          const int bw = (g.Np - col0) < BN_MAX ? (g.Np - col0) : BN_MAX;
-          col0 += (int)rank * (bw >> 1);
-        }
+        const int row0 = tile * BM;
+        const int col0 = nb * BN_MAX;
         for (int ks = 0; ks < g.k_stages; ++ks, ++it) {
           const int s = it % n_stages;
           const unsigned ph = (it / n_stages) & 1;
@@ -250,50 +200,50 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       }
     }
   } else if (warp == 1) {
-    // ---------------------------------------------------------------- MMA issuer (of a pair: the leader's)
-    if (lane == 0 && rank == 0) {
+    // ---------------------------------------------------------------- MMA issuer
+    if (lane == 0) {
       int it = 0, unit = 0;
-      for (int w = unit0; w < n_tiles * n_blocks && !*abort_flag; w += units_step, ++unit) {
+      for (int w = blockIdx.x; w < n_tiles * n_blocks && !*abort_flag; w += gridDim.x, ++unit) {
         const int nb = w % n_blocks;
         const int bw = (g.Np - nb * BN_MAX) < BN_MAX ? (g.Np - nb * BN_MAX) : BN_MAX;
         const int buf = unit & 1;
-        if (unit >= 2 && !mbar_wait<PAIR>(&bars->acc_empty[buf], ((unit >> 1) & 1) ^ 1, abort_flag)) break;
+        if (unit >= 2 && !mbar_wait(&bars->acc_empty[buf], ((unit >> 1) & 1) ^ 1, abort_flag)) break;
         tc_fence_after();
         const unsigned tmem_d = tmem_base + (unsigned)(buf * BN_MAX);
         const unsigned idesc = (1u << 4) | ((BF16 ? 1u : 2u) << 7) | ((BF16 ? 1u : 2u) << 10) |
-                               ((unsigned)(bw >> 3) << 17) | ((unsigned)(TILE >> 4) << 24);
+                               ((unsigned)(bw >> 3) << 17) | ((unsigned)(BM >> 4) << 24);
         bool ok = true;
         for (int ks = 0; ks < g.k_stages; ++ks, ++it) {
           const int s = it % n_stages;
           const unsigned ph = (it / n_stages) & 1;
-          if (!mbar_wait<PAIR>(&bars->conv[s], ph, abort_flag)) { ok = false; break; }
+          if (!mbar_wait(&bars->conv[s], ph, abort_flag)) { ok = false; break; }
           tc_fence_after();
           const unsigned base = smem_u32(stage_ptr(s));
           if (BF16) {
             const unsigned long long da = umma_desc<128>(base + 2 * TILE_A_BYTES), db = umma_desc<128>(base + 3 * TILE_A_BYTES);
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) umma<PAIR>(tmem_d, da + 2 * kk, db + 2 * kk, idesc, (ks | kk) != 0, false);
+            for (int kk = 0; kk < 4; ++kk) umma(tmem_d, da + 2 * kk, db + 2 * kk, idesc, (ks | kk) != 0, false);
           } else {
             const unsigned long long a_hi = umma_desc<ROW32>(base), a_lo = umma_desc<ROW32>(base + A32_BYTES);
             const unsigned long long b_hi = umma_desc<ROW32>(base + 2 * A32_BYTES), b_lo = umma_desc<ROW32>(base + 2 * A32_BYTES + g.b_box_bytes);
 #pragma unroll
             for (int kk = 0; kk < KS32 / 8; ++kk) {
-              umma<PAIR>(tmem_d, a_lo + 2 * kk, b_hi + 2 * kk, idesc, (ks | kk) != 0, true);
-              umma<PAIR>(tmem_d, a_hi + 2 * kk, b_lo + 2 * kk, idesc, 1u, true);
-              umma<PAIR>(tmem_d, a_hi + 2 * kk, b_hi + 2 * kk, idesc, 1u, true);
+              umma(tmem_d, a_lo + 2 * kk, b_hi + 2 * kk, idesc, (ks | kk) != 0, true);
+              umma(tmem_d, a_hi + 2 * kk, b_lo + 2 * kk, idesc, 1u, true);
+              umma(tmem_d, a_hi + 2 * kk, b_hi + 2 * kk, idesc, 1u, true);
             }
           }
-          umma_commit<PAIR>(&bars->empty[s]);    // stage reusable once these MMAs have read it
+          umma_commit(&bars->empty[s]);    // stage reusable once these MMAs have read it
         }
         if (!ok) break;
-        umma_commit<PAIR>(&bars->acc_full[buf]);  // accumulator of this block complete
+        umma_commit(&bars->acc_full[buf]);  // accumulator of this block complete
       }
     }
   } else if (warp < 6) {
     // ---------------------------------------------------------------- converter (128 threads)
     const int t = threadIdx.x - 64;
     int it = 0;
-    for (int w = unit0; w < n_tiles * n_blocks && !*abort_flag; w += units_step) {
+    for (int w = blockIdx.x; w < n_tiles * n_blocks && !*abort_flag; w += gridDim.x) {
       bool ok = true;
       for (int ks = 0; ks < g.k_stages; ++ks, ++it) {
         const int s = it % n_stages;
@@ -334,7 +284,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
           }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> visible to the tensor core
-        if (PAIR) mbar_arrive_leader(&bars->conv[s]); else mbar_arrive(&bars->conv[s]);
+        mbar_arrive(&bars->conv[s]);
       }
       if (!ok) break;
     }
@@ -342,10 +292,9 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     // ---------------------------------------------------------------- epilogue (warps 6..9, TMEM lanes 32 * (warp % 4))
     const int q = warp & 3;
     int unit = 0, out_it = 0;
-    for (int w = unit0; w < n_tiles * n_blocks && !*abort_flag; w += units_step, ++unit) {
+    for (int w = blockIdx.x; w < n_tiles * n_blocks && !*abort_flag; w += gridDim.x, ++unit) {
     const int tile = w / n_blocks, nb = w % n_blocks;
-    const int row_w = tile * TILE + (int)rank * BM + q * 32;   // first row of this warp
-    const int r = row_w + lane;
+    const int r = tile * BM + q * 32 + lane;
     float c_out = 1.f, self_mul = 1.f;
     int vrow = -1;        // finish mode: the vertex this lane's row belongs to
     if (g.finish) {
@@ -429,13 +378,13 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         __syncwarp();
         if (lane == 0) {                      // rows beyond n and columns beyond N are clipped by the tensor map
           asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
-                       ::"l"(&map_out), "r"(cbase), "r"(row_w), "r"(smem_u32(tile_smem)) : "memory");
+                       ::"l"(&map_out), "r"(cbase), "r"(tile * BM + q * 32), "r"(smem_u32(tile_smem)) : "memory");
           asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
         ++out_it;
       }
       tc_fence_before();
-      if (PAIR) mbar_arrive_leader(&bars->acc_empty[buf]); else mbar_arrive(&bars->acc_empty[buf]);
+      mbar_arrive(&bars->acc_empty[buf]);
     }
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // all stores of this warp are complete
@@ -453,11 +402,9 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     }
     __syncthreads();
   }
-  if (PAIR) cluster_sync();   // no MMA reads this CTA's operands, and no arrival of this CTA is on its way, once it leaves
   if (warp == 1) {
     tc_fence_after();
-    if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
-    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
   }
 }
 
@@ -499,8 +446,9 @@ bool make_map(CUtensorMap* m, const void* base, CUtensorMapDataType dt, int elem
 
 // Stages that fit the shared memory sized for STAGES full-width stages.
 void set_stages(GemmArgs& g, bool bf16) {
+  const int budget = STAGES * (bf16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32);
   g.stage_bytes = bf16 ? 3 * TILE_A_BYTES + g.b_box_bytes : 2 * A32_BYTES + 2 * g.b_box_bytes;
-  int n = STAGE_BUDGET / g.stage_bytes;
+  int n = budget / g.stage_bytes;
   g.stages = n < STAGES ? STAGES : n > MAX_STAGES ? MAX_STAGES : n;
 }
 
@@ -510,7 +458,6 @@ struct WImage {
   void* lo = nullptr;   // fp32 mode: residual
   int Np = 0, Kp = 0;
   CUtensorMap map_hi, map_lo;
-  CUtensorMap half_hi, half_lo;   // boxes of half a block, for pairs of CTAs
 };
 
 }  // namespace
@@ -529,10 +476,8 @@ int prepare_tc_weights(taurus_ctx* c, void** slot, const std::vector<float>& cat
       for (int j = 0; j < N; ++j) img[(size_t)j * w->Kp + k] = __float2bfloat16(cat[(size_t)k * N + j]);
     if (cudaMalloc(&w->hi, cnt * 2) != cudaSuccess) return TAURUS_ERR_NOMEM;
     if (cudaMemcpy(w->hi, img.data(), cnt * 2, cudaMemcpyHostToDevice) != cudaSuccess) return TAURUS_ERR_CUDA;
-    if (!make_map(&w->map_hi, w->hi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, w->Np, w->Kp, w->Kp, bw, 64) ||
-        !make_map(&w->half_hi, w->hi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, w->Np, w->Kp, w->Kp, bw / 2, 64)) return TAURUS_ERR_CUDA;
+    if (!make_map(&w->map_hi, w->hi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, w->Np, w->Kp, w->Kp, bw, 64)) return TAURUS_ERR_CUDA;
     w->map_lo = w->map_hi;
-    w->half_lo = w->half_hi;
   } else {
     std::vector<float> hi(cnt, 0.f), lo(cnt, 0.f);
     for (int k = 0; k < K; ++k)
@@ -549,9 +494,7 @@ int prepare_tc_weights(taurus_ctx* c, void** slot, const std::vector<float>& cat
     if (cudaMemcpy(w->hi, hi.data(), cnt * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(w->lo, lo.data(), cnt * 4, cudaMemcpyHostToDevice) != cudaSuccess) return TAURUS_ERR_CUDA;
     if (!make_map(&w->map_hi, w->hi, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, w->Np, w->Kp, w->Kp, bw, KS32) ||
-        !make_map(&w->map_lo, w->lo, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, w->Np, w->Kp, w->Kp, bw, KS32) ||
-        !make_map(&w->half_hi, w->hi, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, w->Np, w->Kp, w->Kp, bw / 2, KS32) ||
-        !make_map(&w->half_lo, w->lo, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, w->Np, w->Kp, w->Kp, bw / 2, KS32)) return TAURUS_ERR_CUDA;
+        !make_map(&w->map_lo, w->lo, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, w->Np, w->Kp, w->Kp, bw, KS32)) return TAURUS_ERR_CUDA;
   }
   return TAURUS_OK;
 }
@@ -575,46 +518,6 @@ bool project_tc_usable(const taurus_ctx* c, int layer, const float* X, int ldx) 
   return true;
 }
 
-// Pairs of CTAs where the tiles of one CTA each would make more than two waves: below that the SMs are better used one by one
-// (1 024 rows x 128 columns are eight units).  Not beside row transfers, whose SMs would leave halves of pairs idle.
-static bool use_pair(const taurus_ctx* c, int n, int Np) {
-  const long long units = (long long)((n + BM - 1) / BM) * ((Np + BN_MAX - 1) / BN_MAX);
-  return !c->pipelined && Np % 32 == 0 && units > 2ll * c->sm_count;
-}
-
-template <bool BF16, bool PAIR>
-static int launch_tc(taurus_ctx* c, const CUtensorMap& x, const CUtensorMap& b0, const CUtensorMap& b1, const CUtensorMap& out, const GemmArgs& g, cudaStream_t st) {
-  const int smem = STAGE_BUDGET + OUT_STAGING_BYTES + (int)sizeof(Barriers) + 1024;
-  bool& set = c->tc_smem_set[(BF16 ? 2 : 0) + (PAIR ? 1 : 0)];
-  if (!set) {   // once per context (the attribute belongs to the context's device)
-    if (cudaFuncSetAttribute(project_tc_kernel<BF16, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) { cudaGetLastError(); return TAURUS_ERR_CUDA; }
-    set = true;
-  }
-  const int tile = PAIR ? 2 * BM : BM;
-  const int n_units = ((g.n + tile - 1) / tile) * ((g.Np + BN_MAX - 1) / BN_MAX);
-  const int sms = c->sm_count - (c->pipelined ? TAURUS_XFER_BLOCKS : 0);   // the SMs of the row transfers have no shared memory left
-  const int most = PAIR ? sms / 2 : sms;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((n_units < most ? n_units : most) * (PAIR ? 2 : 1)));
-  cfg.blockDim = dim3(NUM_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = PAIR ? 1 : 0;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, project_tc_kernel<BF16, PAIR>, x, b0, b1, out, g);
-  if (e != cudaSuccess) { taurus_note_cuda_error(e, "project_tc_kernel"); return TAURUS_ERR_CUDA; }
-  c->launches += 1;
-  return TAURUS_OK;
-}
-static int launch_tc_any(taurus_ctx* c, bool bf16, bool pair, const CUtensorMap& x, const CUtensorMap& b0, const CUtensorMap& b1, const CUtensorMap& out,
-                         const GemmArgs& g, cudaStream_t st) {
-  if (bf16) return pair ? launch_tc<true, true>(c, x, b0, b1, out, g, st) : launch_tc<true, false>(c, x, b0, b1, out, g, st);
-  return pair ? launch_tc<false, true>(c, x, b0, b1, out, g, st) : launch_tc<false, false>(c, x, b0, b1, out, g, st);
-}
-
 int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, cudaStream_t st) {
   const bool bf16 = c->gemm_mode == TAURUS_GEMM_BF16;
   WImage* w = static_cast<WImage*>(c->tc_image[layer]);
@@ -626,13 +529,26 @@ int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long lo
   if (!make_map(&map_out, out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, N, N, 32, 32)) return TAURUS_ERR_CUDA;
   GemmArgs g;
   g.PT = out; g.n = n; g.N = N; g.Np = w->Np; g.k_stages = w->Kp / (bf16 ? 64 : KS32);
-  const bool pair = use_pair(c, n, w->Np);
-  g.b_box_bytes = (w->Np < BN_MAX ? w->Np : BN_MAX) / (pair ? 2 : 1) * (bf16 ? 128 : ROW32);
+  g.b_box_bytes = (w->Np < BN_MAX ? w->Np : BN_MAX) * (bf16 ? 128 : ROW32);
   set_stages(g, bf16);
   g.Hp = Hp; g.mode = c->mode; g.fanout = c->fanout[layer]; g.bias = c->d_bias[layer];
   g.row_ptr = c->d_row_ptr; g.din = c->d_din; g.src_begin = src_begin; g.ctl = c->d_ctl;
   g.finish = 0; g.fin = GemmFinish(); g.done_count = nullptr;
-  return launch_tc_any(c, bf16, pair, map_x, pair ? w->half_hi : w->map_hi, pair ? w->half_lo : w->map_lo, map_out, g, st);
+  const int smem = STAGES * (bf16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32) + OUT_STAGING_BYTES + (int)sizeof(Barriers) + 1024;
+  const int n_tiles = (n + BM - 1) / BM;
+  const int n_units = n_tiles * ((w->Np + BN_MAX - 1) / BN_MAX);
+  const int sms = c->sm_count - (c->pipelined ? TAURUS_XFER_BLOCKS : 0);   // the SMs of the row transfers have no shared memory left
+  const int grid = n_units < sms ? n_units : sms;
+  if (!c->tc_smem_set) {   // once per context (the attribute belongs to the context's device)
+    cudaError_t e = bf16 ? cudaFuncSetAttribute(project_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
+                         : cudaFuncSetAttribute(project_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) { cudaGetLastError(); return TAURUS_ERR_CUDA; }
+    c->tc_smem_set = true;
+  }
+  if (bf16) project_tc_kernel<true><<<grid, NUM_THREADS, smem, st>>>(map_x, w->map_hi, w->map_lo, map_out, g);
+  else project_tc_kernel<false><<<grid, NUM_THREADS, smem, st>>>(map_x, w->map_hi, w->map_lo, map_out, g);
+  c->launches += 1;
+  return TAURUS_OK;
 }
 
 // Plain product on the tensor cores: out[n x N] (pitch ld_out floats) = X[n x K] (pitch ldx) . columns
@@ -654,8 +570,7 @@ int launch_gemm_plain_tc(taurus_ctx* c, void* image, int col0, int N, const floa
   WImage* w = static_cast<WImage*>(image);
   const int rows_left = w->Np - col0;                       // image rows (= output columns) from col0 on
   const int Np = std::min(taurus_round_up(N, 16), rows_left);
-  const bool pair = use_pair(c, n, Np);
-  const int bw = (Np < BN_MAX ? Np : BN_MAX) / (pair ? 2 : 1);   // rows of a weight box: of a pair, each CTA's half
+  const int bw = Np < BN_MAX ? Np : BN_MAX;
   const int elem = bf16 ? 2 : 4;
   CUtensorMap map_x, map_out, map_hi, map_lo;
   if (!make_map(&map_x, X, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, K, ldx, BM, bf16 ? 32 : KS32)) return TAURUS_ERR_CUDA;
@@ -677,5 +592,19 @@ int launch_gemm_plain_tc(taurus_ctx* c, void* image, int col0, int N, const floa
   g.row_ptr = c->d_row_ptr; g.din = c->d_din; g.src_begin = 0; g.ctl = c->d_ctl;
   g.finish = finish ? 1 : 0; g.fin = finish ? *finish : GemmFinish();
   g.done_count = done_count;
-  return launch_tc_any(c, bf16, pair, map_x, map_hi, map_lo, map_out, g, st);
+  const int smem = STAGES * (bf16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32) + OUT_STAGING_BYTES + (int)sizeof(Barriers) + 1024;
+  const int n_tiles = (n + BM - 1) / BM;
+  const int n_units = n_tiles * ((Np + BN_MAX - 1) / BN_MAX);
+  const int sms = c->sm_count - (c->pipelined ? TAURUS_XFER_BLOCKS : 0);   // the SMs of the row transfers have no shared memory left
+  const int grid = n_units < sms ? n_units : sms;
+  if (!c->tc_smem_set) {
+    cudaError_t e = bf16 ? cudaFuncSetAttribute(project_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
+                         : cudaFuncSetAttribute(project_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) { cudaGetLastError(); return TAURUS_ERR_CUDA; }
+    c->tc_smem_set = true;
+  }
+  if (bf16) project_tc_kernel<true><<<grid, NUM_THREADS, smem, st>>>(map_x, map_hi, map_lo, map_out, g);
+  else project_tc_kernel<false><<<grid, NUM_THREADS, smem, st>>>(map_x, map_hi, map_lo, map_out, g);
+  c->launches += 1;
+  return TAURUS_OK;
 }

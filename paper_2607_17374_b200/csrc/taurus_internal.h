@@ -194,7 +194,7 @@ struct taurus_ctx {
   float* d_Wcat[TAURUS_MAX_LAYERS] = {nullptr};
   float* d_bias[TAURUS_MAX_LAYERS] = {nullptr};
   bool xfer_smem_set = false;                      // the same for the row transfer kernel
-  bool tc_smem_set[4] = {false, false, false, false};                        // dynamic shared memory limit of the projection kernel raised
+  bool tc_smem_set = false;                        // dynamic shared memory limit of the projection kernel raised
   void* tc_image[TAURUS_MAX_LAYERS] = {nullptr};   // tensor-core operand images of Wcat (owned by kernels_gemm_tc.cu)
   void* tc_image_af[TAURUS_MAX_LAYERS] = {nullptr};   // SAGE aggregate-first layers: image of [W_neigh ; W_self] stacked along K
   float* d_Waf[TAURUS_MAX_LAYERS] = {nullptr};       //   the same matrix row-major [2 Kp x Hp] for the FFMA kernel
