@@ -103,7 +103,15 @@ typedef struct {
 
 typedef struct {
   int64_t chunk_sources;    /* largest number of sources one push may carry (Sect. 3.3)                    */
-  int64_t pool_slots;       /* capacity of the accumulator slot pool (hot store, Sect. 3.5.2)              */
+  int64_t pool_slots;       /* capacity of the accumulator slot pool (hot store, Sect. 3.5.2).  With pool_slots >= V nothing is
+                               ever evicted, and the library keeps the rows the sources send in place of accumulators and sums
+                               a vertex's in-list once, when its last message has arrived (same messages, states and accounting,
+                               sums in another order).  Device memory then: V rows of the widest layer's sent row (2 x the output
+                               width where a SAGE layer projects first, else the accumulator's width) and per edge 4 B (sampled
+                               layers: 8) plus 12 B per (grid chunk, destination) group, at most one per edge and vertex; up to
+                               48 B per edge more while taurus_graph_init runs.  Chosen where that is at most half of the
+                               device memory free at that point, or no more than accumulators take; dropped for accumulators when
+                               one of its allocations fails, with TAURUS_FLAG_PUSH_FORM or TAURUS_FLAG_NO_GROUPING                */
   int64_t hub_count;        /* vertices pinned in the hub store: the largest by (in_degree desc, id asc)   */
   const int32_t* fanout;    /* [L] per-layer fanout, 0 = exact; NULL = all exact; at most 64 (host pointer) */
   uint64_t seed;            /* seed of the neighbour-sampling hash                                         */
@@ -131,7 +139,7 @@ enum {
 enum {
   TAURUS_FLAG_SIMT_GEMM = 2,    /* use the plain fp32 FFMA projection kernel instead of the tensor-core one         */
   TAURUS_FLAG_NO_GROUPING = 4,  /* do not build the destination-grouped edge order: every chunk takes the CSR-order kernels */
-  TAURUS_FLAG_PROJECT_FIRST = 8 /* always project a chunk before scattering it.  Without this flag a layer whose
+  TAURUS_FLAG_PROJECT_FIRST = 8, /* always project a chunk before scattering it.  Without this flag a layer whose
                                    input rows are at most 3/4 as wide as its output rows aggregates the (scaled) input rows and
                                    applies the weights to the finished rows instead (exact by linearity, Sect. 3.6 / 3.9): the
                                    accumulators, the scatter traffic and every evicted row shrink by d_in / d_out.  SAGE layers
@@ -140,6 +148,7 @@ enum {
                                    for the life of the context.  They take this order only while that store fits in the
                                    device memory free at taurus_graph_init beside an estimate of everything else the context
                                    allocates; taurus_get_layer_plan tells which order a layer got */
+  TAURUS_FLAG_PUSH_FORM = 16 /* accumulate by scatter also where the pool holds every vertex (see pool_slots) */
 };
 
 /* Integer accounting of one layer pass (Sect. 4.4-4.7 report these quantities). */

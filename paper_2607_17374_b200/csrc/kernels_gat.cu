@@ -35,7 +35,7 @@ __global__ void gat_split_kernel(const float* __restrict__ PT, int ldpt, int n, 
       const size_t at = (size_t)(src_begin + r) * heads + gl();
       att_s[at] = s;
       att_t[at] = t;
-      att_max[at] = s;   // the self message takes part in the maximum
+      if (att_max) att_max[at] = s;   // the self message takes part in the maximum
     }
   }
 }
@@ -112,7 +112,7 @@ __global__ void gat_scores_kernel(const float* __restrict__ X, int ldx, int n, i
     if (gl() == 0) {
       att_s[src_begin + r] = s;
       att_t[src_begin + r] = t;
-      att_max[src_begin + r] = s;
+      if (att_max) att_max[src_begin + r] = s;
     }
   }
 }

@@ -22,8 +22,8 @@
 #include "taurus_internal.h"
 
 #define FULL 0xffffffffu
-#define HEAVY_DEGREE 256     // in-lists longer than this are summed in segments
-#define HEAVY_SEGMENT 128
+#define HEAVY_DEGREE TAURUS_HEAVY_DEGREE
+#define HEAVY_SEGMENT TAURUS_HEAVY_SEGMENT
 
 namespace {
 

@@ -1201,7 +1201,7 @@ __global__ void window_edges_kernel(long long V, long long window, const long lo
 
 long long max_window_edges(taurus_ctx* c) {
   unsigned long long* d = nullptr;
-  if (cudaMalloc(&d, sizeof(unsigned long long)) != cudaSuccess) return -1;
+  if (cudaMalloc(&d, sizeof(unsigned long long)) != cudaSuccess) return -2;   // no memory
   cudaMemset(d, 0, sizeof(unsigned long long));
   window_edges_kernel<<<c->sm_count * 8, 256>>>(c->V, c->chunk_sources, c->d_row_ptr, d);
   unsigned long long h = 0;

@@ -108,7 +108,31 @@ extern "C" void taurus_destroy(taurus_ctx* c) {
   delete c;
 }
 
-static int init_impl(taurus_ctx* c, const taurus_graph* g, const taurus_model* m, const taurus_run* r) {
+// Device memory of the pull form: what it keeps, what its build takes on top, and what the push form keeps in its place.
+struct ResidentBytes { double kept, build, push; };
+static ResidentBytes resident_bytes(const taurus_ctx* c, int max_fanout, int af_kmax) {
+  const double V = (double)c->V, E = (double)c->E, items = E + V;   // at most one item per edge and vertex
+  const bool sampled = max_fanout > 0, sage = c->mode == TAURUS_SAGE_MEAN;
+  int row = 4, sum = 4;                                             // floats of a stored row, of a summed row
+  for (int l = 0; l < c->L; ++l) {
+    row = std::max(row, resident_row(c, l));
+    sum = std::max(sum, taurus_round_up(c->agg_first[l] ? c->dims[l] : c->dims[l + 1], 4));
+  }
+  const double heavy = std::min(V, E / TAURUS_HEAVY_DEGREE);        // vertices with long in-lists, at most
+  ResidentBytes r;
+  // rows, items, in-list sources and offsets (offsets: where no layer is sampled), long in-lists with their segments, kept
+  // sources and entries of sampled layers
+  r.kept = V * row * 4.0 + items * 12.0 + E * 4.0 + (sampled ? V * max_fanout * 4.0 + E / 8.0 : V * 8.0) + heavy * (sum * 4.0 + 8.0) +
+           (E / TAURUS_HEAVY_SEGMENT + heavy) * 16.0;
+  r.build = V * 8.0 + (sampled ? 0.0 : E * 16.0) + items * 32.0;    // sorts (their own scratch is as large as what they sort), order of the items
+  // accumulators, slots, locations, grouped edge order, chunk projection, input rows of aggregate-first SAGE layers
+  r.push = ((double)c->pool_slots + c->hub_count) * c->Hmax * 4.0 + (double)c->pool_slots * 16.0 + V * 4.0 + E * (sampled ? 16.125 : 12.0) +
+           (c->mode == TAURUS_GAT ? V * c->heads * 4.0 : (double)c->chunk_sources * c->Hmax * 8.0) + (sage ? V * af_kmax * 4.0 : 0.0);
+  return r;
+}
+
+// push_form: the pull form of resident pools is not to be used (an allocation it needed failed).
+static int init_impl(taurus_ctx* c, const taurus_graph* g, const taurus_model* m, const taurus_run* r, bool push_form) {
   cudaDeviceProp prop;
   CU(cudaGetDevice(&c->device));
   CU(cudaGetDeviceProperties(&prop, c->device));
@@ -244,28 +268,33 @@ static int init_impl(taurus_ctx* c, const taurus_graph* g, const taurus_model* m
   }
 
   // per-vertex state
-  ALLOC(c->d_pend, V); ALLOC(c->d_state, V); ALLOC(c->d_loc, V); ALLOC(c->d_touch, V); ALLOC(c->d_reload, V);
+  ALLOC(c->d_pend, V); ALLOC(c->d_state, V); ALLOC(c->d_touch, V); ALLOC(c->d_reload, V);
   ALLOC(c->d_rank_hist, (V + 63) / 64);
-  // A pool that holds every vertex keeps the rows the sources send instead of accumulators (kernels_resident.cu), where the
-  // in-lists and their build fit beside them; else the push form.
+  // A pool that holds every vertex keeps the rows the sources send instead of accumulators (kernels_resident.cu): the pull
+  // form.  It takes 2 x the row memory where SAGE projects first (P and T of every vertex) and, with its items, up to 12 B
+  // more per edge, so it is chosen where it leaves at least half of the memory free at this point to the rest of the
+  // program, or takes no more than the push form; taurus_graph_init comes back here without it if an allocation fails all the same.
   const bool grouping = !(c->flags & TAURUS_FLAG_NO_GROUPING);
-  int store_floats = 0;
-  for (int l = 0; l < c->L; ++l) store_floats = std::max(store_floats, resident_row(c, l));
   int max_fanout = 0;
   for (int l = 0; l < c->L; ++l) max_fanout = std::max(max_fanout, c->fanout[l]);
-  if (grouping && c->pool_slots >= V && E + V < (1ll << 31) && V * std::max(max_fanout, 1) < (1ll << 31)) {
-    const double rows_b = (double)V * store_floats * 4.0 + (double)c->drain_rows * (c->Hmax + (af_kmax > 0 ? 2 * af_kmax : 0)) * 4.0;
-    const double graph_b = (double)(E + V) * (12.0 + 36.0) + (double)E * 8.0 + (double)V * max_fanout * 4.0;   // in-lists and items, and their build
+  if (grouping && !push_form && !(c->flags & TAURUS_FLAG_PUSH_FORM) && c->pool_slots >= V && E + V < (1ll << 31) && V * std::max(max_fanout, 1) < (1ll << 31)) {
+    const ResidentBytes r = resident_bytes(c, max_fanout, af_kmax);
     CU(cudaMemGetInfo(&free_b, &total_b));
-    c->resident = rows_b + graph_b + 2e9 < 0.95 * (double)free_b || rows_b + graph_b < 0.5 * (double)free_b;
+    c->resident = r.kept + r.build <= 0.5 * (double)free_b || (r.kept <= r.push && r.kept + r.build <= 0.9 * (double)free_b);
   }
   // pool, hub store
-  if (c->resident) ALLOC(c->d_store, (size_t)V * store_floats);
-  else ALLOC(c->d_acc, (size_t)(c->pool_slots + c->hub_count) * c->Hmax);
+  if (c->resident) {
+    int store_floats = 0;
+    for (int l = 0; l < c->L; ++l) store_floats = std::max(store_floats, resident_row(c, l));
+    ALLOC(c->d_store, (size_t)V * store_floats);
+  } else {
+    ALLOC(c->d_loc, V);
+    ALLOC(c->d_acc, (size_t)(c->pool_slots + c->hub_count) * c->Hmax);
+  }
   {
     // a push of at most chunk_sources sources touches at most its edges plus its own vertices
     long long max_edges = max_window_edges(c);
-    if (max_edges < 0) return TAURUS_ERR_CUDA;
+    if (max_edges < 0) return max_edges == -2 ? TAURUS_ERR_NOMEM : TAURUS_ERR_CUDA;
     c->touched_capacity = std::min<long long>(V, max_edges + c->chunk_sources);
     ALLOC(c->d_touched_list, c->touched_capacity);
   }
@@ -322,10 +351,11 @@ static int init_impl(taurus_ctx* c, const taurus_graph* g, const taurus_model* m
     CU(cudaEventCreateWithFlags(&c->fin_done[i], cudaEventDisableTiming));
     CU(cudaEventCreateWithFlags(&c->out_done[i], cudaEventDisableTiming));
   }
-  ALLOC(c->d_PT, (size_t)c->chunk_sources * 2 * c->Hmax);
+  if (!c->resident || c->mode == TAURUS_GAT) ALLOC(c->d_PT, (size_t)c->chunk_sources * 2 * c->Hmax);   // (a resident pool's projection writes the store)
   if (c->mode == TAURUS_GAT) {
     const size_t nh = (size_t)V * c->heads;
-    ALLOC(c->d_att_s, nh); ALLOC(c->d_att_t, nh); ALLOC(c->d_att_max, nh); ALLOC(c->d_att_tm, nh); ALLOC(c->d_att_z, nh);
+    ALLOC(c->d_att_s, nh); ALLOC(c->d_att_t, nh); ALLOC(c->d_att_tm, nh); ALLOC(c->d_att_z, nh);
+    if (!c->resident) ALLOC(c->d_att_max, nh);   // running maximum of the edge sweeps
   }
   if (af_kmax > 0) {
     const bool sage = c->mode == TAURUS_SAGE_MEAN;
@@ -412,15 +442,19 @@ extern "C" int taurus_graph_init(taurus_ctx** out, const taurus_graph* g, const 
   if (r->drain_rows < 1 || r->drain_rows >= (1ll << 31)) return TAURUS_ERR_INVALID_ARG;
   if (r->evict_policy < TAURUS_EVICT_FEWEST_PENDING || r->evict_policy > TAURUS_EVICT_RANDOM) return TAURUS_ERR_INVALID_ARG;
   if (r->pool_slots + r->hub_count >= (1ll << 31)) return TAURUS_ERR_INVALID_ARG;
-  taurus_ctx* c = new (std::nothrow) taurus_ctx();
-  if (!c) return TAURUS_ERR_NOMEM;
-  c->pend_chunk = new (std::nothrow) PendingChunk();
-  if (!c->pend_chunk) { delete c; return TAURUS_ERR_NOMEM; }
-  int rc;
-  try { rc = init_impl(c, g, m, r); } catch (const std::bad_alloc&) { rc = TAURUS_ERR_NOMEM; }
-  if (rc != TAURUS_OK) { taurus_destroy(c); return rc; }
-  *out = c;
-  return TAURUS_OK;
+  for (bool push_form : {false, true}) {
+    taurus_ctx* c = new (std::nothrow) taurus_ctx();
+    if (!c) return TAURUS_ERR_NOMEM;
+    c->pend_chunk = new (std::nothrow) PendingChunk();
+    if (!c->pend_chunk) { delete c; return TAURUS_ERR_NOMEM; }
+    int rc;
+    try { rc = init_impl(c, g, m, r, push_form); } catch (const std::bad_alloc&) { rc = TAURUS_ERR_NOMEM; }
+    if (rc == TAURUS_OK) { *out = c; return TAURUS_OK; }
+    const bool again = rc == TAURUS_ERR_NOMEM && c->resident;   // the push form of the same pool may still fit
+    taurus_destroy(c);
+    if (!again) return rc;
+  }
+  return TAURUS_ERR_NOMEM;
 }
 
 // Reads the device control block up to the chunks' own counters, once everything on `st` and the output stream is through,

@@ -16,6 +16,8 @@
 #define TAURUS_PUSH_EVENTS 12                   // CUDA events per timed push
 #define TAURUS_PHASES 9                         // durations reported per timed push
 #define TAURUS_XFER_BLOCKS 4                     // SMs that carry rows across the host link (one block each, all of its shared memory)
+#define TAURUS_HEAVY_DEGREE 256                  // resident pools: in-lists longer than this are summed in segments
+#define TAURUS_HEAVY_SEGMENT 128
 #define TAURUS_SEL_BITS 11                      // radix-select digit width
 #define TAURUS_SEL_BINS (1 << TAURUS_SEL_BITS)
 #define TAURUS_SEL_LEVELS 6                     // 6 x 11 = 66 bits >= the 62-bit (score, id) key
@@ -218,7 +220,7 @@ struct taurus_ctx {
   int heads = 1;                // GAT: attention heads
   float* d_att_s = nullptr;     // [V] att_src . h'
   float* d_att_t = nullptr;     // [V] att_dst . h'
-  float* d_att_max = nullptr;   // [V] running maximum of att_src . h'_u over the neighbourhood
+  float* d_att_max = nullptr;   // [V] running maximum of att_src . h'_u over the neighbourhood (null in resident pools)
   float2* d_att_tm = nullptr;   // [V] (t, maximum score)
   float* d_att_w[TAURUS_MAX_LAYERS] = {nullptr};   // per layer: W att_src then W att_dst, dims[l] floats each (scores without the transformed rows)
   double* d_att_z = nullptr;    // [V x heads] normaliser
