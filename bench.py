@@ -41,13 +41,12 @@ import taurus_gen as tg  # noqa: E402
 
 METRIC = "edges/sec per GNN layer (GTEPS)"
 
-# DRAM bytes (read + write) of the 256-float scatter_grouped_kernel instance per algorithmic byte, from the ncu capture
-# summarised in profiles/scatter_grouped_kernel_mid_1200k.md (two launches: 2.691 and 2.721 GB measured against 2.143 and
-# 2.164 GB algorithmic).  The figure belongs to the kernel source with the digest below (sha256 of csrc/kernels_group.cu,
-# first 16 hex digits); when the source has changed since the capture the bench prints traffic = null instead of a
-# stale number.
-SCATTER_TRAFFIC_OVER_ALGORITHMIC = 1.257
-SCATTER_CAPTURE_SOURCE = "85d27983976ae3e5"
+# DRAM bytes (read + write) per requested byte of the 256-float gather_kernel instance, from the ncu capture summarised in
+# profiles/gather_kernel_mid_1200k.md.  The figure belongs to the kernel source with the digest below (sha256 of
+# csrc/kernels_resident.cu, first 16 hex digits); when the source has changed since the capture the bench prints
+# traffic = null instead of a stale number.
+GATHER_TRAFFIC_OVER_REQUESTED = None
+GATHER_CAPTURE_SOURCE = ""
 
 
 def source_digest(name: str) -> str:
@@ -368,6 +367,14 @@ def scatter_bytes(groups, edges, n_src, width, self_row):
     return groups * (8 * width + 8) + edges * 8 + n_src * (4 * width + (12 * width if self_row else 0) + 8)
 
 
+def gather_bytes(messages, V, width, out_width, self_row):
+    """Bytes the gather of a pool that holds every vertex asks for: per propagated edge one stored row of the source (4 width) and
+    its index (4); per vertex its own row (4 width, where the layer has a self message in row form), its in-list offsets, list entry
+    and degree words (28) and its finished row once (4 out_width).  Neighbouring destinations share sources, so part of the row
+    reads are L2 hits: the rate can exceed what HBM delivers."""
+    return messages * (4 * width + 4) + V * ((4 * width if self_row else 0) + 28 + 4 * out_width)
+
+
 def link_peaks(env, mb=256, reps=3):
     """Pinned-memory copy bandwidth of this machine, GB/s: host -> device alone, device -> host alone, and both at once on
     two streams (per direction).  Plain asynchronous copies of `mb` MB, best of `reps`."""
@@ -615,6 +622,7 @@ def run_full_pass(args, env, w):
     stream = torch.cuda.current_stream()
     edges_per_layer = []
     groups_per_layer = []
+    push_launches = []                                 # of the last push of every layer of the first step
 
     def step(feat0, final_out, collect_stats=False):
         """One pass over all layers.  feat0 is the layer-0 feature matrix (device for `value`, pinned host for e2e);
@@ -639,14 +647,20 @@ def run_full_pass(args, env, w):
                 runs[l].reset()
                 ctx.layer_set_run_output(runs[l])
                 for (s, e) in chunks:
+                    n0 = ctx.launch_count()
                     if l == 0 or gat:      # gat: pass 3 streams the transformed rows of pass 1
                         ctx.push_chunk(s, e, src[s:e], stream)
                     else:
                         ctx.push_chunk_from_runs(s, e, runs[l - 1], stream)
+                if collect_stats:
+                    push_launches.append(ctx.launch_count() - n0)
             else:
                 ctx.layer_set_dense_output(out, d_out)   # finalised rows go straight to their place in the matrix
                 for (s, e) in chunks:
+                    n0 = ctx.launch_count()
                     ctx.push_chunk(s, e, src[s:e], stream)
+                if collect_stats:
+                    push_launches.append(ctx.launch_count() - n0)
             st = ctx.layer_end()
             if collect_stats:
                 edges_per_layer.append(st["total_messages"])
@@ -667,7 +681,7 @@ def run_full_pass(args, env, w):
     # ---- device-resident timing
     sampler = ClockSampler(env.local)
     sampler.start()
-    # Inside the timed region the library records the two events around every scatter launch and nothing else: an
+    # Inside the timed region the library records the two events around every scatter (or gather) launch and nothing else: an
     # event after each of a push's phases costs about 2 us of the stream, 4-5 % of a step of 114 pushes.  The phase
     # split comes from one more, untimed step with all events on.
     ctx.set_timing(2)
@@ -692,25 +706,27 @@ def run_full_pass(args, env, w):
     ms_max = max_over_ranks(ms, world, dev)
     value = whole_job_value(msgs_per_step, args.steps, world, ms_max)
 
-    # ---- roofline of the dominant kernel (the scatter), from the events recorded inside the timed region
+    # ---- roofline of the dominant kernel, from the events recorded inside the timed region: the gather where the pool holds
+    # every vertex and the library keeps the sources' rows, the scatter where it accumulates (--no-grouping, too little memory)
     n_push = len(chunks) * L * args.steps
     ph = phases[:n_push].reshape(args.steps, L, len(chunks), 9)
-    scatter_ms = ph[..., 5]
-    # In CSR order a "group" is one edge.  The per-edge cold-miss model (12 + 2 * 4 width per edge) is kept beside it.
-    layer_bytes, edge_model_bytes = [], []
+    sum_ms = ph[..., 5]
+    pull = min(push_launches) <= 5                     # rows, accounting, gather (and the transform); the accumulating form takes six and more
+    layer_bytes = []
     for l in range(L):
         Wd = acc_width[l]
-        self_row = not (agg_first[l] and w.mode == tg.SAGE_MEAN)   # aggregate-first SAGE adds its self term after the transform
-        layer_bytes.append(scatter_bytes(groups_per_layer[l], edges_per_layer[l], V, Wd, self_row))
-        edge_model_bytes.append(edges_per_layer[l] * (12 + 8 * Wd) + V * (4 * Wd + 8))
-    alg_bytes_step = float(sum(layer_bytes))
-    scatter_total_ms = float(scatter_ms.sum()) / args.steps
+        if pull:
+            sage_af = agg_first[l] and w.mode == tg.SAGE_MEAN   # the finished sum is followed by the vertex's own row
+            out_w = (2 * Wd if sage_af else Wd) if agg_first[l] else w.dims[l + 1]
+            layer_bytes.append(gather_bytes(edges_per_layer[l], V, Wd, out_w, True))
+        else:
+            self_row = not (agg_first[l] and w.mode == tg.SAGE_MEAN)   # aggregate-first SAGE adds its self term after the transform
+            layer_bytes.append(scatter_bytes(groups_per_layer[l], edges_per_layer[l], V, Wd, self_row))
+    sum_total_ms = float(sum_ms.sum()) / args.steps
     pk = peaks()
-    grouped = not args.no_grouping
-    # The dominant kernel is the scatter instance with the largest total time: layers with the same accumulator width
-    # run the same template instance.  `achieved` = its algorithmic bytes / its CUDA-event time; the other instances
-    # are listed per layer, and the figure over all scatter launches is kept as all_scatter_gbs.
-    per_layer_ms = [float(scatter_ms[:, l].sum()) / args.steps for l in range(L)]
+    # The dominant kernel is the instance with the largest total time: layers with the same row width run the same template
+    # instance.  `achieved` = its bytes / its CUDA-event time; the other instances are listed per layer.
+    per_layer_ms = [float(sum_ms[:, l].sum()) / args.steps for l in range(L)]
     by_width = {}
     for l in range(L):
         by_width.setdefault(acc_width[l], []).append(l)
@@ -719,24 +735,24 @@ def run_full_pass(args, env, w):
     dom_ms = sum(per_layer_ms[l] for l in dom)
     dom_bytes = float(sum(layer_bytes[l] for l in dom))
     achieved = dom_bytes / (dom_ms * 1e-3) / 1e9
-    kname = ("scatter_grouped_kernel" if grouped else "scatter_kernel") + " (accumulator rows of %d floats, layers %s)" % (dom_w, dom)
-    capture_valid = grouped and dom_w == 256 and source_digest("kernels_group.cu") == SCATTER_CAPTURE_SOURCE
+    kname = ("gather_kernel (stored rows" if pull else ("scatter_kernel" if args.no_grouping else "scatter_grouped_kernel") + " (accumulator rows") + \
+        " of %d floats, layers %s)" % (dom_w, dom)
+    capture_valid = pull and dom_w == 256 and GATHER_TRAFFIC_OVER_REQUESTED is not None and source_digest("kernels_resident.cu") == GATHER_CAPTURE_SOURCE
     roofline = dict(bound="hbm", kernel=kname, achieved=achieved,
                     peak=pk["hbm_gbs"], unit="GB/s", frac=achieved / pk["hbm_gbs"], peak_source=pk["source"],
-                    traffic=SCATTER_TRAFFIC_OVER_ALGORITHMIC * dom_bytes / (len(chunks) * len(dom)) if capture_valid else None,
+                    bytes_note="requested bytes: one stored row per message, one finished row per vertex; rows shared by neighbouring "
+                               "destinations are partly L2 hits" if pull else "algorithmic bytes of the row reductions",
+                    traffic=GATHER_TRAFFIC_OVER_REQUESTED * dom_bytes / (len(chunks) * len(dom)) if capture_valid else None,
                     traffic_note=("ncu dram read+write per launch of the 256-float kernel on a 1.2 M-vertex instance, scaled by the "
-                                  "algorithmic bytes of a launch "
-                                  "(profiles/scatter_grouped_kernel_mid_1200k.md)") if capture_valid else
-                                 "no capture of this kernel source (profiles/scatter_grouped_kernel_mid_1200k.md names the source it measured)",
+                                  "requested bytes of a launch (profiles/gather_kernel_mid_1200k.md)") if capture_valid else
+                                 "no capture of this kernel source",
                     launches_per_step=len(chunks) * len(dom), avg_launch_ms=dom_ms / (len(chunks) * len(dom)),
                     algorithmic_bytes_per_launch=dom_bytes / (len(chunks) * len(dom)),
                     share_of_step=dom_ms / (ms_max / args.steps),
-                    all_scatter_gbs=alg_bytes_step / (scatter_total_ms * 1e-3) / 1e9,
-                    edge_model_gbs=float(sum(edge_model_bytes)) / (scatter_total_ms * 1e-3) / 1e9,
-                    per_layer=[dict(layer=l, scatter_ms=per_layer_ms[l],
-                                    gbs=layer_bytes[l] / (per_layer_ms[l] * 1e-3) / 1e9,
-                                    groups=int(groups_per_layer[l]), accumulator_floats=acc_width[l], aggregate_first=bool(agg_first[l]),
-                                    gteps_scatter_only=edges_per_layer[l] / (per_layer_ms[l] * 1e-3) / 1e9)
+                    all_layers_gbs=float(sum(layer_bytes)) / (sum_total_ms * 1e-3) / 1e9,
+                    per_layer=[dict(layer=l, ms=per_layer_ms[l], gbs=layer_bytes[l] / (per_layer_ms[l] * 1e-3) / 1e9,
+                                    groups=int(groups_per_layer[l]), row_floats=acc_width[l], aggregate_first=bool(agg_first[l]),
+                                    gteps_kernel_only=edges_per_layer[l] / (per_layer_ms[l] * 1e-3) / 1e9)
                                for l in range(L)])
     phase_ms = dict(zip(PHASES, [float(x) for x in ph_all.sum(axis=(0, 1, 2))]))
 
@@ -800,11 +816,13 @@ def run_full_pass(args, env, w):
                             mode=["sage_mean", "gcn_sym", "gin_sum", "gat"][w.mode], output=args.output, evict_policy=args.evict_policy,
                             step="one pass over every layer and chunk of the workload",
                             messages_per_step=msgs_per_step,
-                            l2="inputs larger than L2 (accumulators %.1f GB)" % (w.pool_slots * 4 * max(w.dims[1:]) / 1e9),
+                            l2="inputs larger than L2 (rows of one layer %.1f GB)" % (V * 4 * max(w.dims[1:]) / 1e9),
                             parallelism="replicas only" if world > 1 else "1 gpu",
                             phase_note="phase_ms, layer_ms and phase_ms_per_layer: one extra step after the timed ones with an event after "
                                        "every phase of every push (those events lengthen the step by 4-5 %, so the timed steps record "
-                                       "only the events around the scatter launches that the roofline uses)",
+                                       "only the events around the gather or scatter launches that the roofline uses); on a pool "
+                                       "that holds every vertex classify_select is the wait for the accounting beside copy-in and "
+                                       "projection, and scatter the gather (which finishes project-first rows)",
                             layer_ms=[float(ph_all[:, l, :, :8].sum()) for l in range(L)], phase_ms=phase_ms,
                             phase_ms_per_layer=[dict(zip(PHASES, [round(float(x), 3) for x in ph_all[:, l].sum(axis=(0, 1))]))
                                                 for l in range(L)]),

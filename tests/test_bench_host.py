@@ -31,6 +31,13 @@ def test_scatter_bytes_by_hand():
     assert bench.scatter_bytes(10, 25, 4, 8, False) == 10 * (64 + 8) + 25 * 8 + 4 * (32 + 8)
 
 
+def test_gather_bytes_by_hand():
+    # 25 messages of rows of 8 floats (32 bytes and a 4-byte index each), 4 vertices: own row (32), 28 bytes of words, finished
+    # row of 6 floats (24)
+    assert bench.gather_bytes(25, 4, 8, 6, True) == 25 * 36 + 4 * (32 + 28 + 24)
+    assert bench.gather_bytes(25, 4, 8, 16, False) == 25 * 36 + 4 * (28 + 64)
+
+
 def test_which_workloads_are_timed_in_windows():
     assert not bench.windowed(tg.WORKLOADS["mid"]) and not bench.windowed(tg.WORKLOADS["tiny"])
     for name in ("large", "sampled", "stress"):
