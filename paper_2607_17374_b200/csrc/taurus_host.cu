@@ -461,13 +461,14 @@ extern "C" int taurus_graph_init(taurus_ctx** out, const taurus_graph* g, const 
 // and returns its sticky error.  One copy into pinned memory and one wait: the calls that block (drains, layer_end, stats)
 // are paid per chunk or per layer.  with_stats: the reload histogram comes along.
 static int finish_chunk(taurus_ctx* c, cudaStream_t st);
+static int sticky_error(const taurus_ctx* c) { return c->half_applied ? c->half_applied : c->h_ctl->error; }
 static int read_ctl(taurus_ctx* c, cudaStream_t st, bool with_stats = false) {
   { int rc = finish_chunk(c, st); if (rc) return rc; }   // the last chunk's finalise may still be waiting for a successor
   if (with_stats) launch_reload_histogram(c, st);
   CU(cudaMemcpyAsync(c->h_ctl, c->d_ctl, offsetof(DevCtl, pc), cudaMemcpyDeviceToHost, st));
   CU(cudaStreamSynchronize(st));
   CU(cudaStreamSynchronize(c->out_stream));
-  return c->h_ctl->error;
+  return sticky_error(c);
 }
 
 extern "C" int taurus_layer_begin(taurus_ctx* c, int32_t layer, void* cuda_stream) {
@@ -487,6 +488,7 @@ extern "C" int taurus_layer_begin(taurus_ctx* c, int32_t layer, void* cuda_strea
   c->half_used[0] = c->half_used[1] = false;
   c->x_used[0] = c->x_used[1] = false;
   memset(c->h_ctl, 0, sizeof(DevCtl));
+  c->half_applied = TAURUS_OK;
   c->next_src = 0; c->chunk_seq = 0; c->ub_since_drain = 0; c->last_stream = st;
   launch_layer_reset(c, layer, st);
   c->d_mask_cur = nullptr;
@@ -610,13 +612,13 @@ static int hand_off(taurus_ctx* c, const ChunkArgs& a, int l, long long bound, c
   return run_rc;
 }
 
-static int finish_chunk(taurus_ctx* c, cudaStream_t st) {
-  if (!c->pending) return TAURUS_OK;
-  c->pending = false;
+// The deferred part of the chunk pushed last.  *applied: as in push_enqueue.
+static int finish_enqueue(taurus_ctx* c, cudaStream_t st, bool* applied) {
   const PendingChunk& p = *c->pend_chunk;
   const ChunkArgs& a = p.a;
   const int l = p.layer;
   cudaEvent_t* pev = p.timed_index >= 0 && c->timing != 2 ? &c->phase_ev[(size_t)p.timed_index * TAURUS_PUSH_EVENTS] : nullptr;
+  *applied = true;
   if (c->pipelined) {
     CU(cudaStreamWaitEvent(st, c->xfer_done, 0));   // reloaded partial sums have been added to the chunk's rows
     if (pev) cudaEventRecord(pev[8], st);           // (without transfers the finalise follows event 7 directly)
@@ -624,14 +626,24 @@ static int finish_chunk(taurus_ctx* c, cudaStream_t st) {
   if (a.dense_half >= 0 && c->half_used[a.dense_half]) CU(cudaStreamWaitEvent(st, c->out_done[a.dense_half], 0));
   if (p.af) {
     int rc = launch_af_finalise(c, a, l, std::min<long long>(p.bound, a.grad_cap), st);
-    if (rc) { c->h_ctl->error = rc; return rc; }   // the chunk is half applied: the layer has to be begun again
+    if (rc) return rc;
   } else {
     launch_finalise(c, a, st);
   }
   const int run_rc = hand_off(c, a, l, p.bound, st);
   if (pev) cudaEventRecord(pev[9], st);
   CU(cudaGetLastError());
+  *applied = false;   // an error of the run store is about rows already finished
   return run_rc;
+}
+
+static int finish_chunk(taurus_ctx* c, cudaStream_t st) {
+  if (!c->pending) return TAURUS_OK;
+  c->pending = false;
+  bool applied = false;
+  const int rc = finish_enqueue(c, st, &applied);
+  if (rc && applied) c->half_applied = rc;
+  return rc;
 }
 
 // S1: features of sources [s, e) ([n x K], rows contiguous) to the device.  Host chunks are copied on the library's
@@ -658,33 +670,12 @@ static int stage_chunk(taurus_ctx* c, const float* features, taurus_runs* src_ru
   return TAURUS_OK;
 }
 
-// One chunk through S1..S7.  The features come from `features` (host or device memory) or, when `src_runs` is
-// given, from the sorted runs of the previous layer by merge-on-read.
-static int push_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const float* features, taurus_runs* src_runs, void* cuda_stream) {
-  if (!c || (!features && !src_runs)) return TAURUS_ERR_INVALID_ARG;
-  if (c->layer < 0) return TAURUS_ERR_ORDER;
-  if (src_begin != c->next_src) return TAURUS_ERR_ORDER;
-  if (src_end <= src_begin || src_end > c->V || src_end - src_begin > c->chunk_sources) return TAURUS_ERR_INVALID_ARG;
-  if (features && (reinterpret_cast<uintptr_t>(features) & 3) != 0) return TAURUS_ERR_INVALID_ARG;
-  const bool gat = c->mode == TAURUS_GAT;   // pass 3: the features are the transformed rows h'
-  if (gat && !c->gat_ready) return TAURUS_ERR_ORDER;
-  if (src_runs && (runs_width(src_runs) != c->dims[c->layer + (gat ? 1 : 0)] || runs_vertices(src_runs) != c->V ||
-                   runs_max_chunk(src_runs) < src_end - src_begin || src_runs == c->run_out))
-    return TAURUS_ERR_INVALID_ARG;
-  if (c->h_ctl->error) return c->h_ctl->error;
-  const long long bound = completion_bound(c, src_begin, src_end);
-  const bool direct_dense = c->dense_out && c->dense_is_device;   // rows are finalised straight into the caller's matrix
-  const bool halves = (c->dense_out && !direct_dense) || c->run_out;
-  if (halves ? bound > c->drain_rows / 2 : (direct_dense ? bound : c->ub_since_drain + bound) > c->drain_rows) return TAURUS_ERR_DRAIN_FULL;
-  cudaStream_t st = (cudaStream_t)cuda_stream;
-  CU(cudaSetDevice(c->device));
+// One chunk through S1..S7 on `st`, after push_core's checks.  *applied: set while the chunk has been enqueued in part, so that an
+// error in between leaves a layer that cannot go on.
+static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const float* features, taurus_runs* src_runs, long long bound,
+                        bool direct_dense, bool halves, cudaStream_t st, bool* applied) {
+  const bool gat = c->mode == TAURUS_GAT;
   const int l = c->layer;
-  if (c->agg_first[l] && !direct_dense && !halves && !c->d_af_O) {
-    // rows drained by the caller: their place in the graduation buffer is a device-side count, so the transform of
-    // the finished rows writes a scratch matrix first.  Allocated here, before anything of the chunk is enqueued, so
-    // that a failure leaves the layer untouched.
-    ALLOC(c->d_af_O, (size_t)c->drain_rows * c->Hmax);
-  }
   if (st != c->last_stream) {   // keep chunk order across streams
     CU(cudaEventRecord(c->order_event, c->last_stream));
     CU(cudaStreamWaitEvent(st, c->order_event, 0));
@@ -715,6 +706,7 @@ static int push_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const fl
     const bool cell = src_begin % c->chunk_sources == 0 && src_end == std::min<long long>(c->V, src_begin + c->chunk_sources);
     CU(cudaStreamWaitEvent(c->account_stream, c->account_go, 0));
     if (acc.dense_half >= 0 && c->half_used[acc.dense_half]) CU(cudaStreamWaitEvent(c->account_stream, c->out_done[acc.dense_half], 0));
+    *applied = true;
     launch_account(c, acc, cell ? src_begin / c->chunk_sources : -1, c->account_stream);
     CU(cudaEventRecord(c->account_done, c->account_stream));
   }
@@ -732,7 +724,7 @@ static int push_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const fl
       launch_store_rows(c, X, ldx, n, K, w, src_begin, false, rows, st);
     } else if (project_tc_usable(c, l, X, ldx)) {
       int rc = launch_project_tc(c, l, X, ldx, src_begin, n, rows, st);
-      if (rc) { c->h_ctl->error = rc; return rc; }   // the chunk is half applied
+      if (rc) return rc;
     } else {
       launch_project_simt(c, l, X, ldx, src_begin, n, rows, st);
     }
@@ -741,16 +733,17 @@ static int push_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const fl
     CU(cudaStreamWaitEvent(st, c->account_done, 0));
     if (timing) cudaEventRecord(pev[3], st);
     if (scatter_timing) cudaEventRecord(pev[5], st);
-    { int rc = launch_gather(c, a, c->d_store, w, af ? c->d_af_A : nullptr, std::min<long long>(bound, a.grad_cap), st); if (rc) { c->h_ctl->error = rc; return rc; } }
+    { int rc = launch_gather(c, a, c->d_store, w, af ? c->d_af_A : nullptr, std::min<long long>(bound, a.grad_cap), st); if (rc) return rc; }
     if (scatter_timing) cudaEventRecord(pev[6], st);
     if (timing) cudaEventRecord(pev[7], st);
     if (af) {
       int rc = launch_af_finalise(c, a, l, std::min<long long>(bound, a.grad_cap), st);
-      if (rc) { c->h_ctl->error = rc; return rc; }   // the chunk is half applied: the layer has to be begun again
+      if (rc) return rc;
     }
     const int rc = hand_off(c, a, l, bound, st);
     if (timing) cudaEventRecord(pev[9], st);
     CU(cudaGetLastError());
+    *applied = false;   // wholly: an error of the run store is about rows already finished
     c->next_src = src_end;
     c->chunk_seq += 1;
     if (!halves && !direct_dense) c->ub_since_drain += bound;
@@ -795,10 +788,11 @@ static int push_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const fl
   if (xbuf >= 0 && !x_in_use) { CU(cudaEventRecord(c->x_free[xbuf], st)); c->x_used[xbuf] = true; }
   if (timing) cudaEventRecord(pev[2], st);
   // S3, S4
+  *applied = true;
   const bool grouped = c->d_gdst != nullptr && src_begin % c->chunk_sources == 0 &&
                        src_end == std::min<long long>(c->V, src_begin + c->chunk_sources);
   if (grouped) launch_classify_grouped(c, a, st); else launch_classify(c, a, st);
-  { int rc = launch_make_room(c, a, st, timing ? pev[3] : nullptr); if (rc) { c->h_ctl->error = rc; return rc; } }   // pev[3]: victims chosen and placed, rows not yet moved
+  { int rc = launch_make_room(c, a, st, timing ? pev[3] : nullptr); if (rc) return rc; }   // pev[3]: victims chosen and placed, rows not yet moved
   // The chunk before this one: its rows have been crossing the host link since its slots were handed out.  Its
   // finalise runs now, before this chunk takes over the slots it released.
   int run_rc = finish_chunk(c, st);
@@ -809,7 +803,7 @@ static int push_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const fl
     CU(cudaEventRecord(c->moves_ready, st));
     CU(cudaStreamWaitEvent(c->xfer_stream, c->moves_ready, 0));
     if (timing) cudaEventRecord(pev[10], c->xfer_stream);
-    { int rc = launch_transfer(c, a, c->xfer_stream); if (rc) { c->h_ctl->error = rc; return rc; } }
+    { int rc = launch_transfer(c, a, c->xfer_stream); if (rc) return rc; }
     if (timing) cudaEventRecord(pev[11], c->xfer_stream);
     CU(cudaEventRecord(c->xfer_done, c->xfer_stream));
   }
@@ -825,10 +819,45 @@ static int push_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const fl
   c->pending = true;
   if (!c->pipelined) { int rc = finish_chunk(c, st); if (!run_rc) run_rc = rc; }
   CU(cudaGetLastError());
+  *applied = false;
   c->next_src = src_end;
   c->chunk_seq += 1;
   if (!halves && !direct_dense) c->ub_since_drain += bound;
   return run_rc;
+}
+
+// The features come from `features` (host or device memory) or, when `src_runs` is
+// given, from the sorted runs of the previous layer by merge-on-read.
+static int push_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const float* features, taurus_runs* src_runs, void* cuda_stream) {
+  if (!c || (!features && !src_runs)) return TAURUS_ERR_INVALID_ARG;
+  if (c->layer < 0) return TAURUS_ERR_ORDER;
+  if (c->half_applied) return c->half_applied;
+  if (src_begin != c->next_src) return TAURUS_ERR_ORDER;
+  if (src_end <= src_begin || src_end > c->V || src_end - src_begin > c->chunk_sources) return TAURUS_ERR_INVALID_ARG;
+  if (features && (reinterpret_cast<uintptr_t>(features) & 3) != 0) return TAURUS_ERR_INVALID_ARG;
+  const bool gat = c->mode == TAURUS_GAT;   // pass 3: the features are the transformed rows h'
+  if (gat && !c->gat_ready) return TAURUS_ERR_ORDER;
+  if (src_runs && (runs_width(src_runs) != c->dims[c->layer + (gat ? 1 : 0)] || runs_vertices(src_runs) != c->V ||
+                   runs_max_chunk(src_runs) < src_end - src_begin || src_runs == c->run_out))
+    return TAURUS_ERR_INVALID_ARG;
+  if (sticky_error(c)) return sticky_error(c);
+  const long long bound = completion_bound(c, src_begin, src_end);
+  const bool direct_dense = c->dense_out && c->dense_is_device;   // rows are finalised straight into the caller's matrix
+  const bool halves = (c->dense_out && !direct_dense) || c->run_out;
+  if (halves ? bound > c->drain_rows / 2 : (direct_dense ? bound : c->ub_since_drain + bound) > c->drain_rows) return TAURUS_ERR_DRAIN_FULL;
+  cudaStream_t st = (cudaStream_t)cuda_stream;
+  CU(cudaSetDevice(c->device));
+  const int l = c->layer;
+  if (c->agg_first[l] && !direct_dense && !halves && !c->d_af_O) {
+    // rows drained by the caller: their place in the graduation buffer is a device-side count, so the transform of
+    // the finished rows writes a scratch matrix first.  Allocated here, before anything of the chunk is enqueued, so
+    // that a failure leaves the layer untouched.
+    ALLOC(c->d_af_O, (size_t)c->drain_rows * c->Hmax);
+  }
+  bool applied = false;
+  const int rc = push_enqueue(c, src_begin, src_end, features, src_runs, bound, direct_dense, halves, st, &applied);
+  if (rc && applied) c->half_applied = rc;   // every later call returns it: the layer has to be begun again
+  return rc;
 }
 
 static int gat_project_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, const float* features, taurus_runs* src_runs,

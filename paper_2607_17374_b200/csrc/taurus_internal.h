@@ -314,6 +314,7 @@ struct taurus_ctx {
   long long log_capacity = 0;
   // host bookkeeping
   int layer = -1;
+  int half_applied = 0;              // code of a push that failed with its chunk enqueued in part; cleared by taurus_layer_begin
   long long next_src = 0;
   long long chunk_seq = 0;
   const std::vector<long long>* rank_cum = nullptr;   // current layer: completions by block of 64 completion ranks, prefix sums
