@@ -537,7 +537,7 @@ int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long lo
   const int smem = STAGES * (bf16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32) + OUT_STAGING_BYTES + (int)sizeof(Barriers) + 1024;
   const int n_tiles = (n + BM - 1) / BM;
   const int n_units = n_tiles * ((w->Np + BN_MAX - 1) / BN_MAX);
-  const int sms = c->sm_count - (c->pipelined ? TAURUS_XFER_BLOCKS : 0);   // the SMs of the row transfers have no shared memory left
+  const int sms = c->sm_count - c->xfer_blocks;   // the SMs of the row transfers have no shared memory left
   const int grid = n_units < sms ? n_units : sms;
   if (!c->tc_smem_set) {   // once per context (the attribute belongs to the context's device)
     cudaError_t e = bf16 ? cudaFuncSetAttribute(project_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
@@ -595,7 +595,7 @@ int launch_gemm_plain_tc(taurus_ctx* c, void* image, int col0, int N, const floa
   const int smem = STAGES * (bf16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32) + OUT_STAGING_BYTES + (int)sizeof(Barriers) + 1024;
   const int n_tiles = (n + BM - 1) / BM;
   const int n_units = n_tiles * ((Np + BN_MAX - 1) / BN_MAX);
-  const int sms = c->sm_count - (c->pipelined ? TAURUS_XFER_BLOCKS : 0);   // the SMs of the row transfers have no shared memory left
+  const int sms = c->sm_count - c->xfer_blocks;   // the SMs of the row transfers have no shared memory left
   const int grid = n_units < sms ? n_units : sms;
   if (!c->tc_smem_set) {
     cudaError_t e = bf16 ? cudaFuncSetAttribute(project_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)

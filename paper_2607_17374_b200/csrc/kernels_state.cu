@@ -730,14 +730,22 @@ static __device__ __forceinline__ void xf_load(void* dst, const void* src, unsig
 // the host row.
 // Bound by the host link, and by what it does to the kernels beside it: rows waiting for the link fill the queues between
 // the SMs and L2, and everything else on the GPU waits in them.  So the rows in flight are kept to what the link needs,
-// on four SMs of their own (a block takes all the shared memory of its SM, so no block of another kernel shares it).
-// 600 k vertices, 4 096-source chunks, pool 0.27 V, 147 pushes of each of two layers (rows of 128 and 256 floats): one
-// block of eight warps per SM with 4 float4 per lane and direction in flight took 250 us a push and stretched the scatter
-// beside it from 30 to 260 us, 135 ms a pass; blocks of this kernel: 2 115 ms, 3 101, 4 98.7, 6 98.9, 8 99.1 with the one-
-// launch make-room step, 4 115.6, 16 124, 64 135 without it.  Fewer entries per block cost more than they relieve (32
-// instead of 112 rows of 1 KB in each of four blocks: 283 ms).
-// An extent whose last row has come back is listed for the free stack (taken back two chunks later by
-// extent_plan_kernel).
+// on a few SMs of their own (a block takes all the shared memory of its SM, so no block of another kernel shares it): eight;
+// sixteen and thirty-two where a push can touch more than 128 and 512 MB of rows (xfer_blocks_for).  ms a pass, and for the last
+// column ms a window of 32 pushes (190 k rows of 1 KB each way per push; GB/s in the busier direction):
+//   vertices / sources a push / row floats   600k/4k/128,256   900k/16k/256   1M/16k/64   1.5M/16k/256   1.5M/64k/256   111M/64k/256
+//   rows a push can touch                          67 MB         270 MB         64 MB        270 MB           1 GB            1 GB
+//   4 blocks                                       99.3           23.7          29.9         138.5            65.3         284  (22.8)
+//   8                                              98.0           23.6          26.9         126.1            58.3         195  (33.8)
+//   16                                             99.8           23.6          29.4         120.7            55.5         187  (35.1)
+//   32                                            102.5           24.7          30.5         122.1            56.2         185  (35.7)
+//   64                                                                                                                     184  (35.9)
+//   a block of eight warps on every SM, four
+//   float4 per lane and direction in flight       112.6           24.0          30.8         126.8            59.0         197  (36.3)
+// The last of these drives the link a little harder, but stretches the scatter beside it from 16 to 43 ms and the victim select
+// from 28 to 111 ms a window.  No better: one buffer per thread, 60 % of them for incoming rows (within 2 % at 8 to 32 blocks);
+// entries taken from a counter instead of dealt (191 ms at 16); fewer rows per block on more SMs (56 on 32: 189, 28 on 64: 190).
+// An extent whose last row has come back is listed for the free stack (taken back two chunks later by extent_plan).
 #define XF_SMEM (224 * 1024)
 #define XF_THREADS 256
 __global__ void __launch_bounds__(XF_THREADS) transfer_kernel(ChunkArgs a, int lanes) {   // lanes: entries in flight per block
@@ -782,11 +790,18 @@ __global__ void __launch_bounds__(XF_THREADS) transfer_kernel(ChunkArgs a, int l
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
+// SMs for the row transfers of a context: by the bytes of accumulator rows that one push can touch (table at transfer_kernel).
+int xfer_blocks_for(const taurus_ctx* c) {
+  const double bytes = (double)c->touched_capacity * c->Hmax * 4.0;
+  const int blocks = bytes > 512e6 ? 32 : bytes > 128e6 ? 16 : 8;
+  return blocks < c->sm_count / 2 ? blocks : c->sm_count / 2;
+}
+
 int launch_make_room(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, cudaEvent_t before_moves) {
   if (c->pool_slots < c->V - c->hub_count) {
     // one block per SM that the row transfers leave free; blocks that a small pool has no tile for only cost barrier time
     long long blocks = (a.pool_slots + MR_TILE - 1) / MR_TILE;
-    if (blocks > c->sm_count - TAURUS_XFER_BLOCKS) blocks = c->sm_count - TAURUS_XFER_BLOCKS;
+    if (blocks > c->sm_count - c->xfer_blocks) blocks = c->sm_count - c->xfer_blocks;
     if (blocks < 1) blocks = 1;
     ChunkArgs args = a;
     void* params[1] = {&args};
@@ -815,7 +830,7 @@ int launch_transfer(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) { taurus_note_cuda_error(e, "transfer_kernel"); return TAURUS_ERR_CUDA; }
     c->xfer_smem_set = true;
   }
-  transfer_kernel<<<TAURUS_XFER_BLOCKS, XF_THREADS, XF_SMEM, st>>>(a, lanes);
+  transfer_kernel<<<c->xfer_blocks, XF_THREADS, XF_SMEM, st>>>(a, lanes);
   c->launches += 1;
   return TAURUS_OK;
 }

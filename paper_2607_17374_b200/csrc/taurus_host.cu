@@ -334,6 +334,7 @@ static int init_impl(taurus_ctx* c, const taurus_graph* g, const taurus_model* m
     CU(cudaStreamCreateWithPriority(&c->xfer_stream, cudaStreamNonBlocking, prio_high));
     CU(cudaEventCreateWithFlags(&c->moves_ready, cudaEventDisableTiming));
     CU(cudaEventCreateWithFlags(&c->xfer_done, cudaEventDisableTiming));
+    c->xfer_blocks = xfer_blocks_for(c);
     c->pipelined = true;
     cudaError_t e = cudaHostAlloc((void**)&c->h_store, (size_t)c->n_ext * ext_rows * c->Hmax * sizeof(float), cudaHostAllocMapped);
     if (e != cudaSuccess) { cuda_ok(e, "cudaHostAlloc(evicted-row store)"); c->h_store = nullptr; return TAURUS_ERR_NOMEM; }

@@ -15,7 +15,6 @@
 #define TAURUS_MAX_TIMED_PUSHES 16384
 #define TAURUS_PUSH_EVENTS 12                   // CUDA events per timed push
 #define TAURUS_PHASES 9                         // durations reported per timed push
-#define TAURUS_XFER_BLOCKS 4                     // SMs that carry rows across the host link (one block each, all of its shared memory)
 #define TAURUS_HEAVY_DEGREE 256                  // resident pools: in-lists longer than this are summed in segments
 #define TAURUS_HEAVY_SEGMENT 128
 #define TAURUS_SEL_BITS 11                      // radix-select digit width
@@ -195,8 +194,8 @@ struct taurus_ctx {
   // weights per layer: Wcat is [Kp x Ncat] row-major fp32 (P columns then T columns), bias [Hp]
   float* d_Wcat[TAURUS_MAX_LAYERS] = {nullptr};
   float* d_bias[TAURUS_MAX_LAYERS] = {nullptr};
-  bool xfer_smem_set = false;                      // the same for the row transfer kernel
   bool tc_smem_set = false;                        // dynamic shared memory limit of the projection kernel raised
+  bool xfer_smem_set = false;                      // the same for the row transfer kernel
   void* tc_image[TAURUS_MAX_LAYERS] = {nullptr};   // tensor-core operand images of Wcat (owned by kernels_gemm_tc.cu)
   void* tc_image_af[TAURUS_MAX_LAYERS] = {nullptr};   // SAGE aggregate-first layers: image of [W_neigh ; W_self] stacked along K
   float* d_Waf[TAURUS_MAX_LAYERS] = {nullptr};       //   the same matrix row-major [2 Kp x Hp] for the FFMA kernel
@@ -273,6 +272,7 @@ struct taurus_ctx {
   int4* d_xfer_list = nullptr;
   float* d_stage_out = nullptr;
   cudaStream_t xfer_stream = nullptr;   // rows cross the host link here while the compute stream goes on
+  int xfer_blocks = 0;                  // SMs that carry them (one block each, all of its shared memory)
   cudaEvent_t moves_ready = nullptr, xfer_done = nullptr;
   bool pipelined = false;               // bounded pool with a host store: finalise of chunk k is deferred behind chunk k + 1's select
   bool pending = false;                 // a chunk's finalise (and what follows it) is still to be enqueued
@@ -339,6 +339,7 @@ static inline int taurus_proj_width(int mode, int Hp, int heads = 1) {
 // ---- kernels_state.cu
 void launch_layer_reset(taurus_ctx* c, int layer, cudaStream_t st);
 void launch_classify(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);
+int xfer_blocks_for(const taurus_ctx* c);                                    // after touched_capacity is known
 int launch_make_room(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, cudaEvent_t before_moves = nullptr);   // plan, select, placement, [event]
 void launch_alloc(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);       // slots handed out, victims' rows staged, new rows cleared
 int launch_transfer(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);    // staged rows to the host store, reloaded rows added into their slots
