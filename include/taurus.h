@@ -166,8 +166,10 @@ typedef struct {
                                   IN_BUFFER, NOT_STARTED, EVICTED (non-hub) and hub vertices    */
   int64_t free_slots;          /* free pool slots now                                            */
   int64_t chunks;              /* chunks pushed                                                  */
-  int64_t scatter_groups;      /* accumulator-row reductions the scatter issued for propagated messages: one per
-                                  message in CSR order, one per (chunk, destination) group in grouped order    */
+  int64_t scatter_groups;      /* groups of propagated messages: one per message where a push is not a cell of the chunk grid (or
+                                  without grouping), else one per (chunk, destination) pair.  Where accumulators are kept each
+                                  group is one reduction of an accumulator row (a group cut by the split of the work counts for
+                                  each piece); where sent rows are kept (see pool_slots) no reduction is issued for them */
 } taurus_stats;
 
 /* Columns of one per-chunk record returned by taurus_get_chunk_log. */
@@ -197,7 +199,9 @@ int taurus_layer_begin(taurus_ctx* ctx, int32_t layer, void* cuda_stream);
  * memory (pinned host memory makes the copy asynchronous).  Chunks must arrive in ascending, contiguous
  * order starting at 0, at most chunk_sources per push.  All work is enqueued on `cuda_stream`
  * (a cudaStream_t, NULL = default stream) and the call returns without waiting; `features` must stay
- * valid and unchanged until that work has run (synchronise the stream, or drain).  Returns
+ * valid and unchanged until that work has run (synchronise the stream, or drain).  A push that fails with part of its
+ * work enqueued (TAURUS_ERR_CUDA, TAURUS_ERR_INTERNAL) leaves a layer that cannot go on: every later call on it returns the
+ * code until taurus_layer_begin; after any other error the same push may be made again.  Returns
  * TAURUS_ERR_DRAIN_FULL, before changing any state, when the vertices this chunk completes might not
  * fit the graduation buffer: drain and push the same chunk again.
  * Where rows can be evicted (pool_slots < V - hub_count) the chunk's evicted and reloaded rows cross the host link on
@@ -375,7 +379,8 @@ int taurus_reorder(int64_t V, int64_t E, const int64_t* row_ptr, const int32_t* 
  * overlaps it, two binary searches (first id >= s, first id >= e) delimit a contiguous slice, the slice is
  * copied to the device in one transfer, and the slices are merged by vertex id.  The run store stands for the
  * paper's run files on SSD: pinned host memory (TAURUS_RUNS_HOST) or device memory (TAURUS_RUNS_DEVICE); the
- * ids of all runs are always kept in pinned host memory, where the searches run.
+ * ids of all runs are always kept in pinned host memory, where the searches run (with TAURUS_RUNS_DEVICE also in device
+ * memory, 4 B a row, where the merge reads them).
  *
  * Run k of a range holds that range's arrivals k * partition_rows .. (k + 1) * partition_rows - 1 (arrival
  * order = order of the rows within each append, appends in call order), so the set of runs is a function of
@@ -464,6 +469,9 @@ int64_t taurus_launch_count(const taurus_ctx* ctx);
  * rows staged, new rows cleared), 5 scatter, 6 completion list, 7 the chunk's own finalise, 8 the chunk's row
  * transfers over the host link (evicted rows out, reloaded rows in; on the library's transfer stream, beside
  * k = 5, 6 of this chunk and k = 0..2 of the next); *out_pushes = pushes written (at most capacity_pushes).
+ * Where the library keeps sent rows (see pool_slots) the accounting of a chunk runs on a stream of its own beside its copy-in and
+ * projection: k = 2 is what is left of it when those are through, k = 5 the sums of the finished vertices (with bias and
+ * activation, and as finished rows, in layers that project first), k = 7 the transform of aggregate-first layers; k = 3, 4, 6, 8 are 0.
  * An event between two kernels costs about 2 us of the stream (twelve per push: 4-5 % of a pass whose pushes take half a
  * millisecond); taurus_set_timing(ctx, 2) records only the two events around the scatter, and taurus_get_phase_ms then
  * fills k = 5 and leaves the other columns 0.  on = 0 ends the window; another value is TAURUS_ERR_INVALID_ARG.  The

@@ -396,8 +396,9 @@ scatter_grouped_kernel(ChunkArgs a, const int2* __restrict__ g_edge, const uint3
   };
 
   // Where row transfers of the previous chunk may be running beside this kernel (bounded pool), spans are handed out
-  // from a counter rather than by warp number: SMs that also host transfer warps get through fewer of them (measured on
-  // "large": scatter 105 -> 34 ms per 32-chunk window).  A span is requested only when the warp is ready for it: a chunk
+  // from a counter rather than by warp number: warps near the host link's requests get through fewer of them (measured on
+  // "large" with transfer warps on every SM: scatter 105 -> 34 ms per 32-chunk window; 16 ms with the transfers on SMs of
+  // their own).  A span is requested only when the warp is ready for it: a chunk
   // has about two spans per warp there, and a warp that asked ahead would sit on a span while it is slow.  Elsewhere the
   // spans are dealt by warp number: same-address atomics cost about 3 ns each, 75 us per launch at the 25 k spans of a
   // "mid" chunk.
