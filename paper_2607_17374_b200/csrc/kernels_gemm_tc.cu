@@ -518,7 +518,7 @@ bool project_tc_usable(const taurus_ctx* c, int layer, const float* X, int ldx) 
   return true;
 }
 
-int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, cudaStream_t st) {
+int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, int ldo, cudaStream_t st) {
   const bool bf16 = c->gemm_mode == TAURUS_GEMM_BF16;
   WImage* w = static_cast<WImage*>(c->tc_image[layer]);
   const int K = c->dims[layer], Hp = taurus_round_up(c->dims[layer + 1], 4);
@@ -526,7 +526,7 @@ int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long lo
   CUtensorMap map_x;
   if (!make_map(&map_x, X, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, K, ldx, BM, bf16 ? 32 : KS32)) return TAURUS_ERR_CUDA;
   CUtensorMap map_out;
-  if (!make_map(&map_out, out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, N, N, 32, 32)) return TAURUS_ERR_CUDA;
+  if (!make_map(&map_out, out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, N, ldo, 32, 32)) return TAURUS_ERR_CUDA;
   GemmArgs g;
   g.PT = out; g.n = n; g.N = N; g.Np = w->Np; g.k_stages = w->Kp / (bf16 ? 64 : KS32);
   g.b_box_bytes = (w->Np < BN_MAX ? w->Np : BN_MAX) * (bf16 ? 128 : ROW32);

@@ -32,6 +32,30 @@ __device__ __forceinline__ float r_lrelu(float x, float slope) { return x > 0.f 
 __device__ __forceinline__ void red_v4(float* addr, const float4& v) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
+// Four floats as two packed pairs; each half of a packed operation is rounded like the scalar one.
+struct Pairs { unsigned long long a, b; };
+__device__ __forceinline__ Pairs pairs_of(const float4& v) {
+  Pairs p;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(p.a) : "f"(v.x), "f"(v.y));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(p.b) : "f"(v.z), "f"(v.w));
+  return p;
+}
+__device__ __forceinline__ float4 floats_of(const Pairs& p) {
+  float4 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(p.a));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.z), "=f"(v.w) : "l"(p.b));
+  return v;
+}
+__device__ __forceinline__ void add4(Pairs& s, const Pairs& r) {
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(s.a) : "l"(r.a));
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(s.b) : "l"(r.b));
+}
+__device__ __forceinline__ void mul4(Pairs& s, float w) {
+  unsigned long long ww;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(ww) : "f"(w));
+  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(s.a) : "l"(ww));
+  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(s.b) : "l"(ww));
+}
 __device__ __forceinline__ void add4(float4& s, const float4& r) { s.x += r.x; s.y += r.y; s.z += r.z; s.w += r.w; }
 __device__ __forceinline__ void fma4(float4& s, float w, const float4& r) {
   s.x = fmaf(w, r.x, s.x); s.y = fmaf(w, r.y, s.y); s.z = fmaf(w, r.z, s.z); s.w = fmaf(w, r.w, s.w);
@@ -292,8 +316,16 @@ struct Item {                // fetched by one lane each: one chain of dependent
 };
 struct HeadTerm { float t, top, scale, self, bw; };   // GAT: destination term and maximum of the scores; the same three per head
 
+// A value that every lane of the warp holds alike, told to the compiler: the reduction's result is a uniform register, and
+// branches on it need no reconvergence code (which was more than half of this kernel's instructions).
+__device__ __forceinline__ int uniform(int x) { return __reduce_max_sync(FULL, x); }
+__device__ __forceinline__ unsigned uniform(unsigned x) { return __reduce_or_sync(FULL, x); }
+
 __device__ __forceinline__ void copy16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy16_if(unsigned dst, const void* src, int yes) {   // dst: address in shared memory
+  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %2, 0;\n@p cp.async.cg.shared.global [%0], [%1], 16;\n}" ::"r"(dst), "l"(src), "r"(yes) : "memory");
 }
 __device__ __forceinline__ void copy4(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
@@ -306,6 +338,10 @@ __device__ __forceinline__ void copy4(void* dst, const void* src) {
 // With the same loads held in registers (4 rows per warp, 32 warps per SM) DRAM ran at 38 %, L2 at 27 %, the schedulers
 // issued in 20 % of the cycles.  The U rows of a step are added up before they join the running sum and long in-lists
 // are cut: fewer additions in sequence than the push form has.
+// Issue slots are what is left beside the row reads, so control that is the same for the whole warp is told to the compiler as
+// such (`uniform`), additions are packed in pairs, and lanes behind the end of a row are predicated off (copying its last 16
+// bytes again instead halved the rate of 48-float rows that sit in L2).  Instructions per message of 256 / 100 floats on 800 k
+// vertices, 40 M edges: 53 / 33 before, 43 / 24 now; all gathers of 2.45 M vertices, 124 M edges, three layers: 31.8 -> 27.1 ms.
 // GAT: most heads the ring is sized for (0: no attention).  The scores of a block of 32 sources travel with the block's
 // first step; the lanes turn them into coefficients, one source each, when the block is reached.
 template <int VPL, int U, int D, int GAT>
@@ -317,7 +353,7 @@ struct Ring {
 };
 
 template <int LPE, int VPL, int U, int D, int GAT>
-__global__ void __launch_bounds__(32 * G_WARPS) gather_kernel(const __grid_constant__ GatherArgs g) {
+__global__ void __launch_bounds__(32 * G_WARPS, VPL == 1 ? 6 : VPL == 2 ? 5 : VPL == 4 ? 4 : 2) gather_kernel(const __grid_constant__ GatherArgs g) {
   extern __shared__ __align__(16) unsigned char g_smem[];
   ChunkCtl* const pc = g.pc;
   if (g.ctl->error) return;
@@ -327,7 +363,7 @@ __global__ void __launch_bounds__(32 * G_WARPS) gather_kernel(const __grid_const
   const int lane = rl(), sub = lane / LPE, c4 = lane % LPE, wid = threadIdx.x >> 5;
   R& ring = reinterpret_cast<R*>(g_smem)[wid];
   const int warps = (int)((gridDim.x * blockDim.x) >> 5);
-  const int n = pc->done_count, nh = g.heavy ? pc->heavy_count : 0;
+  const int n = uniform(pc->done_count), nh = g.heavy ? uniform(pc->heavy_count) : 0;
   const int total = n + nh;
   bool on[VPL];
   int hk[VPL];
@@ -337,19 +373,27 @@ __global__ void __launch_bounds__(32 * G_WARPS) gather_kernel(const __grid_const
     hk[k] = 0;
     if (GAT && g.heads > 1) { hk[k] = (c4 + k * LPE) / g.head_vec; if (hk[k] >= g.heads) hk[k] = g.heads - 1; }
   }
-  // lanes behind the end of a row carry its last float4 along (same sectors, never stored): no predicates in the stream
-  int col[VPL];
-#pragma unroll
-  for (int k = 0; k < VPL; ++k) col[k] = (on[k] ? c4 + k * LPE : g.vec - 1) * 16;
-  const char* const rows = reinterpret_cast<const char*>(g.rows);
+  // lanes behind the end of a row copy nothing and add up what the ring happens to hold (never stored)
+  const char* const rows = reinterpret_cast<const char*>(g.rows) + c4 * 16;
+  constexpr unsigned SLOT = U * VPL * 512;
+  const unsigned slots = (unsigned)__cvta_generic_to_shared(&ring.row[0][0][0][lane]);
   const unsigned pitch = (unsigned)g.pitch * 16u;
   const bool sage = g.mode == TAURUS_SAGE_MEAN;
   const int own_off = sage && !g.A ? g.vec * 16 : 0;   // SAGE, projected rows: the self message T_v sits behind P_v
 
-  int per = total / (warps * 2);
-  per = per < 1 ? 1 : per > BATCH ? BATCH : per;
-  for (int i0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per; i0 < total; i0 += warps * per) {
-    const int cnt = total - i0 < per ? total - i0 : per;
+  // Batches: the first of a warp is its own number, the others come from a counter, asked for while the batch before is summed
+  // (dealt out in turn, the slowest warp of a launch of 10 ms finished 13 % after the average one).  Few items: up to four at
+  // once, since a batch pays one chain of dependent reads whatever its size (12 548 items of 32 floats, 3 552 warps: one at
+  // a time 18.9 us, four 13.8); more: two batches a warp or more, for the balance (338 884: eight at most 247 us, dealt out 277).
+  const int once = (total + warps - 1) / warps < 4 ? (total + warps - 1) / warps : 4;
+  int per = total / (warps * 2) < BATCH ? total / (warps * 2) : BATCH;
+  per = per < once ? once : per;
+  per = per < 1 ? 1 : per;
+  const int n_batches = (total + per - 1) / per;
+  int ticket = 0;
+  for (int batch = uniform((int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5)); batch < n_batches; batch = uniform(lane == 0 ? ticket : 0)) {
+    if (lane == 0) ticket = (int)atomicAdd(&pc->span_next, 1u) + warps;
+    const int i0 = batch * per, cnt = total - i0 < per ? total - i0 : per;
     __syncwarp();
     if (lane < cnt) {
       Item x;
@@ -393,14 +437,17 @@ __global__ void __launch_bounds__(32 * G_WARPS) gather_kernel(const __grid_const
     }
 
     // sources, 32 at a time: `u` the block the producer is in, `un` the one after it (item fj, entries from fb on)
-    int u = 0, un = 0, fj = 0, fb = -32;
+    int u = 0, un = 0, fj = 0, fb = -32, flen = uniform(ring.item[0].len);
     auto fetch = [&]() {
       fb += 32;
-      while (fj < cnt && fb >= ring.item[fj].len) { ++fj; fb = 0; }
-      if (fj < cnt) un = fb + lane < ring.item[fj].len ? g.src[ring.item[fj].begin + fb + lane] : 0;
+      while (fj < cnt && fb >= flen) {
+        if (++fj < cnt) flen = uniform(ring.item[fj].len);
+        fb = 0;
+      }
+      if (fj < cnt) un = fb + lane < flen ? g.src[ring.item[fj].begin + fb + lane] : 0;
     };
     // producer: next step to request (item pj, entries from pp on; pp at the end: the own row)
-    int pj = -1, pp = 0, plen = 0, slot = 0;
+    int pj = -1, pp = 0, plen = 0;
     int pblk = 0, cblk = 0;     // GAT: block slots of the producer and the consumer
     auto next_block = [&]() {
       u = un;
@@ -416,41 +463,41 @@ __global__ void __launch_bounds__(32 * G_WARPS) gather_kernel(const __grid_const
       fetch();
     };
     auto enter = [&]() {
-      do ++pj; while (pj < cnt && ring.item[pj].len < 0);
+      do {
+        ++pj;
+        if (pj < cnt) plen = uniform(ring.item[pj].len);
+      } while (pj < cnt && plen < 0);
       if (pj < cnt) {
         pp = 0;
-        plen = ring.item[pj].len;
         if (plen > 0) next_block();
       }
     };
-    auto produce = [&](int to) {
+    auto produce = [&](unsigned to) {
       if (pj < cnt) {
         if (pp < plen) {
-          const int at = (pp & 31) + sub;
-          if (pp + STEP <= plen) {
+          const int at = (pp & 31) + sub, left = plen - pp;
+          if (left >= STEP) {
 #pragma unroll
             for (int q = 0; q < U; ++q) {
               const char* src = rows + (unsigned long long)(unsigned)__shfl_sync(FULL, u, at + q * EPS) * pitch;
 #pragma unroll
-              for (int k = 0; k < VPL; ++k) copy16(&ring.row[to][q][k][lane], src + col[k]);
+              for (int k = 0; k < VPL; ++k) copy16_if(to + (q * VPL + k) * 512, src + k * LPE * 16, on[k]);
             }
           } else {
 #pragma unroll
             for (int q = 0; q < U; ++q) {
               const char* src = rows + (unsigned long long)(unsigned)__shfl_sync(FULL, u, at + q * EPS) * pitch;
-              if (pp + q * EPS + sub < plen)
 #pragma unroll
-                for (int k = 0; k < VPL; ++k) copy16(&ring.row[to][q][k][lane], src + col[k]);
+              for (int k = 0; k < VPL; ++k) copy16_if(to + (q * VPL + k) * 512, src + k * LPE * 16, on[k] && q * EPS + sub < left);
             }
           }
           pp += STEP;
           if (pp < plen && (pp & 31) == 0) next_block();
         } else {
-          if (sub == 0 && ring.item[pj].row < 0) {
-            const char* src = rows + (size_t)ring.item[pj].v * pitch + own_off;
+          const bool whole = sub == 0 && ring.item[pj].row < 0;
+          const char* src = rows + (size_t)ring.item[pj].v * pitch + own_off;
 #pragma unroll
-            for (int k = 0; k < VPL; ++k) copy16(&ring.row[to][0][k][lane], src + col[k]);
-          }
+          for (int k = 0; k < VPL; ++k) copy16_if(to + k * 512, src + k * LPE * 16, on[k] && whole);
           enter();
         }
       }
@@ -459,15 +506,21 @@ __global__ void __launch_bounds__(32 * G_WARPS) gather_kernel(const __grid_const
     fetch();
     enter();
 #pragma unroll 1
-    for (int d = 0; d < D; ++d) produce(d);
+    for (int d = 0; d < D; ++d) produce(slots + d * SLOT);
+    unsigned now = slots, before = slots + D * SLOT;   // slots of this step and of the one before it
+    auto advance = [&]() {
+      produce(before);   // the step before this one: its rows have been added
+      before = now;
+      now = now == slots + D * SLOT ? slots : now + SLOT;
+    };
 
 #pragma unroll 1
     for (int j = 0; j < cnt; ++j) {
-      const int len = ring.item[j].len;
+      const int len = uniform(ring.item[j].len);
       if (len < 0) continue;
-      float4 sum[VPL];
+      Pairs acc[VPL];
 #pragma unroll
-      for (int k = 0; k < VPL; ++k) sum[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int k = 0; k < VPL; ++k) acc[k].a = acc[k].b = 0ull;
 #pragma unroll 1
       for (int p = 0; p < len; p += STEP) {
         asm volatile("cp.async.wait_group %0;" ::"n"(D - 1) : "memory");
@@ -482,50 +535,48 @@ __global__ void __launch_bounds__(32 * G_WARPS) gather_kernel(const __grid_const
         auto add_step = [&](auto full) {
 #pragma unroll
           for (int k = 0; k < VPL; ++k) {
-            float4 r[U];
+            Pairs r[U];
 #pragma unroll
             for (int q = 0; q < U; ++q) {
+              r[q].a = r[q].b = 0ull;
               if (full || p + q * EPS + sub < len) {
-                r[q] = ring.row[slot][q][k][lane];
-                if (GAT) {
-                  const float w = ring.att[GAT ? cblk : 0][((p & 31) + q * EPS + sub) * g.heads + hk[k]];
-                  r[q].x *= w; r[q].y *= w; r[q].z *= w; r[q].w *= w;
-                }
-              } else {
-                r[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(r[q].a), "=l"(r[q].b) : "r"(now + (unsigned)((q * VPL + k) * 512)) : "memory");
+                if (GAT) mul4(r[q], ring.att[GAT ? cblk : 0][((p & 31) + q * EPS + sub) * g.heads + hk[k]]);
               }
             }
 #pragma unroll
             for (int o = 1; o < U; o <<= 1)
 #pragma unroll
               for (int q = 0; q + o < U; q += 2 * o) add4(r[q], r[q + o]);
-            add4(sum[k], r[0]);
+            add4(acc[k], r[0]);
           }
         };
         if (p + STEP <= len) add_step(std::true_type()); else add_step(std::false_type());
-        produce(slot == 0 ? D : slot - 1);   // the slot of the step before this one: its rows have been added
-        slot = slot == D ? 0 : slot + 1;
+        advance();
       }
       // the sub-groups' sums
+      float4 sum[VPL];
 #pragma unroll
-      for (int o = LPE; o < 32; o <<= 1)
+      for (int k = 0; k < VPL; ++k) {
 #pragma unroll
-        for (int k = 0; k < VPL; ++k) {
-          sum[k].x += __shfl_xor_sync(FULL, sum[k].x, o); sum[k].y += __shfl_xor_sync(FULL, sum[k].y, o);
-          sum[k].z += __shfl_xor_sync(FULL, sum[k].z, o); sum[k].w += __shfl_xor_sync(FULL, sum[k].w, o);
+        for (int o = LPE; o < 32; o <<= 1) {
+          Pairs y;
+          y.a = __shfl_xor_sync(FULL, acc[k].a, o); y.b = __shfl_xor_sync(FULL, acc[k].b, o);
+          add4(acc[k], y);
         }
+        sum[k] = floats_of(acc[k]);
+      }
       // the own row
       asm volatile("cp.async.wait_group %0;" ::"n"(D - 1) : "memory");
       float4 x[VPL];
 #pragma unroll
       for (int k = 0; k < VPL; ++k) {
         x[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (sub == 0 && on[k]) x[k] = ring.row[slot][0][k][lane];
+        if (sub == 0 && on[k]) asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[k].x), "=f"(x[k].y), "=f"(x[k].z), "=f"(x[k].w) : "r"(now + k * 512u) : "memory");
       }
-      produce(slot == 0 ? D : slot - 1);
-      slot = slot == D ? 0 : slot + 1;
+      advance();
 
-      const int v = ring.item[j].v, i = ring.item[j].i, row = ring.item[j].row;
+      const int v = ring.item[j].v, i = ring.item[j].i, row = uniform(ring.item[j].row);
       if (row >= 0) {
         // partial sums meet in a row of their own; the segment that arrives last finishes the vertex
         float4* const part = g.heavy_rows + (size_t)row * g.vec;
@@ -546,7 +597,7 @@ __global__ void __launch_bounds__(32 * G_WARPS) gather_kernel(const __grid_const
             if (on[k]) {
               sum[k] = __ldcg(part + c4 + k * LPE);
               part[c4 + k * LPE] = make_float4(0.f, 0.f, 0.f, 0.f);
-              x[k] = *reinterpret_cast<const float4*>(rows + (size_t)v * pitch + own_off + col[k]);
+              x[k] = *reinterpret_cast<const float4*>(rows + (size_t)v * pitch + own_off + k * LPE * 16);
             }
       }
       // finished row
@@ -624,7 +675,8 @@ int launch_g2(taurus_ctx* c, const GatherArgs& g, long long bound, int width_cla
 // ------------------------------------------------------------------------------------------------ rows into the store
 // out[r] = scale * X[r], zero-padded from K to Kp columns; scale = 1, or 1 / sqrt(out-degree + 1) with GCN.
 __global__ void store_rows_kernel(const float* __restrict__ X, long long ldx, int n, int K, int Kp, long long src_begin, int gcn,
-                                  const long long* __restrict__ row_ptr, float* __restrict__ out) {
+                                  const long long* __restrict__ row_ptr, float* __restrict__ out,
+                                  int ldo) {
   const long long stride = (long long)gridDim.x * blockDim.x;
   const int vec = Kp >> 2;
   const bool wide = (ldx & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
@@ -640,7 +692,7 @@ __global__ void store_rows_kernel(const float* __restrict__ X, long long ldx, in
       const float s = (float)(1.0 / sqrt((double)(row_ptr[u + 1] - row_ptr[u]) + 1.0));
       x.x *= s; x.y *= s; x.z *= s; x.w *= s;
     }
-    reinterpret_cast<float4*>(out)[i] = x;
+    *reinterpret_cast<float4*>(out + r * ldo + c) = x;
   }
 }
 
@@ -843,11 +895,10 @@ bool take_mem(T** p, size_t n) { return cudaMalloc((void**)p, (n > 0 ? n : 1) * 
 
 }  // namespace
 
-// Columns of a row of the store for layer l.
+// Floats between rows of the store for layer l: whole 32-byte sectors.
 int resident_row(const taurus_ctx* c, int l) {
   const int Kp = taurus_round_up(c->dims[l], 4), Hp = taurus_round_up(c->dims[l + 1], 4);
-  if (c->agg_first[l]) return Kp;
-  return c->mode == TAURUS_SAGE_MEAN ? 2 * Hp : Hp;
+  return taurus_round_up(c->agg_first[l] ? Kp : c->mode == TAURUS_SAGE_MEAN ? 2 * Hp : Hp, 8);
 }
 
 // In-lists (csc_ptr, csc_src; with csc_eid where a layer is sampled: built already), items of the chunk grid, heavy vertices.
@@ -930,9 +981,9 @@ void launch_resident_reset(taurus_ctx* c, int layer, cudaStream_t st) {
   c->launches += 1;
 }
 
-void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int K, int Kp, long long src_begin, bool gcn, float* out, cudaStream_t st) {
+void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int K, int Kp, long long src_begin, bool gcn, float* out, int ldo, cudaStream_t st) {
   const int grid = (int)std::min<long long>(((long long)n * (Kp >> 2) + 255) / 256, (long long)c->sm_count * 8);
-  store_rows_kernel<<<grid, 256, 0, st>>>(X, ldx, n, K, Kp, src_begin, gcn ? 1 : 0, c->d_row_ptr, out);
+  store_rows_kernel<<<grid, 256, 0, st>>>(X, ldx, n, K, Kp, src_begin, gcn ? 1 : 0, c->d_row_ptr, out, ldo);
   c->launches += 1;
 }
 
@@ -971,19 +1022,18 @@ int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitc
   g.d_out = a.d_out; g.act = a.act; g.mode = a.mode; g.heads = a.heads; g.head_vec = a.head_vec;
   g.gin_self = a.gin_self; g.leaky = a.leaky;
   c->launches += 1;
-  // Rows split over as many lanes as they have float4, steps of about 2 KB per warp.  Measured on the passes of 2.45 M
-  // vertices / 124 M edges (48, 100, 256 floats) and 500 k / 12.5 M (64): 48 floats 16 x 1 lanes, 4 rows, 3 steps 4.1 ms,
-  // 4 x 3 lanes 4.3 to 5.1; 64: 2 rows, 4 steps 0.53, others 0.55 to 0.78; 100: 4 rows, 2 steps 8.5, others 8.4 to 8.8
-  // (64 k completed rows of 128 floats 0.68 against 0.75 to 0.94); 256: 2 rows, 3 steps 16.4, others 16.4 to 16.9.
+  // Rows split over as many lanes as they have float4, steps of about 2 KB per warp.  Measured (ms of all launches of a pass):
+  // 48 floats, 2.45 M vertices, 124 M edges: 16 lanes x 1 float4, 4 rows a step, 3 steps 3.9; 8 x 2 4.6 to 5.2.  64 floats, 500 k
+  // vertices, 12.5 M edges: 4 rows, 3 steps 0.47; 2 rows, 4 steps 0.50; 8 x 2 0.54.  100 floats (first graph): 32 x 1, 4 rows, 3 steps
+  // 7.5; 16 x 2 7.7.  256 floats: 2 rows, 4 steps 15.8; 4 rows, 3 steps 15.8, slower where in-lists are short.
   const int Hp = a.Hp;
   if (Hp <= 16) return launch_g2<4, 1, 2, 4>(c, g, bound, 0, st);
   if (Hp <= 32) return launch_g2<8, 1, 2, 4>(c, g, bound, 1, st);
-  if (Hp <= 48) return launch_g2<16, 1, 4, 3>(c, g, bound, 2, st);
-  if (Hp <= 64) return launch_g2<16, 1, 2, 4>(c, g, bound, 3, st);
-  if (Hp <= 128) return launch_g2<32, 1, 4, 3>(c, g, bound, 4, st);
-  if (Hp <= 256) return launch_g2<32, 2, 2, 4>(c, g, bound, 5, st);
-  if (Hp <= 512) return launch_g2<32, 4, 1, 4>(c, g, bound, 6, st);
-  return launch_g2<32, 8, 1, 3>(c, g, bound, 7, st);
+  if (Hp <= 64) return launch_g2<16, 1, 4, 3>(c, g, bound, 2, st);
+  if (Hp <= 128) return launch_g2<32, 1, 4, 3>(c, g, bound, 3, st);
+  if (Hp <= 256) return launch_g2<32, 2, 2, 4>(c, g, bound, 4, st);
+  if (Hp <= 512) return launch_g2<32, 4, 1, 4>(c, g, bound, 5, st);
+  return launch_g2<32, 8, 1, 3>(c, g, bound, 6, st);
 }
 
 void launch_resident_attention(taurus_ctx* c, cudaStream_t st) {

@@ -684,6 +684,7 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
   }
   const int K = gat ? c->dims[l + 1] : c->dims[l];
   const int n = (int)(src_end - src_begin);
+  const int proj_w = taurus_proj_width(c->mode, taurus_round_up(c->dims[l + 1], 4), c->heads);
   cudaEvent_t* pev = nullptr;
   if (c->timing && c->timed_pushes < TAURUS_MAX_TIMED_PUSHES) {
     const size_t need = (size_t)(c->timed_pushes + 1) * TAURUS_PUSH_EVENTS;
@@ -719,15 +720,15 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
     const int w = resident_row(c, l);
     float* rows = c->d_store + (size_t)src_begin * w;
     if (af) {
-      a.Hout = a.Hp; a.Hp = w; a.self_bias = 0;
-      launch_store_rows(c, X, ldx, n, c->dims[l], w, src_begin, c->mode == TAURUS_GCN_SYM, rows, st);   // (GAT: pass 1 handed the input rows back, pitch dims[l + 1])
+      a.Hout = a.Hp; a.Hp = taurus_round_up(c->dims[l], 4); a.self_bias = 0;
+      launch_store_rows(c, X, ldx, n, c->dims[l], a.Hp, src_begin, c->mode == TAURUS_GCN_SYM, rows, w, st);   // (GAT: pass 1 handed the input rows back, pitch dims[l + 1])
     } else if (gat) {
-      launch_store_rows(c, X, ldx, n, K, w, src_begin, false, rows, st);
+      launch_store_rows(c, X, ldx, n, K, a.Hp, src_begin, false, rows, w, st);
     } else if (project_tc_usable(c, l, X, ldx)) {
-      int rc = launch_project_tc(c, l, X, ldx, src_begin, n, rows, st);
+      int rc = launch_project_tc(c, l, X, ldx, src_begin, n, rows, w, st);
       if (rc) return rc;
     } else {
-      launch_project_simt(c, l, X, ldx, src_begin, n, rows, st);
+      launch_project_simt(c, l, X, ldx, src_begin, n, rows, w, st);
     }
     if (xbuf >= 0) { CU(cudaEventRecord(c->x_free[xbuf], st)); c->x_used[xbuf] = true; }
     if (timing) cudaEventRecord(pev[2], st);
@@ -781,10 +782,10 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
     if (K == a.Hp && (reinterpret_cast<uintptr_t>(X) & 15) == 0) { a.PT = X; x_in_use = true; }
     else launch_gat_repack(c, X, n, K, a.Hp, st);
   } else if (project_tc_usable(c, l, X, ldx)) {
-    int rc = launch_project_tc(c, l, X, ldx, src_begin, n, c->d_PT, st);
+    int rc = launch_project_tc(c, l, X, ldx, src_begin, n, c->d_PT, proj_w, st);
     if (rc) return rc;
   } else {
-    launch_project_simt(c, l, X, ldx, src_begin, n, c->d_PT, st);
+    launch_project_simt(c, l, X, ldx, src_begin, n, c->d_PT, proj_w, st);
   }
   if (xbuf >= 0 && !x_in_use) { CU(cudaEventRecord(c->x_free[xbuf], st)); c->x_used[xbuf] = true; }
   if (timing) cudaEventRecord(pev[2], st);
@@ -879,6 +880,7 @@ static int gat_project_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, c
     c->last_stream = st;
   }
   const int n = (int)(src_end - src_begin);
+  const int proj_w = taurus_proj_width(c->mode, Hp, c->heads);
   const float* X = nullptr;
   int xbuf = -1;
   { int rc = stage_chunk(c, features, src_runs, src_begin, src_end, K, st, &X, &xbuf); if (rc) return rc; }
@@ -890,10 +892,10 @@ static int gat_project_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, c
     return TAURUS_OK;
   }
   if (project_tc_usable(c, l, X, K)) {
-    int rc = launch_project_tc(c, l, X, K, src_begin, n, c->d_PT, st);
+    int rc = launch_project_tc(c, l, X, K, src_begin, n, c->d_PT, proj_w, st);
     if (rc) return rc;
   } else {
-    launch_project_simt(c, l, X, K, src_begin, n, c->d_PT, st);
+    launch_project_simt(c, l, X, K, src_begin, n, c->d_PT, proj_w, st);
   }
   if (xbuf >= 0) { CU(cudaEventRecord(c->x_free[xbuf], st)); c->x_used[xbuf] = true; }
   launch_gat_split(c, n, Hp, d_out, src_begin, hprime_out, ld, st);

@@ -243,7 +243,7 @@ struct taurus_ctx {
   std::vector<long long> item_ptr;
   cudaStream_t account_stream = nullptr;   // the accounting of a push runs here, beside its copy and projection
   cudaEvent_t account_go = nullptr, account_done = nullptr;
-  int gather_per_sm[8][3] = {{0}};         // gather: blocks per SM by row width class and attention variant, 0 = not launched yet
+  int gather_per_sm[7][3] = {{0}};         // gather: blocks per SM by row width class and attention variant, 0 = not launched yet
   int32_t* d_heavy_list = nullptr; // vertices with long in-lists
   long long n_heavy = 0, n_heavy_segments = 0;
   int4* d_heavy = nullptr;         // segments of one push
@@ -378,7 +378,7 @@ void launch_gat_repack(taurus_ctx* c, const float* X, int n, int d_out, int Hp, 
 // ---- kernels_scatter.cu
 void launch_scatter(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);
 // ---- kernels_gemm_simt.cu
-void launch_project_simt(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, cudaStream_t st);
+void launch_project_simt(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, int ldo, cudaStream_t st);
 void launch_gemm_plain_simt(taurus_ctx* c, const float* W, int ldw, int N, const float* X, int ldx, int K, int n, float* out, long long ld_out,
                             cudaStream_t st);   // out = X . W[:, 0..N), W row-major with pitch ldw
 // ---- kernels_gemm_tc.cu
@@ -401,12 +401,12 @@ int launch_gemm_plain_tc(taurus_ctx* c, void* image, int col0, int N, const floa
 int prepare_tc_weights(taurus_ctx* c, void** slot, const std::vector<float>& cat, int K, int N);   // image of cat [K x N] into *slot
 void free_tc_weights(taurus_ctx* c);
 bool project_tc_usable(const taurus_ctx* c, int layer, const float* X, int ldx);
-int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, cudaStream_t st);   // out [n x projection width], 16-byte aligned
+int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, int ldo, cudaStream_t st);   // out [n x projection width], pitch ldo (a multiple of 4), 16-byte aligned
 // ---- kernels_resident.cu
 int resident_row(const taurus_ctx* c, int layer);                            // floats per row of the store
 int build_resident(taurus_ctx* c);
 void launch_resident_reset(taurus_ctx* c, int layer, cudaStream_t st);
-void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int K, int Kp, long long src_begin, bool gcn, float* out, cudaStream_t st);
+void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int K, int Kp, long long src_begin, bool gcn, float* out, int ldo, cudaStream_t st);
 void launch_account(taurus_ctx* c, const ChunkArgs& a, long long cell, cudaStream_t st);
 int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitch, float* A, long long bound, cudaStream_t st);
 void launch_resident_attention(taurus_ctx* c, cudaStream_t st);
