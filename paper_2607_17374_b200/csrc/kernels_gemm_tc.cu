@@ -2,15 +2,15 @@
 // epilogue, for one pushed chunk (Sect. 3.6 puts the layer transform on the GPU; here it runs before the
 // aggregation, which is legal by linearity, SAGEConv paragraph of Sect. 3.9).
 //
-// Persistent kernel: one CTA per SM walks (128-row tile of X, block of up to 256 output columns) units.  Roles (10 warps):
+// Persistent kernel: one CTA per SM walks (128-row tile of X, block of up to 256 output columns) units.  Roles (14 warps):
 //   warp 0        TMA producer: cp.async.bulk.tensor loads of the raw fp32 X tile and the W operand tiles
 //   warp 1        MMA issuer: tcgen05.mma, accumulators in TMEM (two buffers of up to 256 columns)
 //   warps 2..5    converter: turns the raw fp32 X tile in shared memory into tensor-core operands
 //                   fp32 mode : hi = x with the low 13 mantissa bits cleared (in place), lo = x - hi (exact);
 //                               acc += lo.Whi + hi.Wlo + hi.Whi   (three kind::tf32 MMAs, small terms first)
 //                   bf16 mode : bf16(x), one kind::f16 MMA
-//   warps 6..9    epilogue: tcgen05.ld of the accumulator, per-row scaling / bias, 32 x 32 tiles staged in shared
-//                 memory and written with TMA stores (full 128-byte lines)
+//   warps 6..13   epilogue, two per quadrant of TMEM lanes: tcgen05.ld of the accumulator, per-row scaling / bias, 32 x 32
+//                 tiles transposed through shared memory and written four rows at a time (full 128-byte lines)
 // The output columns of a tile are processed in blocks of up to 256; (tile, block) units alternate between two
 // TMEM accumulator buffers, so the epilogue of one unit overlaps the main loop of the next, also across tiles.
 //
@@ -20,6 +20,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "taurus_internal.h"
@@ -32,26 +33,28 @@ constexpr int STAGES = 2;            // stages of 128-byte operand rows with ful
 constexpr int MAX_STAGES = 8;        // shorter operand rows and narrower weight tiles leave room for more stages in the same memory
 constexpr int TILE_A_BYTES = BM * 128;           // 128 rows x 128 B
 constexpr int TILE_B_BYTES = BN_MAX * 128;       // 256 rows x 128 B
-// fp32 mode: K columns per stage, 32 (128-byte operand rows, 128-byte swizzle) or 16 (64-byte rows and swizzle: stages half
-// as large, twice as many in flight).  Both are exact and measure the same (projection of the "mid" workload 6.1 against
-// 6.3 ms per step): the three TF32 MMAs of a K step read their operands from shared memory without reuse between them
-// (12 KB per 128 x 256 x 8 MMA, one MMA per 134 cycles at the pipe's rate = 92 B per cycle), and with the TMA fill and the
-// operand split on top the SM's 128 B per cycle of shared memory are the limit, not the depth of the pipeline.
-constexpr int KS32 = 32;
-constexpr int ROW32 = KS32 * 4;                  // operand row bytes in fp32 mode
-constexpr int A32_BYTES = BM * ROW32;            // one fp32-mode feature tile (raw / hi, or lo)
+// fp32 mode: KS, the K columns per stage, is 32 (128-byte operand rows, 128-byte swizzle) or 16 (64-byte rows and swizzle: stages
+// half as large, twice as many in flight).  Both are exact.  The three TF32 MMAs of a K step read their operands from shared
+// memory without reuse between them (12 KB per 128 x 256 x 8 MMA, one MMA per 134 cycles at the pipe's rate = 92 B per cycle), and
+// the TMA fill and the operand split come on top of the SM's 128 B per cycle: 2 125 cycles of shared memory to 1 536 of
+// the pipe per 32 columns.  K up to 64 takes 32, fewer hand-offs (1 024 rows, K = 64: 6.3 against 6.7 us), wider rows 16, a deeper
+// pipeline (projections of 1.5 M vertices, 128-256-256-256: 5.04 against 5.26 ms a pass; of 2.45 M, 100-256-256-47: 6.65 and 6.95).
+// The epilogue of one warp per quadrant with TMA stores, which waited 2 400 cycles per 32 columns, had hidden that: 6.40 and 8.25.
+constexpr int stage_columns(int K) { return K <= 64 ? 32 : 16; }
 constexpr unsigned WAIT_LIMIT = 1u << 24;
-constexpr int NUM_THREADS = 320;
+constexpr int EPI_WARPS = 8;         // two per quadrant of TMEM lanes, which take turns with the columns
+constexpr int NUM_THREADS = 32 * (6 + EPI_WARPS);
 constexpr int OUT_TILE_BYTES = 32 * 128;        // epilogue staging tile: 32 rows x 32 fp32, 128B-swizzled
-constexpr int OUT_STAGING_BYTES = 4 * 2 * OUT_TILE_BYTES;   // 4 epilogue warps x 2 tiles
+constexpr int OUT_STAGING_BYTES = EPI_WARPS * OUT_TILE_BYTES;
 
 struct __align__(8) Barriers {
   unsigned long long full[MAX_STAGES], conv[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2];
+  __align__(16) float bias[BN_MAX];   // of the CTA's columns (a CTA keeps to one block of columns)
   unsigned int tmem_base;
   int abort_flag;
 };
 
-// shared memory per stage: fp32 mode  A_hi(raw) 16K | A_lo 16K | B_hi 32K | B_lo 32K       = 96 KB (32 K-columns)
+// shared memory per stage: fp32 mode  A_hi(raw) 16K | A_lo 16K | B_hi 32K | B_lo 32K       = 96 KB (KS = 32)
 //                          bf16 mode  A_raw0 16K | A_raw1 16K | A_bf16 16K | B_bf16 32K     = 80 KB (64 K-columns)
 // with weight tiles of 256 columns; the memory is sized for two such stages, and a launch whose weight tiles are
 // narrower runs as many stages as fit (GemmArgs::stages, stage_bytes).
@@ -115,16 +118,29 @@ __device__ __forceinline__ void umma(unsigned tmem_d, unsigned long long a, unsi
 __device__ __forceinline__ void umma_commit(unsigned long long* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// 32 columns of the accumulator, one row per lane.
+__device__ __forceinline__ void tmem_ld32(unsigned (&v)[32], unsigned taddr) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
+        "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+        "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(taddr) : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 struct GemmArgs {
-  float* PT;            // [n x N]
+  float* PT;            // [n x N], pitch ldo
+  long long ldo;
   int n, N, Np;         // rows, output columns, columns padded to a multiple of 16
-  int k_stages;         // K padded / (KS32 fp32 mode, 64 bf16 mode)
+  int k_stages;         // K in stages of KS (fp32 mode) or 64 (bf16 mode) columns
   int b_box_bytes;      // bytes one W-operand TMA box delivers (box rows x operand row bytes)
   int stages;           // operand stages in flight (2 .. MAX_STAGES)
-  int stage_bytes;      // fp32 mode 2 * A32_BYTES + 2 * b_box_bytes, bf16 mode 3 * TILE_A_BYTES + b_box_bytes
+  int stage_bytes;      // fp32 mode 2 * BM * KS * 4 + 2 * b_box_bytes, bf16 mode 3 * TILE_A_BYTES + b_box_bytes
   int Hp, mode, fanout;
   const float* bias;
   const long long* row_ptr;
@@ -136,12 +152,13 @@ struct GemmArgs {
   GemmFinish fin;
 };
 
-template <bool BF16>
+template <bool BF16, int KS>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_b0,
-                  const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ CUtensorMap map_out, GemmArgs g) {
+                  const __grid_constant__ CUtensorMap map_b1, GemmArgs g) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  constexpr int ROW = KS * 4, A32_BYTES = BM * ROW;   // fp32 mode: bytes of an operand row, of a feature tile (raw / hi, or lo)
   constexpr int STAGE_BYTES_MAX = BF16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32;
   const int STAGE_BYTES = g.stage_bytes;
   const int n_stages = g.stages;
@@ -157,13 +174,19 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&bars->full[s], 1); mbar_init(&bars->conv[s], 128); mbar_init(&bars->empty[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&bars->acc_full[b], 1); mbar_init(&bars->acc_empty[b], 128); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&bars->acc_full[b], 1); mbar_init(&bars->acc_empty[b], 32 * EPI_WARPS); }
     bars->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {   // TMEM allocation by one full warp
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem_base)), "r"(tmem_cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  // Bias of the CTA's columns (the grid is a multiple of n_blocks).  Read from memory where it is added, between stores to shared
+  // memory, it was eight round trips in a row per 32 columns.
+  for (int j = threadIdx.x; j < BN_MAX; j += NUM_THREADS) {
+    const int c = (int)(blockIdx.x % n_blocks) * BN_MAX + j;
+    bars->bias[j] = c >= g.N || g.mode == TAURUS_GAT ? 0.f : g.finish ? g.fin.bias[c] : g.bias && c >= g.Hp ? g.bias[c - g.Hp] : 0.f;
   }
   tc_fence_before();
   __syncthreads();
@@ -192,9 +215,9 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
             tma_load_2d(st + 3 * TILE_A_BYTES, &map_b0, ks * 64, col0, &bars->full[s]);
           } else {
             mbar_expect_tx(&bars->full[s], A32_BYTES + 2 * g.b_box_bytes);
-            tma_load_2d(st, &map_x, ks * KS32, row0, &bars->full[s]);
-            tma_load_2d(st + 2 * A32_BYTES, &map_b0, ks * KS32, col0, &bars->full[s]);
-            tma_load_2d(st + 2 * A32_BYTES + g.b_box_bytes, &map_b1, ks * KS32, col0, &bars->full[s]);
+            tma_load_2d(st, &map_x, ks * KS, row0, &bars->full[s]);
+            tma_load_2d(st + 2 * A32_BYTES, &map_b0, ks * KS, col0, &bars->full[s]);
+            tma_load_2d(st + 2 * A32_BYTES + g.b_box_bytes, &map_b1, ks * KS, col0, &bars->full[s]);
           }
         }
       }
@@ -224,10 +247,10 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) umma(tmem_d, da + 2 * kk, db + 2 * kk, idesc, (ks | kk) != 0, false);
           } else {
-            const unsigned long long a_hi = umma_desc<ROW32>(base), a_lo = umma_desc<ROW32>(base + A32_BYTES);
-            const unsigned long long b_hi = umma_desc<ROW32>(base + 2 * A32_BYTES), b_lo = umma_desc<ROW32>(base + 2 * A32_BYTES + g.b_box_bytes);
+            const unsigned long long a_hi = umma_desc<ROW>(base), a_lo = umma_desc<ROW>(base + A32_BYTES);
+            const unsigned long long b_hi = umma_desc<ROW>(base + 2 * A32_BYTES), b_lo = umma_desc<ROW>(base + 2 * A32_BYTES + g.b_box_bytes);
 #pragma unroll
-            for (int kk = 0; kk < KS32 / 8; ++kk) {
+            for (int kk = 0; kk < KS / 8; ++kk) {
               umma(tmem_d, a_lo + 2 * kk, b_hi + 2 * kk, idesc, (ks | kk) != 0, true);
               umma(tmem_d, a_hi + 2 * kk, b_lo + 2 * kk, idesc, 1u, true);
               umma(tmem_d, a_hi + 2 * kk, b_hi + 2 * kk, idesc, 1u, true);
@@ -289,9 +312,11 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       if (!ok) break;
     }
   } else {
-    // ---------------------------------------------------------------- epilogue (warps 6..9, TMEM lanes 32 * (warp % 4))
-    const int q = warp & 3;
-    int unit = 0, out_it = 0;
+    // ---------------------------------------------------------------- epilogue (warps 6..13, TMEM lanes 32 * (warp % 4))
+    const int q = warp & 3, half = (warp - 6) >> 2;
+    // this warp's staging tile: 32 rows (lane = row) x 32 columns, 16-byte chunk c of row r at chunk c ^ (r & 7)
+    unsigned char* const tile_smem = out_staging + (warp - 6) * OUT_TILE_BYTES;
+    int unit = 0;
     for (int w = blockIdx.x; w < n_tiles * n_blocks && !*abort_flag; w += gridDim.x, ++unit) {
     const int tile = w / n_blocks, nb = w % n_blocks;
     const int r = tile * BM + q * 32 + lane;
@@ -300,7 +325,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     if (g.finish) {
       if (r < g.n && r < *g.done_count && !g.ctl->error) {
         vrow = g.fin.done_list[r];
-        if (nb == 0) g.fin.state[vrow] = TAURUS_COMPLETED;
+        if (nb == 0 && half == 0) g.fin.state[vrow] = TAURUS_COMPLETED;
       }
     } else if (r < g.n) {
       const long long u = g.src_begin + r;
@@ -317,77 +342,55 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       const int buf = unit & 1;
       if (!mbar_wait(&bars->acc_full[buf], (unit >> 1) & 1, abort_flag)) break;
       tc_fence_after();
-      for (int c0 = 0; c0 < bw; c0 += 32) {
+      const int columns = bw < g.N - nb * BN_MAX ? bw : g.N - nb * BN_MAX;   // without the padding of the last block
+#pragma unroll 1
+      for (int c0 = half * 32; c0 < columns; c0 += 64) {
         unsigned v[32];
-        const unsigned taddr = tmem_base + ((unsigned)(q * 32) << 16) + (unsigned)(buf * BN_MAX + c0);
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-            "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-              "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
-              "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-              "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-            : "r"(taddr) : "memory");
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        tmem_ld32(v, tmem_base + ((unsigned)(q * 32) << 16) + (unsigned)(buf * BN_MAX + c0));
         const int cbase = nb * BN_MAX + c0;
-        if (cbase >= g.N) continue;           // padding columns of the last block
-        // this warp's staging tile: 32 rows (lane = row) x 32 columns, 16-byte chunk c of row r at chunk c ^ (r & 7)
-        unsigned char* tile_smem = out_staging + (q * 2 + (out_it & 1)) * OUT_TILE_BYTES;
-        if (g.finish) {
-          // transpose through the staging tile, then the warp writes four rows per step, each as one 128-byte piece of
-          // the row's place in the vertex-ordered matrix
+        float o[32];
+        if (cbase + 32 <= g.Hp && !g.finish) {   // P columns: c_out(u) * (x W_neigh)
+#pragma unroll
+          for (int j = 0; j < 32; ++j) o[j] = __uint_as_float(v[j]) * c_out;
+        } else {
 #pragma unroll
           for (int j = 0; j < 32; j += 4) {
-            const int c = cbase + j;
-            const float4 b = c < g.N ? *reinterpret_cast<const float4*>(g.fin.bias + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-            float4 o = make_float4(__uint_as_float(v[j]) + b.x, __uint_as_float(v[j + 1]) + b.y, __uint_as_float(v[j + 2]) + b.z,
-                                   __uint_as_float(v[j + 3]) + b.w);
-            if (g.fin.act) { o.x = fmaxf(o.x, 0.f); o.y = fmaxf(o.y, 0.f); o.z = fmaxf(o.z, 0.f); o.w = fmaxf(o.w, 0.f); }
-            *reinterpret_cast<float4*>(tile_smem + lane * 128 + (((j >> 2) ^ (lane & 7)) << 4)) = o;
+            const float4 b = *reinterpret_cast<const float4*>(&bars->bias[c0 + j]);   // zero in P columns
+            // T columns: (x W_self + b) * max(|M(u)|, 1); finished rows: act(x W + b); GAT: the attention scalars as they are
+            const float mul = g.finish ? 1.f : cbase + j >= g.Hp ? self_mul : c_out;
+            o[j] = (__uint_as_float(v[j]) + b.x) * mul; o[j + 1] = (__uint_as_float(v[j + 1]) + b.y) * mul;
+            o[j + 2] = (__uint_as_float(v[j + 2]) + b.z) * mul; o[j + 3] = (__uint_as_float(v[j + 3]) + b.w) * mul;
           }
-          __syncwarp();
+          if (g.finish && g.fin.act)
 #pragma unroll
-          for (int it = 0; it < 8; ++it) {
-            const int rr = it * 4 + (lane >> 3), ch = lane & 7;
+            for (int j = 0; j < 32; ++j) o[j] = fmaxf(o[j], 0.f);
+        }
+#pragma unroll
+        for (int j = 0; j < 32; j += 4)
+          *reinterpret_cast<float4*>(tile_smem + lane * 128 + (((j >> 2) ^ (lane & 7)) << 4)) = make_float4(o[j], o[j + 1], o[j + 2], o[j + 3]);
+        // Transposed through the staging tile: the warp writes four rows per step, each as one 128-byte piece.  (TMA stores of the
+        // tile queue up behind the operand loads.)
+        __syncwarp();
+        const int ch = lane & 7;
+        const bool in = cbase + ch * 4 < g.N;
+#pragma unroll
+        for (int it = 0; it < 8; ++it) {
+          const int rr = it * 4 + (lane >> 3);
+          const float4 y = *reinterpret_cast<const float4*>(tile_smem + rr * 128 + ((ch ^ (rr & 7)) << 4));
+          if (g.finish) {
             const int vv = __shfl_sync(0xffffffffu, vrow, rr);
-            const float4 y = *reinterpret_cast<const float4*>(tile_smem + rr * 128 + ((ch ^ (rr & 7)) << 4));
-            if (vv >= 0 && cbase + ch * 4 < g.N)
-              *reinterpret_cast<float4*>(g.fin.dense + (size_t)vv * g.fin.dense_ld + cbase + ch * 4) = y;
+            if (vv >= 0 && in) *reinterpret_cast<float4*>(g.fin.dense + (size_t)vv * g.fin.dense_ld + cbase + ch * 4) = y;
+          } else {
+            const int row = tile * BM + q * 32 + rr;
+            if (row < n_rows && in) *reinterpret_cast<float4*>(g.PT + (size_t)row * g.ldo + cbase + ch * 4) = y;
           }
-          __syncwarp();   // the tile is rewritten in the next round
-          continue;
         }
-        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");   // the store that last used this tile has read it
-        __syncwarp();
-#pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-          float4 o;
-          float* po = &o.x;
-          const int c = cbase + j;
-          if (c >= g.Hp && c < g.N) {         // T columns: (x W_self + b) * max(|M(u)|, 1); GAT: the two attention scalars as they are
-            const float4 b = g.mode == TAURUS_GAT ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(g.bias + (c - g.Hp));
-            po[0] = (__uint_as_float(v[j]) + b.x) * self_mul; po[1] = (__uint_as_float(v[j + 1]) + b.y) * self_mul;
-            po[2] = (__uint_as_float(v[j + 2]) + b.z) * self_mul; po[3] = (__uint_as_float(v[j + 3]) + b.w) * self_mul;
-          } else {                            // P columns: c_out(u) * (x W_neigh)
-            po[0] = __uint_as_float(v[j]) * c_out; po[1] = __uint_as_float(v[j + 1]) * c_out;
-            po[2] = __uint_as_float(v[j + 2]) * c_out; po[3] = __uint_as_float(v[j + 3]) * c_out;
-          }
-          *reinterpret_cast<float4*>(tile_smem + lane * 128 + (((j >> 2) ^ (lane & 7)) << 4)) = o;
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) {                      // rows beyond n and columns beyond N are clipped by the tensor map
-          asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
-                       ::"l"(&map_out), "r"(cbase), "r"(tile * BM + q * 32), "r"(smem_u32(tile_smem)) : "memory");
-          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-        }
-        ++out_it;
+        __syncwarp();   // the tile is rewritten in the next round
       }
       tc_fence_before();
       mbar_arrive(&bars->acc_empty[buf]);
     }
     }
-    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // all stores of this warp are complete
   }
 
   // ---------------------------------------------------------------- teardown
@@ -430,7 +433,7 @@ EncodeTiledFn encode_fn() {
 }
 
 // 2-D row-major tensor [rows x cols] of `elem` bytes, box [box_rows x box_cols], 128-byte swizzle, zero fill
-// on loads, clipping on stores.
+// on loads.
 bool make_map(CUtensorMap* m, const void* base, CUtensorMapDataType dt, int elem, long long rows, long long cols,
               long long ld_elems, int box_rows, int box_cols) {
   EncodeTiledFn fn = encode_fn();
@@ -445,18 +448,33 @@ bool make_map(CUtensorMap* m, const void* base, CUtensorMapDataType dt, int elem
 }
 
 // Stages that fit the shared memory sized for STAGES full-width stages.
-void set_stages(GemmArgs& g, bool bf16) {
+void set_stages(GemmArgs& g, bool bf16, int ks) {
   const int budget = STAGES * (bf16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32);
-  g.stage_bytes = bf16 ? 3 * TILE_A_BYTES + g.b_box_bytes : 2 * A32_BYTES + 2 * g.b_box_bytes;
+  g.stage_bytes = bf16 ? 3 * TILE_A_BYTES + g.b_box_bytes : 2 * BM * ks * 4 + 2 * g.b_box_bytes;
   int n = budget / g.stage_bytes;
   g.stages = n < STAGES ? STAGES : n > MAX_STAGES ? MAX_STAGES : n;
+}
+
+int launch_tc(taurus_ctx* c, int grid, int smem, cudaStream_t st, const CUtensorMap& map_x, const CUtensorMap& map_hi, const CUtensorMap& map_lo,
+              const GemmArgs& g, bool bf16, int ks) {
+  if (!c->tc_smem_set) {   // once per context (the attribute belongs to the context's device)
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const cudaError_t e0 = bf16 ? cudaFuncSetAttribute(project_tc_kernel<true, 32>, at, smem) : cudaFuncSetAttribute(project_tc_kernel<false, 32>, at, smem);
+    const cudaError_t e1 = bf16 ? e0 : cudaFuncSetAttribute(project_tc_kernel<false, 16>, at, smem);
+    if (e0 != cudaSuccess || e1 != cudaSuccess) { cudaGetLastError(); return TAURUS_ERR_CUDA; }
+    c->tc_smem_set = true;
+  }
+  if (bf16) project_tc_kernel<true, 32><<<grid, NUM_THREADS, smem, st>>>(map_x, map_hi, map_lo, g);
+  else if (ks == 32) project_tc_kernel<false, 32><<<grid, NUM_THREADS, smem, st>>>(map_x, map_hi, map_lo, g);
+  else project_tc_kernel<false, 16><<<grid, NUM_THREADS, smem, st>>>(map_x, map_hi, map_lo, g);
+  return TAURUS_OK;
 }
 
 // Per-layer tensor-core images of Wcat, K-major: [Np x Kp].
 struct WImage {
   void* hi = nullptr;   // fp32 mode: tf32-exact high part; bf16 mode: bf16 weights
   void* lo = nullptr;   // fp32 mode: residual
-  int Np = 0, Kp = 0;
+  int Np = 0, Kp = 0, ks = 0;   // ks: K columns per stage
   CUtensorMap map_hi, map_lo;
 };
 
@@ -467,7 +485,8 @@ int prepare_tc_weights(taurus_ctx* c, void** slot, const std::vector<float>& cat
   WImage* w = new WImage();
   *slot = w;
   w->Np = taurus_round_up(N, 16);
-  w->Kp = taurus_round_up(K, bf16 ? 64 : KS32);
+  w->ks = bf16 ? 64 : stage_columns(K);
+  w->Kp = taurus_round_up(K, w->ks);
   const size_t cnt = (size_t)w->Np * w->Kp;
   const int bw = w->Np < BN_MAX ? w->Np : BN_MAX;
   if (bf16) {
@@ -493,8 +512,8 @@ int prepare_tc_weights(taurus_ctx* c, void** slot, const std::vector<float>& cat
     if (cudaMalloc(&w->hi, cnt * 4) != cudaSuccess || cudaMalloc(&w->lo, cnt * 4) != cudaSuccess) return TAURUS_ERR_NOMEM;
     if (cudaMemcpy(w->hi, hi.data(), cnt * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(w->lo, lo.data(), cnt * 4, cudaMemcpyHostToDevice) != cudaSuccess) return TAURUS_ERR_CUDA;
-    if (!make_map(&w->map_hi, w->hi, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, w->Np, w->Kp, w->Kp, bw, KS32) ||
-        !make_map(&w->map_lo, w->lo, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, w->Np, w->Kp, w->Kp, bw, KS32)) return TAURUS_ERR_CUDA;
+    if (!make_map(&w->map_hi, w->hi, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, w->Np, w->Kp, w->Kp, bw, w->ks) ||
+        !make_map(&w->map_lo, w->lo, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, w->Np, w->Kp, w->Kp, bw, w->ks)) return TAURUS_ERR_CUDA;
   }
   return TAURUS_OK;
 }
@@ -524,29 +543,21 @@ int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long lo
   const int K = c->dims[layer], Hp = taurus_round_up(c->dims[layer + 1], 4);
   const int N = taurus_proj_width(c->mode, Hp, c->heads);
   CUtensorMap map_x;
-  if (!make_map(&map_x, X, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, K, ldx, BM, bf16 ? 32 : KS32)) return TAURUS_ERR_CUDA;
-  CUtensorMap map_out;
-  if (!make_map(&map_out, out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, N, ldo, 32, 32)) return TAURUS_ERR_CUDA;
+  if (!make_map(&map_x, X, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, K, ldx, BM, bf16 ? 32 : w->ks)) return TAURUS_ERR_CUDA;
   GemmArgs g;
-  g.PT = out; g.n = n; g.N = N; g.Np = w->Np; g.k_stages = w->Kp / (bf16 ? 64 : KS32);
-  g.b_box_bytes = (w->Np < BN_MAX ? w->Np : BN_MAX) * (bf16 ? 128 : ROW32);
-  set_stages(g, bf16);
+  g.PT = out; g.ldo = ldo; g.n = n; g.N = N; g.Np = w->Np; g.k_stages = w->Kp / w->ks;
+  g.b_box_bytes = (w->Np < BN_MAX ? w->Np : BN_MAX) * (bf16 ? 128 : w->ks * 4);
+  set_stages(g, bf16, w->ks);
   g.Hp = Hp; g.mode = c->mode; g.fanout = c->fanout[layer]; g.bias = c->d_bias[layer];
   g.row_ptr = c->d_row_ptr; g.din = c->d_din; g.src_begin = src_begin; g.ctl = c->d_ctl;
   g.finish = 0; g.fin = GemmFinish(); g.done_count = nullptr;
   const int smem = STAGES * (bf16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32) + OUT_STAGING_BYTES + (int)sizeof(Barriers) + 1024;
   const int n_tiles = (n + BM - 1) / BM;
-  const int n_units = n_tiles * ((w->Np + BN_MAX - 1) / BN_MAX);
+  const int n_blocks = (w->Np + BN_MAX - 1) / BN_MAX, n_units = n_tiles * n_blocks;
   const int sms = c->sm_count - c->xfer_blocks;   // the SMs of the row transfers have no shared memory left
-  const int grid = n_units < sms ? n_units : sms;
-  if (!c->tc_smem_set) {   // once per context (the attribute belongs to the context's device)
-    cudaError_t e = bf16 ? cudaFuncSetAttribute(project_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
-                         : cudaFuncSetAttribute(project_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) { cudaGetLastError(); return TAURUS_ERR_CUDA; }
-    c->tc_smem_set = true;
-  }
-  if (bf16) project_tc_kernel<true><<<grid, NUM_THREADS, smem, st>>>(map_x, w->map_hi, w->map_lo, map_out, g);
-  else project_tc_kernel<false><<<grid, NUM_THREADS, smem, st>>>(map_x, w->map_hi, w->map_lo, map_out, g);
+  const int grid = n_units < sms ? n_units : std::max(1, sms / n_blocks) * n_blocks;   // a CTA keeps to one block of columns
+  const int rc = launch_tc(c, grid, smem, st, map_x, w->map_hi, w->map_lo, g, bf16, w->ks);
+  if (rc) return rc;
   c->launches += 1;
   return TAURUS_OK;
 }
@@ -572,39 +583,32 @@ int launch_gemm_plain_tc(taurus_ctx* c, void* image, int col0, int N, const floa
   const int Np = std::min(taurus_round_up(N, 16), rows_left);
   const int bw = Np < BN_MAX ? Np : BN_MAX;
   const int elem = bf16 ? 2 : 4;
-  CUtensorMap map_x, map_out, map_hi, map_lo;
-  if (!make_map(&map_x, X, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, K, ldx, BM, bf16 ? 32 : KS32)) return TAURUS_ERR_CUDA;
-  if (!make_map(&map_out, out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, N, ld_out, 32, 32)) return TAURUS_ERR_CUDA;
+  CUtensorMap map_x, map_hi, map_lo;
+  if (!make_map(&map_x, X, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, K, ldx, BM, bf16 ? 32 : w->ks)) return TAURUS_ERR_CUDA;
   const char* hi = static_cast<const char*>(w->hi) + (size_t)col0 * w->Kp * elem;
   if (!make_map(&map_hi, hi, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, elem, rows_left, w->Kp, w->Kp, bw,
-                bf16 ? 64 : KS32))
+                w->ks))
     return TAURUS_ERR_CUDA;
   map_lo = map_hi;
   if (!bf16) {
     const char* lo = static_cast<const char*>(w->lo) + (size_t)col0 * w->Kp * elem;
-    if (!make_map(&map_lo, lo, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, rows_left, w->Kp, w->Kp, bw, KS32)) return TAURUS_ERR_CUDA;
+    if (!make_map(&map_lo, lo, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, rows_left, w->Kp, w->Kp, bw, w->ks)) return TAURUS_ERR_CUDA;
   }
   GemmArgs g;
-  g.PT = out; g.n = n; g.N = N; g.Np = Np; g.k_stages = w->Kp / (bf16 ? 64 : KS32);
-  g.b_box_bytes = bw * (bf16 ? 128 : ROW32);
-  set_stages(g, bf16);
+  g.PT = out; g.ldo = ld_out; g.n = n; g.N = N; g.Np = Np; g.k_stages = w->Kp / w->ks;
+  g.b_box_bytes = bw * (bf16 ? 128 : w->ks * 4);
+  set_stages(g, bf16, w->ks);
   g.Hp = N; g.mode = TAURUS_GIN_SUM; g.fanout = 0; g.bias = nullptr;
   g.row_ptr = c->d_row_ptr; g.din = c->d_din; g.src_begin = 0; g.ctl = c->d_ctl;
   g.finish = finish ? 1 : 0; g.fin = finish ? *finish : GemmFinish();
   g.done_count = done_count;
   const int smem = STAGES * (bf16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32) + OUT_STAGING_BYTES + (int)sizeof(Barriers) + 1024;
   const int n_tiles = (n + BM - 1) / BM;
-  const int n_units = n_tiles * ((Np + BN_MAX - 1) / BN_MAX);
+  const int n_blocks = (Np + BN_MAX - 1) / BN_MAX, n_units = n_tiles * n_blocks;
   const int sms = c->sm_count - c->xfer_blocks;   // the SMs of the row transfers have no shared memory left
-  const int grid = n_units < sms ? n_units : sms;
-  if (!c->tc_smem_set) {
-    cudaError_t e = bf16 ? cudaFuncSetAttribute(project_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
-                         : cudaFuncSetAttribute(project_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) { cudaGetLastError(); return TAURUS_ERR_CUDA; }
-    c->tc_smem_set = true;
-  }
-  if (bf16) project_tc_kernel<true><<<grid, NUM_THREADS, smem, st>>>(map_x, map_hi, map_lo, map_out, g);
-  else project_tc_kernel<false><<<grid, NUM_THREADS, smem, st>>>(map_x, map_hi, map_lo, map_out, g);
+  const int grid = n_units < sms ? n_units : std::max(1, sms / n_blocks) * n_blocks;   // a CTA keeps to one block of columns
+  const int rc = launch_tc(c, grid, smem, st, map_x, map_hi, map_lo, g, bf16, w->ks);
+  if (rc) return rc;
   c->launches += 1;
   return TAURUS_OK;
 }
