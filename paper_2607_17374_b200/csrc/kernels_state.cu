@@ -1057,8 +1057,10 @@ void launch_finalise(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
 
 // ------------------------------------------------------------------------------------------------ drain helpers
 // Row i of the graduation buffer goes to dense[id * ld ...]: the vertex-ordered matrix the next layer streams.
+// empty: the count of waiting rows, set to zero here (a drain is one launch less that way); NULL: left to the caller.
 __global__ void place_rows_kernel(const long long* ids, const float* rows, int Hp, int d_out, float* dense, long long ld,
-                                  long long count) {
+                                  long long count, long long* empty) {
+  if (empty && blockIdx.x == 0 && threadIdx.x == 0) *empty = 0;   // (the count itself came as an argument)
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
   const bool vec_ok = (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(dense) & 15) == 0);
   for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < count; i += warps) {
@@ -1076,11 +1078,12 @@ __global__ void place_rows_kernel(const long long* ids, const float* rows, int H
   }
 }
 
-void launch_place_rows(taurus_ctx* c, float* dense, long long ld, int d_out, int Hp, long long count, cudaStream_t st) {
+void launch_place_rows(taurus_ctx* c, float* dense, long long ld, int d_out, int Hp, long long count, bool empty, cudaStream_t st) {
   if (count <= 0) return;
   long long blocks = (count + 7) / 8;
   if (blocks > c->sm_count * 16) blocks = c->sm_count * 16;
-  place_rows_kernel<<<(int)blocks, 256, 0, st>>>(c->d_grad_ids, c->d_grad_rows, Hp, d_out, dense, ld, count);
+  place_rows_kernel<<<(int)blocks, 256, 0, st>>>(c->d_grad_ids, c->d_grad_rows, Hp, d_out, dense, ld, count,
+                                                    empty ? &c->d_ctl->grad_count : nullptr);
   c->launches += 1;
 }
 

@@ -966,8 +966,8 @@ static int drain_common(taurus_ctx* c, long long capacity, long long* out_count,
   return TAURUS_OK;
 }
 
-static int drain_reset(taurus_ctx* c) {
-  CU(cudaMemsetAsync(reinterpret_cast<char*>(c->d_ctl) + offsetof(DevCtl, grad_count), 0, sizeof(long long), c->last_stream));
+static int drain_reset(taurus_ctx* c, bool emptied = false) {
+  if (!emptied) CU(cudaMemsetAsync(reinterpret_cast<char*>(c->d_ctl) + offsetof(DevCtl, grad_count), 0, sizeof(long long), c->last_stream));
   CU(cudaStreamSynchronize(c->last_stream));
   c->ub_since_drain = 0;
   return TAURUS_OK;
@@ -1006,11 +1006,11 @@ extern "C" int taurus_drain_dense(taurus_ctx* c, float* dense_rows, int64_t ld, 
   if (count > 0) {
     const int d_out = c->dims[c->layer + 1], Hp = taurus_round_up(d_out, 4);
     cudaStream_t st = c->last_stream;
-    launch_place_rows(c, dense_dev, ld, d_out, Hp, count, st);
+    launch_place_rows(c, dense_dev, ld, d_out, Hp, count, out_ids == nullptr, st);
     if (out_ids) CU(cudaMemcpyAsync(out_ids, c->d_grad_ids, (size_t)count * sizeof(long long), cudaMemcpyDefault, st));
     CU(cudaGetLastError());
   }
-  return drain_reset(c);
+  return drain_reset(c, count == 0 || out_ids == nullptr);
 }
 
 extern "C" int taurus_layer_set_dense_output(taurus_ctx* c, float* dense_rows, int64_t ld) {

@@ -346,7 +346,7 @@ int launch_transfer(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);    // s
 void launch_finalise(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);    // finalise + commit (after launch_compact_done)
 void launch_compact_done(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, bool write_record);   // completions listed (and the chunk record written)
 void launch_commit(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);
-void launch_place_rows(taurus_ctx* c, float* dense, long long ld, int d_out, int Hp, long long count, cudaStream_t st);
+void launch_place_rows(taurus_ctx* c, float* dense, long long ld, int d_out, int Hp, long long count, bool empty, cudaStream_t st);   // empty: no row waits any more
 void launch_place_half(taurus_ctx* c, int half, int d_out, int Hp, cudaStream_t st);   // dense-output mode
 void launch_reload_histogram(taurus_ctx* c, cudaStream_t st);               // fills ctl->reload_hist
 void launch_completion_ranks(taurus_ctx* c, cudaStream_t st);                // fills d_rank_hist
