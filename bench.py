@@ -46,7 +46,7 @@ METRIC = "edges/sec per GNN layer (GTEPS)"
 # csrc/kernels_resident.cu, first 16 hex digits); when the source has changed since the capture the bench prints
 # traffic = null instead of a stale number.
 GATHER_TRAFFIC_OVER_REQUESTED = 0.681
-GATHER_CAPTURE_SOURCE = "be171bf5d21b1eaa"
+GATHER_CAPTURE_SOURCE = "83b8ddff6c8ad272"
 
 
 def source_digest(name: str) -> str:
