@@ -15,7 +15,7 @@
 // TMEM accumulator buffers, so the epilogue of one unit overlaps the main loop of the next, also across tiles.
 //
 // Every wait on an mbarrier is bounded: after WAIT_LIMIT polls the kernel raises a CTA-wide abort flag,
-// records TAURUS_ERR_INTERNAL in the control block, waits (bounded) for its TMA copies in flight, frees its
+// records TAURUS_ERR_INTERNAL in the control block, waits (bounded) for its TMA copies and MMAs in flight, frees its
 // TMEM and returns.  Every TMA load is a plain load of the issuing CTA alone.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "stage_waits.h"
 #include "taurus_internal.h"
 
 namespace {
@@ -52,6 +53,7 @@ struct __align__(8) Barriers {
   __align__(16) float bias[BN_MAX];   // of the CTA's columns (a CTA keeps to one block of columns)
   unsigned int tmem_base;
   int abort_flag;
+  int loads, mmas;   // uses of the operand ring whose copies / whose MMAs have been issued (written when their warp is through)
 };
 
 // shared memory per stage: fp32 mode  A_hi(raw) 16K | A_lo 16K | B_hi 32K | B_lo 32K       = 96 KB (KS = 32)
@@ -221,6 +223,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
           }
         }
       }
+      bars->loads = it;
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
@@ -261,6 +264,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         if (!ok) break;
         umma_commit(&bars->acc_full[buf]);  // accumulator of this block complete
       }
+      bars->mmas = it;
     }
   } else if (warp < 6) {
     // ---------------------------------------------------------------- converter (128 threads)
@@ -398,10 +402,9 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   if (*abort_flag) {
     if (threadIdx.x == 0) {
       atomicCAS(&g.ctl->error, 0, TAURUS_ERR_INTERNAL);
-      // give copies that may still be in flight a bounded time to land before the shared memory is released
-      for (int s = 0; s < n_stages; ++s)
-        for (unsigned i = 0; i < (1u << 16); ++i)
-          if (mbar_try(&bars->full[s], 0) || mbar_try(&bars->full[s], 1)) break;
+      // the copies and MMAs on their way get a bounded time to end before shared memory and TMEM are released
+      wait_last_phases(bars->loads, n_stages, 1u << 16, [&](int s, unsigned parity) { return mbar_try(&bars->full[s], parity); });
+      wait_last_phases(bars->mmas, n_stages, 1u << 16, [&](int s, unsigned parity) { return mbar_try(&bars->empty[s], parity); });
     }
     __syncthreads();
   }
