@@ -29,6 +29,11 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def resource_log(src: str) -> str:
+    """Where the build keeps what ptxas said about a source's kernels (registers, shared memory, spills)."""
+    return os.path.join(_PKG, "build", os.path.basename(src)[:-3] + ".ptxas")
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every .cu under csrc/ into one shared library next to the package (no-op when up to date)."""
     if not force and not _stale():
@@ -45,13 +50,15 @@ def build(force: bool = False, verbose: bool = False) -> str:
             glob.glob(os.path.join(INCLUDE, "*.h"))
         if not force and os.path.exists(obj) and all(os.path.getmtime(obj) >= os.path.getmtime(d) for d in deps):
             continue
-        cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-I", INCLUDE, "-I", CSRC, "-c", src, "-o", obj]
+        cmd = [nvcc] + NVCC_FLAGS + ["-Xptxas", "-v", "-I", INCLUDE, "-I", CSRC, "-c", src, "-o", obj]
         procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     failed = False
     for src, p in procs:
         out, _ = p.communicate()
         if p.returncode != 0 or verbose:
             sys.stderr.write(out)
+        with open(resource_log(src), "w") as f:
+            f.write(out)
         failed |= p.returncode != 0
     if failed:
         raise RuntimeError("nvcc failed")

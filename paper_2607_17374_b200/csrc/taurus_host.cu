@@ -721,9 +721,9 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
     float* rows = c->d_store + (size_t)src_begin * w;
     if (af) {
       a.Hout = a.Hp; a.Hp = taurus_round_up(c->dims[l], 4); a.self_bias = 0;
-      launch_store_rows(c, X, ldx, n, c->dims[l], a.Hp, src_begin, c->mode == TAURUS_GCN_SYM, rows, w, st);   // (GAT: pass 1 handed the input rows back, pitch dims[l + 1])
+      launch_store_rows(c, X, ldx, n, c->dims[l], src_begin, c->mode == TAURUS_GCN_SYM, rows, w, st);   // (GAT: pass 1 handed the input rows back, pitch dims[l + 1])
     } else if (gat) {
-      launch_store_rows(c, X, ldx, n, K, a.Hp, src_begin, false, rows, w, st);
+      launch_store_rows(c, X, ldx, n, K, src_begin, false, rows, w, st);
     } else if (project_tc_usable(c, l, X, ldx)) {
       int rc = launch_project_tc(c, l, X, ldx, src_begin, n, rows, w, st);
       if (rc) return rc;

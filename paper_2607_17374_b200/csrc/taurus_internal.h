@@ -406,7 +406,7 @@ int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long lo
 int resident_row(const taurus_ctx* c, int layer);                            // floats per row of the store
 int build_resident(taurus_ctx* c);
 void launch_resident_reset(taurus_ctx* c, int layer, cudaStream_t st);
-void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int K, int Kp, long long src_begin, bool gcn, float* out, int ldo, cudaStream_t st);
+void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int K, long long src_begin, bool gcn, float* out, int ldo, cudaStream_t st);
 void launch_account(taurus_ctx* c, const ChunkArgs& a, long long cell, cudaStream_t st);
 int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitch, float* A, long long bound, cudaStream_t st);
 void launch_resident_attention(taurus_ctx* c, cudaStream_t st);
