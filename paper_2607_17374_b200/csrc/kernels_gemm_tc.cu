@@ -154,12 +154,26 @@ struct GemmArgs {
   GemmFinish fin;
 };
 
+// A CTA leaves room for a block of the accounting on its SM, and with it for the small kernels of the output stream: without it the two
+// took turns.  Passes of 1.5 M vertices, 128-256-256-256, fanout 15-10-5: 12.9 -> 12.1 ms; of 2.45 M, 100-256-256-47: 36.9 -> 36.2;
+// eight pushes of 65 536 rows, 256 -> 2 x 48: 823 -> 720 us.  (96 registers measure the same; at 112 the scheduler with four of the
+// CTA's warps has no room for the two of the other block, although the SM as a whole has.)
+constexpr int PROJECT_REGISTERS = 104;
+constexpr int shared_bytes(bool bf16) { return STAGES * (bf16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32) + OUT_STAGING_BYTES + (int)sizeof(Barriers); }
+static_assert(shared_bytes(false) + TAURUS_BLOCK_SHARED + TAURUS_ACCOUNT_SHARED + TAURUS_BLOCK_SHARED <= TAURUS_SM_SHARED, "shared memory for a block of the accounting");
+static_assert(shared_bytes(true) <= shared_bytes(false), "either operand type");
+static_assert(taurus_quarter_registers(NUM_THREADS, PROJECT_REGISTERS) + taurus_quarter_registers(TAURUS_ACCOUNT_THREADS, TAURUS_ACCOUNT_REGISTERS) <=
+              TAURUS_QUARTER_REGISTERS, "registers for a block of the accounting");
+
 template <bool BF16, int KS>
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+__global__ void __maxnreg__(PROJECT_REGISTERS)
 project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_b0,
                   const __grid_constant__ CUtensorMap map_b1, GemmArgs g) {
-  extern __shared__ unsigned char smem_raw[];
-  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  extern __shared__ __align__(1024) unsigned char smem[];   // (the swizzled operand tiles want 1 024)
+  if ((smem_u32(smem) & 1023u) != 0) {
+    if (threadIdx.x == 0) atomicCAS(&g.ctl->error, 0, TAURUS_ERR_INTERNAL);
+    return;
+  }
   constexpr int ROW = KS * 4, A32_BYTES = BM * ROW;   // fp32 mode: bytes of an operand row, of a feature tile (raw / hi, or lo)
   constexpr int STAGE_BYTES_MAX = BF16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32;
   const int STAGE_BYTES = g.stage_bytes;
@@ -554,7 +568,7 @@ int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long lo
   g.Hp = Hp; g.mode = c->mode; g.fanout = c->fanout[layer]; g.bias = c->d_bias[layer];
   g.row_ptr = c->d_row_ptr; g.din = c->d_din; g.src_begin = src_begin; g.ctl = c->d_ctl;
   g.finish = 0; g.fin = GemmFinish(); g.done_count = nullptr;
-  const int smem = STAGES * (bf16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32) + OUT_STAGING_BYTES + (int)sizeof(Barriers) + 1024;
+  const int smem = shared_bytes(bf16);
   const int n_tiles = (n + BM - 1) / BM;
   const int n_blocks = (w->Np + BN_MAX - 1) / BN_MAX, n_units = n_tiles * n_blocks;
   const int sms = c->sm_count - c->xfer_blocks;   // the SMs of the row transfers have no shared memory left
@@ -605,7 +619,7 @@ int launch_gemm_plain_tc(taurus_ctx* c, void* image, int col0, int N, const floa
   g.row_ptr = c->d_row_ptr; g.din = c->d_din; g.src_begin = 0; g.ctl = c->d_ctl;
   g.finish = finish ? 1 : 0; g.fin = finish ? *finish : GemmFinish();
   g.done_count = done_count;
-  const int smem = STAGES * (bf16 ? STAGE_BYTES_BF16 : STAGE_BYTES_FP32) + OUT_STAGING_BYTES + (int)sizeof(Barriers) + 1024;
+  const int smem = shared_bytes(bf16);
   const int n_tiles = (n + BM - 1) / BM;
   const int n_blocks = (Np + BN_MAX - 1) / BN_MAX, n_units = n_tiles * n_blocks;
   const int sms = c->sm_count - c->xfer_blocks;   // the SMs of the row transfers have no shared memory left

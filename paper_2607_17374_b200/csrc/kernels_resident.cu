@@ -94,7 +94,7 @@ __device__ __forceinline__ int mask_bits(const uint32_t* mask, unsigned long lon
 }
 
 // Edges and own vertices of a push that is not a grid cell: pending counts by atomics, first touches listed.
-__global__ void __launch_bounds__(256) account_edges_kernel(ChunkArgs a) {
+__global__ void __launch_bounds__(TAURUS_ACCOUNT_THREADS, 8) account_edges_kernel(ChunkArgs a) {
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
   if (ctl->error) return;
@@ -148,16 +148,22 @@ __global__ void __launch_bounds__(256) account_edges_kernel(ChunkArgs a) {
 enum { C_HS, C_NS, C_GS, C_MSGS, C_HUB, C_GROUPS, C_FREED, C_COUNT };
 #define ITEMS 4
 
+struct AccountShared {
+  int cnt[2][8], base[2], last;
+  unsigned int sum[C_COUNT];
+};
+static_assert(sizeof(AccountShared) <= TAURUS_ACCOUNT_SHARED, "a block fits beside a CTA of the projection,");
+static_assert(4 * TAURUS_QUARTER_REGISTERS / (5 * TAURUS_ACCOUNT_THREADS) / 8 * 8 <= TAURUS_ACCOUNT_REGISTERS, "with the registers its launch bounds allow");
+static_assert(TAURUS_ACCOUNT_THREADS == 8 * 32, "eight warps (AccountShared::cnt)");
+
 template <bool LISTED>
-__global__ void __launch_bounds__(256) account_kernel(ChunkArgs a, Items it, long long i0, long long n_items, const uint32_t* __restrict__ cmask,
+__global__ void __launch_bounds__(TAURUS_ACCOUNT_THREADS, 5) account_kernel(ChunkArgs a, Items it, long long i0, long long n_items, const uint32_t* __restrict__ cmask,
                                                       int4* __restrict__ heavy, int32_t* __restrict__ heavy_left) {
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
   if (ctl->error) return;
-  __shared__ int s_cnt[2][8], s_base[2];
-  __shared__ unsigned int s_sum[C_COUNT];
-  __shared__ int s_last;
-  if (threadIdx.x < C_COUNT) s_sum[threadIdx.x] = 0;
+  __shared__ AccountShared s;
+  if (threadIdx.x < C_COUNT) s.sum[threadIdx.x] = 0;
   const long long n = LISTED ? (long long)pc->touched_count : n_items;
   const long long stride = (long long)gridDim.x * blockDim.x * ITEMS;
   const int warp = threadIdx.x >> 5;
@@ -209,15 +215,15 @@ __global__ void __launch_bounds__(256) account_kernel(ChunkArgs a, Items it, lon
       wd += __popc(md[q]);
     }
     // appended per block: single-address atomics would bound this kernel
-    if (rl() == 0) s_cnt[par][warp] = wd;
+    if (rl() == 0) s.cnt[par][warp] = wd;
     __syncthreads();
     if (threadIdx.x == 0) {
       int t = 0;
-      for (int w = 0; w < 8; ++w) { const int c = s_cnt[par][w]; s_cnt[par][w] = t; t += c; }
-      s_base[par] = t ? atomicAdd(&pc->done_count, t) : 0;
+      for (int w = 0; w < 8; ++w) { const int c = s.cnt[par][w]; s.cnt[par][w] = t; t += c; }
+      s.base[par] = t ? atomicAdd(&pc->done_count, t) : 0;
     }
     __syncthreads();
-    int at = s_base[par] + s_cnt[par][warp];
+    int at = s.base[par] + s.cnt[par][warp];
 #pragma unroll
     for (int q = 0; q < ITEMS; ++q) {
       if (done[q]) {
@@ -241,15 +247,15 @@ __global__ void __launch_bounds__(256) account_kernel(ChunkArgs a, Items it, lon
   for (int c = 0; c < C_COUNT; ++c) {
     unsigned x = sum[c];
     for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
-    if (rl() == 0 && x) atomicAdd(&s_sum[c], x);
+    if (rl() == 0 && x) atomicAdd(&s.sum[c], x);
   }
   __syncthreads();
-  if (threadIdx.x < C_COUNT && s_sum[threadIdx.x]) atomicAdd(&pc->acc[threadIdx.x], (unsigned long long)s_sum[threadIdx.x]);
+  if (threadIdx.x < C_COUNT && s.sum[threadIdx.x]) atomicAdd(&pc->acc[threadIdx.x], (unsigned long long)s.sum[threadIdx.x]);
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&pc->done_blocks, 1u) == gridDim.x - 1;
+  if (threadIdx.x == 0) s.last = atomicAdd(&pc->done_blocks, 1u) == gridDim.x - 1;
   __syncthreads();
-  if (!s_last) return;
+  if (!s.last) return;
   // the counters of the next chunk (the other set; its last reader, the chunk before this one, is through)
   ChunkCtl* next = pc == &ctl->pc[0] ? &ctl->pc[1] : &ctl->pc[0];
   for (int i = threadIdx.x; i < (int)(offsetof(ChunkCtl, sel_k) / 4); i += blockDim.x) reinterpret_cast<int32_t*>(next)[i] = 0;
@@ -997,13 +1003,13 @@ void launch_account(taurus_ctx* c, const ChunkArgs& a, long long cell, cudaStrea
   if (cell >= 0) {
     const long long i0 = c->item_ptr[(size_t)cell], n = c->item_ptr[(size_t)cell + 1] - i0;
     const int grid = (int)std::max<long long>(1, std::min<long long>((n + 256 * ITEMS - 1) / (256 * ITEMS), (long long)c->sm_count * 6));
-    account_kernel<false><<<grid, 256, 0, st>>>(a, it, i0, n, cmask, heavy, c->d_heavy_left);
+    account_kernel<false><<<grid, TAURUS_ACCOUNT_THREADS, 0, st>>>(a, it, i0, n, cmask, heavy, c->d_heavy_left);
     c->launches += 1;
     return;
   }
-  account_edges_kernel<<<c->sm_count * 8, 256, 0, st>>>(a);
+  account_edges_kernel<<<c->sm_count * 8, TAURUS_ACCOUNT_THREADS, 0, st>>>(a);
   const int grid = (int)std::max<long long>(1, std::min<long long>((a.touched_capacity + 256 * ITEMS - 1) / (256 * ITEMS), (long long)c->sm_count * 6));
-  account_kernel<true><<<grid, 256, 0, st>>>(a, it, 0, 0, cmask, heavy, c->d_heavy_left);
+  account_kernel<true><<<grid, TAURUS_ACCOUNT_THREADS, 0, st>>>(a, it, 0, 0, cmask, heavy, c->d_heavy_left);
   c->launches += 2;
 }
 

@@ -17,6 +17,14 @@
 #define TAURUS_PHASES 9                         // durations reported per timed push
 #define TAURUS_HEAVY_DEGREE 256                  // resident pools: in-lists longer than this are summed in segments
 #define TAURUS_HEAVY_SEGMENT 128
+// The accounting of a push runs beside the projection of its rows, whose CTAs take most of every SM: a block of it fits into what
+// they leave (asserted beside either kernel).
+#define TAURUS_SM_SHARED (228 * 1024)            // shared memory of an SM, and what every block takes of it beside its own
+#define TAURUS_BLOCK_SHARED 1024
+#define TAURUS_QUARTER_REGISTERS 16384           // registers of one of an SM's four schedulers, which a block's warps are dealt out to
+#define TAURUS_ACCOUNT_THREADS 256
+#define TAURUS_ACCOUNT_REGISTERS 48
+#define TAURUS_ACCOUNT_SHARED 128
 #define TAURUS_SEL_BITS 11                      // radix-select digit width
 #define TAURUS_SEL_BINS (1 << TAURUS_SEL_BITS)
 #define TAURUS_SEL_LEVELS 6                     // 6 x 11 = 66 bits >= the 62-bit (score, id) key
@@ -329,6 +337,9 @@ struct taurus_ctx {
   std::vector<std::vector<long long>> rank_cum_cache;   // per layer: rank_cum computed at the first layer_begin
   int sm_count = 148;
 };
+
+// Registers of the scheduler that gets most of a block's warps.
+constexpr int taurus_quarter_registers(int threads, int registers) { return (threads / 32 + 3) / 4 * 32 * registers; }
 
 static inline int taurus_round_up(int x, int m) { return (x + m - 1) / m * m; }
 // Columns of the projection output: [P | T] for SAGE, [h' | (att_src.h', att_dst.h') per head, padded to 4] for GAT, P otherwise.
