@@ -157,8 +157,9 @@ static_assert(4 * TAURUS_QUARTER_REGISTERS / (5 * TAURUS_ACCOUNT_THREADS) / 8 * 
 static_assert(TAURUS_ACCOUNT_THREADS == 8 * 32, "eight warps (AccountShared::cnt)");
 
 template <bool LISTED>
-__global__ void __launch_bounds__(TAURUS_ACCOUNT_THREADS, 5) account_kernel(ChunkArgs a, Items it, long long i0, long long n_items, const uint32_t* __restrict__ cmask,
-                                                      int4* __restrict__ heavy, int32_t* __restrict__ heavy_left) {
+__global__ void __launch_bounds__(TAURUS_ACCOUNT_THREADS, LISTED ? 6 : 5)
+account_kernel(ChunkArgs a, Items it, long long i0, long long n_items, const uint32_t* __restrict__ cmask, int4* __restrict__ heavy,
+               int32_t* __restrict__ heavy_left) {
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
   if (ctl->error) return;
