@@ -30,6 +30,13 @@ namespace {
 
 constexpr int BM = 128;            // rows per CTA tile (UMMA M)
 constexpr int BN_MAX = 256;        // output columns per block (UMMA N)
+// A product of more columns is cut into blocks of nearly the same width: a CTA keeps to one block (its bias, its weights' tiles), so a
+// narrow last block (256 + 256 + 16 columns) leaves the CTAs that have it idle most of the time.  Eight launches of 65 536 rows,
+// 132 -> 264 columns: 256 + 16 463 us, 144 + 128 362; 516 -> 520: 256 + 256 + 16 1 850, 3 x 176 1 610 to 1 650 (2 x 192 + 144 1 740).
+constexpr int block_columns(int Np) {
+  const int blocks = (Np + BN_MAX - 1) / BN_MAX;
+  return ((Np + blocks - 1) / blocks + 15) / 16 * 16;
+}
 constexpr int STAGES = 2;            // stages of 128-byte operand rows with full-width (256-column) weight tiles: sizes the shared memory
 constexpr int MAX_STAGES = 8;        // shorter operand rows and narrower weight tiles leave room for more stages in the same memory
 constexpr int TILE_A_BYTES = BM * 128;           // 128 rows x 128 B
@@ -139,6 +146,7 @@ struct GemmArgs {
   float* PT;            // [n x N], pitch ldo
   long long ldo;
   int n, N, Np;         // rows, output columns, columns padded to a multiple of 16
+  int bn;               // columns per block (the last one may have fewer)
   int k_stages;         // K in stages of KS (fp32 mode) or 64 (bf16 mode) columns
   int b_box_bytes;      // bytes one W-operand TMA box delivers (box rows x operand row bytes)
   int stages;           // operand stages in flight (2 .. MAX_STAGES)
@@ -185,7 +193,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   int n_rows = g.n;
   if (g.done_count) { const int nd = *g.done_count; n_rows = nd < g.n ? nd : g.n; }   // same value in every thread
   const int n_tiles = (n_rows + BM - 1) / BM;
-  const int n_blocks = (g.Np + BN_MAX - 1) / BN_MAX;
+  const int n_blocks = (g.Np + g.bn - 1) / g.bn;
   const int tmem_cols = 512;   // two accumulator buffers of 256 columns; one CTA per SM
 
   if (threadIdx.x == 0) {
@@ -201,8 +209,8 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   // Bias of the CTA's columns (the grid is a multiple of n_blocks).  Read from memory where it is added, between stores to shared
   // memory, it was eight round trips in a row per 32 columns.
   for (int j = threadIdx.x; j < BN_MAX; j += NUM_THREADS) {
-    const int c = (int)(blockIdx.x % n_blocks) * BN_MAX + j;
-    bars->bias[j] = c >= g.N || g.mode == TAURUS_GAT ? 0.f : g.finish ? g.fin.bias[c] : g.bias && c >= g.Hp ? g.bias[c - g.Hp] : 0.f;
+    const int c = (int)(blockIdx.x % n_blocks) * g.bn + j;
+    bars->bias[j] = j >= g.bn || c >= g.N || g.mode == TAURUS_GAT ? 0.f : g.finish ? g.fin.bias[c] : g.bias && c >= g.Hp ? g.bias[c - g.Hp] : 0.f;
   }
   tc_fence_before();
   __syncthreads();
@@ -218,7 +226,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       for (int w = blockIdx.x; w < n_tiles * n_blocks && !*abort_flag; w += gridDim.x) {
         const int tile = w / n_blocks, nb = w % n_blocks;
         const int row0 = tile * BM;
-        const int col0 = nb * BN_MAX;
+        const int col0 = nb * g.bn;
         for (int ks = 0; ks < g.k_stages; ++ks, ++it) {
           const int s = it % n_stages;
           const unsigned ph = (it / n_stages) & 1;
@@ -245,7 +253,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       int it = 0, unit = 0;
       for (int w = blockIdx.x; w < n_tiles * n_blocks && !*abort_flag; w += gridDim.x, ++unit) {
         const int nb = w % n_blocks;
-        const int bw = (g.Np - nb * BN_MAX) < BN_MAX ? (g.Np - nb * BN_MAX) : BN_MAX;
+        const int bw = (g.Np - nb * g.bn) < g.bn ? (g.Np - nb * g.bn) : g.bn;
         const int buf = unit & 1;
         if (unit >= 2 && !mbar_wait(&bars->acc_empty[buf], ((unit >> 1) & 1) ^ 1, abort_flag)) break;
         tc_fence_after();
@@ -356,16 +364,15 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       }
     }
     {
-      const int bw = (g.Np - nb * BN_MAX) < BN_MAX ? (g.Np - nb * BN_MAX) : BN_MAX;
       const int buf = unit & 1;
       if (!mbar_wait(&bars->acc_full[buf], (unit >> 1) & 1, abort_flag)) break;
       tc_fence_after();
-      const int columns = bw < g.N - nb * BN_MAX ? bw : g.N - nb * BN_MAX;   // without the padding of the last block
+      const int columns = g.bn < g.N - nb * g.bn ? g.bn : g.N - nb * g.bn;   // without the padding of the last block
 #pragma unroll 1
       for (int c0 = half * 32; c0 < columns; c0 += 64) {
         unsigned v[32];
         tmem_ld32(v, tmem_base + ((unsigned)(q * 32) << 16) + (unsigned)(buf * BN_MAX + c0));
-        const int cbase = nb * BN_MAX + c0;
+        const int cbase = nb * g.bn + c0;
         float o[32];
         if (cbase + 32 <= g.Hp && !g.finish) {   // P columns: c_out(u) * (x W_neigh)
 #pragma unroll
@@ -390,7 +397,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
         // tile queue up behind the operand loads.)
         __syncwarp();
         const int ch = lane & 7;
-        const bool in = cbase + ch * 4 < g.N;
+        const bool in = c0 + ch * 4 < columns;
 #pragma unroll
         for (int it = 0; it < 8; ++it) {
           const int rr = it * 4 + (lane >> 3);
@@ -505,7 +512,7 @@ int prepare_tc_weights(taurus_ctx* c, void** slot, const std::vector<float>& cat
   w->ks = bf16 ? 64 : stage_columns(K);
   w->Kp = taurus_round_up(K, w->ks);
   const size_t cnt = (size_t)w->Np * w->Kp;
-  const int bw = w->Np < BN_MAX ? w->Np : BN_MAX;
+  const int bw = block_columns(w->Np);
   if (bf16) {
     std::vector<__nv_bfloat16> img(cnt, __float2bfloat16(0.f));
     for (int k = 0; k < K; ++k)
@@ -563,14 +570,15 @@ int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long lo
   if (!make_map(&map_x, X, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, K, ldx, BM, bf16 ? 32 : w->ks)) return TAURUS_ERR_CUDA;
   GemmArgs g;
   g.PT = out; g.ldo = ldo; g.n = n; g.N = N; g.Np = w->Np; g.k_stages = w->Kp / w->ks;
-  g.b_box_bytes = (w->Np < BN_MAX ? w->Np : BN_MAX) * (bf16 ? 128 : w->ks * 4);
+  g.bn = block_columns(w->Np);
+  g.b_box_bytes = g.bn * (bf16 ? 128 : w->ks * 4);
   set_stages(g, bf16, w->ks);
   g.Hp = Hp; g.mode = c->mode; g.fanout = c->fanout[layer]; g.bias = c->d_bias[layer];
   g.row_ptr = c->d_row_ptr; g.din = c->d_din; g.src_begin = src_begin; g.ctl = c->d_ctl;
   g.finish = 0; g.fin = GemmFinish(); g.done_count = nullptr;
   const int smem = shared_bytes(bf16);
   const int n_tiles = (n + BM - 1) / BM;
-  const int n_blocks = (w->Np + BN_MAX - 1) / BN_MAX, n_units = n_tiles * n_blocks;
+  const int n_blocks = (w->Np + g.bn - 1) / g.bn, n_units = n_tiles * n_blocks;
   const int sms = c->sm_count - c->xfer_blocks;   // the SMs of the row transfers have no shared memory left
   const int grid = n_units < sms ? n_units : std::max(1, sms / n_blocks) * n_blocks;   // a CTA keeps to one block of columns
   const int rc = launch_tc(c, grid, smem, st, map_x, w->map_hi, w->map_lo, g, bf16, w->ks);
@@ -598,7 +606,7 @@ int launch_gemm_plain_tc(taurus_ctx* c, void* image, int col0, int N, const floa
   WImage* w = static_cast<WImage*>(image);
   const int rows_left = w->Np - col0;                       // image rows (= output columns) from col0 on
   const int Np = std::min(taurus_round_up(N, 16), rows_left);
-  const int bw = Np < BN_MAX ? Np : BN_MAX;
+  const int bw = block_columns(Np);
   const int elem = bf16 ? 2 : 4;
   CUtensorMap map_x, map_hi, map_lo;
   if (!make_map(&map_x, X, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, n, K, ldx, BM, bf16 ? 32 : w->ks)) return TAURUS_ERR_CUDA;
@@ -613,6 +621,7 @@ int launch_gemm_plain_tc(taurus_ctx* c, void* image, int col0, int N, const floa
   }
   GemmArgs g;
   g.PT = out; g.ldo = ld_out; g.n = n; g.N = N; g.Np = Np; g.k_stages = w->Kp / w->ks;
+  g.bn = bw;
   g.b_box_bytes = bw * (bf16 ? 128 : w->ks * 4);
   set_stages(g, bf16, w->ks);
   g.Hp = N; g.mode = TAURUS_GIN_SUM; g.fanout = 0; g.bias = nullptr;
@@ -621,7 +630,7 @@ int launch_gemm_plain_tc(taurus_ctx* c, void* image, int col0, int N, const floa
   g.done_count = done_count;
   const int smem = shared_bytes(bf16);
   const int n_tiles = (n + BM - 1) / BM;
-  const int n_blocks = (Np + BN_MAX - 1) / BN_MAX, n_units = n_tiles * n_blocks;
+  const int n_blocks = (Np + bw - 1) / bw, n_units = n_tiles * n_blocks;
   const int sms = c->sm_count - c->xfer_blocks;   // the SMs of the row transfers have no shared memory left
   const int grid = n_units < sms ? n_units : std::max(1, sms / n_blocks) * n_blocks;   // a CTA keeps to one block of columns
   const int rc = launch_tc(c, grid, smem, st, map_x, map_hi, map_lo, g, bf16, w->ks);

@@ -1,12 +1,16 @@
 """The projection in fp32 mode (operands split into two TF32 values) at the edges of its tiles and stages: one row to several tiles per
-CTA, K on both sides of the two stage widths and with short last stages, one to four blocks of output columns, columns that fill
-no 32.  Against the product in 64 bits, element by element of the magnitude sum: a value cut after 11 + 11 bits is off by at
+CTA, K on both sides of the two stage widths and with short last stages, one to eight blocks of output columns, columns that fill
+no 32, bias and per-row factors.  Against the product in 64 bits, element by element of the magnitude sum: a value cut after 11 + 11 bits is off by at
 most 2^-20, on either side, the dropped lo.lo by 2^-20, and K additions by 2^-24 each: 2^-18 + K 2^-24 covers them."""
+from dataclasses import replace
+
 import numpy as np
 import pytest
 import torch
 
 import paper_2607_17374_b200 as tb
+import taurus_gen as tg
+from test_gpu_parity import _full_check
 
 pytestmark = pytest.mark.gpu
 
@@ -44,3 +48,43 @@ def test_shapes(V, K, N):
     rng = np.random.default_rng(K * 1000 + N + V)
     x, W = rng.standard_normal((V, K)).astype(np.float32), (rng.standard_normal((K, N)) / K ** 0.5).astype(np.float32)
     _check(x, W, _project(x, W))
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("K,N", [(132, 130), (228, 260), (232, 300), (516, 258), (260, 340), (800, 1024)])   # 2 (264), 3, 3, 3, 3, 8 blocks of columns
+def test_blocks_of_columns(K, N, bf16):
+    """SAGE rows [P | T] of several blocks, enough rows that a CTA takes several tiles; biases and in-degrees that show which columns
+    they went to.  bf16 operands: 2^-9 on either side of a product."""
+    V = 20_003
+    dev, gen = torch.device("cuda:0"), torch.Generator()
+    gen.manual_seed(K + N)
+    din = torch.randint(0, 5, (V,), generator=gen)
+    dst = torch.repeat_interleave(torch.arange(V), din)
+    src = torch.randint(0, V, (dst.numel(),), generator=gen)
+    order = torch.argsort(src, stable=True)
+    row_ptr = torch.zeros(V + 1, dtype=torch.int64)
+    row_ptr[1:] = torch.cumsum(torch.bincount(src, minlength=V), 0)
+    x = torch.randn(V, K, generator=gen)
+    Wn, Ws = (torch.randn(K, N, generator=gen) / K ** 0.5 for _ in range(2))
+    bias = torch.randn(N, generator=gen)
+    ctx = tb.Context(V, dst.numel(), row_ptr.to(dev), dst[order].to(torch.int32).to(dev), din.to(torch.int32).to(dev), tb.SAGE_MEAN, [K, N], [Wn], [Ws], [bias],
+                     [0], V, V, 0, None, 1, 0, V, tb.GEMM_BF16 if bf16 else tb.GEMM_FP32)
+    out = torch.empty(V, N, device=dev)
+    ctx.layer_begin(0)
+    ctx.layer_set_dense_output(out, N)
+    ctx.push_chunk(0, V, x.to(dev))
+    ctx.layer_end()
+
+    def layer(x, Wn, Ws, b):
+        mean = torch.zeros(V, K, dtype=torch.float64, device=dev).index_add_(0, dst.to(dev), x[src.to(dev)]) / din.to(dev).clamp(min=1)[:, None]
+        return mean @ Wn + x @ Ws + b
+    t = [a.to(dev).double() for a in (x, Wn, Ws, bias)]
+    ref, mag = layer(*t), layer(*(a.abs() for a in t))
+    rel = (2.0 ** -8 + 2.0 ** -17 if bf16 else 2.0 ** -18) + (K + 16) * 2.0 ** -24   # K additions of a product, a few of its rows
+    assert bool(((out.double() - ref).abs() <= rel * mag).all()), float(((out.double() - ref).abs() / mag).max())
+
+
+def test_attention_scalars_in_the_second_block():
+    w = tg.scaled(tg.WORKLOADS["mid"], 20_000, chunk=20_000)
+    w = replace(w, E=6 * 20_000, dims=(200, 256), fanout=(0,), pool_slots=20_000, hub_count=0, mode=tg.GAT, gat_heads=4)
+    _full_check(w, tg.make_graph(w), dense_output=True)
