@@ -43,12 +43,15 @@ constexpr int TILE_A_BYTES = BM * 128;           // 128 rows x 128 B
 constexpr int TILE_B_BYTES = BN_MAX * 128;       // 256 rows x 128 B
 // fp32 mode: KS, the K columns per stage, is 32 (128-byte operand rows, 128-byte swizzle) or 16 (64-byte rows and swizzle: stages
 // half as large, twice as many in flight).  Both are exact.  The three TF32 MMAs of a K step read their operands from shared
-// memory without reuse between them (12 KB per 128 x 256 x 8 MMA, one MMA per 134 cycles at the pipe's rate = 92 B per cycle), and
-// the TMA fill and the operand split come on top of the SM's 128 B per cycle: 2 125 cycles of shared memory to 1 536 of
-// the pipe per 32 columns.  K up to 64 takes 32, fewer hand-offs (1 024 rows, K = 64: 6.3 against 6.7 us), wider rows 16, a deeper
-// pipeline (projections of 1.5 M vertices, 128-256-256-256: 5.04 against 5.26 ms a pass; of 2.45 M, 100-256-256-47: 6.65 and 6.95).
-// The epilogue of one warp per quadrant with TMA stores, which waited 2 400 cycles per 32 columns, had hidden that: 6.40 and 8.25.
-constexpr int stage_columns(int K) { return K <= 64 ? 32 : 16; }
+// memory without reuse between them (12 KB per 128 x 256 x 8 MMA, one MMA per 128 cycles at the pipe's rate = 96 B per cycle), and
+// the TMA fill and the operand split come on top of the SM's 128 B per cycle: 2 176 cycles of shared memory to 1 536 of
+// the pipe per 32 columns.  Stages of 32 mean half as many hand-offs and are the better ones while three of them fit (blocks of up
+// to 128 columns); with two, wide rows want the deeper pipeline, and K up to 64 does not fill it.  us a launch of 65 536 rows, 32 / 16:
+//   columns    16           96           128          160          192          256          2 x 192       2 x 256
+//   K = 128    17.2 / 21.2  20.3 / 23.1  22.2 / 24.3  27.2 / 26.6
+//   K = 256    27.5 / 36.3  32.8 / 38.3  35.0 / 39.1  44.7 / 41.9  47.6 / 47.3  54.3 / 52.4
+//   K = 512    47.1 / 65.0  57.1 / 68.1  59.2 / 69.8  79.8 / 73.3  84.1 / 82.5  95.9 / 88.3  134.9 / 140.2  156.2 / 145.6
+constexpr int stage_columns(int K, int block) { return K <= 64 || block <= 128 ? 32 : 16; }
 constexpr unsigned WAIT_LIMIT = 1u << 24;
 constexpr int EPI_WARPS = 8;         // two per quadrant of TMEM lanes, which take turns with the columns
 constexpr int NUM_THREADS = 32 * (6 + EPI_WARPS);
@@ -69,6 +72,7 @@ struct __align__(8) Barriers {
 // narrower runs as many stages as fit (GemmArgs::stages, stage_bytes).
 constexpr int STAGE_BYTES_FP32 = 2 * TILE_A_BYTES + 2 * TILE_B_BYTES;
 constexpr int STAGE_BYTES_BF16 = 3 * TILE_A_BYTES + TILE_B_BYTES;
+static_assert(3 * (2 * TILE_A_BYTES + 2 * 128 * 128) <= STAGES * STAGE_BYTES_FP32, "three stages of 32 columns with blocks of 128 (stage_columns)");
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -509,10 +513,10 @@ int prepare_tc_weights(taurus_ctx* c, void** slot, const std::vector<float>& cat
   WImage* w = new WImage();
   *slot = w;
   w->Np = taurus_round_up(N, 16);
-  w->ks = bf16 ? 64 : stage_columns(K);
+  const int bw = block_columns(w->Np);
+  w->ks = bf16 ? 64 : stage_columns(K, bw);
   w->Kp = taurus_round_up(K, w->ks);
   const size_t cnt = (size_t)w->Np * w->Kp;
-  const int bw = block_columns(w->Np);
   if (bf16) {
     std::vector<__nv_bfloat16> img(cnt, __float2bfloat16(0.f));
     for (int k = 0; k < K; ++k)
