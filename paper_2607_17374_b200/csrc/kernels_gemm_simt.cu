@@ -15,9 +15,10 @@
 #define SIMT_STAGES 3
 
 // A block of 128 threads takes 32 rows x 64 columns, a thread 4 x 4 of them.  Panels of 32 K-columns arrive by cp.async (4 bytes
-// at a time from X, whose rows need no alignment), three in flight: the launches this kernel is for are small, and one panel after
-// the other, loaded and waited for, was 3.9 us each.  Additions are packed in pairs of columns, fma by fma in the order of K.
-// 10 007 rows, 130 -> 48: 35 -> 14.3 us; 700 rows, 47 -> 72: 9.5 -> 4.8 us.
+// at a time from X, whose rows need no alignment), three in flight: one panel after the other, loaded and waited for, was 3.9 us
+// each, most of a small launch.  Additions are packed in pairs of columns, fma by fma in the order of K.  With blocks of 64 x 64, a
+// panel of 16 at a time, and now: 10 007 rows, 130 -> 48: 35 and 14.3 us; 700 rows, 47 -> 72: 9.5 and 4.8 us.  65 536 rows (a layer
+// whose width is no multiple of 4 comes here with its full chunks): 130 -> 264 259 and 193 us, 47 -> 72 50 and 42.
 __global__ void __launch_bounds__(128) project_simt_kernel(const float* __restrict__ X, int ldx, int K, const float* __restrict__ W,
                                                            int ldw, int N, float* __restrict__ PT, long long ldo, int n, int Hp, int mode,
                                                            const float* __restrict__ bias, const long long* __restrict__ row_ptr,

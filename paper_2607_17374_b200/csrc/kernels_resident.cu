@@ -34,12 +34,6 @@ __device__ __forceinline__ void red_v4(float* addr, const float4& v) {
 }
 // Four floats as two packed pairs; each half of a packed operation is rounded like the scalar one.
 struct Pairs { unsigned long long a, b; };
-__device__ __forceinline__ Pairs pairs_of(const float4& v) {
-  Pairs p;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(p.a) : "f"(v.x), "f"(v.y));
-  asm("mov.b64 %0, {%1, %2};" : "=l"(p.b) : "f"(v.z), "f"(v.w));
-  return p;
-}
 __device__ __forceinline__ float4 floats_of(const Pairs& p) {
   float4 v;
   asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(p.a));
@@ -326,7 +320,6 @@ struct HeadTerm { float t, top, scale, self, bw; };   // GAT: destination term a
 // A value that every lane of the warp holds alike, told to the compiler: the reduction's result is a uniform register, and
 // branches on it need no reconvergence code (which was more than half of this kernel's instructions).
 __device__ __forceinline__ int uniform(int x) { return __reduce_max_sync(FULL, x); }
-__device__ __forceinline__ unsigned uniform(unsigned x) { return __reduce_or_sync(FULL, x); }
 
 __device__ __forceinline__ void copy16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
@@ -1034,7 +1027,8 @@ int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitc
   // Rows split over as many lanes as they have float4, steps of about 2 KB per warp.  Measured (ms of all launches of a pass):
   // 48 floats, 2.45 M vertices, 124 M edges: 16 lanes x 1 float4, 4 rows a step, 3 steps 3.9; 8 x 2 4.6 to 5.2.  64 floats, 500 k
   // vertices, 12.5 M edges: 4 rows, 3 steps 0.47; 2 rows, 4 steps 0.50; 8 x 2 0.54.  100 floats (first graph): 32 x 1, 4 rows, 3 steps
-  // 7.5; 16 x 2 7.7.  256 floats: 2 rows, 4 steps 15.8; 4 rows, 3 steps 15.8, slower where in-lists are short.
+  // 7.5; 16 x 2 7.7.  256 floats: 2 rows, 4 steps 15.8; 4 rows, 3 steps 15.8, slower where in-lists are short.  GATConv (a step
+  // less, for the scores), 64 floats, one head: 4 rows, 2 steps 0.66; 2 rows, 3 steps 0.71.
   const int Hp = a.Hp;
   if (Hp <= 16) return launch_g2<4, 1, 2, 4>(c, g, bound, 0, st);
   if (Hp <= 32) return launch_g2<8, 1, 2, 4>(c, g, bound, 1, st);
