@@ -1,7 +1,8 @@
-"""The projection in fp32 mode (operands split into two TF32 values) at the edges of its tiles and stages: one row to several tiles per
-CTA, K on both sides of the two stage widths and with short last stages, one to eight blocks of output columns, columns that fill
-no 32, bias and per-row factors.  Against the product in 64 bits, element by element of the magnitude sum: a value cut after 11 + 11 bits is off by at
-most 2^-20, on either side, the dropped lo.lo by 2^-20, and K additions by 2^-24 each: 2^-18 + K 2^-24 covers them."""
+"""The projection in fp32 mode (operands split into two fp16 values, rows and columns scaled by powers of two) at the edges of its tiles
+and stages: one row to several tiles per CTA, K with short last stages, one to eight blocks of output columns, columns that fill no 32,
+bias and per-row factors; rows and columns of very different magnitudes.  Against the product in 64 bits, element by element of the
+magnitude sum: a value cut after 11 + 11 bits is off by at most 2^-20, on either side, the dropped lo.lo by 2^-20, and K additions by
+2^-24 each: 2^-18 + K 2^-24 covers them."""
 from dataclasses import replace
 
 import numpy as np
@@ -48,6 +49,57 @@ def test_shapes(V, K, N):
     rng = np.random.default_rng(K * 1000 + N + V)
     x, W = rng.standard_normal((V, K)).astype(np.float32), (rng.standard_normal((K, N)) / K ** 0.5).astype(np.float32)
     _check(x, W, _project(x, W))
+
+
+def _rows(kind, V, K, rng):
+    x = rng.standard_normal((V, K))
+    if kind == "grow":        # a power of two of the row that has to give way again and again
+        x *= 10.0 ** np.linspace(-8, 9, K)
+    elif kind == "steps":     # ... at every K step, with empty ones in front
+        x *= 10.0 ** (4 * (np.arange(K) // 32 % 4)) * (np.arange(K) >= 32)
+    elif kind == "late":      # ... in some rows only, in the last column
+        x[:, -1] *= np.where(rng.random(V) < 0.1, 1e6, 1.0)
+    elif kind == "rows":
+        x *= 10.0 ** rng.uniform(-30, 30, V)[:, None]
+    elif kind == "zeros":
+        x *= rng.random((V, K)) < 0.01
+    return x.astype(np.float32)
+
+
+@pytest.mark.parametrize("K,N", [(36, 20), (96, 128), (256, 256), (300, 340)])
+@pytest.mark.parametrize("kind", ["grow", "steps", "late", "rows", "zeros"])
+def test_rows_of_many_magnitudes(kind, K, N):
+    """What a row's power of two leaves of an element is off by at most 2^-33 of the largest one."""
+    V = 40_003
+    rng = np.random.default_rng(K + N)
+    x, W = _rows(kind, V, K, rng), (rng.standard_normal((K, N)) / K ** 0.5).astype(np.float32)
+    got = _project(x, W)
+    x64, W64 = x.astype(np.float64), W.astype(np.float64)
+    ref, mag = x64 @ W64, np.abs(x64) @ np.abs(W64)
+    bound = (2.0 ** -18 + K * 2.0 ** -24) * mag + 2.0 ** -32 * np.abs(x64).max(1)[:, None] * np.abs(W64).sum(0)
+    assert (np.abs(got - ref) <= bound).all(), float((np.abs(got - ref) / np.maximum(bound, 1e-300)).max())
+
+
+@pytest.mark.parametrize("spread", [0, 2, 15])   # 15: the columns of W need powers of two of their own
+def test_columns_of_many_magnitudes(spread):
+    V, K, N = 20_003, 100, 132
+    rng = np.random.default_rng(spread)
+    x = _rows("rows", V, K, rng) if spread < 15 else rng.standard_normal((V, K)).astype(np.float32)
+    W = (rng.standard_normal((K, N)) * 10.0 ** rng.uniform(-spread, spread / 4, N)).astype(np.float32)
+    W[:, 5] = 0
+    _check(x, W, _project(x, W))
+
+
+def test_rows_that_are_not_finite():
+    V, K, N = 5_000, 96, 64
+    rng = np.random.default_rng(1)
+    x, W = rng.standard_normal((V, K)).astype(np.float32), rng.standard_normal((K, N)).astype(np.float32)
+    clean = _project(x, W)
+    x[7, 3], x[800, 90], x[801, 0], x[4_999, 40] = np.inf, -np.inf, np.nan, np.nan
+    got = _project(x, W)
+    bad = np.zeros(V, bool)
+    bad[[7, 800, 801, 4_999]] = True
+    assert np.isnan(got[bad]).all() and (got[~bad] == clean[~bad]).all()
 
 
 @pytest.mark.parametrize("bf16", [False, True])
