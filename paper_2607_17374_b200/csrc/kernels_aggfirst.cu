@@ -140,7 +140,7 @@ __global__ void af_finish_kernel(ChunkArgs a, const float* __restrict__ O, long 
 }  // namespace
 
 void launch_af_prep(taurus_ctx* c, const float* X, int ldx, int n, int K, int Kp, long long src_begin, float* out, cudaStream_t st) {
-  af_prep_kernel<<<c->sm_count * 8, 256, 0, st>>>(X, ldx, n, K, Kp, src_begin, c->mode, c->d_row_ptr, out);
+  af_prep_kernel<<<c->sm_count * 8, 256, c->pipelined ? TAURUS_OFF_XFER : 0, st>>>(X, ldx, n, K, Kp, src_begin, c->mode, c->d_row_ptr, out);
   c->launches += 1;
 }
 

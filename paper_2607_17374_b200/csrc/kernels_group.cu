@@ -276,29 +276,40 @@ void launch_classify_grouped(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st)
 // added to the running group sum or, at a destination change, the sum is flushed with one vector reduction
 // per lane and one integer reduction on the pending count.  The loop body is kept to a few tens of
 // instructions per edge: an earlier version with lane-parallel edge loads and shuffles was issue-bound.
-#define SPAN_EDGES 128   // edges per warp span (all sub-groups together)
+#define SPAN_EDGES 128   // most edges per warp span (all sub-groups together)
 
 // With GAT every message is weighted by exp(LeakyReLU(s_u + t_v) - max_v), recomputed from per-vertex scalars
 // (the 1 / normaliser factor is applied at finalise).
 // GAT: 0 no attention, 1 one head (one weight per message), 2 several heads (each lane weights its float4 columns by the
 // coefficient of the head they belong to; the per-vertex scalars are [V x heads]).
+// One block per SM (80 registers a thread): the blocks of the row transfers, which want an SM each, find theirs empty.  With three blocks of 256
+// they waited for the scatter to end on some SM, half of its time, once every warp of it had work.
+constexpr int sg_threads(int vpl) { return vpl <= 2 ? 768 : vpl == 3 ? 512 : 256; }
 template <int LPE, int VPL, bool SAMPLED, bool DIRECT, int GAT>
-__global__ void __launch_bounds__(256, (VPL <= 2 ? 3 : VPL == 3 ? 2 : 1))
-scatter_grouped_kernel(ChunkArgs a, const int2* __restrict__ g_edge, const uint32_t* __restrict__ gmask) {
+__global__ void __launch_bounds__(sg_threads(VPL), 1) scatter_grouped_kernel(ChunkArgs a, const int2* __restrict__ g_edge, const uint32_t* __restrict__ gmask) {
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
   if (ctl->error) return;
+  __shared__ unsigned int s_total[3];           // groups, messages, messages of hubs
+  if (threadIdx.x < 3) s_total[threadIdx.x] = 0;
+  __syncthreads();
   constexpr int EPS = 32 / LPE;                 // sub-groups per warp
-  constexpr int STRETCH = SPAN_EDGES / EPS;     // edges one sub-group walks per span
   const int lane = lane_id();
   const int sub = lane / LPE;
   const int c4 = lane % LPE;
   const int nvec = a.Hp >> 2;
   const long long e0 = a.row_ptr[a.src_begin], e1 = a.row_ptr[a.src_end];
   const long long n_src = a.src_end - a.src_begin;
-  const long long spans = (e1 - e0 + SPAN_EDGES - 1) / SPAN_EDGES;
-  const long long self_tiles = (n_src + 31) >> 5;
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
+  // Edges one sub-group walks per span, and self messages per tile: no more than give every warp one.  A warp has four edges in
+  // flight, so a chunk of few edges is bound by how many warps walk it: with 128 a warp throughout, 244 k edges (16 384 sources, rows of
+  // 256 floats) kept half of the warps busy, 59 k an eighth.  us a launch, beside row transfers: 121 -> 90 and 118 -> 64.
+  const long long share = (e1 - e0 + warps * EPS - 1) / (warps * EPS);
+  const int stretch = share >= SPAN_EDGES / EPS ? SPAN_EDGES / EPS : share <= 8 ? 8 : (int)(share + 3) & ~3;
+  const long long spans = (e1 - e0 + stretch * EPS - 1) / (stretch * EPS);
+  int tile = 32;
+  while (tile > 8 && n_src < tile * warps) tile >>= 1;
+  const long long self_tiles = (n_src + tile - 1) / tile;
   const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int loc_limit = (int)(a.pool_slots + a.hub_count);
   const int pool = (int)a.pool_slots;
@@ -395,24 +406,21 @@ scatter_grouped_kernel(ChunkArgs a, const int2* __restrict__ g_edge, const uint3
       if (lane_on[k]) row[k] = ld_v4_hint(p + k * LPE * 16, pol_last);
   };
 
-  // Where row transfers of the previous chunk may be running beside this kernel (bounded pool), spans are handed out
-  // from a counter rather than by warp number: warps near the host link's requests get through fewer of them (measured on
-  // "large" with transfer warps on every SM: scatter 105 -> 34 ms per 32-chunk window; 16 ms with the transfers on SMs of
-  // their own).  A span is requested only when the warp is ready for it: a chunk
-  // has about two spans per warp there, and a warp that asked ahead would sit on a span while it is slow.  Elsewhere the
-  // spans are dealt by warp number: same-address atomics cost about 3 ns each, 75 us per launch at the 25 k spans of a
-  // "mid" chunk.
+  // Where row transfers may be running beside this kernel (bounded pool), the spans behind the first of every warp are handed out from
+  // a counter rather than by warp number: warps near the host link's requests get through fewer of them.  A span is requested
+  // only when the warp is ready for it.  Elsewhere the spans are dealt by warp number: same-address atomics cost about 3 ns
+  // each, 75 us per launch at the 25 k spans of a "mid" chunk.
   const bool dyn = a.dynamic_spans != 0;
   for (long long it = 0;; ++it) {
     long long span = warp0 + it * warps;
-    if (dyn) {
+    if (dyn && it > 0 && spans > warps) {
       unsigned int got = 0;
       if (lane == 0) got = atomicAdd(&pc->span_next, 1u);
-      span = (long long)__shfl_sync(FULL, got, 0);
+      span = warps + (long long)__shfl_sync(FULL, got, 0);
     }
     if (span >= spans) break;
-    long long x = e0 + span * SPAN_EDGES + (long long)sub * STRETCH;
-    const long long x_end = (x + STRETCH < e1) ? x + STRETCH : e1;
+    long long x = e0 + (span * EPS + sub) * stretch;
+    const long long x_end = (x + stretch < e1) ? x + stretch : e1;
     const int2* ge = g_edge + x;
     int left = x_end > x ? (int)(x_end - x) : 0;
 #pragma unroll 1
@@ -448,22 +456,22 @@ scatter_grouped_kernel(ChunkArgs a, const int2* __restrict__ g_edge, const uint3
 
   // self messages (one per chunk vertex)
   for (long long it = 0;; ++it) {
-    long long t = warp0 + it * warps;
-    if (dyn) {
+    long long t = warps - 1 - warp0 + it * warps;   // the warps behind the last span first
+    if (dyn && it > 0 && self_tiles > warps) {
       unsigned int got = 0;
       if (lane == 0) got = atomicAdd(&pc->self_next, 1u);
-      t = (long long)__shfl_sync(FULL, got, 0);
+      t = warps + (long long)__shfl_sync(FULL, got, 0);
     }
     if (t >= self_tiles) break;
-    const long long u = a.src_begin + t * 32 + lane;
-    int v = u < a.src_end ? (int)u : -1;
+    const long long u = a.src_begin + t * tile + lane;
+    int v = lane < tile && u < a.src_end ? (int)u : -1;
     int l = -1;
     if (v >= 0) {
       l = a.loc[v];
       if (l < 0 || l >= loc_limit) { bad = 1; l = -1; }
       else atomicAdd(&a.pend[v], -1);
     }
-    for (int step = 0; step < 32; step += EPS) {
+    for (int step = 0; step < tile; step += EPS) {
       const int j = step + sub;
       const int lj = __shfl_sync(FULL, l, j);
       const int vj = __shfl_sync(FULL, v, j);
@@ -513,22 +521,23 @@ scatter_grouped_kernel(ChunkArgs a, const int2* __restrict__ g_edge, const uint3
     bad |= __shfl_xor_sync(FULL, bad, o);
   }
   if (lane == 0) {
-    if (groups) atomicAdd((unsigned long long*)&ctl->scatter_groups, (unsigned long long)groups);
-    if (msgs) atomicAdd((unsigned long long*)&ctl->total_messages, (unsigned long long)msgs);
-    if (hub_msgs) atomicAdd((unsigned long long*)&ctl->hub_messages, (unsigned long long)hub_msgs);
+    if (groups) atomicAdd(&s_total[0], groups);
+    if (msgs) atomicAdd(&s_total[1], msgs);
+    if (hub_msgs) atomicAdd(&s_total[2], hub_msgs);
     if (bad) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
   }
+  __syncthreads();   // counted per block: one address takes an atomic every 3 ns, 32 us of them with three a warp
+  if (threadIdx.x < 3 && s_total[threadIdx.x])
+    atomicAdd((unsigned long long*)(threadIdx.x == 0 ? &ctl->scatter_groups : threadIdx.x == 1 ? &ctl->total_messages : &ctl->hub_messages),
+              (unsigned long long)s_total[threadIdx.x]);
 }
 
 template <int LPE, int VPL, bool SAMPLED, bool DIRECT, int GAT>
 static void launch_sg(taurus_ctx* c, const ChunkArgs& a, const uint32_t* gm, cudaStream_t st) {
-  static int blocks_per_sm = 0;
-  if (blocks_per_sm == 0) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, scatter_grouped_kernel<LPE, VPL, SAMPLED, DIRECT, GAT>, 256, 0) != cudaSuccess ||
-        blocks_per_sm < 1)
-      blocks_per_sm = 1;
-  }
-  scatter_grouped_kernel<LPE, VPL, SAMPLED, DIRECT, GAT><<<c->sm_count * blocks_per_sm, 256, 0, st>>>(a, c->d_gedge, gm);
+  // one block of all the warps that fit on an SM; beside row transfers only on the SMs that those leave free, with shared memory
+  // that keeps it off theirs
+  const int grid = c->pipelined ? c->sm_count - c->xfer_blocks : c->sm_count;
+  scatter_grouped_kernel<LPE, VPL, SAMPLED, DIRECT, GAT><<<grid, sg_threads(VPL), c->pipelined ? TAURUS_OFF_XFER : 0, st>>>(a, c->d_gedge, gm);
 }
 
 template <int LPE, int VPL>

@@ -662,7 +662,7 @@ __global__ void alloc_kernel(ChunkArgs a) {
   per = per < 1 ? 1 : per > 32 ? 32 : per;
   for (long long i0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per; i0 < n; i0 += warps * per) {
     const long long i = i0 + lane_id();
-    int slot = -1, out_hrow = -1;
+    int slot = -1, out_hrow = -1, extra_hrow = -1;
     if (lane_id() < per && i < n) {
       const int v = a.need_list[i];
       int victim = -1;
@@ -674,7 +674,8 @@ __global__ void alloc_kernel(ChunkArgs a) {
         atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
       } else {
         const int in_hrow = a.state[v] == TAURUS_EVICTED ? -2 - a.loc[v] : -1;
-        if (a.xfer_list) a.xfer_list[i] = make_int4(slot, in_hrow, out_hrow, 0);
+        if (i >= deficit) extra_hrow = in_hrow;
+        else if (a.xfer_list) a.xfer_list[i] = make_int4(slot, in_hrow, out_hrow, 0);
         if (out_hrow >= 0) {
           a.loc[victim] = -2 - out_hrow;
           a.state[victim] = TAURUS_EVICTED;
@@ -687,6 +688,13 @@ __global__ void alloc_kernel(ChunkArgs a) {
         if (a.slot_touch) a.slot_touch[slot] = a.epoch;   // slot_pend follows in compact_done: v is on the touched list
         a.state[v] = TAURUS_IN_BUFFER;
       }
+    }
+    const unsigned mx = __ballot_sync(FULL, extra_hrow >= 0);
+    if (mx && a.xfer_list) {
+      int at = 0;
+      if (lane_id() == 0) at = atomicAdd(&pc->xfer_extra, __popc(mx));
+      at = __shfl_sync(FULL, at, 0) + __popc(mx & ((1u << lane_id()) - 1));
+      if (extra_hrow >= 0) a.xfer_list[deficit + at] = make_int4(slot, extra_hrow, -1, 0);
     }
     const int rows = n - i0 < per ? (int)(n - i0) : per;
     for (int j = 0; j < rows; ++j) {
@@ -745,8 +753,10 @@ static __device__ __forceinline__ void xf_load(void* dst, const void* src, unsig
 // The last of these drives the link a little harder, but stretches the scatter beside it from 16 to 43 ms and the victim select
 // from 28 to 111 ms a window.  No better: one buffer per thread, 60 % of them for incoming rows (within 2 % at 8 to 32 blocks);
 // entries taken from a counter instead of dealt (191 ms at 16); fewer rows per block on more SMs (56 on 32: 189, 28 on 64: 190).
+// Only entries with a row to move are listed: a chunk that moves none was 40 to 75 us of walking its need list, beside the scatter.
 // An extent whose last row has come back is listed for the free stack (taken back two chunks later by extent_plan).
 #define XF_SMEM (224 * 1024)
+static_assert(XF_SMEM + 2048 + 2 * TAURUS_BLOCK_SHARED + TAURUS_OFF_XFER > TAURUS_SM_SHARED, "no block that asks for TAURUS_OFF_XFER fits beside one of the transfers");
 #define XF_THREADS 256
 __global__ void __launch_bounds__(XF_THREADS) transfer_kernel(ChunkArgs a, int lanes) {   // lanes: entries in flight per block
   extern __shared__ __align__(128) unsigned char xf_rows[];
@@ -755,7 +765,7 @@ __global__ void __launch_bounds__(XF_THREADS) transfer_kernel(ChunkArgs a, int l
   ChunkCtl* pc = a.pc;
   if (ctl->error) return;
   if ((int)threadIdx.x >= lanes) return;
-  const int n = pc->need_count;
+  const int n = pc->deficit + pc->xfer_extra;
   const unsigned bytes = (unsigned)a.Hp * 4u;
   unsigned char* in = xf_rows + (size_t)threadIdx.x * 2 * bytes;
   unsigned char* out = in + bytes;
@@ -765,9 +775,13 @@ __global__ void __launch_bounds__(XF_THREADS) transfer_kernel(ChunkArgs a, int l
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   const int par = a.epoch & 1;
   unsigned phase = 0;
-  for (long long i = (long long)threadIdx.x * gridDim.x + blockIdx.x; i < n; i += (long long)lanes * gridDim.x) {
-    const int4 x = a.xfer_list[i];   // (slot, host row coming back or -1, host row to fill or -1)
-    if (x.y < 0 && x.z < 0) continue;
+  const int step = lanes * (int)gridDim.x;
+  int4 next = make_int4(0, -1, -1, 0);
+  int i = (int)(threadIdx.x * gridDim.x + blockIdx.x);
+  if (i < n) next = a.xfer_list[i];
+  for (; i < n; i += step) {
+    const int4 x = next;   // (slot, host row coming back or -1, host row to fill or -1)
+    if (i + step < n) next = a.xfer_list[i + step];
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the stores of the last entry have read the buffers
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
                  ::"r"(xf_smem(bar)), "r"((x.y >= 0 ? bytes : 0u) + (x.z >= 0 ? bytes : 0u)) : "memory");
@@ -1030,7 +1044,7 @@ __global__ void commit_kernel(ChunkArgs a, int with_counts) {
   else if (a.dense_half >= 0) ctl->out_count[a.dense_half] = pc->done_count;
   else ctl->grad_count += pc->done_count;
   pc->hs = pc->ns = pc->ev = pc->gs = 0;
-  pc->need_count = 0; pc->done_count = 0; pc->touched_count = 0; pc->deficit = 0; pc->victim_count = 0; pc->reloaded = 0;
+  pc->need_count = 0; pc->done_count = 0; pc->touched_count = 0; pc->deficit = 0; pc->victim_count = 0; pc->reloaded = 0; pc->xfer_extra = 0;
   pc->span_next = 0; pc->self_next = 0;
   pc->grid_arrivals = 0; pc->done_blocks = 0; pc->room_go = 0; pc->room_fail = 0;
 }
@@ -1040,7 +1054,7 @@ void launch_compact_done(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, boo
   // a warp takes 32 * CD_ITEMS entries per round: no more blocks than the longest list of any chunk can feed
   const long long need = (a.touched_capacity + 8 * 32 * CD_ITEMS - 1) / (8 * 32 * CD_ITEMS);
   const int blocks = (int)(need < 1 ? 1 : need < c->sm_count * 8 ? need : c->sm_count * 8);
-  compact_done_kernel<<<blocks, 256, 0, st>>>(a, write_record ? 1 : 0);
+  compact_done_kernel<<<blocks, 256, c->pipelined ? TAURUS_OFF_XFER : 0, st>>>(a, write_record ? 1 : 0);
   c->launches += 1;
 }
 void launch_commit(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {

@@ -25,6 +25,7 @@
 #define TAURUS_ACCOUNT_THREADS 256
 #define TAURUS_ACCOUNT_REGISTERS 48
 #define TAURUS_ACCOUNT_SHARED 128
+#define TAURUS_OFF_XFER 1024                     // dynamic shared memory of a block that is to stay off the SMs of the row transfers
 #define TAURUS_SEL_BITS 11                      // radix-select digit width
 #define TAURUS_SEL_BINS (1 << TAURUS_SEL_BITS)
 #define TAURUS_SEL_LEVELS 6                     // 6 x 11 = 66 bits >= the 62-bit (score, id) key
@@ -45,6 +46,7 @@ struct ChunkCtl {
   unsigned int grid_arrivals; // make-room step: blocks that reached its barriers so far
   unsigned int done_blocks;   // completion list: blocks that have finished
   int32_t room_go, room_fail; // make-room step: the plan went through / the host store could not take the victims
+  int32_t xfer_extra;     // reloads into slots from the free stack (entries of the transfer list behind those of the victims)
   int32_t heavy_count;    // resident pools: segments of long in-lists to sum
   long long grad_base;    // resident pools: first row of the chunk's finished rows in the graduation buffer
   unsigned long long acc[8];  // resident pools: sums over the blocks of the account kernel
@@ -122,7 +124,8 @@ struct ChunkArgs {
   int32_t* new_ext;         // [victim_capacity >> ext_shift + buckets] this chunk: extents taken from the stack
   int2* vic_place;          // [victim_capacity] this chunk: (bucket, rank among the chunk's victims of that bucket)
   int32_t* ext_ret[2];      // [n_ext] each: extents emptied by the transfers of the chunks of each parity
-  // Row transfers of the chunk: entry i = (slot, host row to add into it or -1, host row that takes stage_out[i] or -1)
+  // Row transfers of the chunk: entry i = (slot, host row to add into it or -1, host row that takes stage_out[i] or -1); the entries of the
+  // victims first, then the other reloads
   int4* xfer_list;          // [need capacity]
   float* stage_out;         // [victim_capacity x Hp] victims' rows on their way to the host store
   const long long* csc_ptr; // [V + 1] in-lists (ascending source id): offsets,
