@@ -459,14 +459,15 @@ extern "C" int taurus_graph_init(taurus_ctx** out, const taurus_graph* g, const 
 }
 
 // Reads the device control block up to the chunks' own counters, once everything on `st` and the output stream is through,
-// and returns its sticky error.  One copy into pinned memory and one wait: the calls that block (drains, layer_end, stats)
+// and returns its sticky error.  One launch that writes it to pinned memory and one wait: the calls that block (drains, layer_end, stats)
 // are paid per chunk or per layer.  with_stats: the reload histogram comes along.
 static int finish_chunk(taurus_ctx* c, cudaStream_t st);
 static int sticky_error(const taurus_ctx* c) { return c->half_applied ? c->half_applied : c->h_ctl->error; }
 static int read_ctl(taurus_ctx* c, cudaStream_t st, bool with_stats = false) {
   { int rc = finish_chunk(c, st); if (rc) return rc; }   // the last chunk's finalise may still be waiting for a successor
   if (with_stats) launch_reload_histogram(c, st);
-  CU(cudaMemcpyAsync(c->h_ctl, c->d_ctl, offsetof(DevCtl, pc), cudaMemcpyDeviceToHost, st));
+  launch_report(c, st);
+  CU(cudaGetLastError());
   CU(cudaStreamSynchronize(st));
   CU(cudaStreamSynchronize(c->out_stream));
   return sticky_error(c);
@@ -476,11 +477,17 @@ extern "C" int taurus_layer_begin(taurus_ctx* c, int32_t layer, void* cuda_strea
   if (!c || layer < 0 || layer >= c->L) return TAURUS_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   CU(cudaSetDevice(c->device));
-  if (c->last_stream != st) CU(cudaStreamSynchronize(c->last_stream));
-  CU(cudaStreamSynchronize(c->copy_stream));
-  CU(cudaStreamSynchronize(c->out_stream));
-  if (c->xfer_stream) CU(cudaStreamSynchronize(c->xfer_stream));
-  if (c->account_stream) CU(cudaStreamSynchronize(c->account_stream));   // (a push that failed half way leaves it unjoined)
+  // Everything before the layer is over when this call returns; its own kernels are only enqueued.  A layer that ended has left
+  // nothing behind on the library's streams.
+  CU(cudaStreamSynchronize(st));
+  if (!c->quiet) {
+    if (c->last_stream != st) CU(cudaStreamSynchronize(c->last_stream));
+    CU(cudaStreamSynchronize(c->copy_stream));
+    CU(cudaStreamSynchronize(c->out_stream));
+    if (c->xfer_stream) CU(cudaStreamSynchronize(c->xfer_stream));
+    if (c->account_stream) CU(cudaStreamSynchronize(c->account_stream));   // (a push that failed half way leaves it unjoined)
+  }
+  c->quiet = false;
   c->pending = false;   // an abandoned layer's last chunk is dropped with it
   c->layer = layer;
   c->dense_out = nullptr; c->dense_ld = 0;
@@ -488,7 +495,7 @@ extern "C" int taurus_layer_begin(taurus_ctx* c, int32_t layer, void* cuda_strea
   c->gat_next_src = 0; c->gat_ready = false;
   c->half_used[0] = c->half_used[1] = false;
   c->x_used[0] = c->x_used[1] = false;
-  memset(c->h_ctl, 0, sizeof(DevCtl));
+  memset((void*)c->h_ctl, 0, offsetof(DevCtl, pc));   // (the rest is never read here)
   c->half_applied = TAURUS_OK;
   c->next_src = 0; c->chunk_seq = 0; c->ub_since_drain = 0; c->last_stream = st;
   launch_layer_reset(c, layer, st);
@@ -512,7 +519,6 @@ extern "C" int taurus_layer_begin(taurus_ctx* c, int32_t layer, void* cuda_strea
   }
   c->rank_cum = &c->rank_cum_cache[(size_t)layer];
   CU(cudaGetLastError());
-  CU(cudaStreamSynchronize(st));
   return TAURUS_OK;
 }
 
@@ -966,8 +972,8 @@ static int drain_common(taurus_ctx* c, long long capacity, long long* out_count,
   return TAURUS_OK;
 }
 
-static int drain_reset(taurus_ctx* c, bool emptied = false) {
-  if (!emptied) CU(cudaMemsetAsync(reinterpret_cast<char*>(c->d_ctl) + offsetof(DevCtl, grad_count), 0, sizeof(long long), c->last_stream));
+static int drain_reset(taurus_ctx* c) {
+  CU(cudaMemsetAsync(reinterpret_cast<char*>(c->d_ctl) + offsetof(DevCtl, grad_count), 0, sizeof(long long), c->last_stream));
   CU(cudaStreamSynchronize(c->last_stream));
   c->ub_since_drain = 0;
   return TAURUS_OK;
@@ -999,6 +1005,22 @@ extern "C" int taurus_drain_dense(taurus_ctx* c, float* dense_rows, int64_t ld, 
   if (kind == PK_HOST_PINNED) {
     if (!cuda_ok(cudaHostGetDevicePointer((void**)&dense_dev, dense_rows, 0), "cudaHostGetDevicePointer")) return TAURUS_ERR_INVALID_ARG;
   }
+  if (!out_ids && out_count && capacity_rows >= 0 && c->layer >= 0 && !c->half_applied) {   // no ids to copy: nothing of it needs the count on the host first
+    *out_count = 0;
+    CU(cudaSetDevice(c->device));
+    cudaStream_t st = c->last_stream;
+    { int rc = finish_chunk(c, st); if (rc) return rc; }
+    const int d_out = c->dims[c->layer + 1];
+    launch_drain_rows(c, dense_dev, ld, d_out, taurus_round_up(d_out, 4), c->ub_since_drain, capacity_rows, st);
+    CU(cudaGetLastError());
+    CU(cudaStreamSynchronize(st));
+    CU(cudaStreamSynchronize(c->out_stream));
+    if (sticky_error(c)) return sticky_error(c);
+    *out_count = c->h_ctl->grad_count;
+    if (*out_count > capacity_rows) return TAURUS_ERR_INVALID_ARG;
+    c->ub_since_drain = 0;
+    return TAURUS_OK;
+  }
   long long count = 0, oc = 0;
   int rc = drain_common(c, capacity_rows, &oc, &count);
   if (out_count) *out_count = oc;
@@ -1006,11 +1028,11 @@ extern "C" int taurus_drain_dense(taurus_ctx* c, float* dense_rows, int64_t ld, 
   if (count > 0) {
     const int d_out = c->dims[c->layer + 1], Hp = taurus_round_up(d_out, 4);
     cudaStream_t st = c->last_stream;
-    launch_place_rows(c, dense_dev, ld, d_out, Hp, count, out_ids == nullptr, st);
-    if (out_ids) CU(cudaMemcpyAsync(out_ids, c->d_grad_ids, (size_t)count * sizeof(long long), cudaMemcpyDefault, st));
+    launch_place_rows(c, dense_dev, ld, d_out, Hp, count, st);
+    CU(cudaMemcpyAsync(out_ids, c->d_grad_ids, (size_t)count * sizeof(long long), cudaMemcpyDefault, st));
     CU(cudaGetLastError());
   }
-  return drain_reset(c, count == 0 || out_ids == nullptr);
+  return drain_reset(c);
 }
 
 extern "C" int taurus_layer_set_dense_output(taurus_ctx* c, float* dense_rows, int64_t ld) {
@@ -1066,6 +1088,7 @@ extern "C" int taurus_layer_end(taurus_ctx* c, taurus_stats* stats) {
   if (err) return err;
   if (stats) { int rc = fill_stats(c, stats); if (rc) return rc; }
   if (c->next_src != c->V || c->h_ctl->completed != c->V || c->h_ctl->free_top != c->pool_slots) return TAURUS_ERR_ORDER;
+  c->quiet = true;   // every stream of the layer has been joined into the one just waited for
   return TAURUS_OK;
 }
 

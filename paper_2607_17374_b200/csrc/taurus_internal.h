@@ -64,6 +64,8 @@ struct ChunkCtl {
 struct DevCtl {
   int32_t error;            // sticky TAURUS_ERR_* found on the device
   int32_t heavy_rows;       // resident pools: partial rows of long in-lists handed out in this layer
+  unsigned int drain_blocks;   // drain into a matrix: blocks that have finished
+  int32_t unused;
   int32_t ext_ret_count[2]; // extents emptied by the row transfers of the chunks of each parity, waiting to go back on the free stack
   long long free_top;       // entries on the free-slot stack
   long long ext_free_top;   // entries on the free-extent stack of the host store
@@ -325,6 +327,7 @@ struct taurus_ctx {
   long long log_capacity = 0;
   // host bookkeeping
   int layer = -1;
+  bool quiet = false;                // nothing has been enqueued since a blocking call of the layer ended
   int half_applied = 0;              // code of a push that failed with its chunk enqueued in part; cleared by taurus_layer_begin
   long long next_src = 0;
   long long chunk_seq = 0;
@@ -360,7 +363,9 @@ int launch_transfer(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);    // s
 void launch_finalise(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);    // finalise + commit (after launch_compact_done)
 void launch_compact_done(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, bool write_record);   // completions listed (and the chunk record written)
 void launch_commit(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);
-void launch_place_rows(taurus_ctx* c, float* dense, long long ld, int d_out, int Hp, long long count, bool empty, cudaStream_t st);   // empty: no row waits any more
+void launch_place_rows(taurus_ctx* c, float* dense, long long ld, int d_out, int Hp, long long count, cudaStream_t st);
+void launch_drain_rows(taurus_ctx* c, float* dense, long long ld, int d_out, int Hp, long long bound, long long capacity, cudaStream_t st);   // at most `bound` rows wait; reports to h_ctl
+void launch_report(taurus_ctx* c, cudaStream_t st);                         // the control block up to the chunks' counters to h_ctl
 void launch_place_half(taurus_ctx* c, int half, int d_out, int Hp, cudaStream_t st);   // dense-output mode
 void launch_reload_histogram(taurus_ctx* c, cudaStream_t st);               // fills ctl->reload_hist
 void launch_completion_ranks(taurus_ctx* c, cudaStream_t st);                // fills d_rank_hist

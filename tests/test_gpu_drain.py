@@ -59,3 +59,31 @@ def test_drains_without_ids(mode, pool, step):
         assert got == counts
         assert [p.size for p in placed] == [n for n, has in zip(counts, with_ids) if has]
         assert row_error(out, want)[0] <= 1e-4
+
+
+@pytest.mark.parametrize("pinned", [False, True])
+def test_a_drain_that_does_not_fit_takes_nothing(pinned):
+    """Capacity below the rows that wait: refused, whole, and the next drain has them all.  Many blocks and one."""
+    import torch
+    import paper_2607_17374_b200 as tb
+    for V, chunk in ((30_000, 8_192), (40, 40)):
+        w = tg.scaled(tg.WORKLOADS["large"], V, chunk=chunk)
+        w = replace(w, dims=(40, 37), fanout=(0,), hub_count=1, mode=tg.GIN_SUM, pool_slots=V)
+        g, model = tg.make_graph(w), tg.make_model(w, bias_scale=0.3)
+        x0 = tg.features(w.seed, 0, 0, V, w.dims[0])
+        feat = torch.from_numpy(x0).cuda()
+        ctx = tb.Context(V, g.E, g.row_ptr, g.col_idx, g.in_degree, w.mode, w.dims, model.W_neigh, model.W_self, model.bias, model.act, w.chunk,
+                         w.pool_slots, w.hub_count, w.fanout, w.seed, 0, V, w.gemm_mode, 0, 0, w.gin_eps)
+        dense = torch.zeros((V, 37), pin_memory=True) if pinned else torch.zeros((V, 37), device="cuda")
+        total = 0
+        ctx.layer_begin(0)
+        for s in range(0, V, chunk):
+            ctx.push_chunk(s, min(s + chunk, V), feat[s:s + chunk])
+            before = dense.clone()
+            if s + chunk >= V:
+                with pytest.raises(tb.TaurusError):
+                    ctx.drain_dense(dense, 37, V - total - 1)
+                assert torch.equal(dense, before)
+            total += ctx.drain_dense(dense, 37, V - total)
+        assert total == V and ctx.layer_end()["completed"] == V
+        assert row_error(dense.cpu().numpy(), run_oracle(w, g, model, x0)["outs"][0])[0] <= 1e-4
