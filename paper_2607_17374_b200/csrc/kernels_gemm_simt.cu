@@ -7,6 +7,7 @@
 //   T_u = (x_u W_self + b) * max(|M(u)|, 1)     (SAGE)    self message, pre-multiplied by 1 / c_in(u) so
 //                                                          that finalise is one multiply by c_in
 //   (GCN has no T columns: its self message P_u + b / c_in(u) is formed by the scatter kernel.)
+#include "account.cuh"
 #include "taurus_internal.h"
 
 #define BM 32
@@ -19,14 +20,19 @@
 // each, most of a small launch.  Additions are packed in pairs of columns, fma by fma in the order of K.  With blocks of 64 x 64, a
 // panel of 16 at a time, and now: 10 007 rows, 130 -> 48: 35 and 14.3 us; 700 rows, 47 -> 72: 9.5 and 4.8 us.  65 536 rows (a layer
 // whose width is no multiple of 4 comes here with its full chunks): 130 -> 264 259 and 193 us, 47 -> 72 50 and 42.
+// ACCOUNT: the first blocks do the accounting of the push.  A block's tile is one of `across` side by side.
+template <bool ACCOUNT>
 __global__ void __launch_bounds__(128) project_simt_kernel(const float* __restrict__ X, int ldx, int K, const float* __restrict__ W,
                                                            int ldw, int N, float* __restrict__ PT, long long ldo, int n, int Hp, int mode,
                                                            const float* __restrict__ bias, const long long* __restrict__ row_ptr,
-                                                           const int32_t* __restrict__ din, int fanout, long long src_begin) {
+                                                           const int32_t* __restrict__ din, int fanout, long long src_begin, int across,
+                                                           const __grid_constant__ AccountArgs<ACCOUNT> account) {
   __shared__ __align__(16) float sA[SIMT_STAGES][BM][BK + 4];   // [row][k]
+  if (account_here<128>(account, *reinterpret_cast<AccountShared*>(sA))) return;
+  const int tile = (int)blockIdx.x - account.blocks();
   __shared__ __align__(16) float sB[SIMT_STAGES][BK][BN];
   const int t = threadIdx.x, tx = t % 16, ty = t / 16;
-  const int row0 = blockIdx.x * BM, col0 = blockIdx.y * BN;
+  const int row0 = tile / across * BM, col0 = tile % across * BN;
   auto load = [&](int s, int k0) {   // zero behind the ends
     if (k0 < K) {
 #pragma unroll
@@ -107,12 +113,18 @@ __global__ void __launch_bounds__(128) project_simt_kernel(const float* __restri
   }
 }
 
-void launch_project_simt(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, int ldo, cudaStream_t st) {
+void launch_project_simt(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, int ldo, cudaStream_t st,
+                         const AccountWork* acc) {
   const int Hp = taurus_round_up(c->dims[layer + 1], 4);
   const int N = taurus_proj_width(c->mode, Hp, c->heads);
-  dim3 grid((n + BM - 1) / BM, (N + BN - 1) / BN);
-  project_simt_kernel<<<grid, 128, 0, st>>>(X, ldx, c->dims[layer], c->d_Wcat[layer], N, N, out, ldo, n, Hp, c->mode,
-                                            c->d_bias[layer], c->d_row_ptr, c->d_din, c->fanout[layer], src_begin);
+  const int across = (N + BN - 1) / BN, tiles = (n + BM - 1) / BM * across;
+  if (acc)
+    launch_early(acc->early, project_simt_kernel<true>, tiles + acc->blocks, 128, 0, st, X, ldx, c->dims[layer], (const float*)c->d_Wcat[layer], N, N, out, (long long)ldo, n, Hp,
+                 c->mode, (const float*)c->d_bias[layer], (const long long*)c->d_row_ptr, (const int32_t*)c->d_din, c->fanout[layer], src_begin, across,
+                 AccountArgs<true>{*acc});
+  else
+    project_simt_kernel<false><<<tiles, 128, 0, st>>>(X, ldx, c->dims[layer], c->d_Wcat[layer], N, N, out, ldo, n, Hp, c->mode, c->d_bias[layer], c->d_row_ptr,
+                                                      c->d_din, c->fanout[layer], src_begin, across, AccountArgs<false>());
   c->launches += 1;
 }
 
@@ -120,7 +132,8 @@ void launch_project_simt(taurus_ctx* c, int layer, const float* X, int ldx, long
 void launch_gemm_plain_simt(taurus_ctx* c, const float* W, int ldw, int N, const float* X, int ldx, int K, int n, float* out,
                             long long ld_out, cudaStream_t st) {
   if (n <= 0) return;
-  dim3 grid((n + BM - 1) / BM, (N + BN - 1) / BN);
-  project_simt_kernel<<<grid, 128, 0, st>>>(X, ldx, K, W, ldw, N, out, ld_out, n, N, TAURUS_GIN_SUM, nullptr, c->d_row_ptr, c->d_din, 0, 0);
+  const int across = (N + BN - 1) / BN;
+  project_simt_kernel<false><<<(n + BM - 1) / BM * across, 128, 0, st>>>(X, ldx, K, W, ldw, N, out, ld_out, n, N, TAURUS_GIN_SUM, nullptr, c->d_row_ptr, c->d_din,
+                                                                         0, 0, across, AccountArgs<false>());
   c->launches += 1;
 }

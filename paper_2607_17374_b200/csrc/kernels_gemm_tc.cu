@@ -44,6 +44,7 @@
 #include <cmath>
 #include <vector>
 
+#include "account.cuh"
 #include "stage_waits.h"
 #include "taurus_internal.h"
 
@@ -217,14 +218,18 @@ static_assert(3 * (2 * TILE_A_BYTES + TILE_B_BYTES) <= OPERAND_BYTES, "three sta
 static_assert(taurus_quarter_registers(NUM_THREADS, PROJECT_REGISTERS) + taurus_quarter_registers(TAURUS_ACCOUNT_THREADS, TAURUS_ACCOUNT_REGISTERS) <=
               TAURUS_QUARTER_REGISTERS, "registers for a block of the accounting");
 
-template <bool BF16>
+// ACCOUNT: the first CTAs do the accounting of the push.
+template <bool BF16, bool ACCOUNT>
 __global__ void __maxnreg__(PROJECT_REGISTERS)
-project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_b, const __grid_constant__ GemmArgs g) {
+project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_b, const __grid_constant__ GemmArgs g,
+                  const __grid_constant__ AccountArgs<ACCOUNT> account) {
   extern __shared__ __align__(1024) unsigned char smem[];   // (the swizzled operand tiles want 1 024)
   if ((smem_u32(smem) & 1023u) != 0) {
     if (threadIdx.x == 0) atomicCAS(&g.ctl->error, 0, TAURUS_ERR_INTERNAL);
     return;
   }
+  if (account_here<TAURUS_ACCOUNT_THREADS>(account, *reinterpret_cast<AccountShared*>(smem))) return;
+  const int cta = (int)blockIdx.x - account.blocks(), ctas = (int)gridDim.x - account.blocks();
   constexpr int X_BYTES = BF16 ? 2 * TILE_A_BYTES : TILE_A_BYTES;
   const int x_stages = g.x_stages, w_stages = g.w_stages;
   unsigned char* out_staging = smem + OPERAND_BYTES;
@@ -251,7 +256,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
   // Bias of the CTA's columns (the grid is a multiple of n_blocks).  Read from memory where it is added, between stores to shared
   // memory, it was eight round trips in a row per 32 columns.
   for (int j = threadIdx.x; j < BN_MAX; j += NUM_THREADS) {
-    const int c = (int)(blockIdx.x % n_blocks) * g.bn + j;
+    const int c = cta % n_blocks * g.bn + j;
     bars->bias[j] = j >= g.bn || c >= g.N || g.mode == TAURUS_GAT ? 0.f : g.finish ? g.fin.bias[c] : g.bias && c >= g.Hp ? g.bias[c - g.Hp] : 0.f;
     if (!BF16 && g.col_exp) bars->col_exp[j] = j >= g.bn || c >= g.N ? 127 : g.col_exp[c];
   }
@@ -270,7 +275,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
       const int stages = x ? x_stages : w_stages;
       int it = 0;
       Ring ring;
-      for (int w = blockIdx.x; w < n_tiles * n_blocks && !*abort_flag; w += gridDim.x) {
+      for (int w = cta; w < n_tiles * n_blocks && !*abort_flag; w += ctas) {
         const int row0 = w / n_blocks * BM, col0 = w % n_blocks * g.bn;
         for (int ks = 0; ks < g.k_stages; ++ks, ++it, ring.next(stages)) {
           const int s = ring.s;
@@ -294,7 +299,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     if (lane == 0) {
       int it = 0, unit = 0;
       Ring ring, wring;
-      for (int w = blockIdx.x; w < n_tiles * n_blocks && !*abort_flag; w += gridDim.x, ++unit) {
+      for (int w = cta; w < n_tiles * n_blocks && !*abort_flag; w += ctas, ++unit) {
         const int nb = w % n_blocks;
         const int bw = (g.Np - nb * g.bn) < g.bn ? (g.Np - nb * g.bn) : g.bn;
         const int buf = unit & 1;
@@ -332,7 +337,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     const int q = warp & 3, row = q * 32 + lane, swz = row & 7;   // the row is one of the TMEM lanes the warp can reach
     int unit = 0;
     Ring ring;
-    for (int w = blockIdx.x; w < n_tiles * n_blocks; w += gridDim.x, ++unit) {   // (an abort ends it in a wait, for the warp as one)
+    for (int w = cta; w < n_tiles * n_blocks; w += ctas, ++unit) {   // (an abort ends it in a wait, for the warp as one)
       bool ok = true;
       int field = 0;   // fp32 mode: exponent field of the row's power of two; 0: nothing but zeros so far
       for (int ks = 0; ks < g.k_stages; ++ks, ring.next(x_stages)) {
@@ -410,7 +415,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_consta
     // this warp's staging tile: 32 rows (lane = row) x 32 columns, 16-byte chunk c of row r at chunk c ^ (r & 7)
     unsigned char* const tile_smem = out_staging + (warp - EPI_FIRST) * OUT_TILE_BYTES;
     int unit = 0;
-    for (int w = blockIdx.x; w < n_tiles * n_blocks; w += gridDim.x, ++unit) {   // (an abort ends it in the wait, for the warp as one)
+    for (int w = cta; w < n_tiles * n_blocks; w += ctas, ++unit) {   // (an abort ends it in the wait, for the warp as one)
     const int tile = w / n_blocks, nb = w % n_blocks;
     const int r = tile * BM + q * 32 + lane;
     float c_out = 1.f, self_mul = 1.f;
@@ -559,16 +564,27 @@ void set_stages(GemmArgs& g, bool bf16) {
   g.x_stages = std::min((OPERAND_BYTES - g.w_stages * g.b_box_bytes) / x_bytes, MAX_X);
 }
 
-int launch_tc(taurus_ctx* c, int grid, cudaStream_t st, const CUtensorMap& map_x, const CUtensorMap& map_b, const GemmArgs& g, bool bf16) {
-  if (!c->tc_smem_set) {   // once per context (the attribute belongs to the context's device)
-    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    const cudaError_t e = bf16 ? cudaFuncSetAttribute(project_tc_kernel<true>, at, SHARED_BYTES) : cudaFuncSetAttribute(project_tc_kernel<false>, at, SHARED_BYTES);
-    if (e != cudaSuccess) { cudaGetLastError(); return TAURUS_ERR_CUDA; }
-    c->tc_smem_set = true;
+template <bool BF16, bool ACCOUNT>
+int launch_tc2(taurus_ctx* c, int grid, cudaStream_t st, const CUtensorMap& map_x, const CUtensorMap& map_b, const GemmArgs& g, const AccountArgs<ACCOUNT>& acc, bool early) {
+  bool& set = c->tc_smem_set[ACCOUNT ? 1 : 0];   // once per context (the attribute belongs to the context's device)
+  if (!set) {
+    if (cudaFuncSetAttribute(project_tc_kernel<BF16, ACCOUNT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SHARED_BYTES) != cudaSuccess) {
+      cudaGetLastError();
+      return TAURUS_ERR_CUDA;
+    }
+    set = true;
   }
-  if (bf16) project_tc_kernel<true><<<grid, NUM_THREADS, SHARED_BYTES, st>>>(map_x, map_b, g);
-  else project_tc_kernel<false><<<grid, NUM_THREADS, SHARED_BYTES, st>>>(map_x, map_b, g);
+  launch_early(early, project_tc_kernel<BF16, ACCOUNT>, grid, NUM_THREADS, SHARED_BYTES, st, map_x, map_b, g, acc);
   return TAURUS_OK;
+}
+int launch_tc(taurus_ctx* c, int grid, cudaStream_t st, const CUtensorMap& map_x, const CUtensorMap& map_b, const GemmArgs& g, bool bf16,
+              const AccountWork* acc = nullptr) {
+  if (acc) {
+    const AccountArgs<true> with{*acc};
+    return bf16 ? launch_tc2<true, true>(c, grid + acc->blocks, st, map_x, map_b, g, with, acc->early) : launch_tc2<false, true>(c, grid + acc->blocks, st, map_x, map_b, g, with, acc->early);
+  }
+  const AccountArgs<false> without;
+  return bf16 ? launch_tc2<true, false>(c, grid, st, map_x, map_b, g, without, false) : launch_tc2<false, false>(c, grid, st, map_x, map_b, g, without, false);
 }
 
 // Per-layer tensor-core images of Wcat, K-major: a row per output column.
@@ -660,7 +676,13 @@ bool project_tc_usable(const taurus_ctx* c, int layer, const float* X, int ldx) 
   return true;
 }
 
-int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, int ldo, cudaStream_t st) {
+int project_tc_units(const taurus_ctx* c, int layer, int n) {
+  const int Np = static_cast<const WImage*>(c->tc_image[layer])->Np, bn = block_columns(Np);
+  return (n + BM - 1) / BM * ((Np + bn - 1) / bn);
+}
+
+int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, int ldo, cudaStream_t st,
+                      const AccountWork* acc) {
   const bool bf16 = c->gemm_mode == TAURUS_GEMM_BF16;
   WImage* w = static_cast<WImage*>(c->tc_image[layer]);
   const int K = c->dims[layer], Hp = taurus_round_up(c->dims[layer + 1], 4);
@@ -680,7 +702,7 @@ int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long lo
   const int n_blocks = (w->Np + g.bn - 1) / g.bn, n_units = n_tiles * n_blocks;
   const int sms = c->sm_count - c->xfer_blocks;   // the SMs of the row transfers have no shared memory left
   const int grid = n_units < sms ? n_units : std::max(1, sms / n_blocks) * n_blocks;   // a CTA keeps to one block of columns
-  const int rc = launch_tc(c, grid, st, map_x, w->map, g, bf16);
+  const int rc = launch_tc(c, grid, st, map_x, w->map, g, bf16, acc);
   if (rc) return rc;
   c->launches += 1;
   return TAURUS_OK;

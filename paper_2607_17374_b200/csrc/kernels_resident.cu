@@ -19,15 +19,14 @@
 #include <type_traits>
 #include <vector>
 
+#include "account.cuh"
 #include "taurus_internal.h"
 
-#define FULL 0xffffffffu
 #define HEAVY_DEGREE TAURUS_HEAVY_DEGREE
 #define HEAVY_SEGMENT TAURUS_HEAVY_SEGMENT
 
 namespace {
 
-__device__ __forceinline__ int rl() { return threadIdx.x & 31; }
 __device__ __forceinline__ float r_lrelu(float x, float slope) { return x > 0.f ? x : slope * x; }
 __device__ __forceinline__ void red_v4(float* addr, const float4& v) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
@@ -71,214 +70,19 @@ __global__ void resident_reset_kernel(long long V, const int32_t* din, int fanou
 }
 
 // ------------------------------------------------------------------------------------------------ account
-// Items of a grid chunk: every vertex the chunk can touch, in ascending order, each once: destinations of the chunk's edges
-// (begin, count: their entries in the destination's in-list) and the chunk's own vertices (self message; the count may
-// be zero).  No two items share a vertex, so nothing here needs an atomic or an epoch stamp.
-struct Items { const int32_t* v; const uint32_t* begin; const int32_t* count; };
-
-__device__ __forceinline__ int mask_bits(const uint32_t* mask, unsigned long long b, int n) {   // set bits of [b, b + n)
-  if (n <= 0) return 0;
-  const unsigned long long e = b + (unsigned)n - 1;
-  const long long w0 = (long long)(b >> 5), w1 = (long long)(e >> 5);
-  const uint32_t first = 0xffffffffu << (b & 31), last = 0xffffffffu >> (31 - (e & 31));
-  if (w0 == w1) return __popc(mask[w0] & first & last);
-  int c = __popc(mask[w0] & first) + __popc(mask[w1] & last);
-  for (long long w = w0 + 1; w < w1; ++w) c += __popc(mask[w]);
-  return c;
-}
-
-// Edges and own vertices of a push that is not a grid cell: pending counts by atomics, first touches listed.
-__global__ void __launch_bounds__(TAURUS_ACCOUNT_THREADS, 8) account_edges_kernel(ChunkArgs a) {
-  DevCtl* ctl = a.ctl;
-  ChunkCtl* pc = a.pc;
-  if (ctl->error) return;
-  const long long e0 = a.row_ptr[a.src_begin], ne = a.row_ptr[a.src_end] - e0, total = ne + (a.src_end - a.src_begin);
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  __shared__ unsigned int s_msgs, s_hub;
-  if (threadIdx.x == 0) s_msgs = s_hub = 0;
-  __syncthreads();
-  unsigned msgs = 0, hub = 0;
-  int bad = 0;
-  for (long long base = (long long)blockIdx.x * blockDim.x; base < total; base += stride) {
-    const long long i = base + threadIdx.x;
-    int v = -1;
-    if (i < ne) {
-      const long long e = e0 + i;
-      if (a.mask == nullptr || ((a.mask[e >> 5] >> (e & 31)) & 1u)) v = a.col[e];
-      if (v >= 0) { msgs++; if (a.hub && a.hub[v]) hub++; }
-    } else if (i < total) {
-      v = (int)(a.src_begin + (i - ne));
-    }
-    bool first = false;
-    if (v >= 0) {
-      atomicAdd(&a.pend[v], -1);
-      if (a.touch[v] != a.epoch) first = atomicMax(&a.touch[v], a.epoch) != a.epoch;
-    }
-    const unsigned m = __ballot_sync(FULL, first);
-    if (m) {
-      int at = 0;
-      const int leader = __ffs(m) - 1;
-      if (rl() == leader) at = atomicAdd(&pc->touched_count, __popc(m));
-      at = __shfl_sync(FULL, at, leader) + __popc(m & ((1u << rl()) - 1));
-      if (first) { if (at < a.touched_capacity) a.touched_list[at] = v; else bad = 1; }
-    }
-  }
-  if (msgs) atomicAdd(&s_msgs, msgs);
-  if (hub) atomicAdd(&s_hub, hub);
-  if (bad) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
-  __syncthreads();
-  if (threadIdx.x == 0 && s_msgs) {
-    atomicAdd((unsigned long long*)&ctl->total_messages, (unsigned long long)s_msgs);
-    atomicAdd((unsigned long long*)&ctl->scatter_groups, (unsigned long long)s_msgs);   // no groups here: one per message
-    if (s_hub) atomicAdd((unsigned long long*)&ctl->hub_messages, (unsigned long long)s_hub);
-  }
-}
-
-// Pending counts, states, completion list; the last block to finish writes the chunk record and brings the layer totals,
-// the free-slot count and the place of the chunk's rows in the graduation buffer up to date, so that a push needs no
-// launch of its own for them.  LISTED: the items are the touched vertices listed by account_edges_kernel, whose pending
-// counts are already down.  Bound by the scattered words of a vertex (4 B count, 1 B state), which ascending items make
-// nearly sequential; ITEMS per thread keep their reads in flight together.
-enum { C_HS, C_NS, C_GS, C_MSGS, C_HUB, C_GROUPS, C_FREED, C_COUNT };
-#define ITEMS 4
-
-struct AccountShared {
-  int cnt[2][8], base[2], last;
-  unsigned int sum[C_COUNT];
-};
+// (account.cuh; the accounting of a small push runs in the launch that writes its rows)
 static_assert(sizeof(AccountShared) <= TAURUS_ACCOUNT_SHARED, "a block fits beside a CTA of the projection,");
 static_assert(4 * TAURUS_QUARTER_REGISTERS / (5 * TAURUS_ACCOUNT_THREADS) / 8 * 8 <= TAURUS_ACCOUNT_REGISTERS, "with the registers its launch bounds allow");
-static_assert(TAURUS_ACCOUNT_THREADS == 8 * 32, "eight warps (AccountShared::cnt)");
+static_assert(TAURUS_ACCOUNT_THREADS <= 8 * 32, "eight warps (AccountShared::cnt)");
 
-template <bool LISTED>
-__global__ void __launch_bounds__(TAURUS_ACCOUNT_THREADS, LISTED ? 6 : 5)
-account_kernel(ChunkArgs a, Items it, long long i0, long long n_items, const uint32_t* __restrict__ cmask, int4* __restrict__ heavy,
-               int32_t* __restrict__ heavy_left) {
-  DevCtl* ctl = a.ctl;
-  ChunkCtl* pc = a.pc;
-  if (ctl->error) return;
+__global__ void __launch_bounds__(TAURUS_ACCOUNT_THREADS, 8) account_edges_kernel(const __grid_constant__ AccountWork w) {
   __shared__ AccountShared s;
-  if (threadIdx.x < C_COUNT) s.sum[threadIdx.x] = 0;
-  const long long n = LISTED ? (long long)pc->touched_count : n_items;
-  const long long stride = (long long)gridDim.x * blockDim.x * ITEMS;
-  const int warp = threadIdx.x >> 5;
-  const unsigned lt = (1u << rl()) - 1;
-  unsigned sum[C_COUNT] = {0};
-  int bad = 0, par = 0;
-  for (long long base = (long long)blockIdx.x * blockDim.x * ITEMS; base < n; base += stride, par ^= 1) {
-    int v[ITEMS], msgs[ITEMS], dec[ITEMS], p[ITEMS], st[ITEMS];
-#pragma unroll
-    for (int q = 0; q < ITEMS; ++q) {
-      const long long i = base + q * 256 + threadIdx.x;
-      v[q] = -1; msgs[q] = dec[q] = 0;
-      if (i < n) {
-        if (LISTED) v[q] = a.touched_list[i];
-        else {
-          v[q] = it.v[i0 + i];
-          msgs[q] = it.count[i0 + i];
-          if (cmask) msgs[q] = mask_bits(cmask, it.begin[i0 + i], msgs[q]);
-          dec[q] = msgs[q] + (v[q] >= a.src_begin && v[q] < a.src_end ? 1 : 0);
-          if (dec[q] == 0) v[q] = -1;   // a sampled layer kept none of the group's messages
-        }
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < ITEMS; ++q)
-      if (v[q] >= 0) { p[q] = a.pend[v[q]] - dec[q]; st[q] = a.state[v[q]]; }
-    bool done[ITEMS];
-    unsigned md[ITEMS];
-    int wd = 0;
-#pragma unroll
-    for (int q = 0; q < ITEMS; ++q) {
-      done[q] = false;
-      if (v[q] >= 0) {
-        const bool hub = a.hub && a.hub[v[q]];
-        done[q] = p[q] == 0;
-        if (p[q] < 0 || st[q] == TAURUS_COMPLETED) bad = 1;   // a completed vertex cannot receive a message
-        if (!LISTED) a.pend[v[q]] = p[q];
-        const int to = done[q] ? TAURUS_COMPLETED : hub ? TAURUS_ON_GPU : TAURUS_IN_BUFFER;
-        if (to != st[q]) a.state[v[q]] = (uint8_t)to;
-        if (hub) sum[C_GS]++;
-        else if (st[q] == TAURUS_NOT_STARTED) sum[C_NS]++;
-        else sum[C_HS]++;
-        if (done[q] && !hub) sum[C_FREED]++;
-        sum[C_MSGS] += (unsigned)msgs[q];
-        if (msgs[q] > 0) sum[C_GROUPS]++;
-        if (hub) sum[C_HUB] += (unsigned)msgs[q];
-      }
-      md[q] = __ballot_sync(FULL, done[q]);
-      wd += __popc(md[q]);
-    }
-    // appended per block: single-address atomics would bound this kernel
-    if (rl() == 0) s.cnt[par][warp] = wd;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int t = 0;
-      for (int w = 0; w < 8; ++w) { const int c = s.cnt[par][w]; s.cnt[par][w] = t; t += c; }
-      s.base[par] = t ? atomicAdd(&pc->done_count, t) : 0;
-    }
-    __syncthreads();
-    int at = s.base[par] + s.cnt[par][warp];
-#pragma unroll
-    for (int q = 0; q < ITEMS; ++q) {
-      if (done[q]) {
-        const int i = at + __popc(md[q] & lt);
-        if (i < a.grad_cap) a.done_list[i] = v[q]; else bad = 1;
-        if (heavy && i < a.grad_cap) {
-          const int d = a.din[v[q]];
-          if (d > HEAVY_DEGREE) {
-            const int segs = (d + HEAVY_SEGMENT - 1) / HEAVY_SEGMENT;
-            const int row = atomicAdd(&ctl->heavy_rows, 1), e = atomicAdd(&pc->heavy_count, segs);
-            heavy_left[row] = segs;
-            for (int s = 0; s < segs; ++s) heavy[e + s] = make_int4(i, s, row, segs);
-          }
-        }
-      }
-      at += __popc(md[q]);
-    }
-  }
-  if (bad) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
-#pragma unroll
-  for (int c = 0; c < C_COUNT; ++c) {
-    unsigned x = sum[c];
-    for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
-    if (rl() == 0 && x) atomicAdd(&s.sum[c], x);
-  }
-  __syncthreads();
-  if (threadIdx.x < C_COUNT && s.sum[threadIdx.x]) atomicAdd(&pc->acc[threadIdx.x], (unsigned long long)s.sum[threadIdx.x]);
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s.last = atomicAdd(&pc->done_blocks, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!s.last) return;
-  // the counters of the next chunk (the other set; its last reader, the chunk before this one, is through)
-  ChunkCtl* next = pc == &ctl->pc[0] ? &ctl->pc[1] : &ctl->pc[0];
-  for (int i = threadIdx.x; i < (int)(offsetof(ChunkCtl, sel_k) / 4); i += blockDim.x) reinterpret_cast<int32_t*>(next)[i] = 0;
-  if (threadIdx.x != 0) return;
-  __threadfence();
-  long long c[C_COUNT];
-  for (int k = 0; k < C_COUNT; ++k) c[k] = (long long)__ldcg(&pc->acc[k]);
-  const long long done = __ldcg(&pc->done_count);
-  const long long F = ctl->free_top - c[C_NS], at = ctl->chunks, grad = ctl->grad_count, peak = ctl->peak_occupancy;
-  if (a.pool_slots - F > peak) ctl->peak_occupancy = a.pool_slots - F;
-  ctl->free_top = F + c[C_FREED];
-  if (at < a.log_capacity) {
-    long long* r = a.chunk_log + at * TAURUS_CK_COLUMNS;
-    r[TAURUS_CK_HS] = c[C_HS]; r[TAURUS_CK_NS] = c[C_NS]; r[TAURUS_CK_EV] = 0; r[TAURUS_CK_GS] = c[C_GS];
-    r[TAURUS_CK_NEED] = c[C_NS]; r[TAURUS_CK_EVICTED] = 0; r[TAURUS_CK_RELOADED] = 0;
-    r[TAURUS_CK_COMPLETED] = done; r[TAURUS_CK_OCCUPANCY] = a.pool_slots - (F + c[C_FREED]);
-  }
-  ctl->chunks = at + 1;
-  ctl->sum_hs += c[C_HS]; ctl->sum_ns += c[C_NS]; ctl->sum_gs += c[C_GS];
-  ctl->completed += done;
-  if (!LISTED) { ctl->total_messages += c[C_MSGS]; ctl->scatter_groups += c[C_GROUPS]; ctl->hub_messages += c[C_HUB]; }
-  pc->grad_base = a.dense_half >= 0 ? a.grad_off : grad;
-  if (a.dense_direct) { /* rows go straight into the caller's matrix */ }
-  else if (a.dense_half >= 0) ctl->out_count[a.dense_half] = done;
-  else {
-    if (grad + done > a.drain_rows) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
-    ctl->grad_count = grad + done;
-  }
+  account_edges_block<TAURUS_ACCOUNT_THREADS>(w.a, s, (int)blockIdx.x, (int)gridDim.x);
+}
+template <bool LISTED>
+__global__ void __launch_bounds__(TAURUS_ACCOUNT_THREADS, LISTED ? 6 : 5) account_kernel(const __grid_constant__ AccountWork w) {
+  __shared__ AccountShared s;
+  account_block<LISTED, TAURUS_ACCOUNT_THREADS>(w, s, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // ------------------------------------------------------------------------------------------------ gather
@@ -306,6 +110,8 @@ struct GatherArgs {
   long long* grad_ids;
   int d_out, act, mode, heads, head_vec;
   float gin_self, leaky;
+  bool early;                // launched while the kernel before it may still run
+  long long room;            // rows that the graduation buffer holds, where they go there behind others
 };
 
 #define G_WARPS 4            // warps per block
@@ -353,18 +159,25 @@ struct Ring {
 };
 
 template <int LPE, int VPL, int U, int D, int GAT>
-__global__ void __launch_bounds__(32 * G_WARPS, VPL == 1 ? 6 : VPL == 2 ? 5 : VPL == 4 ? 4 : 2) gather_kernel(const __grid_constant__ GatherArgs g) {
+__global__ void __launch_bounds__(32 * G_WARPS, VPL == 1 ? 6 : VPL == 2 ? 5 : VPL == 4 ? 4 : 2) gather_kernel(const __grid_constant__ GatherArgs g, const __grid_constant__ ChunkArgs chunk) {
   extern __shared__ __align__(16) unsigned char g_smem[];
   ChunkCtl* const pc = g.pc;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (the next push may come up, and waits in its turn)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (g.ctl->error) return;
+  if (blockIdx.x == 0) {   // a block for it: in the code of the others it would take registers
+    if (threadIdx.x < 32) account_close(chunk, g.ctl, pc);
+    return;
+  }
   constexpr int EPS = 32 / LPE, STEP = U * EPS;
   static_assert(STEP <= 32 && 32 % STEP == 0, "a block of 32 sources is a whole number of steps");
   typedef Ring<VPL, U, D, GAT> R;
   const int lane = rl(), sub = lane / LPE, c4 = lane % LPE, wid = threadIdx.x >> 5;
   R& ring = reinterpret_cast<R*>(g_smem)[wid];
-  const int warps = (int)((gridDim.x * blockDim.x) >> 5);
+  const int warps = (int)(((gridDim.x - 1) * blockDim.x) >> 5), warp = (int)(((blockIdx.x - 1) * blockDim.x + threadIdx.x) >> 5);
   const int n = uniform(pc->done_count), nh = g.heavy ? uniform(pc->heavy_count) : 0;
   const int total = n + nh;
+  if (g.room > 0 && uniform(pc->grad_base + n > g.room)) return;   // (the close has found the same)
   bool on[VPL];
   int hk[VPL];
 #pragma unroll
@@ -391,7 +204,7 @@ __global__ void __launch_bounds__(32 * G_WARPS, VPL == 1 ? 6 : VPL == 2 ? 5 : VP
   per = per < 1 ? 1 : per;
   const int n_batches = (total + per - 1) / per;
   int ticket = 0;
-  for (int batch = uniform((int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5)); batch < n_batches; batch = uniform(lane == 0 ? ticket : 0)) {
+  for (int batch = uniform(warp); batch < n_batches; batch = uniform(lane == 0 ? ticket : 0)) {
     if (lane == 0) ticket = (int)atomicAdd(&pc->span_next, 1u) + warps;
     const int i0 = batch * per, cnt = total - i0 < per ? total - i0 : per;
     __syncwarp();
@@ -646,7 +459,7 @@ __global__ void __launch_bounds__(32 * G_WARPS, VPL == 1 ? 6 : VPL == 2 ? 5 : VP
 // per_sm: the context's record of the instantiation (blocks per SM, 0 = not launched yet).  The shared-memory limit belongs to
 // the context's device, so nothing is kept process-wide.
 template <int LPE, int VPL, int U, int D, int GAT>
-int launch_g(taurus_ctx* c, const GatherArgs& g, long long bound, int* per_sm, cudaStream_t st) {
+int launch_g(taurus_ctx* c, const GatherArgs& g, const ChunkArgs& a, long long bound, int* per_sm, cudaStream_t st) {
   const size_t smem = sizeof(Ring<VPL, U, D, GAT>) * G_WARPS;
   if (*per_sm == 0) {
     int b = 0;
@@ -659,17 +472,16 @@ int launch_g(taurus_ctx* c, const GatherArgs& g, long long bound, int* per_sm, c
   // no more warps than items: a completed vertex each, and the segments of long in-lists
   const long long items = bound + c->n_heavy_segments;
   const int grid = (int)std::max<long long>(1, std::min<long long>((items + G_WARPS - 1) / G_WARPS, (long long)c->sm_count * *per_sm));
-  gather_kernel<LPE, VPL, U, D, GAT><<<grid, 32 * G_WARPS, smem, st>>>(g);
-  const cudaError_t e = cudaGetLastError();   // the accounting has been enqueued: the push must not look as if nothing had happened
+  const cudaError_t e = launch_early(g.early, gather_kernel<LPE, VPL, U, D, GAT>, grid + 1, 32 * G_WARPS, smem, st, g, a);   // the accounting has been enqueued: the push must not look as if nothing had happened
   if (e != cudaSuccess) { taurus_note_cuda_error(e, "gather_kernel"); return TAURUS_ERR_CUDA; }
   return TAURUS_OK;
 }
 template <int LPE, int VPL, int U, int D>
-int launch_g2(taurus_ctx* c, const GatherArgs& g, long long bound, int width_class, cudaStream_t st) {
+int launch_g2(taurus_ctx* c, const GatherArgs& g, const ChunkArgs& a, long long bound, int width_class, cudaStream_t st) {
   int* const per_sm = c->gather_per_sm[width_class];
-  if (g.mode != TAURUS_GAT) return launch_g<LPE, VPL, U, D, 0>(c, g, bound, per_sm, st);
+  if (g.mode != TAURUS_GAT) return launch_g<LPE, VPL, U, D, 0>(c, g, a, bound, per_sm, st);
   constexpr int DG = D > 3 ? 3 : 2;   // the scores take room in the ring
-  return g.heads <= 4 ? launch_g<LPE, VPL, U, DG, 4>(c, g, bound, per_sm + 1, st) : launch_g<LPE, VPL, U, DG, 16>(c, g, bound, per_sm + 2, st);
+  return g.heads <= 4 ? launch_g<LPE, VPL, U, DG, 4>(c, g, a, bound, per_sm + 1, st) : launch_g<LPE, VPL, U, DG, 16>(c, g, a, bound, per_sm + 2, st);
 }
 
 // ------------------------------------------------------------------------------------------------ rows into the store
@@ -677,12 +489,12 @@ int launch_g2(taurus_ctx* c, const GatherArgs& g, long long bound, int width_cla
 // 1 / sqrt(out-degree + 1) with GCN.  A copy, bound by memory: 8 blocks per SM, all of the launch's grid at once (36 registers
 // let only 6 of them in, and the last quarter of the grid ran by itself: 524 288 rows of 256 floats 222 us, now 178 = 6.0 TB/s; of 100
 // floats 114 and 93).
-__global__ void __launch_bounds__(256, 8) store_rows_kernel(const float* __restrict__ X, long long ldx, int n, int K, long long src_begin, int gcn,
-                                                            const long long* __restrict__ row_ptr, float* __restrict__ out, int ldo) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
+__device__ __forceinline__ void store_rows(const float* __restrict__ X, long long ldx, int n, int K, long long src_begin, int gcn,
+                                           const long long* __restrict__ row_ptr, float* __restrict__ out, int ldo, int block, int blocks) {
+  const long long stride = (long long)blocks * blockDim.x;
   const int vec = ldo >> 2;
   const bool wide = (ldx & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < (long long)n * vec; i += stride) {
+  for (long long i = (long long)block * blockDim.x + threadIdx.x; i < (long long)n * vec; i += stride) {
     const long long r = i / vec;
     const int c = (int)(i - r * vec) * 4;
     const float* src = X + r * ldx + c;
@@ -696,6 +508,18 @@ __global__ void __launch_bounds__(256, 8) store_rows_kernel(const float* __restr
     }
     reinterpret_cast<float4*>(out)[i] = x;
   }
+}
+
+__global__ void __launch_bounds__(256, 8) store_rows_kernel(const float* X, long long ldx, int n, int K, long long src_begin, int gcn, const long long* row_ptr,
+                                                            float* out, int ldo) {
+  store_rows(X, ldx, n, K, src_begin, gcn, row_ptr, out, ldo, (int)blockIdx.x, (int)gridDim.x);
+}
+// The first blocks do the accounting of the push.
+__global__ void __launch_bounds__(256, 4) store_and_account_kernel(const float* X, long long ldx, int n, int K, long long src_begin, int gcn, const long long* row_ptr,
+                                                                   float* out, int ldo, const __grid_constant__ AccountArgs<true> acc) {
+  __shared__ AccountShared s;
+  if (account_here<256>(acc, s)) return;
+  store_rows(X, ldx, n, K, src_begin, gcn, row_ptr, out, ldo, (int)blockIdx.x - acc.blocks(), (int)gridDim.x - acc.blocks());
 }
 
 // ------------------------------------------------------------------------------------------------ attention
@@ -983,33 +807,49 @@ void launch_resident_reset(taurus_ctx* c, int layer, cudaStream_t st) {
   c->launches += 1;
 }
 
-void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int K, long long src_begin, bool gcn, float* out, int ldo, cudaStream_t st) {
+void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int K, long long src_begin, bool gcn, float* out, int ldo, cudaStream_t st,
+                       const AccountWork* acc) {
   const int grid = (int)std::min<long long>(((long long)n * (ldo >> 2) + 255) / 256, (long long)c->sm_count * 8);
-  store_rows_kernel<<<grid, 256, 0, st>>>(X, ldx, n, K, src_begin, gcn ? 1 : 0, c->d_row_ptr, out, ldo);
+  if (acc)
+    launch_early(acc->early, store_and_account_kernel, grid + acc->blocks, 256, 0, st, X, ldx, n, K, src_begin, gcn ? 1 : 0, (const long long*)c->d_row_ptr, out, ldo,
+                 AccountArgs<true>{*acc});
+  else
+    store_rows_kernel<<<grid, 256, 0, st>>>(X, ldx, n, K, src_begin, gcn ? 1 : 0, c->d_row_ptr, out, ldo);
   c->launches += 1;
 }
 
-// Accounting of a push.  `cell`: the chunk's number when it is one cell of the chunk grid, else -1.
+// Accounting of a push.  `cell`: the chunk's number when it is one cell of the chunk grid, else -1: then edge by edge first.
+AccountWork account_work(const taurus_ctx* c, const ChunkArgs& a, long long cell) {
+  AccountWork w;
+  w.a = a;
+  w.cmask = c->d_mask_cur ? c->d_cmask : nullptr;
+  w.heavy = c->n_heavy > 0 && !w.cmask ? c->d_heavy : nullptr;
+  w.heavy_left = c->d_heavy_left;
+  w.it = Items{c->d_item_v, c->d_item_begin, c->d_item_count};
+  w.i0 = cell >= 0 ? c->item_ptr[(size_t)cell] : 0;
+  w.n_items = cell >= 0 ? c->item_ptr[(size_t)cell + 1] - w.i0 : 0;
+  w.blocks = 0;
+  w.early = false;
+  return w;
+}
 void launch_account(taurus_ctx* c, const ChunkArgs& a, long long cell, cudaStream_t st) {
-  const uint32_t* cmask = c->d_mask_cur ? c->d_cmask : nullptr;
-  int4* heavy = c->n_heavy > 0 && !cmask ? c->d_heavy : nullptr;
-  Items it = {c->d_item_v, c->d_item_begin, c->d_item_count};
+  const AccountWork w = account_work(c, a, cell);
   if (cell >= 0) {
-    const long long i0 = c->item_ptr[(size_t)cell], n = c->item_ptr[(size_t)cell + 1] - i0;
-    const int grid = (int)std::max<long long>(1, std::min<long long>((n + 256 * ITEMS - 1) / (256 * ITEMS), (long long)c->sm_count * 6));
-    account_kernel<false><<<grid, TAURUS_ACCOUNT_THREADS, 0, st>>>(a, it, i0, n, cmask, heavy, c->d_heavy_left);
+    const int grid = (int)std::max<long long>(1, std::min<long long>((w.n_items + 256 * ITEMS - 1) / (256 * ITEMS), (long long)c->sm_count * 6));
+    account_kernel<false><<<grid, TAURUS_ACCOUNT_THREADS, 0, st>>>(w);
     c->launches += 1;
     return;
   }
-  account_edges_kernel<<<c->sm_count * 8, TAURUS_ACCOUNT_THREADS, 0, st>>>(a);
+  account_edges_kernel<<<c->sm_count * 8, TAURUS_ACCOUNT_THREADS, 0, st>>>(w);
   const int grid = (int)std::max<long long>(1, std::min<long long>((a.touched_capacity + 256 * ITEMS - 1) / (256 * ITEMS), (long long)c->sm_count * 6));
-  account_kernel<true><<<grid, TAURUS_ACCOUNT_THREADS, 0, st>>>(a, it, 0, 0, cmask, heavy, c->d_heavy_left);
+  account_kernel<true><<<grid, TAURUS_ACCOUNT_THREADS, 0, st>>>(w);
   c->launches += 2;
 }
 
 // Sums and finished rows of the vertices the push completed, at most `bound` (aggregate-first layers: sums into A).
-int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitch, float* A, long long bound, cudaStream_t st) {
+int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitch, float* A, long long bound, bool early, cudaStream_t st) {
   GatherArgs g;
+  g.early = early;
   const bool sampled = c->d_mask_cur != nullptr;
   g.rows = reinterpret_cast<const float4*>(rows); g.pitch = pitch >> 2; g.vec = a.Hp >> 2;
   g.csc_ptr = c->d_csc_ptr; g.src = sampled ? c->d_kept : c->d_csc_src; g.keep = sampled ? a.fanout : 0;
@@ -1023,6 +863,7 @@ int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitc
   g.dense = a.dense_direct; g.dense_ld = a.dense_ld; g.grad_rows = a.grad_rows; g.grad_ids = a.grad_ids;
   g.d_out = a.d_out; g.act = a.act; g.mode = a.mode; g.heads = a.heads; g.head_vec = a.head_vec;
   g.gin_self = a.gin_self; g.leaky = a.leaky;
+  g.room = !A && !a.dense_direct && a.dense_half < 0 ? a.drain_rows : 0;
   c->launches += 1;
   // Rows split over as many lanes as they have float4, steps of about 2 KB per warp.  Measured (ms of all launches of a pass):
   // 48 floats, 2.45 M vertices, 124 M edges: 16 lanes x 1 float4, 4 rows a step, 3 steps 3.9; 8 x 2 4.6 to 5.2.  64 floats, 500 k
@@ -1030,13 +871,13 @@ int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitc
   // 7.5; 16 x 2 7.7.  256 floats: 2 rows, 4 steps 15.8; 4 rows, 3 steps 15.8, slower where in-lists are short.  GATConv (a step
   // less, for the scores), 64 floats, one head: 4 rows, 2 steps 0.66; 2 rows, 3 steps 0.71.
   const int Hp = a.Hp;
-  if (Hp <= 16) return launch_g2<4, 1, 2, 4>(c, g, bound, 0, st);
-  if (Hp <= 32) return launch_g2<8, 1, 2, 4>(c, g, bound, 1, st);
-  if (Hp <= 64) return launch_g2<16, 1, 4, 3>(c, g, bound, 2, st);
-  if (Hp <= 128) return launch_g2<32, 1, 4, 3>(c, g, bound, 3, st);
-  if (Hp <= 256) return launch_g2<32, 2, 2, 4>(c, g, bound, 4, st);
-  if (Hp <= 512) return launch_g2<32, 4, 1, 4>(c, g, bound, 5, st);
-  return launch_g2<32, 8, 1, 3>(c, g, bound, 6, st);
+  if (Hp <= 16) return launch_g2<4, 1, 2, 4>(c, g, a, bound, 0, st);
+  if (Hp <= 32) return launch_g2<8, 1, 2, 4>(c, g, a, bound, 1, st);
+  if (Hp <= 64) return launch_g2<16, 1, 4, 3>(c, g, a, bound, 2, st);
+  if (Hp <= 128) return launch_g2<32, 1, 4, 3>(c, g, a, bound, 3, st);
+  if (Hp <= 256) return launch_g2<32, 2, 2, 4>(c, g, a, bound, 4, st);
+  if (Hp <= 512) return launch_g2<32, 4, 1, 4>(c, g, a, bound, 5, st);
+  return launch_g2<32, 8, 1, 3>(c, g, a, bound, 6, st);
 }
 
 void launch_resident_attention(taurus_ctx* c, cudaStream_t st) {

@@ -8,6 +8,7 @@
 #include <new>
 #include <vector>
 
+#include "account.cuh"
 #include "taurus_internal.h"
 
 static thread_local char g_cuda_err[256] = "";
@@ -656,11 +657,11 @@ static int finish_chunk(taurus_ctx* c, cudaStream_t st) {
 // S1: features of sources [s, e) ([n x K], rows contiguous) to the device.  Host chunks are copied on the library's
 // copy stream into one of two staging buffers, so that the copy of chunk k+1 overlaps the kernels of chunk k; a
 // chunk read from sorted runs is merged into the same buffers; a device pointer is used in place (*xbuf = -1).
-static int stage_chunk(taurus_ctx* c, const float* features, taurus_runs* src_runs, long long s, long long e, int K, cudaStream_t st,
+static int stage_chunk(taurus_ctx* c, const float* features, taurus_runs* src_runs, bool in_place, long long s, long long e, int K, cudaStream_t st,
                        const float** X, int* xbuf) {
   *X = features;
   *xbuf = -1;
-  if (!src_runs && pointer_kind(features) == PK_DEVICE) return TAURUS_OK;
+  if (in_place) return TAURUS_OK;
   const int b = (int)(c->host_pushes & 1);
   if (c->x_used[b]) CU(cudaStreamWaitEvent(c->copy_stream, c->x_free[b], 0));
   if (src_runs) {   // merge-on-read; fails before anything is enqueued when the runs do not cover the chunk
@@ -677,13 +678,37 @@ static int stage_chunk(taurus_ctx* c, const float* features, taurus_runs* src_ru
   return TAURUS_OK;
 }
 
+// Whether the accounting of a push to a resident pool runs in the launch that writes the push's rows from X (device memory: it would wait for a
+// copy), and in how many of its blocks: a stream of its own costs two events and two waits, which a small push has nothing to hide behind.
+// Where the tensor-core kernel writes the rows, whose CTAs take an SM each, all blocks have to be on the device at once; else up to the
+// sizes where the gain has gone.  us a push, degree 12, on two streams / in one launch:
+//   sources                              512         2 048       8 192       16 384      32 768      65 536
+//   64 -> 64, tensor cores               23.3/16.9   26.0/17.0   29.2/21.1   34.3/34.6   (does not fit from here on)
+//   128 -> 256, rows copied              26.2/19.9   33.6/26.8   43.9/37.4   55.0/48.3   71.9/67.2   111.6/110.6
+//   47 -> 33, FFMA kernel                18.6/10.9   25.2/16.8   29.4/22.4   34.3/29.5   48.7/43.9   76.6/72.8
+// Not off the chunk grid, where the accounting is two kernels, one after the other (10 007 sources, 145 k edges, FFMA kernel: 73 us a push and
+// drain on two streams, 77 in the launch of the rows).
+static bool rows_with_account(const taurus_ctx* c, const ChunkArgs& a, const float* X, int n, long long cell, AccountWork* w) {
+  if (cell < 0 || n > 65536) return false;
+  const int l = c->layer;
+  const bool copy = c->agg_first[l] || c->mode == TAURUS_GAT, tc = !copy && project_tc_usable(c, l, X, c->dims[l]);
+  const int per = tc || copy ? 256 * ITEMS : 128 * ITEMS;
+  const long long blocks = std::max<long long>(1, (c->item_ptr[(size_t)cell + 1] - c->item_ptr[(size_t)cell] + per - 1) / per);
+  if (blocks > (tc ? c->sm_count - project_tc_units(c, l, n) : 8 * c->sm_count)) return false;
+  *w = account_work(c, a, cell);
+  w->blocks = (int)blocks;
+  return true;
+}
+
 // One chunk through S1..S7 on `st`, after push_core's checks.  *applied: set while the chunk has been enqueued in part, so that an
 // error in between leaves a layer that cannot go on.
 static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const float* features, taurus_runs* src_runs, long long bound,
                         bool direct_dense, bool halves, cudaStream_t st, bool* applied) {
   const bool gat = c->mode == TAURUS_GAT;
   const int l = c->layer;
+  bool waits = false;           // this push has the stream wait for an event
   if (st != c->last_stream) {   // keep chunk order across streams
+    waits = true;
     CU(cudaEventRecord(c->order_event, c->last_stream));
     CU(cudaStreamWaitEvent(st, c->order_event, 0));
     c->last_stream = st;
@@ -701,21 +726,32 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
   const bool scatter_timing = pev != nullptr;           // level 2 records the two events around the scatter only
   const bool timing = pev != nullptr && c->timing != 2;
   if (timing) cudaEventRecord(pev[0], st);
-  if (c->resident) CU(cudaEventRecord(c->account_go, st));   // everything of the chunk before this one
+  const bool in_place = !src_runs && pointer_kind(features) == PK_DEVICE;
+  const bool cell = src_begin % c->chunk_sources == 0 && src_end == std::min<long long>(c->V, src_begin + c->chunk_sources);
+  AccountWork acc;   // blocks > 0: in the launch that writes the rows
+  acc.blocks = 0;
+  if (c->resident) {
+    const ChunkArgs aa = make_args(c, src_begin, src_end);
+    if (in_place && rows_with_account(c, aa, features, n, cell ? src_begin / c->chunk_sources : -1, &acc)) {
+      if (aa.dense_half >= 0 && c->half_used[aa.dense_half]) { CU(cudaStreamWaitEvent(st, c->out_done[aa.dense_half], 0)); waits = true; }
+      acc.early = !waits && !pev;
+    } else {
+      CU(cudaEventRecord(c->account_go, st));   // everything of the chunk before this one
+    }
+  }
   // S1: features to the device
   const float* X = nullptr;
   int ldx = K;
   int xbuf = -1;
-  { int rc = stage_chunk(c, features, src_runs, src_begin, src_end, K, st, &X, &xbuf); if (rc) return rc; }
-  if (c->resident) {
+  { int rc = stage_chunk(c, features, src_runs, in_place, src_begin, src_end, K, st, &X, &xbuf); if (rc) return rc; }
+  if (c->resident && acc.blocks == 0) {
     // Accounting of the chunk: topology only, so it runs beside the copy and the projection of its rows (20 us of latencies
     // on a chunk of 65 536 sources, 7 us on the smallest, that would otherwise stand in front of the gather).
-    const ChunkArgs acc = make_args(c, src_begin, src_end);
-    const bool cell = src_begin % c->chunk_sources == 0 && src_end == std::min<long long>(c->V, src_begin + c->chunk_sources);
+    const ChunkArgs aa = make_args(c, src_begin, src_end);
     CU(cudaStreamWaitEvent(c->account_stream, c->account_go, 0));
-    if (acc.dense_half >= 0 && c->half_used[acc.dense_half]) CU(cudaStreamWaitEvent(c->account_stream, c->out_done[acc.dense_half], 0));
+    if (aa.dense_half >= 0 && c->half_used[aa.dense_half]) CU(cudaStreamWaitEvent(c->account_stream, c->out_done[aa.dense_half], 0));
     *applied = true;
-    launch_account(c, acc, cell ? src_begin / c->chunk_sources : -1, c->account_stream);
+    launch_account(c, aa, cell ? src_begin / c->chunk_sources : -1, c->account_stream);
     CU(cudaEventRecord(c->account_done, c->account_stream));
   }
   if (timing) cudaEventRecord(pev[1], st);
@@ -725,23 +761,25 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
     const bool af = c->agg_first[l];
     const int w = resident_row(c, l);
     float* rows = c->d_store + (size_t)src_begin * w;
+    const AccountWork* with = acc.blocks > 0 ? &acc : nullptr;
+    if (with) *applied = true;
     if (af) {
       a.Hout = a.Hp; a.Hp = taurus_round_up(c->dims[l], 4); a.self_bias = 0;
-      launch_store_rows(c, X, ldx, n, c->dims[l], src_begin, c->mode == TAURUS_GCN_SYM, rows, w, st);   // (GAT: pass 1 handed the input rows back, pitch dims[l + 1])
+      launch_store_rows(c, X, ldx, n, c->dims[l], src_begin, c->mode == TAURUS_GCN_SYM, rows, w, st, with);   // (GAT: pass 1 handed the input rows back, pitch dims[l + 1])
     } else if (gat) {
-      launch_store_rows(c, X, ldx, n, K, src_begin, false, rows, w, st);
+      launch_store_rows(c, X, ldx, n, K, src_begin, false, rows, w, st, with);
     } else if (project_tc_usable(c, l, X, ldx)) {
-      int rc = launch_project_tc(c, l, X, ldx, src_begin, n, rows, w, st);
+      int rc = launch_project_tc(c, l, X, ldx, src_begin, n, rows, w, st, with);
       if (rc) return rc;
     } else {
-      launch_project_simt(c, l, X, ldx, src_begin, n, rows, w, st);
+      launch_project_simt(c, l, X, ldx, src_begin, n, rows, w, st, with);
     }
     if (xbuf >= 0) { CU(cudaEventRecord(c->x_free[xbuf], st)); c->x_used[xbuf] = true; }
     if (timing) cudaEventRecord(pev[2], st);
-    CU(cudaStreamWaitEvent(st, c->account_done, 0));
+    if (!with) CU(cudaStreamWaitEvent(st, c->account_done, 0));
     if (timing) cudaEventRecord(pev[3], st);
     if (scatter_timing) cudaEventRecord(pev[5], st);
-    { int rc = launch_gather(c, a, c->d_store, w, af ? c->d_af_A : nullptr, std::min<long long>(bound, a.grad_cap), st); if (rc) return rc; }
+    { int rc = launch_gather(c, a, c->d_store, w, af ? c->d_af_A : nullptr, std::min<long long>(bound, a.grad_cap), with && !pev, st); if (rc) return rc; }
     if (scatter_timing) cudaEventRecord(pev[6], st);
     if (timing) cudaEventRecord(pev[7], st);
     if (af) {
@@ -889,7 +927,7 @@ static int gat_project_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, c
   const int proj_w = taurus_proj_width(c->mode, Hp, c->heads);
   const float* X = nullptr;
   int xbuf = -1;
-  { int rc = stage_chunk(c, features, src_runs, src_begin, src_end, K, st, &X, &xbuf); if (rc) return rc; }
+  { int rc = stage_chunk(c, features, src_runs, !src_runs && pointer_kind(features) == PK_DEVICE, src_begin, src_end, K, st, &X, &xbuf); if (rc) return rc; }
   if (c->agg_first[l]) {   // scores from two dot products per row; the input rows go back to the caller for pass 3
     launch_gat_scores(c, l, X, K, n, src_begin, hprime_out, ld, st);
     if (xbuf >= 0) { CU(cudaEventRecord(c->x_free[xbuf], st)); c->x_used[xbuf] = true; }

@@ -207,7 +207,7 @@ struct taurus_ctx {
   // weights per layer: Wcat is [Kp x Ncat] row-major fp32 (P columns then T columns), bias [Hp]
   float* d_Wcat[TAURUS_MAX_LAYERS] = {nullptr};
   float* d_bias[TAURUS_MAX_LAYERS] = {nullptr};
-  bool tc_smem_set = false;                        // dynamic shared memory limit of the projection kernel raised
+  bool tc_smem_set[2] = {false, false};            // dynamic shared memory limit of the projection kernel raised (without, with accounting)
   bool xfer_smem_set = false;                      // the same for the row transfer kernel
   void* tc_image[TAURUS_MAX_LAYERS] = {nullptr};   // tensor-core operand images of Wcat (owned by kernels_gemm_tc.cu)
   void* tc_image_af[TAURUS_MAX_LAYERS] = {nullptr};   // SAGE aggregate-first layers: image of [W_neigh ; W_self] stacked along K
@@ -353,6 +353,19 @@ static inline int taurus_proj_width(int mode, int Hp, int heads = 1) {
   return mode == TAURUS_SAGE_MEAN ? 2 * Hp : mode == TAURUS_GAT ? Hp + taurus_round_up(2 * heads, 4) : Hp;
 }
 
+// Launches a kernel that, with `early`, may come up while the kernel before it on the stream still runs (it waits, inside, before it reads or
+// writes anything): a microsecond between two short kernels.  Not behind a wait for an event.
+template <class... P, class... A>
+static inline cudaError_t launch_early(bool early, void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.attrs = &at; cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ---- kernels_state.cu
 void launch_layer_reset(taurus_ctx* c, int layer, cudaStream_t st);
 void launch_classify(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);
@@ -397,7 +410,9 @@ void launch_gat_repack(taurus_ctx* c, const float* X, int n, int d_out, int Hp, 
 // ---- kernels_scatter.cu
 void launch_scatter(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st);
 // ---- kernels_gemm_simt.cu
-void launch_project_simt(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, int ldo, cudaStream_t st);
+// acc (account.cuh): accounting of the push in the first blocks of the launch, NULL: none
+void launch_project_simt(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, int ldo, cudaStream_t st,
+                         const struct AccountWork* acc = nullptr);
 void launch_gemm_plain_simt(taurus_ctx* c, const float* W, int ldw, int N, const float* X, int ldx, int K, int n, float* out, long long ld_out,
                             cudaStream_t st);   // out = X . W[:, 0..N), W row-major with pitch ldw
 // ---- kernels_gemm_tc.cu
@@ -420,14 +435,18 @@ int launch_gemm_plain_tc(taurus_ctx* c, void* image, int col0, int N, const floa
 int prepare_tc_weights(taurus_ctx* c, void** slot, const std::vector<float>& cat, int K, int N);   // image of cat [K x N] into *slot
 void free_tc_weights(taurus_ctx* c);
 bool project_tc_usable(const taurus_ctx* c, int layer, const float* X, int ldx);
-int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, int ldo, cudaStream_t st);   // out [n x projection width], pitch ldo (a multiple of 4), 16-byte aligned
+int project_tc_units(const taurus_ctx* c, int layer, int n);                 // units of work, one CTA each at most
+int launch_project_tc(taurus_ctx* c, int layer, const float* X, int ldx, long long src_begin, int n, float* out, int ldo, cudaStream_t st,
+                      const struct AccountWork* acc = nullptr);   // out [n x projection width], pitch ldo (a multiple of 4), 16-byte aligned
 // ---- kernels_resident.cu
 int resident_row(const taurus_ctx* c, int layer);                            // floats per row of the store
 int build_resident(taurus_ctx* c);
 void launch_resident_reset(taurus_ctx* c, int layer, cudaStream_t st);
-void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int K, long long src_begin, bool gcn, float* out, int ldo, cudaStream_t st);
+void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int K, long long src_begin, bool gcn, float* out, int ldo, cudaStream_t st,
+                       const struct AccountWork* acc);
+struct AccountWork account_work(const taurus_ctx* c, const ChunkArgs& a, long long cell);   // (account.cuh)
 void launch_account(taurus_ctx* c, const ChunkArgs& a, long long cell, cudaStream_t st);
-int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitch, float* A, long long bound, cudaStream_t st);
+int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitch, float* A, long long bound, bool early, cudaStream_t st);
 void launch_resident_attention(taurus_ctx* c, cudaStream_t st);
 // ---- kernels_group.cu
 int build_grouped_order(taurus_ctx* c, bool keep_edge_ids, bool fill_csc_src);   // fill_csc_src: also writes csc_src (needs csc_ptr)
