@@ -758,6 +758,7 @@ static __device__ __forceinline__ void xf_load(void* dst, const void* src, unsig
 // Only entries with a row to move are listed: a chunk that moves none was 40 to 75 us of walking its need list, beside the scatter.
 // An extent whose last row has come back is listed for the free stack (taken back two chunks later by extent_plan).
 #define XF_SMEM (224 * 1024)
+#define XF_FLIGHT (112 * 1024)   // bytes of rows in flight per block, half of them either way
 static_assert(XF_SMEM + 2048 + 2 * TAURUS_BLOCK_SHARED + TAURUS_OFF_XFER > TAURUS_SM_SHARED, "no block that asks for TAURUS_OFF_XFER fits beside one of the transfers");
 #define XF_THREADS 256
 __global__ void __launch_bounds__(XF_THREADS) transfer_kernel(ChunkArgs a, int lanes) {   // lanes: entries in flight per block
@@ -767,41 +768,39 @@ __global__ void __launch_bounds__(XF_THREADS) transfer_kernel(ChunkArgs a, int l
   ChunkCtl* pc = a.pc;
   if (ctl->error) return;
   if ((int)threadIdx.x >= lanes) return;
-  const int n = pc->deficit + pc->xfer_extra;
+  const bool out = threadIdx.x & 1;   // rows on their way out: those of the victims, which are listed first; else rows coming back
+  const int n = out ? pc->deficit : pc->deficit + pc->xfer_extra, step = (lanes >> 1) * (int)gridDim.x;
   const unsigned bytes = (unsigned)a.Hp * 4u;
-  unsigned char* in = xf_rows + (size_t)threadIdx.x * 2 * bytes;
-  unsigned char* out = in + bytes;
+  unsigned char* const row = xf_rows + (size_t)threadIdx.x * bytes;
   unsigned long long* bar = &bars[threadIdx.x];
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(xf_smem(bar)) : "memory");
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   const int par = a.epoch & 1;
   unsigned phase = 0;
-  const int step = lanes * (int)gridDim.x;
   int4 next = make_int4(0, -1, -1, 0);
-  int i = (int)(threadIdx.x * gridDim.x + blockIdx.x);
+  int i = (int)((threadIdx.x >> 1) * gridDim.x + blockIdx.x);
   if (i < n) next = a.xfer_list[i];
   for (; i < n; i += step) {
     const int4 x = next;   // (slot, host row coming back or -1, host row to fill or -1)
     if (i + step < n) next = a.xfer_list[i + step];
-    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the stores of the last entry have read the buffers
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                 ::"r"(xf_smem(bar)), "r"((x.y >= 0 ? bytes : 0u) + (x.z >= 0 ? bytes : 0u)) : "memory");
-    if (x.y >= 0) xf_load(in, a.host_store + (size_t)x.y * a.Hp, bytes, bar);
-    if (x.z >= 0) xf_load(out, a.stage_out + (size_t)i * a.Hp, bytes, bar);
+    const int hrow = out ? x.z : x.y;
+    if (hrow < 0) continue;
+    float* const host = a.host_store + (size_t)hrow * a.Hp;
+    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the store of the last entry has read the buffer
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(xf_smem(bar)), "r"(bytes) : "memory");
+    xf_load(row, out ? a.stage_out + (size_t)i * a.Hp : host, bytes, bar);
     if (!xf_wait(bar, phase)) { atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL); xf_wait(bar, phase); break; }
     phase ^= 1;
-    if (x.y >= 0)
+    if (out) {
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(host), "r"(xf_smem(row)), "r"(bytes) : "memory");
+    } else {
       asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;"
-                   ::"l"(a.acc + (size_t)x.x * a.Hp), "r"(xf_smem(in)), "r"(bytes) : "memory");
-    if (x.z >= 0)
-      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                   ::"l"(a.host_store + (size_t)x.z * a.Hp), "r"(xf_smem(out)), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-    if (x.y >= 0) {
-      const int e = x.y >> a.ext_shift;
+                   ::"l"(a.acc + (size_t)x.x * a.Hp), "r"(xf_smem(row)), "r"(bytes) : "memory");
+      const int e = hrow >> a.ext_shift;
       if (atomicSub(&a.ext_live[e], 1) == 1) a.ext_ret[par][atomicAdd(&ctl->ext_ret_count[par], 1)] = e;   // last row of the extent
     }
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
   }
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
@@ -834,13 +833,13 @@ int launch_make_room(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, cudaEve
 
 // Slots handed out, victims' rows staged, new rows cleared (S4, device side).
 void launch_alloc(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
-  alloc_kernel<<<c->sm_count * 8, 256, 0, st>>>(a);
+  // bounded pools: one wave (46 registers), every block of which pays the chain of dependent reads once
+  alloc_kernel<<<c->sm_count * (a.direct ? 8 : 5), 256, 0, st>>>(a);
   c->launches += 1;
 }
 // Rows across the host link (bounded pools only).
 int launch_transfer(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
-  int lanes = XF_SMEM / (2 * a.Hp * 4);
-  if (lanes > XF_THREADS) lanes = XF_THREADS;
+  const int lanes = std::min(std::max(XF_FLIGHT / (a.Hp * 4), 32), XF_THREADS) & ~1;
   if (!c->xfer_smem_set) {   // once per context (the attribute belongs to the context's device)
     const cudaError_t e = cudaFuncSetAttribute(transfer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, XF_SMEM);
     if (e != cudaSuccess) { taurus_note_cuda_error(e, "transfer_kernel"); return TAURUS_ERR_CUDA; }
@@ -941,7 +940,8 @@ __global__ void compact_done_kernel(ChunkArgs a, int write_record) {
 // vertex, its slot and its normalisation of one row of the batch (one dependent chain for 32 rows), then the
 // warp walks the batch row by row: out = act(c_in(v) * acc) into the graduation buffer, or straight into the
 // caller's vertex-ordered matrix (Sect. 3.6); the slot is released by compact_done_kernel.
-__global__ void finalise_kernel(ChunkArgs a) {
+static __device__ void commit_chunk(const ChunkArgs& a, DevCtl* ctl, ChunkCtl* pc, int with_counts);
+__global__ void finalise_kernel(ChunkArgs a, int with_counts) {
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
   if (ctl->error) return;
@@ -1013,6 +1013,12 @@ __global__ void finalise_kernel(ChunkArgs a) {
       }
     }
   }
+  // the last block to finish closes the chunk (a launch of its own for that was 5 us between two chunks)
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&pc->final_blocks, 1u) == gridDim.x - 1) { __threadfence(); commit_chunk(a, ctl, pc, with_counts); }
+  }
 }
 
 // After the chunk's completions are listed: fold the chunk's counters into the layer totals, write the chunk record.
@@ -1037,10 +1043,8 @@ static __device__ void commit_counts(const ChunkArgs& a, DevCtl* ctl, ChunkCtl* 
 // One thread, after the chunk's rows are finalised: the graduation buffer's row count, and the chunk's counters are
 // cleared for the chunk after next.  with_counts: the chunk record has not been written yet (no transfers in flight:
 // finalise followed the completion list directly).
-__global__ void commit_kernel(ChunkArgs a, int with_counts) {
-  DevCtl* ctl = a.ctl;
-  ChunkCtl* pc = a.pc;
-  if (threadIdx.x != 0 || ctl->error) return;
+static __device__ void commit_chunk(const ChunkArgs& a, DevCtl* ctl, ChunkCtl* pc, int with_counts) {
+  if (ctl->error) return;
   if (with_counts) commit_counts(a, ctl, pc);
   if (a.dense_direct) { /* rows already sit in the caller's matrix */ }
   else if (a.dense_half >= 0) ctl->out_count[a.dense_half] = pc->done_count;
@@ -1048,7 +1052,10 @@ __global__ void commit_kernel(ChunkArgs a, int with_counts) {
   pc->hs = pc->ns = pc->ev = pc->gs = 0;
   pc->need_count = 0; pc->done_count = 0; pc->touched_count = 0; pc->deficit = 0; pc->victim_count = 0; pc->reloaded = 0; pc->xfer_extra = 0;
   pc->span_next = 0; pc->self_next = 0;
-  pc->grid_arrivals = 0; pc->done_blocks = 0; pc->room_go = 0; pc->room_fail = 0;
+  pc->grid_arrivals = 0; pc->done_blocks = 0; pc->final_blocks = 0; pc->room_go = 0; pc->room_fail = 0;
+}
+__global__ void commit_kernel(ChunkArgs a, int with_counts) {
+  if (threadIdx.x == 0) commit_chunk(a, a.ctl, a.pc, with_counts);
 }
 
 // S6: completions listed, slots released, chunk record written.
@@ -1064,11 +1071,10 @@ void launch_commit(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
   c->launches += 1;
 }
 
-// S7 of a project-first layer (after launch_compact_done): rows finalised, graduation bookkeeping.
+// S7 of a project-first layer (after launch_compact_done): rows finalised, graduation bookkeeping.  One wave of blocks (60 registers).
 void launch_finalise(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
-  finalise_kernel<<<c->sm_count * 8, 256, 0, st>>>(a);
-  commit_kernel<<<1, 32, 0, st>>>(a, c->pipelined ? 0 : 1);
-  c->launches += 2;
+  finalise_kernel<<<c->sm_count * 4, 256, 0, st>>>(a, c->pipelined ? 0 : 1);
+  c->launches += 1;
 }
 
 // ------------------------------------------------------------------------------------------------ drain helpers

@@ -45,6 +45,7 @@ struct ChunkCtl {
   unsigned int self_next; // scatter: next tile of 32 self messages to hand to a warp
   unsigned int grid_arrivals; // make-room step: blocks that reached its barriers so far
   unsigned int done_blocks;   // completion list: blocks that have finished
+  unsigned int final_blocks;  // finalise: the same
   int32_t room_go, room_fail; // make-room step: the plan went through / the host store could not take the victims
   int32_t xfer_extra;     // reloads into slots from the free stack (entries of the transfer list behind those of the victims)
   int32_t heavy_count;    // resident pools: segments of long in-lists to sum
