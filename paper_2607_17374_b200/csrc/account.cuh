@@ -20,7 +20,6 @@ struct AccountWork {
   int4* heavy;                 // segments of long in-lists, NULL: none
   int32_t* heavy_left;
   int blocks;                  // blocks of the launch that do it
-  bool early;                  // the launch may come up while the kernel before it on the stream still runs
 };
 
 namespace {
@@ -237,12 +236,10 @@ template <> struct AccountArgs<true> { AccountWork w; __device__ __forceinline__
 template <> struct AccountArgs<false> { __device__ __forceinline__ int blocks() const { return 0; } };
 // True in the blocks that did it.  s: shared memory of the kernel to use.
 template <int THREADS>
-__device__ __forceinline__ bool account_here(const AccountArgs<false>&, AccountShared&) { return false; }
+__device__ __forceinline__ bool account_here(const AccountArgs<false>&, AccountShared&) { early_start(); return false; }
 template <int THREADS>
 __device__ __forceinline__ bool account_here(const AccountArgs<true>& acc, AccountShared& s) {
-  // Launched while the kernel before it on the stream may still run, and lets the one behind it come up: both wait for what they read.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  early_start();
   if ((int)blockIdx.x >= acc.w.blocks) return false;
   if (threadIdx.x < THREADS) account_block<false, THREADS>(acc.w, s, (int)blockIdx.x, acc.w.blocks);
   return true;

@@ -21,6 +21,7 @@ __device__ __forceinline__ int af_messages(int din, int fanout) { return (fanout
 // S[r][k] = c_out(u) * X[r][k] for k < K, 0 for the padding columns; u = src_begin + r.
 __global__ void af_prep_kernel(const float* __restrict__ X, int ldx, int n, int K, int Kp, long long src_begin, int mode,
                                const long long* __restrict__ row_ptr, float* __restrict__ S) {
+  early_start();
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
     float scale = 1.0f;
@@ -93,6 +94,7 @@ __global__ void af_gather_kernel(ChunkArgs a, float* __restrict__ A, long long r
 // out = act(O_i + b) into the graduation buffer or straight into the caller's vertex-ordered matrix.
 // O has pitch a.Hout; rows of the graduation buffer too.
 __global__ void af_finish_kernel(ChunkArgs a, const float* __restrict__ O, long long rows) {
+  early_start();
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
   if (ctl->error) return;
@@ -140,7 +142,8 @@ __global__ void af_finish_kernel(ChunkArgs a, const float* __restrict__ O, long 
 }  // namespace
 
 void launch_af_prep(taurus_ctx* c, const float* X, int ldx, int n, int K, int Kp, long long src_begin, float* out, cudaStream_t st) {
-  af_prep_kernel<<<c->sm_count * 8, 256, c->pipelined ? TAURUS_OFF_XFER : 0, st>>>(X, ldx, n, K, Kp, src_begin, c->mode, c->d_row_ptr, out);
+  launch_early(c->early, af_prep_kernel, c->sm_count * 8, 256, c->pipelined ? TAURUS_OFF_XFER : 0, st, X, ldx, n, K, Kp, src_begin, c->mode,
+               (const long long*)c->d_row_ptr, out);
   c->launches += 1;
 }
 
@@ -171,7 +174,7 @@ int launch_af_finalise(taurus_ctx* c, const ChunkArgs& a, int layer, long long r
       fin.bias = a.bias; fin.act = a.act;
       int rc = launch_gemm_plain_tc(c, image, 0, a.Hout, c->d_af_A, Ka, Ka, (int)rows, O, a.Hout, st, &fin, &a.pc->done_count);
       if (rc) return rc;
-      if (!a.resident) launch_commit(c, a, st);
+      if (!a.resident) launch_commit(c, a, true, st);
       return TAURUS_OK;
     }
     if (tc) {
@@ -183,9 +186,9 @@ int launch_af_finalise(taurus_ctx* c, const ChunkArgs& a, int layer, long long r
       launch_gemm_plain_simt(c, c->d_Wcat[layer], taurus_proj_width(c->mode, a.Hout, c->heads), a.Hout, c->d_af_A, Ka, c->dims[layer], (int)rows, O,
                              a.Hout, st);
     }
-    af_finish_kernel<<<grid, 256, 0, st>>>(a, O, rows);
+    launch_early(c->early, af_finish_kernel, grid, 256, 0, st, a, (const float*)O, rows);
     c->launches += 1;
   }
-  if (!a.resident) launch_commit(c, a, st);
+  if (!a.resident) launch_commit(c, a, rows > 0, st);   // (with no row to transform, a wait for an event may be what comes before it)
   return TAURUS_OK;
 }

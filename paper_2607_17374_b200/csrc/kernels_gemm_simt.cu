@@ -119,12 +119,13 @@ void launch_project_simt(taurus_ctx* c, int layer, const float* X, int ldx, long
   const int N = taurus_proj_width(c->mode, Hp, c->heads);
   const int across = (N + BN - 1) / BN, tiles = (n + BM - 1) / BM * across;
   if (acc)
-    launch_early(acc->early, project_simt_kernel<true>, tiles + acc->blocks, 128, 0, st, X, ldx, c->dims[layer], (const float*)c->d_Wcat[layer], N, N, out, (long long)ldo, n, Hp,
+    launch_early(c->early, project_simt_kernel<true>, tiles + acc->blocks, 128, 0, st, X, ldx, c->dims[layer], (const float*)c->d_Wcat[layer], N, N, out, (long long)ldo, n, Hp,
                  c->mode, (const float*)c->d_bias[layer], (const long long*)c->d_row_ptr, (const int32_t*)c->d_din, c->fanout[layer], src_begin, across,
                  AccountArgs<true>{*acc});
   else
-    project_simt_kernel<false><<<tiles, 128, 0, st>>>(X, ldx, c->dims[layer], c->d_Wcat[layer], N, N, out, ldo, n, Hp, c->mode, c->d_bias[layer], c->d_row_ptr,
-                                                      c->d_din, c->fanout[layer], src_begin, across, AccountArgs<false>());
+    launch_early(c->early, project_simt_kernel<false>, tiles, 128, 0, st, X, ldx, c->dims[layer], (const float*)c->d_Wcat[layer], N, N, out, (long long)ldo, n, Hp,
+                 c->mode, (const float*)c->d_bias[layer], (const long long*)c->d_row_ptr, (const int32_t*)c->d_din, c->fanout[layer], src_begin, across,
+                 AccountArgs<false>());
   c->launches += 1;
 }
 

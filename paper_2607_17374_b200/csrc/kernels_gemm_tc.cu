@@ -565,7 +565,7 @@ void set_stages(GemmArgs& g, bool bf16) {
 }
 
 template <bool BF16, bool ACCOUNT>
-int launch_tc2(taurus_ctx* c, int grid, cudaStream_t st, const CUtensorMap& map_x, const CUtensorMap& map_b, const GemmArgs& g, const AccountArgs<ACCOUNT>& acc, bool early) {
+int launch_tc2(taurus_ctx* c, int grid, cudaStream_t st, const CUtensorMap& map_x, const CUtensorMap& map_b, const GemmArgs& g, const AccountArgs<ACCOUNT>& acc) {
   bool& set = c->tc_smem_set[ACCOUNT ? 1 : 0];   // once per context (the attribute belongs to the context's device)
   if (!set) {
     if (cudaFuncSetAttribute(project_tc_kernel<BF16, ACCOUNT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SHARED_BYTES) != cudaSuccess) {
@@ -574,17 +574,17 @@ int launch_tc2(taurus_ctx* c, int grid, cudaStream_t st, const CUtensorMap& map_
     }
     set = true;
   }
-  launch_early(early, project_tc_kernel<BF16, ACCOUNT>, grid, NUM_THREADS, SHARED_BYTES, st, map_x, map_b, g, acc);
+  launch_early(c->early, project_tc_kernel<BF16, ACCOUNT>, grid, NUM_THREADS, SHARED_BYTES, st, map_x, map_b, g, acc);
   return TAURUS_OK;
 }
 int launch_tc(taurus_ctx* c, int grid, cudaStream_t st, const CUtensorMap& map_x, const CUtensorMap& map_b, const GemmArgs& g, bool bf16,
               const AccountWork* acc = nullptr) {
   if (acc) {
     const AccountArgs<true> with{*acc};
-    return bf16 ? launch_tc2<true, true>(c, grid + acc->blocks, st, map_x, map_b, g, with, acc->early) : launch_tc2<false, true>(c, grid + acc->blocks, st, map_x, map_b, g, with, acc->early);
+    return bf16 ? launch_tc2<true, true>(c, grid + acc->blocks, st, map_x, map_b, g, with) : launch_tc2<false, true>(c, grid + acc->blocks, st, map_x, map_b, g, with);
   }
   const AccountArgs<false> without;
-  return bf16 ? launch_tc2<true, false>(c, grid, st, map_x, map_b, g, without, false) : launch_tc2<false, false>(c, grid, st, map_x, map_b, g, without, false);
+  return bf16 ? launch_tc2<true, false>(c, grid, st, map_x, map_b, g, without) : launch_tc2<false, false>(c, grid, st, map_x, map_b, g, without);
 }
 
 // Per-layer tensor-core images of Wcat, K-major: a row per output column.

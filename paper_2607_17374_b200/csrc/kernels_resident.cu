@@ -110,7 +110,6 @@ struct GatherArgs {
   long long* grad_ids;
   int d_out, act, mode, heads, head_vec;
   float gin_self, leaky;
-  bool early;                // launched while the kernel before it may still run
   long long room;            // rows that the graduation buffer holds, where they go there behind others
 };
 
@@ -162,8 +161,7 @@ template <int LPE, int VPL, int U, int D, int GAT>
 __global__ void __launch_bounds__(32 * G_WARPS, VPL == 1 ? 6 : VPL == 2 ? 5 : VPL == 4 ? 4 : 2) gather_kernel(const __grid_constant__ GatherArgs g, const __grid_constant__ ChunkArgs chunk) {
   extern __shared__ __align__(16) unsigned char g_smem[];
   ChunkCtl* const pc = g.pc;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // (the next push may come up, and waits in its turn)
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  early_start();
   if (g.ctl->error) return;
   if (blockIdx.x == 0) {   // a block for it: in the code of the others it would take registers
     if (threadIdx.x < 32) account_close(chunk, g.ctl, pc);
@@ -472,7 +470,7 @@ int launch_g(taurus_ctx* c, const GatherArgs& g, const ChunkArgs& a, long long b
   // no more warps than items: a completed vertex each, and the segments of long in-lists
   const long long items = bound + c->n_heavy_segments;
   const int grid = (int)std::max<long long>(1, std::min<long long>((items + G_WARPS - 1) / G_WARPS, (long long)c->sm_count * *per_sm));
-  const cudaError_t e = launch_early(g.early, gather_kernel<LPE, VPL, U, D, GAT>, grid + 1, 32 * G_WARPS, smem, st, g, a);   // the accounting has been enqueued: the push must not look as if nothing had happened
+  const cudaError_t e = launch_early(c->early, gather_kernel<LPE, VPL, U, D, GAT>, grid + 1, 32 * G_WARPS, smem, st, g, a);   // the accounting has been enqueued: the push must not look as if nothing had happened
   if (e != cudaSuccess) { taurus_note_cuda_error(e, "gather_kernel"); return TAURUS_ERR_CUDA; }
   return TAURUS_OK;
 }
@@ -811,7 +809,7 @@ void launch_store_rows(taurus_ctx* c, const float* X, long long ldx, int n, int 
                        const AccountWork* acc) {
   const int grid = (int)std::min<long long>(((long long)n * (ldo >> 2) + 255) / 256, (long long)c->sm_count * 8);
   if (acc)
-    launch_early(acc->early, store_and_account_kernel, grid + acc->blocks, 256, 0, st, X, ldx, n, K, src_begin, gcn ? 1 : 0, (const long long*)c->d_row_ptr, out, ldo,
+    launch_early(c->early, store_and_account_kernel, grid + acc->blocks, 256, 0, st, X, ldx, n, K, src_begin, gcn ? 1 : 0, (const long long*)c->d_row_ptr, out, ldo,
                  AccountArgs<true>{*acc});
   else
     store_rows_kernel<<<grid, 256, 0, st>>>(X, ldx, n, K, src_begin, gcn ? 1 : 0, c->d_row_ptr, out, ldo);
@@ -829,7 +827,6 @@ AccountWork account_work(const taurus_ctx* c, const ChunkArgs& a, long long cell
   w.i0 = cell >= 0 ? c->item_ptr[(size_t)cell] : 0;
   w.n_items = cell >= 0 ? c->item_ptr[(size_t)cell + 1] - w.i0 : 0;
   w.blocks = 0;
-  w.early = false;
   return w;
 }
 void launch_account(taurus_ctx* c, const ChunkArgs& a, long long cell, cudaStream_t st) {
@@ -847,9 +844,8 @@ void launch_account(taurus_ctx* c, const ChunkArgs& a, long long cell, cudaStrea
 }
 
 // Sums and finished rows of the vertices the push completed, at most `bound` (aggregate-first layers: sums into A).
-int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitch, float* A, long long bound, bool early, cudaStream_t st) {
+int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitch, float* A, long long bound, cudaStream_t st) {
   GatherArgs g;
-  g.early = early;
   const bool sampled = c->d_mask_cur != nullptr;
   g.rows = reinterpret_cast<const float4*>(rows); g.pitch = pitch >> 2; g.vec = a.Hp >> 2;
   g.csc_ptr = c->d_csc_ptr; g.src = sampled ? c->d_kept : c->d_csc_src; g.keep = sampled ? a.fanout : 0;

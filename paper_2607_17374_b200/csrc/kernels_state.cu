@@ -616,6 +616,7 @@ __global__ void __launch_bounds__(MR_THREADS, 1) make_room_kernel(ChunkArgs a) {
 // use both directions of the link at the same time.  Entries i >= deficit pop the free stack.  Either way
 // the vertex is IN_BUFFER afterwards.
 __global__ void alloc_kernel(ChunkArgs a) {
+  early_start();
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
   if (ctl->error) return;
@@ -834,7 +835,7 @@ int launch_make_room(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, cudaEve
 // Slots handed out, victims' rows staged, new rows cleared (S4, device side).
 void launch_alloc(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
   // bounded pools: one wave (46 registers), every block of which pays the chain of dependent reads once
-  alloc_kernel<<<c->sm_count * (a.direct ? 8 : 5), 256, 0, st>>>(a);
+  launch_early(c->early, alloc_kernel, c->sm_count * (a.direct ? 8 : 5), 256, 0, st, a);
   c->launches += 1;
 }
 // Rows across the host link (bounded pools only).
@@ -860,6 +861,7 @@ int launch_transfer(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
 static __device__ void commit_counts(const ChunkArgs& a, DevCtl* ctl, ChunkCtl* pc);
 // write_record: the last block to finish folds the chunk's counters into the layer totals.
 __global__ void compact_done_kernel(ChunkArgs a, int write_record) {
+  early_start();
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
   if (ctl->error) return;
@@ -1055,6 +1057,7 @@ static __device__ void commit_chunk(const ChunkArgs& a, DevCtl* ctl, ChunkCtl* p
   pc->grid_arrivals = 0; pc->done_blocks = 0; pc->final_blocks = 0; pc->room_go = 0; pc->room_fail = 0;
 }
 __global__ void commit_kernel(ChunkArgs a, int with_counts) {
+  early_start();
   if (threadIdx.x == 0) commit_chunk(a, a.ctl, a.pc, with_counts);
 }
 
@@ -1063,11 +1066,12 @@ void launch_compact_done(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st, boo
   // a warp takes 32 * CD_ITEMS entries per round: no more blocks than the longest list of any chunk can feed
   const long long need = (a.touched_capacity + 8 * 32 * CD_ITEMS - 1) / (8 * 32 * CD_ITEMS);
   const int blocks = (int)(need < 1 ? 1 : need < c->sm_count * 8 ? need : c->sm_count * 8);
-  compact_done_kernel<<<blocks, 256, c->pipelined ? TAURUS_OFF_XFER : 0, st>>>(a, write_record ? 1 : 0);
+  // (not early beside row transfers: its blocks would sit on the SMs that those are about to take; 20.2 / 21.2 ms a pass)
+  launch_early(c->early && !c->pipelined, compact_done_kernel, blocks, 256, c->pipelined ? TAURUS_OFF_XFER : 0, st, a, write_record ? 1 : 0);
   c->launches += 1;
 }
-void launch_commit(taurus_ctx* c, const ChunkArgs& a, cudaStream_t st) {
-  commit_kernel<<<1, 32, 0, st>>>(a, c->pipelined ? 0 : 1);
+void launch_commit(taurus_ctx* c, const ChunkArgs& a, bool behind_kernel, cudaStream_t st) {
+  launch_early(c->early && behind_kernel, commit_kernel, 1, 32, 0, st, a, c->pipelined ? 0 : 1);
   c->launches += 1;
 }
 

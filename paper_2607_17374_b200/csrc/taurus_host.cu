@@ -734,7 +734,6 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
     const ChunkArgs aa = make_args(c, src_begin, src_end);
     if (in_place && rows_with_account(c, aa, features, n, cell ? src_begin / c->chunk_sources : -1, &acc)) {
       if (aa.dense_half >= 0 && c->half_used[aa.dense_half]) { CU(cudaStreamWaitEvent(st, c->out_done[aa.dense_half], 0)); waits = true; }
-      acc.early = !waits && !pev;
     } else {
       CU(cudaEventRecord(c->account_go, st));   // everything of the chunk before this one
     }
@@ -756,6 +755,7 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
   }
   if (timing) cudaEventRecord(pev[1], st);
   ChunkArgs a = make_args(c, src_begin, src_end);
+  c->early = in_place && !waits && !pev;   // (behind the push before, or whatever the caller has put on the stream)
   if (c->resident) {
     // rows into the store, accounting, sums and finished rows of the vertices this chunk completes
     const bool af = c->agg_first[l];
@@ -777,9 +777,10 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
     if (xbuf >= 0) { CU(cudaEventRecord(c->x_free[xbuf], st)); c->x_used[xbuf] = true; }
     if (timing) cudaEventRecord(pev[2], st);
     if (!with) CU(cudaStreamWaitEvent(st, c->account_done, 0));
+    c->early = with && !pev;
     if (timing) cudaEventRecord(pev[3], st);
     if (scatter_timing) cudaEventRecord(pev[5], st);
-    { int rc = launch_gather(c, a, c->d_store, w, af ? c->d_af_A : nullptr, std::min<long long>(bound, a.grad_cap), with && !pev, st); if (rc) return rc; }
+    { int rc = launch_gather(c, a, c->d_store, w, af ? c->d_af_A : nullptr, std::min<long long>(bound, a.grad_cap), st); if (rc) return rc; }
     if (scatter_timing) cudaEventRecord(pev[6], st);
     if (timing) cudaEventRecord(pev[7], st);
     if (af) {
@@ -835,6 +836,7 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
   if (timing) cudaEventRecord(pev[2], st);
   // S3, S4
   *applied = true;
+  c->early = !pev;
   const bool grouped = c->d_gdst != nullptr && src_begin % c->chunk_sources == 0 &&
                        src_end == std::min<long long>(c->V, src_begin + c->chunk_sources);
   if (grouped) launch_classify_grouped(c, a, st); else launch_classify(c, a, st);
@@ -923,6 +925,7 @@ static int gat_project_core(taurus_ctx* c, int64_t src_begin, int64_t src_end, c
     CU(cudaStreamWaitEvent(st, c->order_event, 0));
     c->last_stream = st;
   }
+  c->early = false;
   const int n = (int)(src_end - src_begin);
   const int proj_w = taurus_proj_width(c->mode, Hp, c->heads);
   const float* X = nullptr;
