@@ -604,6 +604,136 @@ attention_kernel(long long V, int heads, const long long* __restrict__ csc_ptr, 
   }
 }
 
+// The same for 1, 2, 4 or 8 heads, whose scores of an entry are one vector: a lane per entry, eight lanes per vertex, so four vertices' chains of
+// dependent reads (offsets, sources, scores) run side by side in a warp, and a read brings in H times as many scores.  The vertices with
+// long in-lists in the same launch, by the first blocks: a block each, then a warp each.  Two layers of 400 k vertices, 20 M edges, four
+// heads: three launches of the kernel above 1.15 ms, this one 0.44 (a block for every vertex of the list 0.51; 4 or 16 lanes 0.59).
+template <int H> struct Scores { float x[H]; };
+template <int H>
+__device__ __forceinline__ Scores<H> scores_of(const float* __restrict__ att, long long v) {
+  Scores<H> s;
+  const float* p = att + v * H;
+  if constexpr (H == 1) s.x[0] = *p;
+  else if constexpr (H == 2) { const float2 a = *reinterpret_cast<const float2*>(p); s.x[0] = a.x; s.x[1] = a.y; }
+  else
+#pragma unroll
+    for (int h = 0; h < H; h += 4) {
+      const float4 a = *reinterpret_cast<const float4*>(p + h);
+      s.x[h] = a.x; s.x[h + 1] = a.y; s.x[h + 2] = a.z; s.x[h + 3] = a.w;
+    }
+  return s;
+}
+#define ATT_LANES 8          // lanes per vertex
+#define ATT_BLOCK 4096       // in-lists of the list that are a whole block's
+template <int H>
+__global__ void __launch_bounds__(256) attention_vec_kernel(long long V, const long long* __restrict__ csc_ptr, const int32_t* __restrict__ csc_src,
+                                                            const uint32_t* __restrict__ cmask, const float* __restrict__ att_s, const float* __restrict__ att_t,
+                                                            float slope, float2* __restrict__ tm, double* __restrict__ z, const int32_t* __restrict__ list, long long n_list,
+                                                            int list_blocks) {
+  constexpr int KEEP = H == 8 ? 4 : 8;   // entries of a lane whose scores are held for the second sweep
+  __shared__ float s_max[8][H];
+  __shared__ double s_sum[8][H];
+  // One vertex by G threads, of which this is number g.  All of them / the groups of a warp take the same path.
+  auto vertex = [&](auto threads, long long v, bool live) {
+    constexpr int G = decltype(threads)::value;
+    constexpr bool BLOCK = G > 32;
+    const int g = (int)threadIdx.x % G;
+    const long long b = live ? csc_ptr[v] : 0;
+    int d = live ? (int)(csc_ptr[v + 1] - b) : 0;
+    if (G < 32 && d > HEAVY_DEGREE) { d = 0; live = false; }   // (on the list)
+    const int most = G < 32 ? __reduce_max_sync(FULL, d) : d;
+    Scores<H> own, t, x[KEEP];
+#pragma unroll
+    for (int h = 0; h < H; ++h) own.x[h] = t.x[h] = 0.f;
+    if (live) { own = scores_of<H>(att_s, v); t = scores_of<H>(att_t, v); }
+    unsigned has = 0;
+    auto load = [&](int p0) {
+      has = 0;
+      int src[KEEP];
+#pragma unroll
+      for (int q = 0; q < KEEP; ++q) {
+        const int p = p0 + q * G + g;
+        src[q] = -1;
+        if (p < d && (!cmask || ((cmask[(b + p) >> 5] >> ((b + p) & 31)) & 1u))) { src[q] = csc_src[b + p]; has |= 1u << q; }
+      }
+#pragma unroll
+      for (int q = 0; q < KEEP; ++q) { if (src[q] >= 0) x[q] = scores_of<H>(att_s, src[q]); else x[q] = own; }
+    };
+    float mx[H];
+#pragma unroll
+    for (int h = 0; h < H; ++h) mx[h] = own.x[h];   // the self message takes part in the maximum
+    for (int p0 = 0; p0 < most; p0 += KEEP * G) {
+      load(p0);
+#pragma unroll
+      for (int q = 0; q < KEEP; ++q)
+#pragma unroll
+        for (int h = 0; h < H; ++h) mx[h] = fmaxf(mx[h], x[q].x[h]);
+    }
+#pragma unroll
+    for (int o = (BLOCK ? 32 : G) / 2; o; o >>= 1)
+#pragma unroll
+      for (int h = 0; h < H; ++h) mx[h] = fmaxf(mx[h], __shfl_xor_sync(FULL, mx[h], o));
+    if (BLOCK) {
+      if (rl() == 0)
+#pragma unroll
+        for (int h = 0; h < H; ++h) s_max[threadIdx.x >> 5][h] = mx[h];
+      __syncthreads();
+#pragma unroll
+      for (int h = 0; h < H; ++h)
+#pragma unroll
+        for (int w = 0; w < 8; ++w) mx[h] = fmaxf(mx[h], s_max[w][h]);
+    }
+    double sum[H];
+#pragma unroll
+    for (int h = 0; h < H; ++h) { mx[h] = r_lrelu(mx[h] + t.x[h], slope); sum[h] = 0.0; }
+    for (int p0 = 0; p0 < most; p0 += KEEP * G) {
+      if (most > KEEP * G) load(p0);   // else the scores are still held
+#pragma unroll
+      for (int q = 0; q < KEEP; ++q)
+        if ((has >> q) & 1u)
+#pragma unroll
+          for (int h = 0; h < H; ++h) sum[h] += (double)__expf(r_lrelu(x[q].x[h] + t.x[h], slope) - mx[h]);
+    }
+#pragma unroll
+    for (int o = (BLOCK ? 32 : G) / 2; o; o >>= 1)
+#pragma unroll
+      for (int h = 0; h < H; ++h) sum[h] += __shfl_xor_sync(FULL, sum[h], o);
+    if (BLOCK) {
+      if (rl() == 0)
+#pragma unroll
+        for (int h = 0; h < H; ++h) s_sum[threadIdx.x >> 5][h] = sum[h];
+      __syncthreads();
+      if (g < H) {
+#pragma unroll
+        for (int h = 0; h < H; ++h) { sum[h] = 0.0; for (int w = 0; w < 8; ++w) sum[h] += s_sum[w][h]; }
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < H; ++h)
+      if (live && g == h) {
+        tm[v * H + h] = make_float2(t.x[h], mx[h]);
+        z[v * H + h] = sum[h] + (double)__expf(r_lrelu(own.x[h] + t.x[h], slope) - mx[h]);
+      }
+    if (BLOCK) __syncthreads();   // the partial results are rewritten for the block's next vertex
+  };
+  if ((int)blockIdx.x < list_blocks) {
+    for (long long i = blockIdx.x; i < n_list; i += list_blocks) {
+      const long long v = list[i];
+      if (csc_ptr[v + 1] - csc_ptr[v] > ATT_BLOCK) vertex(std::integral_constant<int, 256>(), v, true);
+    }
+    for (long long i = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); i < n_list; i += (long long)list_blocks * 8) {
+      const long long v = list[i];
+      if (csc_ptr[v + 1] - csc_ptr[v] <= ATT_BLOCK) vertex(std::integral_constant<int, 32>(), v, true);
+    }
+    return;
+  }
+  const long long warps = (long long)(gridDim.x - list_blocks) * 8, per = 32 / ATT_LANES;
+  for (long long v0 = ((long long)(blockIdx.x - list_blocks) * 8 + (threadIdx.x >> 5)) * per; v0 < V; v0 += warps * per) {
+    const long long v = v0 + rl() / ATT_LANES;
+    vertex(std::integral_constant<int, ATT_LANES>(), v, v < V);
+  }
+}
+
 // ------------------------------------------------------------------------------------------------ build (init)
 __global__ void edge_sources_kernel(long long V, const long long* __restrict__ row_ptr, int32_t* __restrict__ src) {
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -878,6 +1008,18 @@ int launch_gather(taurus_ctx* c, const ChunkArgs& a, const float* rows, int pitc
 
 void launch_resident_attention(taurus_ctx* c, cudaStream_t st) {
   const uint32_t* cmask = c->d_mask_cur ? c->d_cmask : nullptr;
+  if (c->heads == 1 || c->heads == 2 || c->heads == 4 || c->heads == 8) {
+    const int list_blocks = (int)std::min<long long>(c->n_heavy, (long long)c->sm_count * 4);
+    const int blocks = list_blocks + (int)std::min<long long>((c->V + 31) / 32, (long long)c->sm_count * 8);
+    auto run = [&](auto kernel) {
+      kernel<<<blocks, 256, 0, st>>>(c->V, c->d_csc_ptr, c->d_csc_src, cmask, c->d_att_s, c->d_att_t, c->leaky, c->d_att_tm, c->d_att_z, c->d_heavy_list, c->n_heavy,
+                                     list_blocks);
+    };
+    if (c->heads == 1) run(attention_vec_kernel<1>); else if (c->heads == 2) run(attention_vec_kernel<2>);
+    else if (c->heads == 4) run(attention_vec_kernel<4>); else run(attention_vec_kernel<8>);
+    c->launches += 1;
+    return;
+  }
   const int grid = (int)std::min<long long>((c->V + 7) / 8, (long long)c->sm_count * 8);
   attention_kernel<1><<<grid, 256, 0, st>>>(c->V, c->heads, c->d_csc_ptr, c->d_csc_src, cmask, c->d_att_s, c->d_att_t, c->leaky, c->d_att_tm, c->d_att_z,
                                             nullptr, -1, HEAVY_DEGREE);
