@@ -508,6 +508,7 @@ extern "C" int taurus_layer_begin(taurus_ctx* c, int32_t layer, void* cuda_strea
   }
   if (c->rank_cum_cache[(size_t)layer].empty()) {
     // completion ranks depend only on the topology and the layer's edge mask: computed once per layer
+    ensure_edge_mask(c, st);
     launch_completion_ranks(c, st);
     CU(cudaGetLastError());
     const long long nb = (c->V + 63) / 64;
@@ -735,6 +736,7 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
     if (in_place && rows_with_account(c, aa, features, n, cell ? src_begin / c->chunk_sources : -1, &acc)) {
       if (aa.dense_half >= 0 && c->half_used[aa.dense_half]) { CU(cudaStreamWaitEvent(st, c->out_done[aa.dense_half], 0)); waits = true; }
     } else {
+      if (!cell) ensure_edge_mask(c, st);
       CU(cudaEventRecord(c->account_go, st));   // everything of the chunk before this one
     }
   }
@@ -1173,6 +1175,8 @@ extern "C" int taurus_get_edge_mask(taurus_ctx* c, uint32_t* out_words) {
   if (!c || !out_words) return TAURUS_ERR_INVALID_ARG;
   if (c->layer < 0) return TAURUS_ERR_ORDER;
   CU(cudaSetDevice(c->device));
+  ensure_edge_mask(c, c->last_stream);
+  CU(cudaGetLastError());
   CU(cudaStreamSynchronize(c->last_stream));
   size_t words = (size_t)((c->E + 31) / 32);
   if (c->d_mask_cur) CU(cudaMemcpy(out_words, c->d_mask_cur, words * sizeof(uint32_t), cudaMemcpyDeviceToHost));
@@ -1187,6 +1191,7 @@ extern "C" int taurus_get_sample_digest(taurus_ctx* c, uint64_t* out_digest) {
   if (!c || !out_digest) return TAURUS_ERR_INVALID_ARG;
   if (c->layer < 0) return TAURUS_ERR_ORDER;
   CU(cudaSetDevice(c->device));
+  ensure_edge_mask(c, c->last_stream);
   CU(cudaStreamSynchronize(c->last_stream));
   unsigned long long* d = nullptr;
   ALLOC(d, (size_t)2 * c->V);

@@ -319,6 +319,7 @@ struct taurus_ctx {
   int2* d_gedge = nullptr;        //   (destination, source - chunk start) pairs
   uint32_t* d_geid = nullptr;     //   CSR edge indices (kept only when some layer is sampled)
   uint32_t* d_gmask = nullptr;    // current layer's edge mask in grouped order
+  bool mask_built = false;        // d_mask holds the current layer's mask (resident pools build it when it is asked for)
   uint32_t* d_mask_cur = nullptr; // d_mask when the current layer is sampled, else NULL (every edge propagated)
   int32_t* d_vtmp = nullptr;     // [V] scratch for layer_begin
   int32_t* d_rank_hist = nullptr;
@@ -469,5 +470,6 @@ int build_in_edge_order(taurus_ctx* c);                                      // 
 int build_csc_ptr(taurus_ctx* c);                                            // csc_ptr alone
 int build_csc_src_from_eid(taurus_ctx* c);                                   // csc_src from csc_eid (both in in-list order)
 void launch_sample_mask(taurus_ctx* c, int layer, cudaStream_t st);
+void ensure_edge_mask(taurus_ctx* c, cudaStream_t st);                       // the layer's mask by CSR edge, where it has not been built
 int sampled_edges_of(taurus_ctx* c, int layer, long long dst, long long* out_eids, int32_t* out_src, int cap, int* n);
 void launch_sample_digest(taurus_ctx* c, unsigned long long* d_digest, cudaStream_t st);   // d_digest [2V], zeroed by the caller
