@@ -214,27 +214,42 @@ static __device__ __forceinline__ int sel_shift_of(unsigned long long lo, unsign
   return top >= TAURUS_SEL_BITS ? top - (TAURUS_SEL_BITS - 1) : 0;
 }
 
-// Minimum / maximum / count of the eligible keys a thread saw, folded into level `lvl` of the control block.
-static __device__ __forceinline__ void sel_fold(ChunkCtl* pc, int lvl, unsigned long long kmin, unsigned long long kmax, int cnt, bool with_count) {
+#define MR_THREADS 1024
+#define MR_ITEMS 2
+#define MR_TILE (MR_THREADS * MR_ITEMS)   // slots or candidates a block takes per step
+
+struct FoldShared { unsigned long long lo[32], hi[32]; int n[32]; };
+
+// Minimum / maximum / count of the eligible keys the threads of a block saw, folded into level `lvl` of the control block.  One atomic of each
+// kind per block: an address takes one every 3 ns, and three per warp of a pool of 162 k slots were 23 us of the 47 of a make-room step.
+static __device__ __forceinline__ void sel_fold(ChunkCtl* pc, int lvl, unsigned long long kmin, unsigned long long kmax, int cnt, bool with_count, FoldShared& s) {
   for (int o = 16; o; o >>= 1) {
     const unsigned long long m = __shfl_xor_sync(FULL, kmin, o), M = __shfl_xor_sync(FULL, kmax, o);
     if (m < kmin) kmin = m;
     if (M > kmax) kmax = M;
     cnt += __shfl_xor_sync(FULL, cnt, o);
   }
-  if (lane_id() == 0 && cnt) {
-    atomicMin(&pc->sel_min[lvl], kmin);
-    atomicMax(&pc->sel_max[lvl], kmax);
-    if (with_count) atomicAdd(&pc->sel_count[lvl], cnt);
+  __syncthreads();   // (its memory may have been in use for the fold before)
+  if (lane_id() == 0) { s.lo[threadIdx.x >> 5] = kmin; s.hi[threadIdx.x >> 5] = kmax; s.n[threadIdx.x >> 5] = cnt; }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    kmin = s.lo[threadIdx.x]; kmax = s.hi[threadIdx.x]; cnt = s.n[threadIdx.x];
+    for (int o = 16; o; o >>= 1) {
+      const unsigned long long m = __shfl_xor_sync(FULL, kmin, o), M = __shfl_xor_sync(FULL, kmax, o);
+      if (m < kmin) kmin = m;
+      if (M > kmax) kmax = M;
+      cnt += __shfl_xor_sync(FULL, cnt, o);
+    }
+    if (threadIdx.x == 0 && cnt) {
+      atomicMin(&pc->sel_min[lvl], kmin);
+      atomicMax(&pc->sel_max[lvl], kmax);
+      if (with_count) atomicAdd(&pc->sel_count[lvl], cnt);
+    }
   }
 }
 
-#define MR_THREADS 1024
-#define MR_ITEMS 2
-#define MR_TILE (MR_THREADS * MR_ITEMS)   // slots or candidates a block takes per step
-
 // Key of every slot; range and number of the eligible ones.
-static __device__ __forceinline__ void select_keys(const ChunkArgs& a, ChunkCtl* pc) {
+static __device__ __forceinline__ void select_keys(const ChunkArgs& a, ChunkCtl* pc, FoldShared& fold) {
   unsigned long long kmin = ~0ull, kmax = 0ull;
   int cnt = 0;
   for (long long base = (long long)blockIdx.x * MR_TILE; base < a.pool_slots; base += (long long)gridDim.x * MR_TILE) {
@@ -261,7 +276,7 @@ static __device__ __forceinline__ void select_keys(const ChunkArgs& a, ChunkCtl*
       a.keys[s] = key;
     }
   }
-  sel_fold(pc, 0, kmin, kmax, cnt, true);
+  sel_fold(pc, 0, kmin, kmax, cnt, true, fold);
 }
 
 // Histogram of the level's digit over the keys entering the level.  Threads of a warp that hit the same bin add
@@ -295,7 +310,7 @@ static __device__ __forceinline__ void select_hist(const ChunkArgs& a, ChunkCtl*
 // the level listed the last victims, 0 when another level follows, -1 when the selection cannot be completed; the
 // answer is the same in every block.
 static __device__ __forceinline__ int select_split(const ChunkArgs& a, ChunkCtl* pc, int level, int shift, unsigned int* sh, unsigned int* part,
-                                                   int* s_digit, long long* s_rest) {
+                                                   int* s_digit, long long* s_rest, FoldShared& fold) {
   const unsigned int* hist = pc->hist[level & 1];
   const long long k = pc->sel_k[level];
   constexpr int PER = TAURUS_SEL_BINS / MR_THREADS;   // consecutive bins per thread
@@ -341,40 +356,55 @@ static __device__ __forceinline__ int select_split(const ChunkArgs& a, ChunkCtl*
   unsigned long long kmin = ~0ull, kmax = 0ull;
   int cnt = 0;
   const unsigned lt = (1u << lane_id()) - 1;
+  // appended per block (one atomic a list and step): counts of the warps in part[0..63], then where each of them starts
   for (long long base = (long long)blockIdx.x * MR_TILE; base < n; base += (long long)gridDim.x * MR_TILE) {
+    int slot[MR_ITEMS];
+    unsigned long long key[MR_ITEMS];
+    unsigned mv[MR_ITEMS], mk[MR_ITEMS];
+    int wv = 0, wk = 0;
 #pragma unroll
     for (int j = 0; j < MR_ITEMS; ++j) {
       const long long i = base + j * MR_THREADS + threadIdx.x;
-      unsigned long long key = ~0ull;
-      int slot = -1;
-      if (i < n) { slot = level == 0 ? (int)i : cand[i]; key = a.keys[slot]; }
-      const bool on = key != ~0ull;
-      const int digit = on ? (int)((unsigned)(key >> shift) & (TAURUS_SEL_BINS - 1)) : TAURUS_SEL_BINS;
-      const bool victim = digit < digit_k || (final && digit == digit_k);
-      const bool keep = !final && digit == digit_k;
-      const unsigned mv = __ballot_sync(FULL, victim), mk = __ballot_sync(FULL, keep);
-      if (mv) {
-        int idx = 0;
-        const int leader = __ffs(mv) - 1;
-        if (lane_id() == leader) idx = atomicAdd(&pc->victim_count, __popc(mv));
-        idx = __shfl_sync(FULL, idx, leader) + __popc(mv & lt);
-        if (victim && idx < a.victim_capacity) a.victims[idx].x = slot;
+      key[j] = ~0ull;
+      slot[j] = -1;
+      if (i < n) { slot[j] = level == 0 ? (int)i : cand[i]; key[j] = a.keys[slot[j]]; }
+      const bool on = key[j] != ~0ull;
+      const int digit = on ? (int)((unsigned)(key[j] >> shift) & (TAURUS_SEL_BINS - 1)) : TAURUS_SEL_BINS;
+      mv[j] = __ballot_sync(FULL, digit < digit_k || (final && digit == digit_k));
+      mk[j] = __ballot_sync(FULL, !final && digit == digit_k);
+      wv += __popc(mv[j]);
+      wk += __popc(mk[j]);
+    }
+    __syncthreads();   // (part may still be read for the step before)
+    if (lane_id() == 0) { part[threadIdx.x >> 5] = (unsigned)wv; part[32 + (threadIdx.x >> 5)] = (unsigned)wk; }
+    __syncthreads();
+    if (threadIdx.x < 64) {   // two warps: victims, candidates
+      const unsigned own = part[threadIdx.x];
+      unsigned x = own;
+      for (int o = 1; o < 32; o <<= 1) { const unsigned y = __shfl_up_sync(FULL, x, o); if (lane_id() >= o) x += y; }
+      int at = 0;
+      if (lane_id() == 31 && x) at = atomicAdd(threadIdx.x < 32 ? &pc->victim_count : &pc->sel_count[level + 1], (int)x);
+      part[threadIdx.x] = (unsigned)__shfl_sync(FULL, at, 31) + x - own;
+    }
+    __syncthreads();
+    int iv = (int)part[threadIdx.x >> 5], ik = (int)part[32 + (threadIdx.x >> 5)];
+#pragma unroll
+    for (int j = 0; j < MR_ITEMS; ++j) {
+      if ((mv[j] >> lane_id()) & 1u) {
+        const int idx = iv + __popc(mv[j] & lt);
+        if (idx < a.victim_capacity) a.victims[idx].x = slot[j];
       }
-      if (mk) {
-        int idx = 0;
-        const int leader = __ffs(mk) - 1;
-        if (lane_id() == leader) idx = atomicAdd(&pc->sel_count[level + 1], __popc(mk));
-        idx = __shfl_sync(FULL, idx, leader) + __popc(mk & lt);
-        if (keep) {
-          next[idx] = slot;   // at most pool_slots keys enter any level
-          if (key < kmin) kmin = key;
-          if (key > kmax) kmax = key;
-          cnt++;
-        }
+      if ((mk[j] >> lane_id()) & 1u) {
+        next[ik + __popc(mk[j] & lt)] = slot[j];   // at most pool_slots keys enter any level
+        if (key[j] < kmin) kmin = key[j];
+        if (key[j] > kmax) kmax = key[j];
+        cnt++;
       }
+      iv += __popc(mv[j]);
+      ik += __popc(mk[j]);
     }
   }
-  sel_fold(pc, level + 1, kmin, kmax, cnt, false);   // the appends have counted the next level already
+  if (!final) sel_fold(pc, level + 1, kmin, kmax, cnt, false, fold);   // the appends have counted the next level already
   return final ? 1 : 0;
 }
 
@@ -411,7 +441,13 @@ static __device__ __forceinline__ void victim_bucket(const ChunkArgs& a, DevCtl*
     long long ns = next_sender(a, v);
     if (ns >= a.V) { atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL); ns = a.V - 1; }   // a victim has a message to come
     const int b = (int)(ns / a.chunk_sources);
-    a.vic_place[i] = make_int2(b, atomicAdd(&a.bk_new[b], 1));
+    // rank in the bucket: the victims of a warp that share one ask together (a fifth of them may be filed under the next chunk)
+    const unsigned here = __activemask(), peers = __match_any_sync(here, b);
+    const int first = __ffs(peers) - 1;
+    int at = 0;
+    if (lane_id() == first) at = atomicAdd(&a.bk_new[b], __popc(peers));
+    at = __shfl_sync(peers, at, first) + __popc(peers & ((1u << lane_id()) - 1));
+    a.vic_place[i] = make_int2(b, at);
   }
 }
 
@@ -561,7 +597,8 @@ __global__ void __launch_bounds__(MR_THREADS, 1) make_room_kernel(ChunkArgs a) {
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
   __shared__ unsigned int sh[TAURUS_SEL_BINS];
-  __shared__ unsigned int part[32];
+  __shared__ unsigned int part[64];
+  __shared__ FoldShared fold;
   __shared__ int s_digit, s_ok;
   __shared__ long long s_rest;
   unsigned int round = 0;
@@ -579,7 +616,7 @@ __global__ void __launch_bounds__(MR_THREADS, 1) make_room_kernel(ChunkArgs a) {
     if (blockIdx.x == 0) extent_plan(a, ctl, 0);
     return;
   }
-  select_keys(a, pc);
+  select_keys(a, pc, fold);
   if (!grid_barrier(ctl, pc, round, &s_ok)) return;
   for (int level = 0;; ++level) {
     if ((long long)pc->sel_count[level] < pc->sel_k[level]) {   // fewer eligible victims than needed
@@ -589,7 +626,7 @@ __global__ void __launch_bounds__(MR_THREADS, 1) make_room_kernel(ChunkArgs a) {
     const int shift = sel_shift_of(pc->sel_min[level], pc->sel_max[level]);
     select_hist(a, pc, level, shift, sh);
     if (!grid_barrier(ctl, pc, round, &s_ok)) return;
-    const int done = select_split(a, pc, level, shift, sh, part, &s_digit, &s_rest);
+    const int done = select_split(a, pc, level, shift, sh, part, &s_digit, &s_rest, fold);
     if (done < 0) {
       if (blockIdx.x == 0 && threadIdx.x == 0) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
       return;
