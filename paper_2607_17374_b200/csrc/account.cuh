@@ -199,13 +199,7 @@ __device__ __forceinline__ void account_block(const AccountWork& work, AccountSh
   if (threadIdx.x < C_COUNT && s.sum[threadIdx.x]) atomicAdd(&pc->acc[threadIdx.x], (unsigned long long)s.sum[threadIdx.x]);
 }
 
-// After the accounting of a chunk, once, by one warp of the kernel behind it (the gather, which every push has): the chunk record, the layer's
-// totals, the free-slot count and the count of waiting rows, and the counters of the next chunk (the other set; its last reader, the chunk
-// before this one, is through) are cleared.  By the accounting's last block to finish it was 1.7 us on the way of every push.
-__device__ __forceinline__ void account_close(const ChunkArgs& a, DevCtl* ctl, ChunkCtl* pc) {
-  ChunkCtl* next = pc == &ctl->pc[0] ? &ctl->pc[1] : &ctl->pc[0];
-  for (int i = rl(); i < (int)(offsetof(ChunkCtl, sel_k) / 4); i += 32) reinterpret_cast<int32_t*>(next)[i] = 0;
-  if (rl() != 0) return;
+__device__ __forceinline__ void account_totals(const ChunkArgs& a, DevCtl* ctl, ChunkCtl* pc) {   // one thread
   long long c[C_COUNT];
   for (int k = 0; k < C_COUNT; ++k) c[k] = (long long)pc->acc[k];
   const long long done = pc->done_count;
@@ -227,6 +221,22 @@ __device__ __forceinline__ void account_close(const ChunkArgs& a, DevCtl* ctl, C
   else {
     if (grad + done > a.drain_rows) atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
     ctl->grad_count = grad + done;
+  }
+}
+// After the accounting of a chunk, once, by one warp of the kernel behind it (the gather, which every push has): the chunk record, the layer's
+// totals, the free-slot count and the count of waiting rows, and the counters of the next chunk (the other set; its last reader, the chunk
+// before this one, is through) are cleared.  By the accounting's last block to finish it was 1.7 us on the way of every push.
+__device__ __forceinline__ void account_close(const ChunkArgs& a, DevCtl* ctl, ChunkCtl* pc) {
+  if (!ctl->error) {
+    ChunkCtl* next = pc == &ctl->pc[0] ? &ctl->pc[1] : &ctl->pc[0];
+    for (int i = rl(); i < (int)(offsetof(ChunkCtl, sel_k) / 4); i += 32) reinterpret_cast<int32_t*>(next)[i] = 0;
+    __syncwarp();
+    if (rl() == 0) account_totals(a, ctl, pc);
+  }
+  if (a.report) {   // what layer_end would otherwise launch a kernel for
+    __threadfence();
+    __syncwarp();
+    report_ctl(ctl, a.report, rl(), 32);
   }
 }
 

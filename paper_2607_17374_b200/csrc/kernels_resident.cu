@@ -162,11 +162,11 @@ __global__ void __launch_bounds__(32 * G_WARPS, VPL == 1 ? 6 : VPL == 2 ? 5 : VP
   extern __shared__ __align__(16) unsigned char g_smem[];
   ChunkCtl* const pc = g.pc;
   early_start();
-  if (g.ctl->error) return;
   if (blockIdx.x == 0) {   // a block for it: in the code of the others it would take registers
     if (threadIdx.x < 32) account_close(chunk, g.ctl, pc);
     return;
   }
+  if (g.ctl->error) return;
   constexpr int EPS = 32 / LPE, STEP = U * EPS;
   static_assert(STEP <= 32 && 32 % STEP == 0, "a block of 32 sources is a whole number of steps");
   typedef Ring<VPL, U, D, GAT> R;

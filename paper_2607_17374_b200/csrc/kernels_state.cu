@@ -1141,12 +1141,7 @@ __global__ void place_rows_kernel(const long long* ids, const float* rows, int H
   place_rows(ids, rows, Hp, d_out, dense, ld, count);
 }
 
-// The words of the control block in front of the chunks' counters, to pinned host memory: what a blocking call waits for.
-#define CTL_WORDS ((int)(offsetof(DevCtl, pc) / 8))
-static __device__ __forceinline__ void report_ctl(const DevCtl* ctl, long long* report) {
-  for (int i = threadIdx.x; i < CTL_WORDS; i += blockDim.x) report[i] = __ldcg(reinterpret_cast<const long long*>(ctl) + i);
-}
-__global__ void report_kernel(const DevCtl* ctl, long long* report) { report_ctl(ctl, report); }
+__global__ void report_kernel(const DevCtl* ctl, long long* report) { report_ctl(ctl, report, threadIdx.x, blockDim.x); }
 
 // A drain into a matrix, in one launch and one wait: the rows that wait (if they fit and no error has been found) are placed, the last block
 // to finish reports the control block as it was and then empties the buffer.  The count stays on the device until then: asked for
@@ -1164,7 +1159,7 @@ __global__ void drain_rows_kernel(DevCtl* ctl, const long long* ids, const float
   }
   __syncthreads();
   if (!last) return;
-  report_ctl(ctl, report);
+  report_ctl(ctl, report, threadIdx.x, blockDim.x);
   __syncthreads();
   if (threadIdx.x == 0) {
     if (go) ctl->grad_count = 0;

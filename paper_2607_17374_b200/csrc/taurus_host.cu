@@ -466,9 +466,11 @@ static int finish_chunk(taurus_ctx* c, cudaStream_t st);
 static int sticky_error(const taurus_ctx* c) { return c->half_applied ? c->half_applied : c->h_ctl->error; }
 static int read_ctl(taurus_ctx* c, cudaStream_t st, bool with_stats = false) {
   { int rc = finish_chunk(c, st); if (rc) return rc; }   // the last chunk's finalise may still be waiting for a successor
-  if (with_stats) launch_reload_histogram(c, st);
-  launch_report(c, st);
-  CU(cudaGetLastError());
+  if (!c->reported) {
+    if (with_stats) launch_reload_histogram(c, st);
+    launch_report(c, st);
+    CU(cudaGetLastError());
+  }
   CU(cudaStreamSynchronize(st));
   CU(cudaStreamSynchronize(c->out_stream));
   return sticky_error(c);
@@ -489,6 +491,7 @@ extern "C" int taurus_layer_begin(taurus_ctx* c, int32_t layer, void* cuda_strea
     if (c->account_stream) CU(cudaStreamSynchronize(c->account_stream));   // (a push that failed half way leaves it unjoined)
   }
   c->quiet = false;
+  c->reported = false;
   c->pending = false;   // an abandoned layer's last chunk is dropped with it
   c->layer = layer;
   c->dense_out = nullptr; c->dense_ld = 0;
@@ -573,6 +576,7 @@ static ChunkArgs make_args(taurus_ctx* c, long long s, long long e) {
   a.dense_ld = c->dense_ld;
   a.d_out = c->dims[l + 1];
   a.Hout = a.Hp; a.self_rows = 1; a.self_bias = 1;
+  a.report = c->resident && e == c->V && !c->agg_first[l] && !c->timing ? reinterpret_cast<long long*>(c->h_ctl) : nullptr;   // (the finish of an aggregate-first layer comes after)
   a.dense_half = halves ? (int)(c->chunk_seq & 1) : -1;
   a.grad_cap = halves ? c->drain_rows / 2 : c->drain_rows;
   a.grad_off = halves ? (long long)a.dense_half * (c->drain_rows / 2) : 0;
@@ -789,6 +793,7 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
       int rc = launch_af_finalise(c, a, l, std::min<long long>(bound, a.grad_cap), st);
       if (rc) return rc;
     }
+    c->reported = a.report != nullptr;
     const int rc = hand_off(c, a, l, bound, st);
     if (timing) cudaEventRecord(pev[9], st);
     CU(cudaGetLastError());
@@ -1016,6 +1021,7 @@ static int drain_common(taurus_ctx* c, long long capacity, long long* out_count,
 }
 
 static int drain_reset(taurus_ctx* c) {
+  c->reported = false;
   CU(cudaMemsetAsync(reinterpret_cast<char*>(c->d_ctl) + offsetof(DevCtl, grad_count), 0, sizeof(long long), c->last_stream));
   CU(cudaStreamSynchronize(c->last_stream));
   c->ub_since_drain = 0;
@@ -1054,6 +1060,7 @@ extern "C" int taurus_drain_dense(taurus_ctx* c, float* dense_rows, int64_t ld, 
     cudaStream_t st = c->last_stream;
     { int rc = finish_chunk(c, st); if (rc) return rc; }
     const int d_out = c->dims[c->layer + 1];
+    c->reported = false;   // (the drain reports itself, and changes the count of waiting rows after it)
     launch_drain_rows(c, dense_dev, ld, d_out, taurus_round_up(d_out, 4), c->ub_since_drain, capacity_rows, st);
     CU(cudaGetLastError());
     CU(cudaStreamSynchronize(st));

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include <vector>
@@ -177,6 +178,7 @@ struct ChunkArgs {
   int32_t Hout;             // padded output width (= Hp for project-first layers)
   int32_t self_rows;        // 1: the scatter adds a self row; 0: it only counts the self message (the self term is added after the transform)
   int32_t resident;         // 1: resident pool, the account kernel has done the graduation bookkeeping
+  long long* report;        // resident pools, last push of a layer whose control block is final with its gather: pinned host memory that takes it, else NULL
   int32_t self_bias;        // 1: the self row carries the bias (project-first); 0: the bias is added after the transform
 };
 
@@ -330,6 +332,7 @@ struct taurus_ctx {
   // host bookkeeping
   int layer = -1;
   bool quiet = false;                // nothing has been enqueued since a blocking call of the layer ended
+  bool reported = false;             // h_ctl has (or, once the stream is through, will have) the control block as the layer left it
   bool early = false;                // the next kernel of the push may be launched early (launch_early): a kernel is what comes before it on the stream
   int half_applied = 0;              // code of a push that failed with its chunk enqueued in part; cleared by taurus_layer_begin
   long long next_src = 0;
@@ -377,6 +380,14 @@ static inline cudaError_t launch_early(bool early, void (*kernel)(P...), int gri
   cfg.attrs = &at; cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
+
+// The words of the control block in front of the chunks' counters, to pinned host memory: what a blocking call waits for.
+#define CTL_WORDS ((int)(offsetof(DevCtl, pc) / 8))
+#ifdef __CUDACC__
+static __device__ __forceinline__ void report_ctl(const DevCtl* ctl, long long* report, int thread, int threads) {
+  for (int i = thread; i < CTL_WORDS; i += threads) report[i] = __ldcg(reinterpret_cast<const long long*>(ctl) + i);
+}
+#endif
 
 // ---- kernels_state.cu
 void launch_layer_reset(taurus_ctx* c, int layer, cudaStream_t st);

@@ -49,3 +49,43 @@ def test_rows_written_and_overwritten_on_the_stream(fanout):
                     bufs[k].fill_(float("nan"))
             assert ctx.layer_end()["completed"] == V
         assert row_error(out.cpu().numpy(), want)[0] <= 1e-4
+
+
+@pytest.mark.parametrize("dims,fanout", [((64, 64), 0), ((24, 72), 0), ((64, 32), 4)])
+def test_what_blocking_calls_find_after_the_last_push(dims, fanout):
+    """The last push of a layer reports the control block by itself: statistics, drains, layer_end and another drain after it, in several orders."""
+    import numpy as np
+    import torch
+    import paper_2607_17374_b200 as tb
+    V, chunk = 5_000, 1_000
+    w = replace(tg.scaled(tg.WORKLOADS["large"], V, chunk=chunk), dims=dims, fanout=(fanout,), pool_slots=V, hub_count=5)
+    g, m = tg.make_graph(w), tg.make_model(w, bias_scale=0.3)
+    x = torch.from_numpy(tg.features(w.seed, 0, 0, V, dims[0])).cuda()
+    ctx = tb.Context(V, g.E, g.row_ptr, g.col_idx, g.in_degree, w.mode, w.dims, m.W_neigh, m.W_self, m.bias, m.act, chunk, V, 5, w.fanout, w.seed, 0, V + 1_024)
+    out = torch.empty(V, dims[1], device="cuda")
+    ids, rows = torch.empty(V, dtype=torch.int64, device="cuda"), torch.empty(V, dims[1], device="cuda")
+    seen = []
+    for order in range(5):
+        ctx.layer_begin(0)
+        if order == 4:
+            ctx.layer_set_dense_output(out, dims[1])
+        for b in range(0, V, chunk):
+            ctx.push_chunk(b, b + chunk, x[b:b + chunk])
+            if order == 0 and b == 2 * chunk:
+                first = ctx.drain_dense(out, dims[1], V)
+        if order == 0:
+            assert ctx.get_stats()["completed"] == V
+            assert ctx.drain_dense(out, dims[1], V) + first == V and ctx.drain_dense(out, dims[1], V) == 0
+        elif order == 1:
+            assert ctx.drain_completed(ids, rows, V) == V and ctx.drain_completed(ids, rows, V) == 0
+        elif order == 2:
+            assert ctx.get_stats()["completed"] == V and ctx.layer_end()["completed"] == V
+            assert ctx.drain_dense(out, dims[1], V) == V and ctx.drain_completed(ids, rows, V) == 0
+        elif order == 3:
+            with pytest.raises(tb.TaurusError):
+                ctx.drain_dense(out, dims[1], V - 1)
+            assert ctx.drain_dense(out, dims[1], V, ids) == V and sorted(ids.tolist()) == list(range(V))
+        st = ctx.layer_end()
+        assert st["completed"] == V and st["chunks"] == V // chunk and st["free_slots"] == V
+        seen.append({k: v for k, v in st.items()})
+    assert all(s == seen[0] for s in seen)
