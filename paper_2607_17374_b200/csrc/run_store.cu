@@ -30,6 +30,15 @@ struct MoveSeg { long long src, n, dst; };   // src: position in the grouped ind
 
 constexpr int SEG_RING = 8;
 
+// Pieces of one launch: in the launch itself while they fit (a table in memory is a copy, an event and a slot of a ring on top: some
+// 10 us of the host's time and 4 of the stream's, two or three times a chunk), else in memory.
+constexpr int SEGS_INLINE = 64;
+struct Segs {
+  const MoveSeg* table;            // NULL: the pieces are here
+  MoveSeg s[SEGS_INLINE];
+  __device__ __forceinline__ MoveSeg at(int i) const { return table ? table[i] : s[i]; }
+};
+
 __device__ __forceinline__ int rs_lane() { return threadIdx.x & 31; }
 
 __device__ __forceinline__ void copy_row(float* __restrict__ dst, const float* __restrict__ src, int width) {
@@ -70,11 +79,100 @@ __global__ void rs_key_kernel(const long long* __restrict__ ids, long long n_bou
   if (blockIdx.x == 0 && threadIdx.x == 0) cnt[P] = count;
 }
 
+// The same, and the grouping, for up to GROUP_RANGES ranges: two launches where a radix sort with its passes, the key kernel, a memset and a
+// copy of the counts were up to ten.  rs_count_kernel: rows per tile and range; its last block to finish adds them up, writes where
+// every range starts, and the totals straight to pinned host memory.  rs_group_kernel: every tile finds its places from the
+// tiles before it and writes them in row order, so the grouping is stable, like the sort.  500 k vertices, 128-128-64 through runs of 16 ranges:
+// 4.10 -> 3.55 ms a pass with the pieces in the launches (tiles of 512 and 2 048 rows 3.55, 3.59).
+constexpr int GROUP_RANGES = 64, GROUP_TILE = 1024, GROUP_MAX = 16384;   // GROUP_MAX: tiles x ranges, what a tile reads to find its places
+__device__ __forceinline__ int rs_range(const long long* __restrict__ ids, long long i, long long count, long long V, long long range_ids, int P) {
+  if (i >= count) return P;
+  const long long id = ids[i];
+  return id < 0 || id >= V ? P + 1 : (int)(id / range_ids);
+}
+__global__ void __launch_bounds__(256) rs_count_kernel(const long long* __restrict__ ids, long long n_bound, const long long* d_count, long long count_host, long long V,
+                                                       long long range_ids, int P, int32_t* __restrict__ tile_cnt, long long* __restrict__ start, unsigned int* ticket,
+                                                       long long* __restrict__ report) {
+  __shared__ unsigned int sh[GROUP_RANGES + 2];
+  __shared__ long long total[GROUP_RANGES + 2];
+  __shared__ int last;
+  if (threadIdx.x < GROUP_RANGES + 2) sh[threadIdx.x] = 0;
+  __syncthreads();
+  const long long given = d_count ? *d_count : count_host, count = given < n_bound ? given : n_bound;
+  const long long first = (long long)blockIdx.x * GROUP_TILE;
+#pragma unroll
+  for (int j = 0; j < GROUP_TILE / 256; ++j) {
+    const int k = rs_range(ids, first + j * 256 + threadIdx.x, count, V, range_ids, P);
+    const unsigned peers = __match_any_sync(0xffffffffu, k);
+    if (k != P && rs_lane() == __ffs(peers) - 1) atomicAdd(&sh[k], (unsigned)__popc(peers));
+  }
+  __syncthreads();
+  for (int p = threadIdx.x; p < P + 2; p += 256) tile_cnt[(long long)blockIdx.x * (P + 2) + p] = (int32_t)sh[p];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int p = threadIdx.x >> 5; p < P + 2; p += 8) {
+    long long t = 0;
+    for (unsigned b = rs_lane(); b < gridDim.x; b += 32) t += __ldcg(&tile_cnt[(long long)b * (P + 2) + p]);
+    for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (rs_lane() == 0) total[p] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    long long at = 0;
+    for (int p = 0; p < P; ++p) { start[p] = at; at += total[p]; report[p] = total[p]; }
+    report[P] = count;
+    report[P + 1] = total[P + 1] + (given > n_bound ? 1 : 0);
+    *ticket = 0;
+  }
+}
+__global__ void __launch_bounds__(256) rs_group_kernel(const long long* __restrict__ ids, long long n_bound, const long long* d_count, long long count_host, long long V,
+                                                       long long range_ids, int P, const int32_t* __restrict__ tile_cnt, const long long* __restrict__ start,
+                                                       int32_t* __restrict__ idx_s) {
+  __shared__ long long base[GROUP_RANGES];
+  __shared__ int warp_cnt[8][GROUP_RANGES];
+  const long long given = d_count ? *d_count : count_host, count = given < n_bound ? given : n_bound;
+  const long long first = (long long)blockIdx.x * GROUP_TILE;
+  if (first >= count) return;
+  const int warp = threadIdx.x >> 5;
+  for (int p = warp; p < P; p += 8) {   // rows of the tiles before this one
+    long long t = 0;
+    for (unsigned b = rs_lane(); b < blockIdx.x; b += 32) t += tile_cnt[(long long)b * (P + 2) + p];
+    for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (rs_lane() == 0) base[p] = start[p] + t;
+  }
+  for (int j = 0; j < GROUP_TILE / 256; ++j) {
+    for (int t = threadIdx.x; t < 8 * GROUP_RANGES; t += 256) (&warp_cnt[0][0])[t] = 0;
+    __syncthreads();
+    const long long i = first + j * 256 + threadIdx.x;
+    const int k = rs_range(ids, i, count, V, range_ids, P);
+    const unsigned peers = __match_any_sync(0xffffffffu, k);
+    const int rank = __popc(peers & ((1u << rs_lane()) - 1));
+    if (k < P && rank == 0) warp_cnt[warp][k] = __popc(peers);
+    __syncthreads();
+    if (k < P) {
+      int before = 0;
+      for (int w = 0; w < warp; ++w) before += warp_cnt[w][k];
+      idx_s[base[k] + before + rank] = (int32_t)i;
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < P) {
+      int t = 0;
+      for (int w = 0; w < 8; ++w) t += warp_cnt[w][threadIdx.x];
+      base[threadIdx.x] += t;
+    }
+    __syncthreads();
+  }
+}
+
 // One piece per range: rows idx_s[src .. src + n) of the append go to partition-buffer rows dst .. dst + n.
-__global__ void rs_move_kernel(const MoveSeg* __restrict__ segs, const int32_t* __restrict__ idx_s, const long long* __restrict__ ids,
+__global__ void rs_move_kernel(const __grid_constant__ Segs segs, const int32_t* __restrict__ idx_s, const long long* __restrict__ ids,
                                const float* __restrict__ rows, long long ld, int width, int32_t* __restrict__ pids,
                                float* __restrict__ prows) {
-  const MoveSeg sg = segs[blockIdx.y];
+  const MoveSeg sg = segs.at((int)blockIdx.y);
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < sg.n; i += warps) {
     const long long r = idx_s[sg.src + i];
@@ -84,9 +182,9 @@ __global__ void rs_move_kernel(const MoveSeg* __restrict__ segs, const int32_t* 
 }
 
 // Buffers that leave together: ids of piece q go to fkeys[dst ..], their partition-buffer row numbers to fvals[dst ..].
-__global__ void rs_collect_kernel(const MoveSeg* __restrict__ segs, const int32_t* __restrict__ pids, int32_t* __restrict__ fkeys,
+__global__ void rs_collect_kernel(const __grid_constant__ Segs segs, const int32_t* __restrict__ pids, int32_t* __restrict__ fkeys,
                                   int32_t* __restrict__ fvals) {
-  const MoveSeg sg = segs[blockIdx.y];
+  const MoveSeg sg = segs.at((int)blockIdx.y);
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < sg.n; i += stride) {
     fkeys[sg.dst + i] = pids[sg.src + i];
@@ -114,9 +212,9 @@ __global__ void rs_place_kernel(long long n, const int32_t* __restrict__ sid, co
 
 // The same for a store in device memory: slice q of the chunk (rows src .. src + n of the store, ids beside them) is read
 // in place, without staging copies (one small copy of ids per slice took 2.6 us of the stream, thirty a chunk).
-__global__ void rs_place_slices_kernel(const MoveSeg* __restrict__ segs, const int32_t* __restrict__ ids, const float* __restrict__ store,
+__global__ void rs_place_slices_kernel(const __grid_constant__ Segs segs, const int32_t* __restrict__ ids, const float* __restrict__ store,
                                        int width, long long s, float* __restrict__ out, long long ld) {
-  const MoveSeg sg = segs[blockIdx.y];
+  const MoveSeg sg = segs.at((int)blockIdx.y);
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < sg.n; i += warps)
     copy_row(out + (size_t)(ids[sg.src + i] - s) * ld, store + (size_t)(sg.src + i) * width, width);
@@ -148,6 +246,9 @@ struct taurus_runs {
   // append scratch
   int32_t *d_key = nullptr, *d_key_s = nullptr, *d_idx = nullptr, *d_idx_s = nullptr;
   long long* d_cnt = nullptr;
+  int32_t* d_tile_cnt = nullptr;   // rows per tile and range (rs_count_kernel), with the ticket of its blocks and the starts of the ranges
+  long long* d_start = nullptr;
+  unsigned int* d_ticket = nullptr;
   long long* h_cnt = nullptr;    // pinned
   MoveSeg* d_segs = nullptr;     // SEG_RING tables of P pieces
   MoveSeg* h_segs = nullptr;     // pinned
@@ -201,7 +302,7 @@ extern "C" void taurus_runs_destroy(taurus_runs* r) {
   cudaFree(r->d_pids); cudaFree(r->d_prows);
   if (r->kind == TAURUS_RUNS_HOST) cudaFreeHost(r->store_host); else cudaFree(r->store_dev);
   cudaFreeHost(r->h_ids); cudaFreeHost(r->h_cnt); cudaFreeHost(r->h_segs);
-  cudaFree(r->d_key); cudaFree(r->d_key_s); cudaFree(r->d_idx); cudaFree(r->d_idx_s); cudaFree(r->d_cnt); cudaFree(r->d_segs);
+  cudaFree(r->d_key); cudaFree(r->d_key_s); cudaFree(r->d_idx); cudaFree(r->d_idx_s); cudaFree(r->d_cnt); cudaFree(r->d_segs); cudaFree(r->d_tile_cnt); cudaFree(r->d_start);
   cudaFree(r->d_fkeys); cudaFree(r->d_fvals); cudaFree(r->d_sid); cudaFree(r->d_sidx); cudaFree(r->d_tmp);
   cudaFree(r->d_stage_rows); cudaFree(r->d_stage_ids); cudaFree(r->d_ids);
   for (int i = 0; i < SEG_RING; ++i) if (r->seg_done[i]) cudaEventDestroy(r->seg_done[i]);
@@ -245,6 +346,12 @@ extern "C" int taurus_runs_create(taurus_runs** out, const taurus_runs_config* c
   if (r->kind == TAURUS_RUNS_DEVICE) RALLOC(r->d_ids, r->store_rows);
   RALLOC(r->d_key, r->max_append); RALLOC(r->d_key_s, r->max_append); RALLOC(r->d_idx, r->max_append); RALLOC(r->d_idx_s, r->max_append);
   RALLOC(r->d_cnt, r->P + 2);
+  if (r->P <= GROUP_RANGES) {
+    RALLOC(r->d_tile_cnt, std::min<long long>(GROUP_MAX / r->P, (r->max_append + GROUP_TILE - 1) / GROUP_TILE) * (r->P + 2));
+    RALLOC(r->d_start, GROUP_RANGES + 1);
+    r->d_ticket = reinterpret_cast<unsigned int*>(r->d_start + GROUP_RANGES);
+    if (cudaMemset(r->d_ticket, 0, sizeof(long long)) != cudaSuccess) { cudaGetLastError(); taurus_runs_destroy(r); return TAURUS_ERR_CUDA; }
+  }
   RPINNED(r->h_cnt, (size_t)r->P + 2);
   RALLOC(r->d_segs, (size_t)SEG_RING * r->P);
   RPINNED(r->h_segs, (size_t)SEG_RING * r->P);
@@ -280,6 +387,17 @@ int runs_phase1(taurus_runs* r, const long long* ids, const float* rows, long lo
                 long long count_host, cudaStream_t st) {
   if (r->pending) return TAURUS_ERR_ORDER;
   if (n_bound < 0 || n_bound > r->max_append || ld < r->width) return TAURUS_ERR_INVALID_ARG;
+  const long long tiles = (n_bound + GROUP_TILE - 1) / GROUP_TILE;
+  if (n_bound > 0 && r->P <= GROUP_RANGES && tiles * r->P <= GROUP_MAX) {
+    rs_count_kernel<<<(int)tiles, 256, 0, st>>>(ids, n_bound, d_count, count_host, r->V, r->range_ids, (int)r->P, r->d_tile_cnt, r->d_start, r->d_ticket, r->h_cnt);
+    RCU(cudaEventRecord(r->cnt_ready, st));
+    rs_group_kernel<<<(int)tiles, 256, 0, st>>>(ids, n_bound, d_count, count_host, r->V, r->range_ids, (int)r->P, r->d_tile_cnt, r->d_start, r->d_idx_s);
+    RCU(cudaGetLastError());
+    r->launches += 2;
+    r->p_ids = ids; r->p_rows = rows; r->p_ld = ld;
+    r->pending = true;
+    return TAURUS_OK;
+  }
   RCU(cudaMemsetAsync(r->d_cnt, 0, (size_t)(r->P + 2) * sizeof(long long), st));
   if (n_bound > 0) {
     const int grid = (int)std::min<long long>((n_bound + 255) / 256, (long long)r->sm_count * 8);
@@ -296,27 +414,40 @@ int runs_phase1(taurus_runs* r, const long long* ids, const float* rows, long lo
   return TAURUS_OK;
 }
 
-// One slot of the piece-table ring, filled by the caller through *hs and uploaded by push_segs.
-static int next_seg_slot(taurus_runs* r, MoveSeg** hs, MoveSeg** ds, int* slot) {
-  *slot = (int)(r->seg_seq % SEG_RING);
-  r->seg_seq += 1;
-  if (r->seg_used[*slot]) RCU(cudaEventSynchronize(r->seg_done[*slot]));
-  *hs = r->h_segs + (size_t)*slot * r->P;
-  *ds = r->d_segs + (size_t)*slot * r->P;
-  return TAURUS_OK;
-}
-static int push_segs(taurus_runs* r, int slot, int nseg, cudaStream_t st) {
-  RCU(cudaMemcpyAsync(r->d_segs + (size_t)slot * r->P, r->h_segs + (size_t)slot * r->P, (size_t)nseg * sizeof(MoveSeg),
-                      cudaMemcpyHostToDevice, st));
-  return TAURUS_OK;
-}
-// Called after the kernel that reads the table has been launched: the slot (host and device copy) may be
-// reused once that kernel has run, on whichever stream the next user works.
-static int release_seg_slot(taurus_runs* r, int slot, cudaStream_t st) {
-  RCU(cudaEventRecord(r->seg_done[slot], st));
-  r->seg_used[slot] = true;
-  return TAURUS_OK;
-}
+// The pieces of one launch, filled through next() and given to a kernel as `segs`: in the launch, or beyond SEGS_INLINE of them in a slot of the
+// ring (host and device copy may be reused once that kernel has run, on whichever stream the next user works).
+struct SegList {
+  Segs segs;
+  MoveSeg* to = nullptr;   // where the caller's pieces go
+  int n = 0, slot = -1;
+  long long most = 0;      // rows of the longest
+  int begin(taurus_runs* r, long long at_most) {
+    to = segs.s;
+    segs.table = nullptr;
+    if (at_most <= SEGS_INLINE) return TAURUS_OK;
+    slot = (int)(r->seg_seq % SEG_RING);
+    r->seg_seq += 1;
+    if (r->seg_used[slot]) RCU(cudaEventSynchronize(r->seg_done[slot]));
+    to = r->h_segs + (size_t)slot * r->P;
+    segs.table = r->d_segs + (size_t)slot * r->P;
+    return TAURUS_OK;
+  }
+  void add(long long src, long long rows, long long dst) { to[n++] = MoveSeg{src, rows, dst}; most = std::max(most, rows); }
+  int upload(taurus_runs* r, cudaStream_t st) const {
+    if (slot < 0) return TAURUS_OK;
+    RCU(cudaMemcpyAsync(r->d_segs + (size_t)slot * r->P, r->h_segs + (size_t)slot * r->P, (size_t)n * sizeof(MoveSeg), cudaMemcpyHostToDevice, st));
+    return TAURUS_OK;
+  }
+  int done(taurus_runs* r, cudaStream_t st) const {   // after the launch
+    if (slot < 0) return TAURUS_OK;
+    RCU(cudaEventRecord(r->seg_done[slot], st));
+    r->seg_used[slot] = true;
+    return TAURUS_OK;
+  }
+  dim3 grid(const taurus_runs* r, long long threads_per_row) const {
+    return dim3((unsigned)std::max<long long>(1, std::min<long long>((most * threads_per_row + 255) / 256, std::max<long long>(1, (long long)r->sm_count * 8 / n))), (unsigned)n);
+  }
+};
 
 // Sorts the listed partition buffers (ascending range numbers) by id and writes each to the store as one run.
 // Buffers are sorted together, as many per radix sort as the scratch holds: the ranges are contiguous in id,
@@ -327,25 +458,22 @@ static int flush_many(taurus_runs* r, const std::vector<long long>& parts, cudaS
   if (r->store_top + total > r->store_rows) return TAURUS_ERR_RUN_STORE_FULL;
   size_t at = 0;
   while (at < parts.size()) {
-    MoveSeg *hs, *ds;
-    int slot;
-    { int rc = next_seg_slot(r, &hs, &ds, &slot); if (rc) return rc; }
-    int nseg = 0;
-    long long m = 0, most = 0;
+    SegList list;
+    { int rc = list.begin(r, (long long)(parts.size() - at)); if (rc) return rc; }
+    long long m = 0;
     const size_t first = at;
     while (at < parts.size()) {
       const long long p = parts[at], n = r->fill[(size_t)p];
       if (n == 0) { ++at; continue; }
       if (m + n > r->flush_cap) break;   // n <= R <= flush_cap, so every batch takes at least one buffer
-      hs[nseg++] = MoveSeg{p * r->R, n, m};
-      m += n; most = std::max(most, n);
+      list.add(p * r->R, n, m);
+      m += n;
       ++at;
     }
     if (m == 0) continue;
-    { int rc = push_segs(r, slot, nseg, st); if (rc) return rc; }
-    const int gx = (int)std::max<long long>(1, std::min<long long>((most + 255) / 256, std::max<long long>(1, (long long)r->sm_count * 8 / nseg)));
-    rs_collect_kernel<<<dim3(gx, nseg), 256, 0, st>>>(ds, r->d_pids, r->d_fkeys, r->d_fvals);
-    { int rc = release_seg_slot(r, slot, st); if (rc) return rc; }
+    { int rc = list.upload(r, st); if (rc) return rc; }
+    rs_collect_kernel<<<list.grid(r, 1), 256, 0, st>>>(list.segs, r->d_pids, r->d_fkeys, r->d_fvals);
+    { int rc = list.done(r, st); if (rc) return rc; }
     size_t tb = r->tmp_bytes;
     RCU(cub::DeviceRadixSort::SortPairs(r->d_tmp, tb, r->d_fkeys, r->d_sid, r->d_fvals, r->d_sidx, (int)m, 0, r->id_bits, st));
     const long long off = r->store_top;
@@ -383,22 +511,17 @@ int runs_phase2(taurus_runs* r, cudaStream_t st) {
   for (long long p = 0; p < r->P; ++p) { src[(size_t)p] = acc; left[(size_t)p] = cnt[p]; acc += cnt[p]; remaining += cnt[p]; }
   std::vector<long long> full;
   while (remaining > 0) {
-    MoveSeg *hs, *ds;
-    int slot;
-    { int rc = next_seg_slot(r, &hs, &ds, &slot); if (rc) return rc; }
-    int nseg = 0;
-    long long most = 0;
+    SegList list;
+    { int rc = list.begin(r, r->P); if (rc) return rc; }
     for (long long p = 0; p < r->P; ++p) {
       const long long take = std::min(left[(size_t)p], r->R - r->fill[(size_t)p]);
       if (take <= 0) continue;
-      hs[nseg++] = MoveSeg{src[(size_t)p], take, p * r->R + r->fill[(size_t)p]};
+      list.add(src[(size_t)p], take, p * r->R + r->fill[(size_t)p]);
       r->fill[(size_t)p] += take; src[(size_t)p] += take; left[(size_t)p] -= take; remaining -= take;
-      most = std::max(most, take);
     }
-    { int rc = push_segs(r, slot, nseg, st); if (rc) return rc; }
-    const int gx = (int)std::max<long long>(1, std::min<long long>((most * 32 + 255) / 256, std::max<long long>(1, (long long)r->sm_count * 8 / nseg)));
-    rs_move_kernel<<<dim3(gx, nseg), 256, 0, st>>>(ds, r->d_idx_s, r->p_ids, r->p_rows, r->p_ld, r->width, r->d_pids, r->d_prows);
-    { int rc = release_seg_slot(r, slot, st); if (rc) return rc; }
+    { int rc = list.upload(r, st); if (rc) return rc; }
+    rs_move_kernel<<<list.grid(r, 32), 256, 0, st>>>(list.segs, r->d_idx_s, r->p_ids, r->p_rows, r->p_ld, r->width, r->d_pids, r->d_prows);
+    { int rc = list.done(r, st); if (rc) return rc; }
     r->launches += 1;
     full.clear();
     for (long long p = 0; p < r->P; ++p)
@@ -454,20 +577,16 @@ int runs_read_into(taurus_runs* r, long long s, long long e, float* out, long lo
   if (r->stage_used) RCU(cudaStreamWaitEvent(st, r->stage_free, 0));
   long long at = 0;
   const size_t w = (size_t)r->width;
-  if (r->kind == TAURUS_RUNS_DEVICE && (long long)slices.size() <= r->P) {   // rows are read from the store in place
-    MoveSeg *hs, *ds;
-    int slot;
-    { int rc2 = next_seg_slot(r, &hs, &ds, &slot); if (rc2) return rc2; }
-    int nseg = 0;
-    long long most = 0;
+  if (r->kind == TAURUS_RUNS_DEVICE && (long long)slices.size() <= std::max<long long>(r->P, SEGS_INLINE)) {   // rows are read from the store in place
+    SegList list;
+    { int rc2 = list.begin(r, (long long)slices.size()); if (rc2) return rc2; }
     for (const Slice& sl : slices) {
-      hs[nseg++] = MoveSeg{sl.off, sl.n, at};
-      at += sl.n; most = std::max(most, sl.n);
+      list.add(sl.off, sl.n, at);
+      at += sl.n;
     }
-    { int rc2 = push_segs(r, slot, nseg, st); if (rc2) return rc2; }
-    const int gx = (int)std::max<long long>(1, std::min<long long>((most * 32 + 255) / 256, std::max<long long>(1, (long long)r->sm_count * 8 / nseg)));
-    rs_place_slices_kernel<<<dim3(gx, nseg), 256, 0, st>>>(ds, r->d_ids, r->store_dev, r->width, s, out, ld);
-    { int rc2 = release_seg_slot(r, slot, st); if (rc2) return rc2; }
+    { int rc2 = list.upload(r, st); if (rc2) return rc2; }
+    rs_place_slices_kernel<<<list.grid(r, 32), 256, 0, st>>>(list.segs, r->d_ids, r->store_dev, r->width, s, out, ld);
+    { int rc2 = list.done(r, st); if (rc2) return rc2; }
   } else {
     for (const Slice& sl : slices) {
       const float* src = r->kind == TAURUS_RUNS_HOST ? r->store_host + (size_t)sl.off * w : r->store_dev + (size_t)sl.off * w;
