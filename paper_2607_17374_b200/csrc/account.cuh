@@ -61,8 +61,8 @@ __device__ __forceinline__ void account_edges_block(const ChunkArgs& a, AccountS
   if (threadIdx.x == 0) s.sum[0] = s.sum[1] = 0;
   account_sync<THREADS>();
   unsigned msgs = 0, hub = 0;
-  int bad = 0;
-  for (long long base = (long long)block * THREADS; base < total; base += stride) {
+  int bad = 0, par = 0;
+  for (long long base = (long long)block * THREADS; base < total; base += stride, par ^= 1) {
     const long long i = base + threadIdx.x;
     int v = -1;
     if (i < ne) {
@@ -77,13 +77,20 @@ __device__ __forceinline__ void account_edges_block(const ChunkArgs& a, AccountS
       atomicAdd(&a.pend[v], -1);
       if (a.touch[v] != a.epoch) first = atomicMax(&a.touch[v], a.epoch) != a.epoch;
     }
+    // appended per block: an address takes an atomic every 3 ns (120 k edges: 8.6 us a launch with one per warp, 6.5 now)
     const unsigned m = __ballot_sync(FULL, first);
-    if (m) {
-      int at = 0;
-      const int leader = __ffs(m) - 1;
-      if (rl() == leader) at = atomicAdd(&pc->touched_count, __popc(m));
-      at = __shfl_sync(FULL, at, leader) + __popc(m & ((1u << rl()) - 1));
-      if (first) { if (at < a.touched_capacity) a.touched_list[at] = v; else bad = 1; }
+    const int warp = threadIdx.x >> 5;
+    if (rl() == 0) s.cnt[par][warp] = __popc(m);
+    account_sync<THREADS>();
+    if (threadIdx.x == 0) {
+      int t = 0;
+      for (int w = 0; w < THREADS / 32; ++w) { const int c = s.cnt[par][w]; s.cnt[par][w] = t; t += c; }
+      s.base[par] = t ? atomicAdd(&pc->touched_count, t) : 0;
+    }
+    account_sync<THREADS>();
+    if (first) {
+      const int at = s.base[par] + s.cnt[par][warp] + __popc(m & ((1u << rl()) - 1));
+      if (at < a.touched_capacity) a.touched_list[at] = v; else bad = 1;
     }
   }
   if (msgs) atomicAdd(&s.sum[0], msgs);

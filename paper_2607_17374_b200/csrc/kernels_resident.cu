@@ -77,11 +77,13 @@ static_assert(TAURUS_ACCOUNT_THREADS <= 8 * 32, "eight warps (AccountShared::cnt
 
 __global__ void __launch_bounds__(TAURUS_ACCOUNT_THREADS, 8) account_edges_kernel(const __grid_constant__ AccountWork w) {
   __shared__ AccountShared s;
+  early_start();
   account_edges_block<TAURUS_ACCOUNT_THREADS>(w.a, s, (int)blockIdx.x, (int)gridDim.x);
 }
 template <bool LISTED>
 __global__ void __launch_bounds__(TAURUS_ACCOUNT_THREADS, LISTED ? 6 : 5) account_kernel(const __grid_constant__ AccountWork w) {
   __shared__ AccountShared s;
+  if (LISTED) early_start();   // (behind the edges)
   account_block<LISTED, TAURUS_ACCOUNT_THREADS>(w, s, (int)blockIdx.x, (int)gridDim.x);
 }
 
@@ -969,7 +971,7 @@ void launch_account(taurus_ctx* c, const ChunkArgs& a, long long cell, cudaStrea
   }
   account_edges_kernel<<<c->sm_count * 8, TAURUS_ACCOUNT_THREADS, 0, st>>>(w);
   const int grid = (int)std::max<long long>(1, std::min<long long>((a.touched_capacity + 256 * ITEMS - 1) / (256 * ITEMS), (long long)c->sm_count * 6));
-  account_kernel<true><<<grid, TAURUS_ACCOUNT_THREADS, 0, st>>>(w);
+  launch_early(true, account_kernel<true>, grid, TAURUS_ACCOUNT_THREADS, 0, st, w);
   c->launches += 2;
 }
 

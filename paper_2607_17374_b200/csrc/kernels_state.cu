@@ -1149,6 +1149,7 @@ __global__ void report_kernel(const DevCtl* ctl, long long* report) { report_ctl
 __global__ void drain_rows_kernel(DevCtl* ctl, const long long* ids, const float* rows, int Hp, int d_out, float* dense, long long ld, long long capacity,
                                   long long* report) {
   __shared__ int last;
+  early_start();
   const long long count = ctl->grad_count;
   const bool go = !ctl->error && count <= capacity;
   if (go) place_rows(ids, rows, Hp, d_out, dense, ld, count);
@@ -1175,7 +1176,8 @@ void launch_place_rows(taurus_ctx* c, float* dense, long long ld, int d_out, int
 }
 void launch_drain_rows(taurus_ctx* c, float* dense, long long ld, int d_out, int Hp, long long bound, long long capacity, cudaStream_t st) {
   const long long blocks = std::max<long long>(1, std::min<long long>((bound + 7) / 8, (long long)c->sm_count * 8));   // one wave: every block takes its turn at the counter
-  drain_rows_kernel<<<(int)blocks, 256, 0, st>>>(c->d_ctl, c->d_grad_ids, c->d_grad_rows, Hp, d_out, dense, ld, capacity, reinterpret_cast<long long*>(c->h_ctl));
+  launch_early(true, drain_rows_kernel, (int)blocks, 256, 0, st, c->d_ctl, (const long long*)c->d_grad_ids, (const float*)c->d_grad_rows, Hp, d_out, dense, ld, capacity,
+               reinterpret_cast<long long*>(c->h_ctl));
   c->launches += 1;
 }
 void launch_report(taurus_ctx* c, cudaStream_t st) {

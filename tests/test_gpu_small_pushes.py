@@ -89,3 +89,37 @@ def test_what_blocking_calls_find_after_the_last_push(dims, fanout):
         assert st["completed"] == V and st["chunks"] == V // chunk and st["free_slots"] == V
         seen.append({k: v for k, v in st.items()})
     assert all(s == seen[0] for s in seen)
+
+
+@pytest.mark.parametrize("pool", ["all", "bounded"])
+def test_rows_that_another_stream_writes_late(pool):
+    """The rows of every push come from another stream, behind a kernel that takes its time, and the push waits for an event of it: directly behind
+    that wait, with the kernels of the push before in front of it."""
+    import torch
+    import paper_2607_17374_b200 as tb
+    V, chunk = 6_000, 500 if pool == "all" else 100
+    w = replace(tg.scaled(tg.WORKLOADS["large"], V, chunk=chunk), dims=(64, 64), fanout=(0,), pool_slots=V if pool == "all" else 4_500, hub_count=9)
+    g, model = tg.make_graph(w), tg.make_model(w, bias_scale=0.3)
+    x0 = tg.features(w.seed, 0, 0, V, 64)
+    want = run_oracle(w, g, model, x0)["outs"][0]
+    x = torch.from_numpy(x0).cuda()
+    ctx = tb.Context(V, g.E, g.row_ptr, g.col_idx, g.in_degree, w.mode, w.dims, model.W_neigh, model.W_self, model.bias, model.act, chunk, w.pool_slots, 9, w.fanout, w.seed,
+                     0 if pool == "all" else V, V + 1_024)
+    ours, other = torch.cuda.Stream(), torch.cuda.Stream()
+    out = torch.empty(V, 64, device="cuda")
+    rows = torch.empty(V, 64, device="cuda")
+    for _ in range(3):
+        rows.fill_(float("nan"))
+        torch.cuda.synchronize()
+        ctx.layer_begin(0, ours)
+        ctx.layer_set_dense_output(out, 64)
+        for b in range(0, V, chunk):
+            with torch.cuda.stream(other):
+                torch.cuda._sleep(200_000)
+                rows[b:b + chunk].copy_(x[b:b + chunk])
+                ready = torch.cuda.Event()
+                ready.record(other)
+            ours.wait_event(ready)
+            ctx.push_chunk(b, b + chunk, rows[b:b + chunk], ours)
+        assert ctx.layer_end()["completed"] == V
+        assert row_error(out.cpu().numpy(), want)[0] <= 1e-4
