@@ -185,7 +185,7 @@ __global__ void plan_kernel(ChunkArgs a) {
   if (threadIdx.x == 0) plan_chunk(a, ctl, pc);
 }
 
-// Victims are the `deficit` smallest keys (score << 31 | id) among IN_BUFFER vertices the chunk does not
+// Victims are the `deficit` smallest keys (score above id) among IN_BUFFER vertices the chunk does not
 // touch (Sect. 3.5.3: fewest pending messages first).  Keys are unique, so an MSB-first radix select finds
 // them exactly.  Level 0 scans the pool; every level lists the keys below the digit that holds rank k as
 // victims and hands the keys inside that digit to the next level, so deeper levels see a small candidate list.
@@ -252,6 +252,7 @@ static __device__ __forceinline__ void sel_fold(ChunkCtl* pc, int lvl, unsigned 
 static __device__ __forceinline__ void select_keys(const ChunkArgs& a, ChunkCtl* pc, FoldShared& fold) {
   unsigned long long kmin = ~0ull, kmax = 0ull;
   int cnt = 0;
+  const int id_bits = 64 - __clzll(a.V);   // the score right above them: zeros in between would be digits of a level that tell nothing apart
   for (long long base = (long long)blockIdx.x * MR_TILE; base < a.pool_slots; base += (long long)gridDim.x * MR_TILE) {
 #pragma unroll
     for (int j = 0; j < MR_ITEMS; ++j) {
@@ -267,7 +268,7 @@ static __device__ __forceinline__ void select_keys(const ChunkArgs& a, ChunkCtl*
           else if (a.evict_policy == TAURUS_EVICT_LRU) score = (unsigned)t;
           else if (a.evict_policy == TAURUS_EVICT_RANDOM) score = evict_hash(a.seed, (unsigned long long)v, (unsigned long long)(a.epoch - 1));
           else score = (unsigned)a.slot_pend[s];   // = pend[v]: v was not touched since the copy was taken
-          key = ((unsigned long long)score << 31) | (unsigned long long)v;
+          key = ((unsigned long long)score << id_bits) | (unsigned long long)v;
           if (key < kmin) kmin = key;
           if (key > kmax) kmax = key;
           cnt++;
