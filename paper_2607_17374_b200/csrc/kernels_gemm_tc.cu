@@ -27,11 +27,13 @@
 // us a launch of 65 536 rows, two tf32 values / now:
 //   K -> N    64 -> 64    100 -> 64   128 -> 128  256 -> 96   256 -> 192  256 -> 256  256 -> 512  512 -> 64   512 -> 256
 //             14.5/14.3   19.1/17.8   22.6/20.8   34.0/28.2   47.1/32.8   52.1/37.4   85.3/61.1   49.5/43.7   88.3/57.6
-// What bounds it: narrow products the row pieces of 128 B that a K step reads (4.5 TB/s, with nothing else in the kernel 35 of the
-// 43.7 us of 512 -> 64), wide ones shared memory: per K step of a 256-column block the TMA fill is 48 KB, the conversion 32, the MMAs'
-// operands 72, the epilogue's transposition 32 = 1 470 cycles of 128 B of the 1 500 a step takes.  Tried and slower: two threads to
-// a row in eight warps (256 -> 512: 70 us), the epilogue's rows straight from registers in 32-byte pieces (78), L2 promotion of 256 B
-// (the same); one ring for X and W was 0.5 to 3 us a launch slower than the two.
+// What bounds it: narrow products the row pieces of 128 B that a K step reads (4.5 TB/s: with nothing else in the kernel 35 of the
+// 43.7 us of 512 -> 64).  Wide ones: nothing is full.  256 -> 512: a K step of a block takes 1 660 cycles, 768 of them MMAs (the pipe is busy 46 % of
+// the active cycles); the L1 pipeline, which the conversion and the epilogue's transposition and stores share, is at 61 %, shared-memory
+// banks at 25 % (reads) and 20 % (writes), L2 at 28 %, DRAM at 27 %.  Without the epilogue a launch takes 47.6 of 63.5 us, without its
+// stores 55.5, without the conversion 56.6, without all but loads and MMAs 40.  Tried and slower: two threads to a row in eight warps
+// (70 us), the epilogue's rows straight from registers in 32-byte pieces (78), the next accumulator piece loaded ahead of the stores and L2 promotion
+// of 256 B (the same); one ring for X and W was 0.5 to 3 us a launch slower than the two.
 //
 // Every wait on an mbarrier is bounded: after WAIT_LIMIT polls the kernel raises a CTA-wide abort flag,
 // records TAURUS_ERR_INTERNAL in the control block, waits (bounded) for its TMA copies and MMAs in flight, frees its

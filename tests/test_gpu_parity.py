@@ -211,7 +211,7 @@ def test_error_paths():
 
 @pytest.mark.parametrize("dims", [(64, 64, 16), (100, 256, 47), (512, 256, 256), (36, 20, 12)])
 def test_projection_kernels_agree_with_the_oracle(dims):
-    """The three projection paths on the same chunk stream: fp32 tensor-core (3 x TF32), bf16 tensor-core, FFMA."""
+    """The three projection paths on the same chunk stream: fp32 tensor-core (two fp16 values), bf16 tensor-core, FFMA."""
     import paper_2607_17374_b200 as tb
     from dataclasses import replace
     w = replace(tg.scaled(tg.WORKLOADS["mid"], 9_000, chunk=1000), dims=dims, fanout=(0,) * (len(dims) - 1))
