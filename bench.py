@@ -518,16 +518,17 @@ def run_windowed(args, env, w):
     sc_s = phase[5] * 1e-3
     moves_share = phase[8] / ms
     # the dominant kernel: the row transfers between the pool and pinned host memory, bound by the host link
-    # The link is full duplex: a launch cannot end before its busier direction has crossed, max(bytes out, bytes in) /
-    # per-direction peak.  `achieved` is therefore the rate of the busier direction; both are listed.
+    # The link is full duplex: a launch cannot end before its busier direction has crossed, bytes / per-direction peak.  Every evicted
+    # row crosses; of the reloaded ones those that the push before evicted do not (they come out of the staging buffer), so the
+    # direction that the counters give exactly is the way out, and `achieved` is its rate; the other is an upper bound.
     roofline = dict(bound="pcie", kernel="transfer_kernel (evicted rows out, reloaded rows in, %d-byte rows)" % row_bytes,
-                    achieved=max(out_gbs, in_gbs), peak=link["both_per_direction_gbs"], unit="GB/s in the busier direction",
-                    frac=max(out_gbs, in_gbs) / link["both_per_direction_gbs"], mean_of_directions_gbs=(out_gbs + in_gbs) / 2,
+                    achieved=out_gbs, peak=link["both_per_direction_gbs"], unit="GB/s, device to host",
+                    frac=out_gbs / link["both_per_direction_gbs"],
                     peak_source="measured in this run: " + link["how"],
-                    device_to_host_gbs=out_gbs, host_to_device_gbs=in_gbs, link=link,
-                    rows_out_per_step=evicted / K, rows_in_per_step=reloaded / K, launches_per_step=window,
-                    avg_launch_ms=float(phase[8]) / (K * window), algorithmic_bytes_per_launch=max(evicted, reloaded) * row_bytes / (K * window),
-                    algorithmic_bytes_note="rows of the busier direction x row bytes (counters of the library)",
+                    device_to_host_gbs=out_gbs, host_to_device_gbs_at_most=in_gbs, link=link,
+                    rows_out_per_step=evicted / K, rows_back_per_step=reloaded / K, launches_per_step=window,
+                    avg_launch_ms=float(phase[8]) / (K * window), algorithmic_bytes_per_launch=evicted * row_bytes / (K * window),
+                    algorithmic_bytes_note="evicted rows x row bytes (counters of the library)",
                     share_of_step=float(moves_share),
                     share_note="the transfers run on their own stream beside the compute stream: their share of the step is how "
                                "much of the step the host link is busy",

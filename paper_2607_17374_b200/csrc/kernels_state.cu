@@ -452,6 +452,10 @@ static __device__ __forceinline__ void victim_bucket(const ChunkArgs& a, DevCtl*
   }
 }
 
+// Row of stage_out for victim entry i of this push: pushes fill it from either end in turn, so a push finds the rows of the one before
+// it where they were as long as the two have room beside each other.
+static __device__ __forceinline__ long long stage_row(const ChunkArgs& a, long long i) { return a.epoch & 1 ? a.victim_capacity - 1 - i : i; }
+
 // One block.  First the tails of the buckets whose grid cell ends inside this push are closed (no victim can be
 // filed there any more: its next sender would lie behind the push); then every bucket that received victims gets
 // the extents it lacks from the free stack.
@@ -470,7 +474,13 @@ static __device__ void extent_plan(const ChunkArgs& a, DevCtl* ctl, int deficit)
     const long long top = ctl->ext_free_top;
     for (int i = threadIdx.x; i < n_ret; i += blockDim.x) a.ext_free[top + i] = a.ext_ret[par][i];
     __syncthreads();
-    if (threadIdx.x == 0) { ctl->ext_free_top = top + n_ret; ctl->ext_ret_count[par] = 0; }
+    if (threadIdx.x == 0) {
+      ctl->ext_free_top = top + n_ret;
+      ctl->ext_ret_count[par] = 0;
+      const long long next = a.src_end / a.chunk_sources;   // grid cell behind this push
+      ctl->staged[par] = deficit;
+      ctl->kept_n[par] = deficit > 0 && next < a.n_buckets ? a.bk_new[next] : 0;
+    }
     __syncthreads();
   }
   // phase 1: close tails
@@ -554,6 +564,7 @@ static __device__ void extent_plan(const ChunkArgs& a, DevCtl* ctl, int deficit)
 // Host row of every victim.
 static __device__ __forceinline__ void victim_place(const ChunkArgs& a, int n) {
   const int E = 1 << a.ext_shift;
+  const int next = (int)(a.src_end / a.chunk_sources);
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const int2 pl = a.vic_place[i];
@@ -562,7 +573,12 @@ static __device__ __forceinline__ void victim_place(const ChunkArgs& a, int n) {
     int ext, idx;
     if (pl.y < room) { ext = base.x; idx = base.y + pl.y; }
     else { const int q = pl.y - room; ext = a.new_ext[a.bk_off[pl.x] + (q >> a.ext_shift)]; idx = q & (E - 1); }
-    a.victims[i].y = (ext << a.ext_shift) + idx;
+    const int hrow = (ext << a.ext_shift) + idx;
+    a.victims[i].y = hrow;
+    if (pl.x == next) {   // the next push may take it back from the staging buffer
+      a.kept[a.epoch & 1][pl.y] = make_int2(hrow, (int)stage_row(a, n - 1 - i));
+      a.ext_rank[ext] = pl.y - idx;   // same value from every victim in the extent
+    }
     a.bk_new[pl.x] = 0;   // same value from every victim of the bucket; nothing reads the count after the plan
   }
 }
@@ -694,36 +710,53 @@ __global__ void alloc_kernel(ChunkArgs a) {
   // copied to the staging buffer (it leaves for its pinned host row in transfer_kernel) and the victim becomes
   // EVICTED; entry i >= deficit pops the free stack.  Either way the slot is cleared and handed to the vertex, which
   // is IN_BUFFER afterwards; the partial sum of a vertex that was EVICTED is ADDED into the slot by transfer_kernel
-  // (sums commute: the scatter may already be adding this chunk's messages to the same row).
+  // (sums commute: the scatter may already be adding this chunk's messages to the same row), unless the push before this one evicted
+  // it and its row is still in the staging buffer: it is the same row, so it goes straight into the slot and does not cross the link.
+  // A fifth of the victims of a push of 4 096 sources of 600 k vertices are back in the next, and the link bounds the pass: 88.2 -> 83.5 ms;
+  // 34 k vertices, 338 a push: 18.2 -> 17.6; 215 k, 999 a push: 41.4 -> 40.4; the two more reads of an entry cost nothing measurable where
+  // few come back (900 k, 16 k a push: 19.7 and 19.7; rows of 16 floats left out: no faster).
   // Batches of up to 32 entries per warp: each lane follows the chain of dependent reads of one entry (vertex, victim,
   // slot, state) and writes its metadata, then the warp walks the batch row by row.
   int reloaded = 0;
+  const int par = a.epoch & 1;
+  const unsigned kept_n = (long long)ctl->staged[par ^ 1] + deficit <= a.victim_capacity ? (unsigned)ctl->kept_n[par ^ 1] : 0u;
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
   int per = (int)((n + warps - 1) / warps);
   per = per < 1 ? 1 : per > 32 ? 32 : per;
   for (long long i0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per; i0 < n; i0 += warps * per) {
     const long long i = i0 + lane_id();
     int slot = -1, out_hrow = -1, extra_hrow = -1;
+    int from = -1, from_ext = -1;   // staged row of the push before this one, extent of its host row
     if (lane_id() < per && i < n) {
+      // a read waits for the one before it only where it needs it: vertex and victim; state, place and owner; rank; list
       const int v = a.need_list[i];
-      int victim = -1;
-      if (i < deficit) {
-        const int2 vic = a.victims[deficit - 1 - i];
-        slot = vic.x; out_hrow = vic.y; victim = a.owner[slot];
-      } else { const long long f = pc->alloc_base - 1 - i; slot = f >= 0 ? a.free_stack[f] : -1; }
+      int2 vic = make_int2(-1, -1);
+      if (i < deficit) vic = a.victims[deficit - 1 - i];
+      else { const long long f = pc->alloc_base - 1 - i; if (f >= 0) vic.x = a.free_stack[f]; }
+      const int st = a.state[v], lv = a.loc[v];
+      slot = vic.x; out_hrow = vic.y;
+      const int victim = out_hrow >= 0 ? a.owner[slot] : -1;
+      int in_hrow = st == TAURUS_EVICTED ? -2 - lv : -1;
       if (slot < 0) {
         atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL);
       } else {
-        const int in_hrow = a.state[v] == TAURUS_EVICTED ? -2 - a.loc[v] : -1;
+        if (in_hrow >= 0) {
+          a.reload_count[v] += 1;
+          reloaded++;
+          if (kept_n > 0) {
+            const int e = in_hrow >> a.ext_shift;
+            const unsigned at = (unsigned)a.ext_rank[e] + (unsigned)(in_hrow & ((1 << a.ext_shift) - 1));
+            if (at < kept_n) {   // ext_rank may be that of an earlier push: only the host row in the list says
+              const int2 k = a.kept[par ^ 1][at];
+              if (k.x == in_hrow) { from = k.y; from_ext = e; in_hrow = -1; }
+            }
+          }
+        }
         if (i >= deficit) extra_hrow = in_hrow;
         else if (a.xfer_list) a.xfer_list[i] = make_int4(slot, in_hrow, out_hrow, 0);
         if (out_hrow >= 0) {
           a.loc[victim] = -2 - out_hrow;
           a.state[victim] = TAURUS_EVICTED;
-        }
-        if (in_hrow >= 0) {
-          a.reload_count[v] += 1;
-          reloaded++;
         }
         a.loc[v] = slot; a.owner[slot] = v; a.slot_epoch[slot] = a.epoch;
         if (a.slot_touch) a.slot_touch[slot] = a.epoch;   // slot_pend follows in compact_done: v is on the touched list
@@ -740,16 +773,18 @@ __global__ void alloc_kernel(ChunkArgs a) {
     const int rows = n - i0 < per ? (int)(n - i0) : per;
     for (int j = 0; j < rows; ++j) {
       const int sj = __shfl_sync(FULL, slot, j);
-      const int oj = __shfl_sync(FULL, out_hrow, j);
+      const int oj = __shfl_sync(FULL, out_hrow, j), fj = __shfl_sync(FULL, from, j);
       if (sj < 0) continue;
       float4* __restrict__ row = reinterpret_cast<float4*>(a.acc + (size_t)sj * a.Hp);
+      const float4* __restrict__ back = reinterpret_cast<const float4*>(a.stage_out + (size_t)(fj >= 0 ? fj : 0) * a.Hp);
       if (oj >= 0) {
-        float4* __restrict__ keep = reinterpret_cast<float4*>(a.stage_out + (size_t)(i0 + j) * a.Hp);
-        for (int k = lane_id(); k < vec; k += 32) { keep[k] = row[k]; row[k] = zero; }
+        float4* __restrict__ keep = reinterpret_cast<float4*>(a.stage_out + (size_t)stage_row(a, i0 + j) * a.Hp);
+        for (int k = lane_id(); k < vec; k += 32) { keep[k] = row[k]; row[k] = fj >= 0 ? back[k] : zero; }
       } else {
-        for (int k = lane_id(); k < vec; k += 32) row[k] = zero;
+        for (int k = lane_id(); k < vec; k += 32) row[k] = fj >= 0 ? back[k] : zero;
       }
     }
+    if (from_ext >= 0 && atomicSub(&a.ext_live[from_ext], 1) == 1) a.ext_ret[par][atomicAdd(&ctl->ext_ret_count[par], 1)] = from_ext;   // as in transfer_kernel
   }
   for (int o = 16; o; o >>= 1) reloaded += __shfl_xor_sync(FULL, reloaded, o);
   if (lane_id() == 0 && reloaded) atomicAdd(&pc->reloaded, reloaded);
@@ -774,14 +809,14 @@ static __device__ __forceinline__ void xf_load(void* dst, const void* src, unsig
 // The rows of one chunk across the host link: the staged row of the victim whose slot a need-list entry took over
 // goes to its pinned host row (device -> host), and the host row of a vertex that was EVICTED is added into its new
 // slot (host -> device), so both directions of the link are busy at once.
-// Every thread carries one entry at a time through its own pair of row buffers in shared memory with untiled bulk
-// copies: host row and staged row in (one barrier for both), then an fp32 add-reduction into the slot and a store to
-// the host row.
+// Every thread carries one row at a time, one way (odd threads out, even ones back), through a buffer of its own in shared memory with
+// untiled bulk copies: in behind an mbarrier, then a store to the host row or an fp32 add-reduction into the slot.  With a pair of
+// buffers a thread a row waited for the slower direction: 94.8 -> 92.8 ms (600k/4k/128,256), 20.7 -> 20.3 (900k/16k/256).
 // Bound by the host link, and by what it does to the kernels beside it: rows waiting for the link fill the queues between
 // the SMs and L2, and everything else on the GPU waits in them.  So the rows in flight are kept to what the link needs,
 // on a few SMs of their own (a block takes all the shared memory of its SM, so no block of another kernel shares it): eight;
-// sixteen and thirty-two where a push can touch more than 128 and 512 MB of rows (xfer_blocks_for).  ms a pass, and for the last
-// column ms a window of 32 pushes (190 k rows of 1 KB each way per push; GB/s in the busier direction):
+// sixteen and thirty-two where a push can touch more than 128 and 512 MB of rows (xfer_blocks_for).  With pairs of buffers, ms a
+// pass, and for the last column ms a window of 32 pushes (190 k rows of 1 KB each way per push; GB/s in the busier direction):
 //   vertices / sources a push / row floats   600k/4k/128,256   900k/16k/256   1M/16k/64   1.5M/16k/256   1.5M/64k/256   111M/64k/256
 //   rows a push can touch                          67 MB         270 MB         64 MB        270 MB           1 GB            1 GB
 //   4 blocks                                       99.3           23.7          29.9         138.5            65.3         284  (22.8)
@@ -792,8 +827,8 @@ static __device__ __forceinline__ void xf_load(void* dst, const void* src, unsig
 //   a block of eight warps on every SM, four
 //   float4 per lane and direction in flight       112.6           24.0          30.8         126.8            59.0         197  (36.3)
 // The last of these drives the link a little harder, but stretches the scatter beside it from 16 to 43 ms and the victim select
-// from 28 to 111 ms a window.  No better: one buffer per thread, 60 % of them for incoming rows (within 2 % at 8 to 32 blocks);
-// entries taken from a counter instead of dealt (191 ms at 16); fewer rows per block on more SMs (56 on 32: 189, 28 on 64: 190).
+// from 28 to 111 ms a window.  No better: 60 % of the buffers for incoming rows (within 2 % at 8 to 32 blocks); entries taken
+// from a counter instead of dealt (191 ms at 16); fewer rows per block on more SMs (56 on 32: 189, 28 on 64: 190).
 // Only entries with a row to move are listed: a chunk that moves none was 40 to 75 us of walking its need list, beside the scatter.
 // An extent whose last row has come back is listed for the free stack (taken back two chunks later by extent_plan).
 #define XF_SMEM (224 * 1024)
@@ -828,7 +863,7 @@ __global__ void __launch_bounds__(XF_THREADS) transfer_kernel(ChunkArgs a, int l
     float* const host = a.host_store + (size_t)hrow * a.Hp;
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the store of the last entry has read the buffer
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(xf_smem(bar)), "r"(bytes) : "memory");
-    xf_load(row, out ? a.stage_out + (size_t)i * a.Hp : host, bytes, bar);
+    xf_load(row, out ? a.stage_out + (size_t)stage_row(a, i) * a.Hp : host, bytes, bar);
     if (!xf_wait(bar, phase)) { atomicCAS(&ctl->error, 0, TAURUS_ERR_INTERNAL); xf_wait(bar, phase); break; }
     phase ^= 1;
     if (out) {

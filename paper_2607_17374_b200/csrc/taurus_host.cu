@@ -75,7 +75,7 @@ extern "C" void taurus_destroy(taurus_ctx* c) {
   cudaFree(c->d_cand[0]); cudaFree(c->d_cand[1]); cudaFree(c->d_ext_free); cudaFree(c->d_ext_live); cudaFree(c->d_bk_tail_ext);
   cudaFree(c->d_bk_tail_fill); cudaFree(c->d_bk_new); cudaFree(c->d_bk_off); cudaFree(c->d_bk_base); cudaFree(c->d_new_ext);
   cudaFree(c->d_vic_place); cudaFree(c->d_csc_src); cudaFree(c->d_ext_ret[0]); cudaFree(c->d_ext_ret[1]); cudaFree(c->d_xfer_list);
-  cudaFree(c->d_stage_out);
+  cudaFree(c->d_stage_out); cudaFree(c->d_stage_kept[0]); cudaFree(c->d_stage_kept[1]); cudaFree(c->d_ext_rank);
   if (c->moves_ready) cudaEventDestroy(c->moves_ready);
   if (c->xfer_done) cudaEventDestroy(c->xfer_done);
   if (c->xfer_stream) cudaStreamDestroy(c->xfer_stream);
@@ -330,6 +330,7 @@ static int init_impl(taurus_ctx* c, const taurus_graph* g, const taurus_model* m
     ALLOC(c->d_ext_ret[0], c->n_ext); ALLOC(c->d_ext_ret[1], c->n_ext);
     ALLOC(c->d_xfer_list, std::min<long long>(c->pool_slots, c->touched_capacity));   // one entry per need-list entry: a chunk needs at most what it touches
     ALLOC(c->d_stage_out, (size_t)c->victim_capacity * c->Hmax);
+    ALLOC(c->d_stage_kept[0], c->victim_capacity); ALLOC(c->d_stage_kept[1], c->victim_capacity); ALLOC(c->d_ext_rank, c->n_ext);
     int prio_low = 0, prio_high = 0;
     CU(cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
     CU(cudaStreamCreateWithPriority(&c->xfer_stream, cudaStreamNonBlocking, prio_high));
@@ -555,6 +556,7 @@ static ChunkArgs make_args(taurus_ctx* c, long long s, long long e) {
   a.bk_new = c->d_bk_new; a.bk_off = c->d_bk_off; a.bk_base = c->d_bk_base; a.new_ext = c->d_new_ext; a.vic_place = c->d_vic_place;
   a.csc_ptr = c->d_csc_ptr; a.csc_src = c->d_csc_src; a.csc_eid = c->d_csc_eid;
   a.ext_ret[0] = c->d_ext_ret[0]; a.ext_ret[1] = c->d_ext_ret[1]; a.xfer_list = c->d_xfer_list; a.stage_out = c->d_stage_out;
+  a.kept[0] = c->d_stage_kept[0]; a.kept[1] = c->d_stage_kept[1]; a.ext_rank = c->d_ext_rank;
   a.chunk_sources = c->chunk_sources; a.n_ext = c->n_ext; a.n_buckets = c->n_buckets; a.ext_shift = c->ext_shift;
   a.grad_ids = c->d_grad_ids; a.grad_rows = c->d_grad_rows; a.done_list = c->d_done_list;
   a.Hp = taurus_round_up(c->dims[l + 1], 4);

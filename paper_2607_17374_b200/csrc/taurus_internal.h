@@ -68,6 +68,8 @@ struct DevCtl {
   int32_t heavy_rows;       // resident pools: partial rows of long in-lists handed out in this layer
   unsigned int drain_blocks;   // drain into a matrix: blocks that have finished
   int32_t unused;
+  int32_t staged[2];        // rows that the last push of each parity left in stage_out,
+  int32_t kept_n[2];        // and those of them that the push behind it takes back first (ranks 0 .. kept_n - 1 of `kept`)
   int32_t ext_ret_count[2]; // extents emptied by the row transfers of the chunks of each parity, waiting to go back on the free stack
   long long free_top;       // entries on the free-slot stack
   long long ext_free_top;   // entries on the free-extent stack of the host store
@@ -131,7 +133,9 @@ struct ChunkArgs {
   // Row transfers of the chunk: entry i = (slot, host row to add into it or -1, host row that takes stage_out[i] or -1); the entries of the
   // victims first, then the other reloads
   int4* xfer_list;          // [need capacity]
-  float* stage_out;         // [victim_capacity x Hp] victims' rows on their way to the host store
+  float* stage_out;         // [victim_capacity x Hp] victims' rows on their way to the host store, from either end in turn (stage_row)
+  int2* kept[2];            // [victim_capacity] pushes of each parity: (host row, staged row) of the victims filed under the next grid cell, by rank
+  int32_t* ext_rank;        // [n_ext] extents of the last of them: rank of the victim in the extent's row 0
   const long long* csc_ptr; // [V + 1] in-lists (ascending source id): offsets,
   const int32_t* csc_src;   // [E]       sources,
   const uint32_t* csc_eid;  // [E]       CSR edge indices (sampled layers: the mask is looked up through them), else NULL
@@ -287,6 +291,8 @@ struct taurus_ctx {
   int32_t* d_ext_ret[2] = {nullptr, nullptr};
   int4* d_xfer_list = nullptr;
   float* d_stage_out = nullptr;
+  int2* d_stage_kept[2] = {nullptr, nullptr};
+  int32_t* d_ext_rank = nullptr;
   cudaStream_t xfer_stream = nullptr;   // rows cross the host link here while the compute stream goes on
   int xfer_blocks = 0;                  // SMs that carry them (one block each, all of its shared memory)
   cudaEvent_t moves_ready = nullptr, xfer_done = nullptr;
