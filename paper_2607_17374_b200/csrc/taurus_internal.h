@@ -214,7 +214,7 @@ struct taurus_ctx {
   // weights per layer: Wcat is [Kp x Ncat] row-major fp32 (P columns then T columns), bias [Hp]
   float* d_Wcat[TAURUS_MAX_LAYERS] = {nullptr};
   float* d_bias[TAURUS_MAX_LAYERS] = {nullptr};
-  bool tc_smem_set[2] = {false, false};            // dynamic shared memory limit of the projection kernel raised (without, with accounting)
+  bool tc_smem_set[4] = {false, false, false, false};   // dynamic shared memory limit of the projection kernel raised (without, with accounting; stages of 16 columns)
   bool xfer_smem_set = false;                      // the same for the row transfer kernel
   void* tc_image[TAURUS_MAX_LAYERS] = {nullptr};   // tensor-core operand images of Wcat (owned by kernels_gemm_tc.cu)
   void* tc_image_af[TAURUS_MAX_LAYERS] = {nullptr};   // SAGE aggregate-first layers: image of [W_neigh ; W_self] stacked along K

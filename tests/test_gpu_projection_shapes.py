@@ -1,8 +1,8 @@
-"""The projection in fp32 mode (operands split into two fp16 values, rows and columns scaled by powers of two) at the edges of its tiles
-and stages: one row to several tiles per CTA, K with short last stages, one to eight blocks of output columns, columns that fill no 32,
-bias and per-row factors; rows and columns of very different magnitudes.  Against the product in 64 bits, element by element of the
-magnitude sum: a value cut after 11 + 11 bits is off by at most 2^-20, on either side, the dropped lo.lo by 2^-20, and K additions by
-2^-24 each: 2^-18 + K 2^-24 covers them."""
+"""The projection in fp32 mode (operands split into two TF32 values) at the edges of its tiles and stages: one row to several tiles per
+CTA, K with short last stages, one to eight blocks of output columns, columns that fill no 32, bias and per-row factors; elements of
+very different magnitudes in a row of X, in a column of W.  Against the product in 64 bits, element by element of the magnitude sum:
+a value cut after 11 + 11 bits is off by at most 2^-20, on either side, the dropped lo.lo by 2^-20, and K additions by 2^-24 each:
+2^-18 + K 2^-24 covers them, whatever the magnitudes."""
 from dataclasses import replace
 
 import numpy as np
@@ -53,7 +53,7 @@ def test_shapes(V, K, N):
 
 def _rows(kind, V, K, rng):
     x = rng.standard_normal((V, K))
-    if kind == "grow":        # a power of two of the row that has to give way again and again
+    if kind == "grow":        # every column larger than the one before it
         x *= 10.0 ** np.linspace(-8, 9, K)
     elif kind == "steps":     # ... at every K step, with empty ones in front
         x *= 10.0 ** (4 * (np.arange(K) // 32 % 4)) * (np.arange(K) >= 32)
@@ -69,18 +69,74 @@ def _rows(kind, V, K, rng):
 @pytest.mark.parametrize("K,N", [(36, 20), (96, 128), (256, 256), (300, 340)])
 @pytest.mark.parametrize("kind", ["grow", "steps", "late", "rows", "zeros"])
 def test_rows_of_many_magnitudes(kind, K, N):
-    """What a row's power of two leaves of an element is off by at most 2^-33 of the largest one."""
     V = 40_003
     rng = np.random.default_rng(K + N)
     x, W = _rows(kind, V, K, rng), (rng.standard_normal((K, N)) / K ** 0.5).astype(np.float32)
-    got = _project(x, W)
-    x64, W64 = x.astype(np.float64), W.astype(np.float64)
-    ref, mag = x64 @ W64, np.abs(x64) @ np.abs(W64)
-    bound = (2.0 ** -18 + K * 2.0 ** -24) * mag + 2.0 ** -32 * np.abs(x64).max(1)[:, None] * np.abs(W64).sum(0)
-    assert (np.abs(got - ref) <= bound).all(), float((np.abs(got - ref) / np.maximum(bound, 1e-300)).max())
+    _check(x, W, _project(x, W))
 
 
-@pytest.mark.parametrize("spread", [0, 2, 15])   # 15: the columns of W need powers of two of their own
+@pytest.mark.parametrize("weights", ["zero", "balancing"])
+@pytest.mark.parametrize("at", [0, 31, 32, -1])
+@pytest.mark.parametrize("size", [1e4, 1e6, 1e9])
+def test_one_raw_column(size, at, weights):
+    """An id, a count or a time stamp among N(0, 1) features, with no weight or with one that brings it back to their size."""
+    V, K, N = 5_003, 100, 72
+    rng = np.random.default_rng(int(size) + at)
+    x, W = rng.standard_normal((V, K)), rng.standard_normal((K, N)) / K ** 0.5
+    x[:, at] *= size
+    W[at] *= 0 if weights == "zero" else 1 / size
+    x, W = x.astype(np.float32), W.astype(np.float32)
+    _check(x, W, _project(x, W))
+
+
+@pytest.mark.parametrize("feature", ["zero", "balancing"])
+@pytest.mark.parametrize("at", [0, 31, 32, -1])
+@pytest.mark.parametrize("size", [1e6, 1e9])
+def test_one_large_weight_a_column(size, at, feature):
+    V, K, N = 5_003, 100, 72
+    rng = np.random.default_rng(int(size) + at)
+    x, W = rng.standard_normal((V, K)), rng.standard_normal((K, N)) / K ** 0.5
+    W[at] *= size
+    x[:, at] *= 0 if feature == "zero" else 1 / size
+    x, W = x.astype(np.float32), W.astype(np.float32)
+    _check(x, W, _project(x, W))
+
+
+def test_worst_element_of_a_hub():
+    """A sum over thousands of projected rows, where an error that the rows have in common adds up, element by element.  On top of a
+    product's own error: the additions of a piece of an in-list (128 entries) and of its pieces, one after the other at most."""
+    V, K, N, hub = 30_000, 64, 32, 20_003
+    rng = np.random.default_rng(5)
+    src = np.concatenate([rng.integers(0, V, hub), rng.integers(0, V, 700), rng.integers(0, V, 3 * V)])
+    dst = np.concatenate([np.full(hub, 17), np.full(700, V - 1), rng.integers(0, V, 3 * V)])
+    order = np.argsort(src, kind="stable")
+    src, dst = src[order], dst[order]
+    row_ptr = np.zeros(V + 1, np.int64)
+    row_ptr[1:] = np.cumsum(np.bincount(src, minlength=V))
+    x, W = (1 + rng.standard_normal((V, K))).astype(np.float32), (rng.standard_normal((K, N)) / K ** 0.5).astype(np.float32)
+    dev = torch.device("cuda:0")
+    ctx = tb.Context(V, len(src), torch.from_numpy(row_ptr).to(dev), torch.from_numpy(dst.astype(np.int32)).to(dev),
+                     torch.from_numpy(np.bincount(dst, minlength=V).astype(np.int32)).to(dev), tb.GIN_SUM, [K, N], [torch.from_numpy(W)], [torch.from_numpy(W)],
+                     [torch.zeros(N)], [0], 8192, V, 0, None, 1, 0, V, tb.GEMM_FP32, 0, 0, 0.0)
+    out = torch.empty(V, N, device=dev)
+    ctx.layer_begin(0)
+    ctx.layer_set_dense_output(out, N)
+    xd = torch.from_numpy(x).to(dev)
+    for b in range(0, V, 8192):
+        ctx.push_chunk(b, min(b + 8192, V), xd[b:b + 8192])
+    ctx.layer_end()
+
+    def layer(x, W):
+        h = x @ W
+        o = h.copy()
+        np.add.at(o, dst, h[src])
+        return o
+    ref, mag = layer(x.astype(np.float64), W.astype(np.float64)), layer(np.abs(x).astype(np.float64), np.abs(W).astype(np.float64))
+    err = np.abs(out.cpu().numpy() - ref)
+    assert (err <= (2.0 ** -18 + (K + 128 + hub // 128 + 16) * 2.0 ** -24) * mag).all(), float((err / mag).max())
+
+
+@pytest.mark.parametrize("spread", [0, 2, 15])
 def test_columns_of_many_magnitudes(spread):
     V, K, N = 20_003, 100, 132
     rng = np.random.default_rng(spread)

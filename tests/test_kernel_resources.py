@@ -45,4 +45,4 @@ def test_a_block_of_the_accounting_fits_beside_a_projection(kernels):
         assert smem == 0
         for beside in ("account_kernel", "account_edges_kernel"):
             for r, s in kernels[beside]:
-                assert _quarter(registers, 480) + _quarter(r, 256) <= QUARTER and s <= 128
+                assert _quarter(registers, 448) + _quarter(r, 256) <= QUARTER and s <= 128
