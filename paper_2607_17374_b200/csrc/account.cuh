@@ -3,6 +3,7 @@
 // the launch that writes the rows for small ones, which are bound by launches and by the events between two streams.
 #pragma once
 
+#include "block_exit.h"
 #include "taurus_internal.h"
 
 #define FULL 0xffffffffu
@@ -25,7 +26,7 @@ struct AccountWork {
 namespace {
 
 __device__ __forceinline__ int rl() { return threadIdx.x & 31; }
-// The first THREADS threads of a block (which may have more; they have gone).
+// The first THREADS threads of a block (which may have more; they have gone).  It waits for that many, so none of them leaves early by itself.
 template <int THREADS>
 __device__ __forceinline__ void account_sync() { asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory"); }
 
@@ -47,7 +48,7 @@ enum { C_HS, C_NS, C_GS, C_MSGS, C_HUB, C_GROUPS, C_FREED, C_COUNT };
 #define ITEMS 4
 
 struct AccountShared {
-  int cnt[2][8], base[2];
+  int cnt[2][8], base[2], go;
   unsigned int sum[C_COUNT];
 };
 // Edges and own vertices of a push that is not a grid cell: pending counts by atomics, first touches listed.
@@ -55,11 +56,10 @@ template <int THREADS>
 __device__ __forceinline__ void account_edges_block(const ChunkArgs& a, AccountShared& s, int block, int blocks) {
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
-  if (ctl->error) return;
+  if (threadIdx.x == 0) s.sum[0] = s.sum[1] = 0;
+  if (!block_goes_on((int)threadIdx.x, &ctl->error, &s.go, account_sync<THREADS>)) return;
   const long long e0 = a.row_ptr[a.src_begin], ne = a.row_ptr[a.src_end] - e0, total = ne + (a.src_end - a.src_begin);
   const long long stride = (long long)blocks * THREADS;
-  if (threadIdx.x == 0) s.sum[0] = s.sum[1] = 0;
-  account_sync<THREADS>();
   unsigned msgs = 0, hub = 0;
   int bad = 0, par = 0;
   for (long long base = (long long)block * THREADS; base < total; base += stride, par ^= 1) {
@@ -115,8 +115,8 @@ __device__ __forceinline__ void account_block(const AccountWork& work, AccountSh
   constexpr int WARPS = THREADS / 32;
   DevCtl* ctl = a.ctl;
   ChunkCtl* pc = a.pc;
-  if (ctl->error) return;
   if (threadIdx.x < C_COUNT) s.sum[threadIdx.x] = 0;
+  if (!block_goes_on((int)threadIdx.x, &ctl->error, &s.go, account_sync<THREADS>)) return;
   if (block == 0 && threadIdx.x == 0) pc->grad_base = a.dense_half >= 0 ? a.grad_off : ctl->grad_count;
   const long long n = LISTED ? (long long)pc->touched_count : n_items;
   const long long stride = (long long)blocks * THREADS * ITEMS;
@@ -234,7 +234,7 @@ __device__ __forceinline__ void account_totals(const ChunkArgs& a, DevCtl* ctl, 
 // totals, the free-slot count and the count of waiting rows, and the counters of the next chunk (the other set; its last reader, the chunk
 // before this one, is through) are cleared.  By the accounting's last block to finish it was 1.7 us on the way of every push.
 __device__ __forceinline__ void account_close(const ChunkArgs& a, DevCtl* ctl, ChunkCtl* pc) {
-  if (!ctl->error) {
+  if (__shfl_sync(FULL, ctl->error, 0) == 0) {   // (one answer for the warp, which meets again below)
     ChunkCtl* next = pc == &ctl->pc[0] ? &ctl->pc[1] : &ctl->pc[0];
     for (int i = rl(); i < (int)(offsetof(ChunkCtl, sel_k) / 4); i += 32) reinterpret_cast<int32_t*>(next)[i] = 0;
     __syncwarp();
