@@ -189,7 +189,8 @@ int taurus_graph_init(taurus_ctx** out, const taurus_graph* graph, const taurus_
 /*
  * Starts layer `layer` (0-based): every vertex NOT_STARTED, pending count |M(v)| + 1 (the +1 is the
  * vertex's own self message, delivered with its chunk), pool empty; builds the layer's edge mask when
- * fanout[layer] > 0 (Sect. 3.9).  Blocking (synchronises `cuda_stream`, then enqueues its own work on it).  A layer may be begun again.
+ * fanout[layer] > 0 (Sect. 3.9).  Blocking: synchronises `cuda_stream` and, where that is another
+ * one, the stream of the calls before, then enqueues its own work on `cuda_stream`.  A layer may be begun again.
  */
 int taurus_layer_begin(taurus_ctx* ctx, int32_t layer, void* cuda_stream);
 

@@ -481,11 +481,11 @@ extern "C" int taurus_layer_begin(taurus_ctx* c, int32_t layer, void* cuda_strea
   if (!c || layer < 0 || layer >= c->L) return TAURUS_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   CU(cudaSetDevice(c->device));
-  // Everything before the layer is over when this call returns; its own kernels are only enqueued.  A layer that ended has left
-  // nothing behind on the library's streams.
+  // Everything before the layer is over when this call returns, on its stream and on the one before's (where the caller may have gone on
+  // with that layer's rows); its own kernels are only enqueued.  A layer that ended has left nothing behind on the library's streams.
   CU(cudaStreamSynchronize(st));
+  if (c->last_stream != st) CU(cudaStreamSynchronize(c->last_stream));
   if (!c->quiet) {
-    if (c->last_stream != st) CU(cudaStreamSynchronize(c->last_stream));
     CU(cudaStreamSynchronize(c->copy_stream));
     CU(cudaStreamSynchronize(c->out_stream));
     if (c->xfer_stream) CU(cudaStreamSynchronize(c->xfer_stream));
