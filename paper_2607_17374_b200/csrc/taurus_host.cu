@@ -805,6 +805,7 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
     if (!halves && !direct_dense) c->ub_since_drain += bound;
     return rc;
   }
+  const long long launches = c->launches;
   // S2: projection (GAT: already done in pass 1; rows narrower than their padded width are repacked).
   // Aggregate-first layers push the (scaled, padded) input rows instead and transform the finished rows in S7.
   bool x_in_use = false;
@@ -845,10 +846,11 @@ static int push_enqueue(taurus_ctx* c, int64_t src_begin, int64_t src_end, const
   if (timing) cudaEventRecord(pev[2], st);
   // S3, S4
   *applied = true;
-  c->early = !pev;
+  if (c->launches != launches) c->early = !pev;   // else rows used in place: what stands in front of the first launch may be a wait for an event
   const bool grouped = c->d_gdst != nullptr && src_begin % c->chunk_sources == 0 &&
                        src_end == std::min<long long>(c->V, src_begin + c->chunk_sources);
   if (grouped) launch_classify_grouped(c, a, st); else launch_classify(c, a, st);
+  c->early = !pev;
   { int rc = launch_make_room(c, a, st, timing ? pev[3] : nullptr); if (rc) return rc; }   // pev[3]: victims chosen and placed, rows not yet moved
   // The chunk before this one: its rows have been crossing the host link since its slots were handed out.  Its
   // finalise runs now, before this chunk takes over the slots it released.
