@@ -77,13 +77,11 @@ static_assert(TAURUS_ACCOUNT_THREADS <= 8 * 32, "eight warps (AccountShared::cnt
 
 __global__ void __launch_bounds__(TAURUS_ACCOUNT_THREADS, 8) account_edges_kernel(const __grid_constant__ AccountWork w) {
   __shared__ AccountShared s;
-  early_start();
   account_edges_block<TAURUS_ACCOUNT_THREADS>(w.a, s, (int)blockIdx.x, (int)gridDim.x);
 }
 template <bool LISTED>
 __global__ void __launch_bounds__(TAURUS_ACCOUNT_THREADS, LISTED ? 6 : 5) account_kernel(const __grid_constant__ AccountWork w) {
   __shared__ AccountShared s;
-  if (LISTED) early_start();   // (behind the edges)
   account_block<LISTED, TAURUS_ACCOUNT_THREADS>(w, s, (int)blockIdx.x, (int)gridDim.x);
 }
 
@@ -971,7 +969,9 @@ void launch_account(taurus_ctx* c, const ChunkArgs& a, long long cell, cudaStrea
   }
   account_edges_kernel<<<c->sm_count * 8, TAURUS_ACCOUNT_THREADS, 0, st>>>(w);
   const int grid = (int)std::max<long long>(1, std::min<long long>((a.touched_capacity + 256 * ITEMS - 1) / (256 * ITEMS), (long long)c->sm_count * 6));
-  launch_early(true, account_kernel<true>, grid, TAURUS_ACCOUNT_THREADS, 0, st, w);
+  // Not early: its waiting blocks would take the room that the CTAs of the projection beside it come into.  ms a pass of 500 k vertices, 6 M edges, 40 000
+  // sources a push, 128 -> 128: early 1.50, behind the edges 1.28; fanout 5 1.30 and 1.02; 120 k vertices, FFMA kernel, 1.74 and 1.71.
+  account_kernel<true><<<grid, TAURUS_ACCOUNT_THREADS, 0, st>>>(w);
   c->launches += 2;
 }
 
