@@ -46,7 +46,7 @@ METRIC = "edges/sec per GNN layer (GTEPS)"
 # csrc/kernels_resident.cu, first 16 hex digits); when the source has changed since the capture the bench prints
 # traffic = null instead of a stale number.
 GATHER_TRAFFIC_OVER_REQUESTED = 0.680
-GATHER_CAPTURE_SOURCE = "96acf553eceeb0f6"
+GATHER_CAPTURE_SOURCE = "a2825bd519cf516a"
 
 
 def source_digest(name: str) -> str:
